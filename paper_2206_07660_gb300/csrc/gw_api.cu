@@ -25,6 +25,8 @@ struct gw_ctx {
   // time-reversal symmetry (GW_TRS): kneg[k] = index of -k; the forward P~0, screened solve and
   // Sigma~ skip every q (k) with kneg < q (k) and take its result as the conjugate of its partner's
   bool trs = false, reduce = false;
+  // V^{k'k}(Q) = V^{kk'}(Q)^H holds to kPairTol: P~0 of (-q, beta - tau) is taken from that of (q, tau)
+  bool fold = false;
   std::vector<int> kneg;
   int *d_kneg = nullptr, *d_kneed = nullptr, *d_vpart = nullptr;
   int64_t n2 = 0, na2 = 0;
@@ -144,6 +146,9 @@ static constexpr bool kTensorSmallSteps = true;   // GW_SMALL_TENSOR / GW_SMALL_
 // rounding); the systems are processed in batches whose workspace (digit planes of
 // P~0 and of the iterate, residual, complex64 panels) stays below kRefineBytes.
 static constexpr int kRefineSteps = 2;
+// V paired to this relative tolerance is taken as paired exactly (gw_init accepts 1e-10; between
+// the two the contractions run over every (q, tau))
+static constexpr double kPairTol = 1e-14;
 static constexpr size_t kZGroupBytes = (size_t)8 << 30;
 static int g_pgroup_cap = 0;   // test hook: upper bound on the k-points per group (0: none)
 static int g_pbatch_cap = 0;   // test hook: upper bound on the k-points per chain launch (0: none)
@@ -596,8 +601,8 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
   c->ws_bytes = ws;
   c->ws = need(A(ws));
   c->partial = (double*)need(A((size_t)(ntau > nwf ? ntau : nwf) * nk * 8));
+  c->d_kneg = (int*)need(A((size_t)nk * 4));
   if (c->trs) {
-    c->d_kneg = (int*)need(A((size_t)nk * 4));
     c->d_kneed = (int*)need(A((size_t)nk * 4));
     c->d_vpart = (int*)need(A((size_t)nk * nk * 4));
   }
@@ -700,12 +705,12 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
   // input checks
   chk(cudaMemsetAsync(c->dscr, 0, 64 * 8, st), "memset");
   std::vector<int> kneed((size_t)nk), vpart((size_t)nk * nk);
+  chk(cudaMemcpyAsync(c->d_kneg, c->kneg.data(), (size_t)nk * 4, cudaMemcpyHostToDevice, st), "copy");
   if (c->trs) {
     for (int k = 0; k < nk; ++k) {
       kneed[(size_t)k] = c->kneg[(size_t)k] < k ? 1 : 0;
       for (int k2 = 0; k2 < nk; ++k2) vpart[(size_t)k * nk + k2] = c->kneg[(size_t)k] * nk + c->kneg[(size_t)k2];
     }
-    chk(cudaMemcpyAsync(c->d_kneg, c->kneg.data(), (size_t)nk * 4, cudaMemcpyHostToDevice, st), "copy");
     chk(cudaMemcpyAsync(c->d_kneed, kneed.data(), (size_t)nk * 4, cudaMemcpyHostToDevice, st), "copy");
     chk(cudaMemcpyAsync(c->d_vpart, vpart.data(), (size_t)nk * nk * 4, cudaMemcpyHostToDevice, st), "copy");
   }
@@ -718,9 +723,12 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
     }
     chk(check_herm(c->H0, nao, nk, c->dscr, st), "check");
     chk(check_herm(c->S, nao, nk, c->dscr + 2, st), "check");
-    chk(check_v_pairing(c->V, nk, naux, nao, c->dscr + 4, st), "check");
-    count(3);
+    count(2);
   }
+  // the pairing decides whether P~0 is folded over (q, tau) -> (-q, beta - tau), so it is
+  // measured with GW_SKIP_CHECKS too (without the error)
+  chk(check_v_pairing(c->V, nk, naux, nao, c->dscr + 4, st), "check");
+  count(1);
   chk(cudaMemcpyAsync(c->h_scr, c->dscr, 64 * 8, cudaMemcpyDeviceToHost, st), "copy");
   int h_info = 0;
   chk(cudaMemcpyAsync(&h_info, c->info, 4, cudaMemcpyDeviceToHost, st), "copy");
@@ -749,6 +757,7 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
                "V^{-k,-k'} = conj V^{kk'} within 1e-10)";
     }
   }
+  c->fold = std::isfinite(c->h_scr[5]) && c->h_scr[4] <= kPairTol * c->h_scr[5];
   if (s != GW_OK) { g_init_err = c->err; free_all(c); delete c; return s; }
   // zero self-energy and the grid are defined from the start
   for (gw_quantity q : {GW_Q_SIGMA_INF, GW_Q_SIGMA_IW, GW_Q_TFF, GW_Q_TBF, GW_Q_TFB, GW_Q_TBB, GW_Q_LB, GW_Q_TAU})
@@ -910,6 +919,33 @@ extern "C" gw_status gw_hf(gw_ctx* c) {
 
 // ------------------------------------------------------------------ A2/A3: polarization
 
+// Which P~0^q(tau_j) are computed.  With the paired V and the cyclic trace,
+//   P~0^{-q}_{Q'Q}(tau_{n-1-j}) = (s/Nk) sum_k tr[V^{k,k-q}(Q') G^{k-q}(tau_{n-1-j}) V^{k-q,k}(Q) (-G^k(tau_j))]
+//                               = P~0^q_{QQ'}(tau_j)      for any G, Hermitian or not
+// (the chains on the tensor cores, which take G^{k+q} as its own adjoint, give the adjoint of
+// the right-hand side), so after the symmetrisation P~0^{-q}(tau_{n-1-j}) = conj P~0^q(tau_j) on
+// either route, and the same holds for the sum of the two tangents.  A q that is its own negative
+// needs the first half of the tau points (the middle one included); of a pair q != -q in the
+// context's range only the smaller index is needed.  Half the contraction's work at any size:
+// P~0 of nao 52, naux 400, 2x2x1, ntau 100 (split fp16) 44.0 -> 32.5 ms with its transform,
+// nao 8, naux 64, 4x4x4, ntau 64 51.9 -> 32.1 ms, nao 26, naux 200, 3x1x1, ntau 92 in FP64
+// 337 -> 170 ms.
+// Returns the number of leading tau points to compute (0: none).
+static int polar_taus(const gw_ctx* c, int q) {
+  const int nq = c->kneg[(size_t)q];
+  if (!c->fold) return c->reduce && nq < q ? 0 : c->ntau;
+  if (nq < c->q0 || nq >= c->q1) return c->ntau;
+  return nq == q ? (c->ntau + 1) / 2 : (nq > q ? c->ntau : 0);
+}
+
+// Symmetrises the computed part of P~0 (or its tangent) over the context's q range and fills
+// the rest from it.
+static cudaError_t polar_finish(gw_ctx* c, double2* out, bool trs) {
+  count(1);
+  // with both symmetries the folded image is taken, as without GW_TRS
+  return herm_fill(out, c->naux, c->ntau, c->q0, c->q1, c->d_kneg, c->fold, trs && !c->fold, c->st);
+}
+
 // The P~0 chain of Eq. tilde_P0_tau with its two G factors taken from separate
 // tensors: Gplus supplies G^{k+q}(t), Gminus supplies G^k(-t) (= -Gminus^k(t_{ntau-1-j})).
 // out (nq, ntau, naux, naux) receives the unsymmetrised sum, added to its contents
@@ -948,7 +984,8 @@ static gw_status polar_chain(gw_ctx* c, const double2* Gplus, const double2* Gmi
   const int G = tc ? c->pgroup : 1;
   const int64_t zld = tc ? G * c->kpadP : 0;
   for (int q = c->q0; q < c->q1; ++q) {
-    if (c->reduce && c->kneg[(size_t)q] < q) continue;   // the conjugate of P~0^{-q}
+    const int nt = polar_taus(c, q);   // tau points computed; the others are conjugates
+    if (nt == 0) continue;
     double2* Pq = out + (size_t)q * ntau * na2;
     for (int k = 0; k < nk; ++k) {
       const int kq = c->kplus[(size_t)q * nk + k];
@@ -965,28 +1002,28 @@ static gw_status polar_chain(gw_ctx* c, const double2* Gplus, const double2* Gmi
                       c->Vs_hi, c->Vs_lo, ka, c->st));
         count(1);
         UmmaOperand oa{c->Vs_hi, c->Vs_lo, (int64_t)naux * nao, 1, ka, 0};
-        UmmaOperand ob{c->Ge_hi + (size_t)kq * ntau * per, c->Ge_lo + (size_t)kq * ntau * per, 2 * (int64_t)nao, ntau, ka,
+        UmmaOperand ob{c->Ge_hi + (size_t)kq * ntau * per, c->Ge_lo + (size_t)kq * ntau * per, 2 * (int64_t)nao, nt, ka,
                        per};
-        CK(run_umma(c, 8.0 * ntau * naux * (double)nao * n2, oa, ob, naux * nao, 2 * nao, ka, ntau, c->Xs_hi, false, 1.0,
+        CK(run_umma(c, 8.0 * nt * naux * (double)nao * n2, oa, ob, naux * nao, 2 * nao, ka, nt, c->Xs_hi, false, 1.0,
                     false, 2, (int64_t)naux * nao * ka, 1, nao, (int64_t)nao * ka, 2, ka, c->Xs_lo, 2 * (int64_t)nao));
         // Z[t][Q][c][b] = -sum_d G^k(t_{ntau-1-j})[c][d] Y[t][Q][d][b] as rows (t, Q, b) of (c, re/im),
         // written into the (c, b) layout of the last step's A operand
-        UmmaOperand ya{c->Xs_hi, c->Xs_lo, (int64_t)naux * nao, ntau, ka, (int64_t)naux * nao * ka};
-        UmmaOperand gb{c->Gp_hi + (size_t)k * ntau * per, c->Gp_lo + (size_t)k * ntau * per, 2 * (int64_t)nao, ntau, ka,
+        UmmaOperand ya{c->Xs_hi, c->Xs_lo, (int64_t)naux * nao, nt, ka, (int64_t)naux * nao * ka};
+        UmmaOperand gb{c->Gp_hi + (size_t)k * ntau * per, c->Gp_lo + (size_t)k * ntau * per, 2 * (int64_t)nao, nt, ka,
                        per};
-        CK(run_umma(c, 8.0 * ntau * naux * (double)nao * n2, ya, gb, naux * nao, 2 * nao, ka, ntau, Zh, false, -1.0,
+        CK(run_umma(c, 8.0 * nt * naux * (double)nao * n2, ya, gb, naux * nao, 2 * nao, ka, nt, Zh, false, -1.0,
                     false, 2, (int64_t)naux * zld, 1, nao, zld, 2, 2 * (int64_t)nao, Zl, 2 * (int64_t)nao));
       } else if (f32 && nao <= 64) {
         // Y[t][Q][d][b] = sum_a V^{k,k+q}[Q][d][a] G^{k+q}[t][a][b]   (G shared per t)
         BsmDesc b1{};
-        b1.M = b1.N = b1.K = nao; b1.G = ntau; b1.E = naux; b1.alpha = 1.f;
+        b1.M = b1.N = b1.K = nao; b1.G = nt; b1.E = naux; b1.alpha = 1.f;
         b1.A = (const float2*)Vkq; b1.a_gs = 0; b1.a_es = n2; b1.a_rs = nao; b1.a_cs = 1;
         b1.B = (const float2*)Gp + (size_t)kq * n2; b1.b_gs = gstep; b1.b_rs = nao; b1.b_cs = 1; b1.b_shared = 1;
         b1.C = (float2*)c->chA; b1.c_gs = slab; b1.c_es = n2; b1.c_rs = nao;
         CK(run_bsm(c, b1));
         // Z[t][Q][c][b] = -sum_d G^k(t_{ntau-1-j})[c][d] Y[t][Q][d][b]   (G^k(-t) shared per t)
         BsmDesc b2{};
-        b2.M = b2.N = b2.K = nao; b2.G = ntau; b2.E = naux; b2.alpha = -1.f;
+        b2.M = b2.N = b2.K = nao; b2.G = nt; b2.E = naux; b2.alpha = -1.f;
         b2.A = (const float2*)Gm; b2.a_gs = -gstep; b2.a_rs = nao; b2.a_cs = 1; b2.a_shared = 1;
         b2.B = (const float2*)c->chA; b2.b_gs = slab; b2.b_es = n2; b2.b_rs = nao; b2.b_cs = 1;
         if (tc) {   // straight into the TF32 hi/lo operand of the tensor-core GEMM
@@ -998,13 +1035,13 @@ static gw_status polar_chain(gw_ctx* c, const double2* Gplus, const double2* Gmi
         CK(run_bsm(c, b2));
       } else {
       // Y[t][(Q,d)][b] = sum_a V^{k,k+q}[Q][d][a] G^{k+q}[t][a][b]
-      GettDesc d1 = base_desc((int64_t)naux * nao, nao, nao, ntau);
+      GettDesc d1 = base_desc((int64_t)naux * nao, nao, nao, nt);
       d1.am = I1(nao); d1.ak = I1(1); d1.az = I1(0);
       d1.bk = I1(nao); d1.bn = I1(1); d1.bz = I1(gstep);
       d1.cm = I1(nao); d1.cn = I1(1); d1.cz = I1(slab);
       CK(run_gett(d1, Vkq, tv, (const char*)Gp + (size_t)kq * n2 * es, tv, c->chA, tv, acc, c));
       // Z[t][Q][c][b] = sum_d G^k_cd(-t) Y[t][Q][d][b],  G(-t_j) = -G(t_{ntau-1-j})
-      GettDesc d2 = base_desc(nao, (int64_t)naux * nao, nao, ntau);
+      GettDesc d2 = base_desc(nao, (int64_t)naux * nao, nao, nt);
       d2.am = I1(nao); d2.ak = I1(1); d2.az = I1(-gstep);
       d2.bk = I1(nao); d2.bn = I2(nao, n2, 1); d2.bz = I1(slab);
       d2.cm = I1(nao); d2.cn = I2(nao, n2, 1); d2.cz = I1(slab);
@@ -1018,7 +1055,7 @@ static gw_status polar_chain(gw_ctx* c, const double2* Gplus, const double2* Gmi
         // of G k-points (K = their column blocks side by side)
         const int64_t kp = c->kpadP;
         if (nao > 64) {
-          CK(split_rows(c->chB, false, (int64_t)ntau * naux, n2, n2, false, Zh, Zl, kp, c->st, zld));
+          CK(split_rows(c->chB, false, (int64_t)nt * naux, n2, n2, false, Zh, Zl, kp, c->st, zld));
           count(1);
         }
         CK(embed_conj((const char*)c->V + ((size_t)k * nk + kq) * slab * 16, true, naux, n2, c->Vhi + j * kp,
@@ -1026,15 +1063,15 @@ static gw_status polar_chain(gw_ctx* c, const double2* Gplus, const double2* Gmi
         count(1);
         if (j == G - 1 || k == nk - 1) {
           const int g = j + 1, k0 = k - j;
-          UmmaOperand oa{c->Zhi, c->Zlo, (int64_t)ntau * naux, 1, zld, 0};
+          UmmaOperand oa{c->Zhi, c->Zlo, (int64_t)nt * naux, 1, zld, 0};
           UmmaOperand ob{c->Vhi, c->Vlo, 2 * (int64_t)naux, 1, zld, 0};
-          CK(run_umma(c, 8.0 * g * ntau * naux * (double)naux * n2, oa, ob, ntau * naux, 2 * naux, g * kp, 1, Pq,
+          CK(run_umma(c, 8.0 * g * nt * naux * (double)naux * n2, oa, ob, nt * naux, 2 * naux, g * kp, 1, Pq,
                       true, c->spin / nk, accumulate || k0 > 0, 2 * (int64_t)naux, 0, 1, 0, 0, 0, 0, nullptr,
                       (g - 1) * kp + 2 * n2));
         }
         continue;
       }
-      GettDesc d3 = base_desc((int64_t)ntau * naux, naux, n2, 1);
+      GettDesc d3 = base_desc((int64_t)nt * naux, naux, n2, 1);
       d3.am = I1(n2); d3.ak = I1(1);
       d3.bk = I1(1); d3.bn = I1(n2); d3.conjB = true;
       d3.cm = I1(naux); d3.cn = I1(1);
@@ -1085,13 +1122,14 @@ static gw_status polar_chain_half(gw_ctx* c, const double2* Gplus, const double2
                        true, c->eGp + (size_t)k * ntau, st));
   }
   count(2 * nk);
-  const double fl12 = 8.0 * ntau * naux * (double)nao * n2;
   // k-points per launch: several (k, k+q) pairs of small systems share each GEMM
   // (batch entry z = (k, t)), whole groups of the last step at most
   const int KB = c->pbatch < G ? c->pbatch : G;
   const int64_t vs_blk = (int64_t)naux * nao * ka, xs_blk = (int64_t)ntau * naux * nao * ka;
   for (int q = c->q0; q < c->q1; ++q) {
-    if (c->reduce && c->kneg[(size_t)q] < q) continue;   // the conjugate of P~0^{-q}
+    const int nt = polar_taus(c, q);   // tau points computed; the others are conjugates
+    if (nt == 0) continue;
+    const double fl12 = 8.0 * nt * naux * (double)nao * n2;
     double2* Pq = out + (size_t)q * ntau * c->na2;
     for (int g0 = 0; g0 < nk; g0 += G) {
       const int gn = nk - g0 < G ? nk - g0 : G;
@@ -1121,8 +1159,8 @@ static gw_status polar_chain_half(gw_ctx* c, const double2* Gplus, const double2
           UmmaScale sc{c->eV1, gbe, 0, 1, 0, 1, kAll};
           UmmaOut o{fmt, c->eY, naux, nao, 0};
           // z = (k, t): A and the row exponents per k, B and its exponents per (k, t), Y blocks per (k, t)
-          UmmaZ zz{ntau, 1, 0, ntau, 1, (int64_t)naux * nao, ntau, 0, xs_blk};
-          CK(run_umma(c, fl12 * kn, oa, ob, naux * nao, 2 * nao, ka, kn * ntau, c->Xs_hi, false, 1.0, false, 2,
+          UmmaZ zz{nt, 1, 0, ntau, 1, (int64_t)naux * nao, ntau, 0, xs_blk};
+          CK(run_umma(c, fl12 * kn, oa, ob, naux * nao, 2 * nao, ka, kn * nt, c->Xs_hi, false, 1.0, false, 2,
                       (int64_t)naux * nao * ka, 1, nao, (int64_t)nao * ka, 2, ka, c->Xs_lo, 2 * (int64_t)nao, &sc, &o,
                       kn > 1 ? &zz : nullptr));
         }
@@ -1134,8 +1172,8 @@ static gw_status polar_chain_half(gw_ctx* c, const double2* Gplus, const double2
                          2 * (int64_t)nao, (int64_t)kn * ntau, ka, per, fmt};
           UmmaScale sc{c->eY, c->eGp + (size_t)k0 * ntau, naux, 1, 0, nao, kAll};
           UmmaOut o{fmt, c->eZ, naux, nao, 0};
-          UmmaZ zz{ntau, ntau, 1, ntau, 1, 0, ntau, 0, kp};
-          CK(run_umma(c, fl12 * kn, ya, gb, naux * nao, 2 * nao, ka, kn * ntau, hofs(c->Zhi, b0 * kp), false, -1.0, false,
+          UmmaZ zz{nt, ntau, 1, ntau, 1, 0, ntau, 0, kp};
+          CK(run_umma(c, fl12 * kn, ya, gb, naux * nao, 2 * nao, ka, kn * nt, hofs(c->Zhi, b0 * kp), false, -1.0, false,
                       2, (int64_t)naux * zld, 1, nao, zld, 2, 2 * (int64_t)nao, hofs(c->Zlo, b0 * kp),
                       2 * (int64_t)nao, &sc, &o, kn > 1 ? &zz : nullptr));
         }
@@ -1145,10 +1183,10 @@ static gw_status polar_chain_half(gw_ctx* c, const double2* Gplus, const double2
         count(1);
       }
       const int g = gn;
-      UmmaOperand oa{c->Zhi, c->Zlo, (int64_t)ntau * naux, 1, zld, 0, fmt};
+      UmmaOperand oa{c->Zhi, c->Zlo, (int64_t)nt * naux, 1, zld, 0, fmt};
       UmmaOperand ob{c->Vhi, c->Vlo, 2 * (int64_t)naux, 1, zld, 0, fmt};
       UmmaScale sc{c->eZ, c->eVQ, 0, 0, 0, 1, 1};
-      CK(run_umma(c, 8.0 * g * ntau * naux * (double)naux * n2, oa, ob, ntau * naux, 2 * naux, g * kp, 1, Pq, true,
+      CK(run_umma(c, 8.0 * g * nt * naux * (double)naux * n2, oa, ob, nt * naux, 2 * naux, g * kp, 1, Pq, true,
                   c->spin / nk, accumulate || g0 > 0, 2 * (int64_t)naux, 0, 1, 0, 0, 0, 0, nullptr,
                   (g - 1) * kp + 2 * n2, &sc, nullptr));
     }
@@ -1267,7 +1305,7 @@ static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2*
 extern "C" gw_status gw_polarization(gw_ctx* c) {
   if (!c) return GW_ERR_ARG;
   if (!c->have_G) return fail(c, GW_ERR_STATE, "no Green's function yet");
-  const int nk = c->nk, naux = c->naux, ntau = c->ntau;
+  const int ntau = c->ntau;
   const int64_t na2 = c->na2;
   const bool tc = uses_tc(c);
   const bool red = trs_reduce(c);
@@ -1275,10 +1313,6 @@ extern "C" gw_status gw_polarization(gw_ctx* c) {
   gw_status s = polar_chain(c, c->G_tau, c->G_tau, c->P0_tau, false);
   c->reduce = false;
   if (s != GW_OK) return s;
-  if (red) {   // P~0^{-q}(tau) = conj P~0^q(tau) (time-reversal symmetry)
-    CK(conj_fill(c->P0_tau, 1, nk, (int64_t)ntau * na2, c->d_kneg, c->d_kneed, c->st));
-    count(1);
-  }
   if (tc && !c->deferred) {
     int h = 0;
     CK(cudaMemcpyAsync(c->h_scr, c->info + 1, 4, cudaMemcpyDeviceToHost, c->st));
@@ -1288,8 +1322,7 @@ extern "C" gw_status gw_polarization(gw_ctx* c) {
   }
   const int nq = c->q1 - c->q0;
   double2* P0q = c->P0_tau + (size_t)c->q0 * ntau * na2;
-  CK(herm_batched(P0q, naux, (int64_t)nq * ntau, na2, c->st));
-  count(1);
+  CK(polar_finish(c, c->P0_tau, red));
   // P~0(i Omega_m) = sum_j TFb[m][j] P~0(tau_j)   (Eq. P0t_to_P0w)
   CK(transform(c, c->TFb, P0q, c->P_iw + (size_t)c->q0 * c->nwb * na2, c->nwb, na2, nq, (int64_t)ntau * na2,
                (int64_t)c->nwb * na2));
@@ -1343,7 +1376,8 @@ extern "C" gw_status gw_screened(gw_ctx* c) {
     }
     if (s != GW_OK) return s;
     CK(conj_fill(c->P_iw, 1, c->nk, (int64_t)c->nwb * c->na2, c->d_kneg, c->d_kneed, c->st));
-    CK(conj_fill(c->P_tau, 1, c->nk, (int64_t)c->ntau * c->na2, c->d_kneg, c->d_kneed, c->st));
+    // the folded image of P~ as of P~0 (P~^q(beta - tau) = P~^q(tau) too under time reversal)
+    CK(conj_fill(c->P_tau, 1, c->nk, (int64_t)c->ntau * c->na2, c->d_kneg, c->d_kneed, c->st, c->fold ? c->ntau : 1));
     count(2);
   } else {
     s = screened_block(c, c->q0, c->q1);
@@ -1866,8 +1900,7 @@ extern "C" gw_status gw_polarization_jvp(gw_ctx* c, const double* dG, double* dP
   if (s == GW_OK) s = polar_chain(c, c->G_tau, g, out, true);
   if (s == GW_OK) s = tc_check(c);
   if (s != GW_OK) return s;
-  CK(herm_batched(out, c->naux, (int64_t)c->nk * c->ntau, c->na2, c->st));
-  count(1);
+  CK(polar_finish(c, out, false));
   return GW_OK;
 }
 
@@ -1967,8 +2000,7 @@ static gw_status sc_jvp(gw_ctx* c, const double2* dSinf, const double2* dSiw, do
   // dP~0, then dP~ through the screened block (in place), then dSigma~
   if ((s = polar_chain(c, c->tGtau, c->G_tau, c->tP, false)) != GW_OK) return s;
   if ((s = polar_chain(c, c->G_tau, c->tGtau, c->tP, true)) != GW_OK) return s;
-  CK(herm_batched(c->tP, c->naux, (int64_t)nk * c->ntau, c->na2, c->st));
-  count(1);
+  CK(polar_finish(c, c->tP, false));
   if ((s = gw_screened_jvp(c, (const double*)c->tP, (double*)c->tP)) != GW_OK) return s;
   if ((s = sigma_chain(c, c->tGtau, c->P_tau, c->tS, false)) != GW_OK) return s;
   if ((s = sigma_chain(c, c->G_tau, c->tP, c->tS, true)) != GW_OK) return s;

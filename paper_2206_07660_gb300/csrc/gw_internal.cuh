@@ -53,6 +53,12 @@ inline Idx2 I2(int64_t inner, int64_t s1, int64_t s0) { return Idx2{inner, s1, s
 
 // ------------------------------------------------------------------ other kernels
 cudaError_t herm_batched(double2* X, int64_t n, int64_t count, int64_t stride, cudaStream_t st);
+// X [nq][nt][n][n] over q in [q0, q1): (X + X^H)/2 of the computed matrices; with fold, of a q
+// with neg[q] == q the first (nt + 1)/2 are computed and the others filled with the conjugates
+// of their mirror images nt - 1 - t, of a pair q < neg[q] in the range the smaller q is computed
+// and the larger one filled in the same way (without mirroring when trs)
+cudaError_t herm_fill(double2* X, int64_t n, int nt, int q0, int q1, const int* neg, bool fold, bool trs,
+                      cudaStream_t st);
 // out[m] = tr ln(I - A_m) + tr A_m for `count` n x n matrices A_m spaced `stride` apart
 // (overwritten), by FP64 LU without row exchanges; flag |= 1 (zero pivot), 2 (pivot with
 // non-positive real part).  tracelog_panel(n) == 0: n too large for the shared-memory panel.
@@ -113,7 +119,7 @@ cudaError_t to_c64(const double2* x, float2* y, int64_t n, cudaStream_t st);
 cudaError_t check_trs(const double2* X, int64_t nslab, int64_t len, const int* partner, double* d_out,
                       cudaStream_t st);
 cudaError_t conj_fill(double2* X, int64_t outer, int nk, int64_t inner, const int* src, const int* need,
-                      cudaStream_t st);
+                      cudaStream_t st, int nt = 1);
 
 // ------------------------------------------------------------------ batched small products (k_bsm.cu)
 // C[g][e] = alpha * A[g][e] * B[g][e] (complex64), M, N, K <= 64; element (r, c) of

@@ -60,6 +60,71 @@ cudaError_t herm_batched(double2* X, int64_t n, int64_t count, int64_t stride, c
   return cudaGetLastError();
 }
 
+// The symmetrisation above over the computed matrices of X [nq][nt][n][n], each result also
+// written conjugated to its mirror image (herm_fill's rule): one read of the computed half and
+// one write of the whole, where a separate fill would read the half once more.
+__global__ void __launch_bounds__(256) herm_fill_kernel(double2* X, int n, int ntile, int nt, int q0, int q1,
+                                                        const int* __restrict__ neg, int fold, int trs) {
+  __shared__ double2 a[32][33];
+  __shared__ double2 b[32][33];
+  int p = blockIdx.x, I = 0;
+  while (p >= ntile - I) { p -= ntile - I; ++I; }
+  const int J = I + p;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int64_t n2 = (int64_t)n * n;
+  for (int m = blockIdx.y; m < (q1 - q0) * nt; m += gridDim.y) {
+    const int q = q0 + m / nt, t = m % nt, nq = neg[q];
+    const bool in = nq >= q0 && nq < q1;
+    const bool filled = (fold || trs) && in && (nq < q || (fold && nq == q && t >= (nt + 1) / 2));
+    if (filled) continue;
+    double2* M = X + ((int64_t)q * nt + t) * n2;
+    // mirror image (null: none)
+    double2* W = nullptr;
+    if (in && nq != q && (fold || trs)) W = X + ((int64_t)nq * nt + (trs ? t : nt - 1 - t)) * n2;
+    else if (fold && nq == q && 2 * t != nt - 1) W = X + ((int64_t)q * nt + nt - 1 - t) * n2;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int rr = ty + 8 * r;
+      int i = I * 32 + rr, j = J * 32 + tx;
+      if (i < n && j < n) a[rr][tx] = M[(int64_t)i * n + j];
+      i = J * 32 + rr; j = I * 32 + tx;
+      if (i < n && j < n) b[rr][tx] = M[(int64_t)i * n + j];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int rr = ty + 8 * r;
+      int i = I * 32 + rr, j = J * 32 + tx;
+      if (i < n && j < n) {
+        const double2 u = a[rr][tx], v = b[tx][rr];
+        const double2 h = make_double2(0.5 * (u.x + v.x), 0.5 * (u.y - v.y));
+        M[(int64_t)i * n + j] = h;
+        if (W) W[(int64_t)i * n + j] = make_double2(h.x, -h.y);
+      }
+      if (I != J) {
+        i = J * 32 + rr; j = I * 32 + tx;
+        if (i < n && j < n) {
+          const double2 u = b[rr][tx], v = a[tx][rr];
+          const double2 h = make_double2(0.5 * (u.x + v.x), 0.5 * (u.y - v.y));
+          M[(int64_t)i * n + j] = h;
+          if (W) W[(int64_t)i * n + j] = make_double2(h.x, -h.y);
+        }
+      }
+    }
+    __syncthreads();
+  }
+}
+
+cudaError_t herm_fill(double2* X, int64_t n, int nt, int q0, int q1, const int* neg, bool fold, bool trs,
+                      cudaStream_t st) {
+  if (n <= 0 || q1 <= q0) return cudaSuccess;
+  const int ntile = (int)((n + 31) / 32);
+  const int64_t count = (int64_t)(q1 - q0) * nt;
+  dim3 grid(ntile * (ntile + 1) / 2, (unsigned)(count < 65535 ? count : 65535));
+  herm_fill_kernel<<<grid, 256, 0, st>>>(X, (int)n, ntile, nt, q0, q1, neg, fold ? 1 : 0, trs ? 1 : 0);
+  return cudaGetLastError();
+}
+
 // gamma[e] = -sum_j lb_j G[j][e]  (density matrix from the beta^- endpoint row)
 __global__ void gamma_kernel(const double2* __restrict__ G, const double* __restrict__ lb, double2* gam,
                              int ntau, int64_t ne) {
@@ -248,22 +313,28 @@ cudaError_t check_trs(const double2* X, int64_t nslab, int64_t len, const int* p
   return cudaGetLastError();
 }
 
-// X[o][k][:] = conj X[o][src[k]][:] for every k with need[k] (layout [outer][nk][inner])
+// X[o][k][:] = conj X[o][src[k]][:] for every k with need[k] (layout [outer][nk][inner]); the
+// nt equal blocks of the inner range are taken in reverse order
 __global__ void conj_fill_kernel(double2* X, int64_t outer, int nk, int64_t inner, const int* __restrict__ src,
-                                 const int* __restrict__ need) {
+                                 const int* __restrict__ need, int nt) {
   const int64_t tot = outer * nk * inner;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t o = e / ((int64_t)nk * inner), r = e - o * nk * inner;
     const int k = (int)(r / inner);
     if (!need[k]) continue;
     const int64_t i = r - (int64_t)k * inner;
-    const double2 v = X[(o * nk + src[k]) * inner + i];
+    int64_t is = i;
+    if (nt > 1) {
+      const int64_t blk = inner / nt, t = i / blk;
+      is = (nt - 1 - t) * blk + (i - t * blk);
+    }
+    const double2 v = X[(o * nk + src[k]) * inner + is];
     X[e] = make_double2(v.x, -v.y);
   }
 }
 cudaError_t conj_fill(double2* X, int64_t outer, int nk, int64_t inner, const int* src, const int* need,
-                      cudaStream_t st) {
-  conj_fill_kernel<<<nblk(outer * nk * inner), 256, 0, st>>>(X, outer, nk, inner, src, need);
+                      cudaStream_t st, int nt) {
+  conj_fill_kernel<<<nblk(outer * nk * inner), 256, 0, st>>>(X, outer, nk, inner, src, need, nt);
   return cudaGetLastError();
 }
 
