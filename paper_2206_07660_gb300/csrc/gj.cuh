@@ -8,23 +8,54 @@ namespace gwk {
 template <typename T> struct gj_real;
 template <> struct gj_real<double2> { using t = double; };
 template <> struct gj_real<float2> { using t = float; };
+template <> struct gj_real<float> { using t = float; };
+template <typename T> struct gj_cplx { static constexpr bool v = true; };
+template <> struct gj_cplx<float> { static constexpr bool v = false; };
 
 template <typename T>
 static __device__ __forceinline__ T cmul(T a, T b) {
-  T r; r.x = a.x * b.x - a.y * b.y; r.y = a.x * b.y + a.y * b.x; return r;
+  if constexpr (gj_cplx<T>::v) {
+    T r; r.x = a.x * b.x - a.y * b.y; r.y = a.x * b.y + a.y * b.x; return r;
+  } else {
+    return a * b;
+  }
 }
 template <typename T>
 static __device__ __forceinline__ T cinv(T a) {
-  const auto d = a.x * a.x + a.y * a.y;
-  T r; r.x = a.x / d; r.y = -a.y / d; return r;
+  if constexpr (gj_cplx<T>::v) {
+    const auto d = a.x * a.x + a.y * a.y;
+    T r; r.x = a.x / d; r.y = -a.y / d; return r;
+  } else {
+    return (T)1 / a;
+  }
 }
 template <typename T>
 static __device__ __forceinline__ T cval(double re, double im) {
-  T r; r.x = (decltype(r.x))re; r.y = (decltype(r.y))im; return r;
+  if constexpr (gj_cplx<T>::v) {
+    T r; r.x = (decltype(r.x))re; r.y = (decltype(r.y))im; return r;
+  } else {
+    return (T)re;
+  }
+}
+template <typename T>
+static __device__ __forceinline__ typename gj_real<T>::t cnorm2(T v) {
+  if constexpr (gj_cplx<T>::v) return v.x * v.x + v.y * v.y;
+  else return v * v;
+}
+// v - f c
+template <typename T>
+static __device__ __forceinline__ T cfms(T v, T f, T c) {
+  if constexpr (gj_cplx<T>::v) {
+    v.x -= f.x * c.x - f.y * c.y;
+    v.y -= f.x * c.y + f.y * c.x;
+    return v;
+  } else {
+    return v - f * c;
+  }
 }
 
 // A: n x n row-major with leading dimension lda (shared memory), complex T
-// (double2 or float2, arithmetic in T's precision).
+// (double2 or float2; float for a real matrix), arithmetic in T's precision.
 // f: n complex scratch, perm: n ints, red_v/red_i: blockDim.x scratch.
 // Returns (in every thread) 1 if a zero pivot was met, else 0.
 template <typename T>
@@ -39,8 +70,7 @@ static __device__ int gj_invert_smem(T* A, int n, int lda, T* f, int* perm, type
     // pivot: argmax_{r >= c} |A[r][c]| (ties -> smallest r)
     R bv = -1; int bi = c;
     for (int r = c + tid; r < n; r += nt) {
-      T v = A[r * lda + c];
-      R m = v.x * v.x + v.y * v.y;
+      const R m = cnorm2(A[r * lda + c]);
       if (m > bv) { bv = m; bi = r; }
     }
     red_v[tid] = bv; red_i[tid] = bi;
@@ -78,9 +108,7 @@ static __device__ int gj_invert_smem(T* A, int n, int lda, T* f, int* perm, type
       T fr = f[r];
       T cj = A[c * lda + j];
       T v = (j == c) ? cval<T>(0.0, 0.0) : A[r * lda + j];
-      v.x -= fr.x * cj.x - fr.y * cj.y;
-      v.y -= fr.x * cj.y + fr.y * cj.x;
-      A[r * lda + j] = v;
+      A[r * lda + j] = cfms(v, fr, cj);
     }
     __syncthreads();
   }

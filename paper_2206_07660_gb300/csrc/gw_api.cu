@@ -27,6 +27,14 @@ struct gw_ctx {
   bool trs = false, reduce = false;
   // V^{k'k}(Q) = V^{kk'}(Q)^H holds to kPairTol: P~0 of (-q, beta - tau) is taken from that of (q, tau)
   bool fold = false;
+  // folded bosonic block (k_fold.cu): kept frequencies and partners, q-points of the range that are
+  // their own negatives (qR) and the other kept ones (qC), digits of the transforms restricted to
+  // them; P_iw holds a folded P~0 / P_tau a folded P~
+  bool wfold = false, p0sym = false;
+  int nrep = 0, nqR = 0, nqC = 0;
+  int *d_rep = nullptr, *d_repn = nullptr, *d_qR = nullptr, *d_qC = nullptr;
+  void *fRd = nullptr, *fCd = nullptr, *bRd = nullptr, *bCd = nullptr;
+  int *fRe = nullptr, *fCe = nullptr, *bRe = nullptr, *bCe = nullptr;
   std::vector<int> kneg;
   int *d_kneg = nullptr, *d_kneed = nullptr, *d_vpart = nullptr;
   int64_t n2 = 0, na2 = 0;
@@ -149,6 +157,9 @@ static constexpr int kRefineSteps = 2;
 // V paired to this relative tolerance is taken as paired exactly (gw_init accepts 1e-10; between
 // the two the contractions run over every (q, tau))
 static constexpr double kPairTol = 1e-14;
+// deviation of a given P~0(i Omega) from its symmetries, relative to its largest value, that is
+// taken as rounding (a few units in the last place of FP64 sums)
+static constexpr double kFoldTol = 4e-15;
 static constexpr size_t kZGroupBytes = (size_t)8 << 30;
 static int g_pgroup_cap = 0;   // test hook: upper bound on the k-points per group (0: none)
 static int g_pbatch_cap = 0;   // test hook: upper bound on the k-points per chain launch (0: none)
@@ -165,6 +176,7 @@ static int chain_pbatch(int nao, int naux, int nk, int ntau) {
   return kb < 1 ? 1 : (int)kb;
 }
 static constexpr size_t kRefineBytes = (size_t)6 << 30;
+static constexpr size_t kFoldBytes = (size_t)1 << 30;
 
 #define CK(x)                                                                        \
   do {                                                                               \
@@ -351,6 +363,222 @@ static cudaError_t transform(gw_ctx* c, const double2* T, const double2* X, doub
   d.bk = I1(ncol); d.bn = I1(1); d.bz = I1(xstride);
   d.cm = I1(ncol); d.cn = I1(1); d.cz = I1(ystride);
   return run_gett(d, T, Ty::C128, X, Ty::C128, Y, Ty::C128, Ty::C128, c);
+}
+
+// ------------------------------------------------------------------ folded bosonic block
+
+static inline size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
+
+// bytes of one q in the folded transforms (digits of its columns, their exponents, the compact
+// output) and of one q's systems in the folded solve with the workspace of one of them
+static size_t fold_fwd_bytes(const gw_ctx* c, bool real) {
+  const int64_t K = real ? (c->ntau + 1) / 2 : c->ntau, out = real ? (c->nrep + 1) / 2 : c->nrep;
+  return al256(emul_digit_bytes(c->na2, K)) + al256((size_t)c->na2 * 4) + al256((size_t)out * c->na2 * 16);
+}
+static size_t fold_back_bytes(const gw_ctx* c, bool real) {
+  return al256(emul_digit_bytes(c->na2, real ? (c->nrep + 1) / 2 : c->nrep)) + al256((size_t)c->na2 * 4);
+}
+static int64_t fold_order(const gw_ctx* c) { return (c->naux + 1) / 2 * 2; }   // order of the real systems
+static size_t fold_x_bytes(const gw_ctx* c, bool real) {
+  const int64_t ne = fold_order(c);
+  return real ? al256((size_t)c->nrep * ne * ne * 8) : al256((size_t)c->nrep * c->na2 * 16);
+}
+static size_t fold_min_bytes(const gw_ctx* c) {
+  size_t b = fold_fwd_bytes(c, false);
+  const size_t r = fold_x_bytes(c, true) + screened_refine_real_bytes(fold_order(c), 1);
+  const size_t z = fold_x_bytes(c, false) + screened_refine_bytes(c->naux, 1);
+  b = b > r ? b : r;
+  b = b > z ? b : z;
+  return b > fold_back_bytes(c, false) ? b : fold_back_bytes(c, false);
+}
+// The folded block serves a paired V on a grid with its two symmetries, with the refinement
+// workspace (else the transforms and the solve run over every q and frequency).
+static inline bool fold_ready(const gw_ctx* c) { return c->fold && c->wfold && c->irws; }
+static inline FoldView fold_view(const gw_ctx* c) {
+  return FoldView{c->naux, c->nwb, c->nrep, c->q0, c->q1, c->d_rep, c->d_repn, c->d_kneg};
+}
+
+// the kept q of the context's range: qR and qC (polar_taus' rule)
+static cudaError_t fold_lists(gw_ctx* c) {
+  std::vector<int> r, z;
+  for (int q = c->q0; q < c->q1; ++q) {
+    const int nq = c->kneg[(size_t)q];
+    if (nq == q) r.push_back(q);
+    else if (nq < c->q0 || nq >= c->q1 || nq > q) z.push_back(q);
+  }
+  c->nqR = (int)r.size(); c->nqC = (int)z.size();
+  cudaError_t e = cudaSuccess;
+  if (c->nqR) e = cudaMemcpyAsync(c->d_qR, r.data(), r.size() * 4, cudaMemcpyHostToDevice, c->st);
+  if (!e && c->nqC) e = cudaMemcpyAsync(c->d_qC, z.data(), z.size() * 4, cudaMemcpyHostToDevice, c->st);
+  return e ? e : cudaStreamSynchronize(c->st);
+}
+
+// Frequencies to keep and the restricted transforms, from the grid's matrices (host copies):
+//   P(i Omega_m) of a real block: rows w_j (Re T_mj, -Im T_mj) over the first half of tau
+//   (w = 2; 1 for a tau point that is its own image), of the others rows T_mj;
+//   P(tau_j) = herm(sum_m c_jm P(i Omega_m)) over the kept m, c_jm = T'_jm + conj T'_j,-m (T'_jm
+//   alone for a frequency without a partner or Omega = 0).
+// wfold stays false when a matrix misses the symmetries T_m,n-1-j = conj T_mj, T_-m,j = conj T_mj.
+static cudaError_t fold_build(gw_ctx* c, const int32_t* bm) {
+  const int nt = c->ntau, nw = c->nwb, h = (nt + 1) / 2;
+  std::vector<double2> F((size_t)nw * nt), B((size_t)nt * nw);
+  cudaError_t e = cudaMemcpyAsync(F.data(), c->TFb, F.size() * 16, cudaMemcpyDeviceToHost, c->st);
+  if (!e) e = cudaMemcpyAsync(B.data(), c->TBb, B.size() * 16, cudaMemcpyDeviceToHost, c->st);
+  if (!e) e = cudaStreamSynchronize(c->st);
+  if (e) return e;
+  std::vector<int> part((size_t)nw, -1), rep, repn;
+  for (int m = 0; m < nw; ++m)
+    for (int l = 0; l < nw; ++l)
+      if (bm[l] == -bm[m] && bm[m] != 0) part[(size_t)m] = l;
+  double dF = 0, mF = 0, dB = 0, mB = 0;
+  auto dev = [](double2 a, double2 b) { return std::fmax(std::fabs(a.x - b.x), std::fabs(a.y + b.y)); };
+  auto mag = [](double2 a) { return std::fmax(std::fabs(a.x), std::fabs(a.y)); };
+  for (int m = 0; m < nw; ++m)
+    for (int j = 0; j < nt; ++j) {
+      const double2 f = F[(size_t)m * nt + j], b = B[(size_t)j * nw + m];
+      dF = std::fmax(dF, dev(f, F[(size_t)m * nt + nt - 1 - j]));
+      if (part[(size_t)m] >= 0) dF = std::fmax(dF, dev(f, F[(size_t)part[(size_t)m] * nt + j]));
+      dB = std::fmax(dB, dev(b, B[(size_t)(nt - 1 - j) * nw + m]));
+      mF = std::fmax(mF, mag(f));
+      mB = std::fmax(mB, mag(b));
+    }
+  if (!(dF <= 1e-13 * mF && dB <= 1e-11 * mB)) return cudaSuccess;
+  for (int m = 0; m < nw; ++m)
+    if (part[(size_t)m] < 0 || bm[m] > 0) { rep.push_back(m); repn.push_back(part[(size_t)m]); }
+  const int nr = c->nrep = (int)rep.size(), nr2 = (nr + 1) / 2 * 2;
+  std::vector<double> fR((size_t)nr2 * 2 * h, 0.0), bR((size_t)2 * h * nr, 0.0);
+  std::vector<double2> fC((size_t)nr * nt), bC((size_t)nt * nr);
+  for (int r = 0; r < nr; ++r) {
+    const int m = rep[(size_t)r], mn = repn[(size_t)r];
+    for (int j = 0; j < nt; ++j) {
+      const double2 f = F[(size_t)m * nt + j];
+      fC[(size_t)r * nt + j] = f;
+      double2 b = B[(size_t)j * nw + m];
+      if (mn >= 0) { const double2 o = B[(size_t)j * nw + mn]; b.x += o.x; b.y -= o.y; }
+      bC[(size_t)j * nr + r] = b;
+      if (j < h) {
+        const double w = 2 * j == nt - 1 ? 1.0 : 2.0;
+        fR[((size_t)r * h + j) * 2] = w * f.x;
+        fR[((size_t)r * h + j) * 2 + 1] = -w * f.y;
+        bR[(size_t)(2 * j) * nr + r] = b.x;
+        bR[(size_t)(2 * j + 1) * nr + r] = b.y;
+      }
+    }
+  }
+  const size_t fRb = emul_digit_bytes(nr2, h), fCb = emul_digit_bytes(2 * (int64_t)nr, nt);
+  const size_t bRb = emul_digit_bytes(2 * (int64_t)h, (nr + 1) / 2), bCb = emul_digit_bytes(2 * (int64_t)nt, nr);
+  c->d_rep = (int*)dalloc(c, (size_t)nr * 4); c->d_repn = (int*)dalloc(c, (size_t)nr * 4);
+  c->d_qR = (int*)dalloc(c, (size_t)c->nk * 4); c->d_qC = (int*)dalloc(c, (size_t)c->nk * 4);
+  c->fRd = dalloc(c, fRb); c->fCd = dalloc(c, fCb); c->bRd = dalloc(c, bRb); c->bCd = dalloc(c, bCb);
+  c->fRe = (int*)dalloc(c, (size_t)nr2 * 4); c->fCe = (int*)dalloc(c, (size_t)nr * 4);
+  c->bRe = (int*)dalloc(c, (size_t)h * 4); c->bCe = (int*)dalloc(c, (size_t)nt * 4);
+  size_t most = fR.size() * 8;   // staging of one source matrix at a time
+  for (size_t b : {fC.size() * 16, bR.size() * 8, bC.size() * 16}) most = b > most ? b : most;
+  void* stage = dalloc(c, most);
+  if (!c->d_rep || !c->d_repn || !c->d_qR || !c->d_qC || !c->fRd || !c->fCd || !c->bRd || !c->bCd || !c->fRe ||
+      !c->fCe || !c->bRe || !c->bCe || !stage)
+    return cudaSuccess;   // without room the unfolded route is kept
+  cudaStream_t st = c->st;
+  e = cudaMemcpyAsync(c->d_rep, rep.data(), (size_t)nr * 4, cudaMemcpyHostToDevice, st);
+  if (!e) e = cudaMemcpyAsync(c->d_repn, repn.data(), (size_t)nr * 4, cudaMemcpyHostToDevice, st);
+  if (!e) e = cudaMemcpyAsync(stage, fR.data(), fR.size() * 8, cudaMemcpyHostToDevice, st);
+  if (!e) e = emul_split_b_real((const double*)stage, nr2, 2 * h, c->fRd, c->fRe, st);
+  if (!e) e = cudaMemcpyAsync(stage, bR.data(), bR.size() * 8, cudaMemcpyHostToDevice, st);
+  if (!e) e = emul_split_b_real((const double*)stage, 2 * h, nr, c->bRd, c->bRe, st);
+  if (!e) e = cudaMemcpyAsync(stage, fC.data(), fC.size() * 16, cudaMemcpyHostToDevice, st);
+  if (!e) e = emul_split_b((const double2*)stage, nr, nt, nt, c->fCd, c->fCe, st);
+  if (!e) e = cudaMemcpyAsync(stage, bC.data(), bC.size() * 16, cudaMemcpyHostToDevice, st);
+  if (!e) e = emul_split_b((const double2*)stage, nt, nr, nr, c->bCd, c->bCe, st);
+  if (!e) e = cudaStreamSynchronize(st);   // the host matrices go out of scope
+  count(4);
+  dfree(c, stage);
+  if (e) return e;
+  c->wfold = true;
+  return fold_lists(c);
+}
+
+// P~0(i Omega) of the context's range from the folded P~0(tau)
+static cudaError_t fold_forward(gw_ctx* c) {
+  const int64_t na2 = c->na2;
+  const FoldView f = fold_view(c);
+  for (int pass = 0; pass < 2; ++pass) {
+    const bool real = pass == 0;
+    const int nq = real ? c->nqR : c->nqC;
+    const int* list = real ? c->d_qR : c->d_qC;
+    const int64_t K = real ? 2 * ((c->ntau + 1) / 2) : 2 * c->ntau, np = real ? (c->nrep + 1) / 2 : c->nrep;
+    const size_t per = fold_fwd_bytes(c, real);
+    int64_t g = (int64_t)(c->irws_bytes / per);
+    if (g > INT32_MAX / na2) g = INT32_MAX / na2;
+    if (nq > 0 && g < 1) return cudaErrorMemoryAllocation;
+    for (int a = 0; a < nq; a += (int)g) {
+      const int nz = (int)(nq - a < g ? nq - a : g);
+      char* p = (char*)c->irws;
+      void* Ad = p;             p += nz * al256(emul_digit_bytes(na2, K / 2));
+      int* Ae = (int*)p;        p += nz * al256((size_t)na2 * 4);
+      double2* Y = (double2*)p;
+      cudaError_t e = emul_transform_multi(real ? c->fRd : c->fCd, real ? c->fRe : c->fCe, np, c->P0_tau, K, false, na2,
+                                           (int64_t)c->ntau * na2, nz, list + a, nullptr, Y, np * na2, nullptr, Ad, Ae,
+                                           c->info + 1, c->st);
+      if (e) return e;
+      e = real ? fold_expand_pairs(c->P_iw, f, list + a, nz, Y, c->st) : fold_expand_cplx(c->P_iw, f, list + a, nz, Y, c->st);
+      if (e) return e;
+      count(2 + emul_launches_real(K));
+    }
+  }
+  return cudaSuccess;
+}
+
+// P~ = (I - P~0)^{-1} - I of the kept systems, written to every image in P_iw, and P~(tau)
+static cudaError_t fold_screened(gw_ctx* c) {
+  const int64_t na2 = c->na2, ne = fold_order(c);
+  const FoldView f = fold_view(c);
+  cudaError_t e;
+  for (int pass = 0; pass < 2; ++pass) {
+    const bool real = pass == 0;
+    const int nq = real ? c->nqR : c->nqC;
+    const int* list = real ? c->d_qR : c->d_qC;
+    // the systems of g q-points, then the refinement workspace (a quarter at most for the first)
+    const size_t per = fold_x_bytes(c, real);
+    int64_t g = (int64_t)(c->irws_bytes / 4 / per);
+    if (g < 1) g = 1;
+    for (int a = 0; a < nq; a += (int)g) {
+      const int nz = (int)(nq - a < g ? nq - a : g);
+      const int64_t cnt = (int64_t)nz * c->nrep;
+      char* X = (char*)c->irws;
+      char* ws = X + nz * per;
+      const size_t wsb = c->irws_bytes - nz * per;
+      int64_t nl = 0;
+      if (real) {
+        if ((e = fold_pack_real(c->P_iw, f, list + a, nz, (double*)X, (int)ne, c->st))) return e;
+        if ((e = screened_refine_real((double*)X, ne, cnt, ws, wsb, kRefineSteps, c->info + 2, c->info + 1, c->st, &nl)))
+          return e;
+        if ((e = fold_expand_real(c->P_iw, f, list + a, nz, (const double*)X, (int)ne, c->st))) return e;
+      } else {
+        if ((e = fold_pack_cplx(c->P_iw, f, list + a, nz, (double2*)X, c->st))) return e;
+        if ((e = screened_refine((double2*)X, c->naux, cnt, ws, wsb, kRefineSteps, c->info + 2, c->info + 1, c->st, &nl)))
+          return e;
+        if ((e = fold_expand_cplx(c->P_iw, f, list + a, nz, (const double2*)X, c->st))) return e;
+      }
+      count((int)nl + 2);
+    }
+    // P~(tau_j), the first half of tau for the real blocks
+    const int64_t K = real ? c->nrep : 2 * c->nrep, np = real ? (c->ntau + 1) / 2 : c->ntau;
+    const size_t pb = fold_back_bytes(c, real);
+    g = (int64_t)(c->irws_bytes / pb);
+    if (g > INT32_MAX / na2) g = INT32_MAX / na2;
+    for (int a = 0; a < nq; a += (int)g) {
+      const int nz = (int)(nq - a < g ? nq - a : g);
+      char* p = (char*)c->irws;
+      void* Ad = p;             p += nz * al256(emul_digit_bytes(na2, (K + 1) / 2));
+      if ((e = emul_transform_multi(real ? c->bRd : c->bCd, real ? c->bRe : c->bCe, np, c->P_iw, K, real, na2,
+                                    (int64_t)c->nwb * na2, nz, list + a, c->d_rep, c->P_tau, (int64_t)c->ntau * na2,
+                                    list + a, Ad, (int*)p, c->info + 1, c->st)))
+        return e;
+      count(1 + emul_launches_real(K));
+    }
+  }
+  count(1);
+  return herm_fill(c->P_tau, c->naux, c->ntau, c->q0, c->q1, c->d_kneg, true, false, c->st);
 }
 
 static int kidx(const int* m, int a, int b, int cc) {
@@ -758,6 +986,26 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
     }
   }
   c->fold = std::isfinite(c->h_scr[5]) && c->h_scr[4] <= kPairTol * c->h_scr[5];
+  if (s == GW_OK && c->fold && c->irws) {
+    chk(fold_build(c, bm_h), "folded block");
+    if (s == GW_OK && c->wfold) {
+      // a small system's refinement workspace may be too small for a transform's digits: all
+      // kept q of it share a launch where kFoldBytes hold them
+      size_t want = fold_min_bytes(c), all = (size_t)nk * fold_fwd_bytes(c, false);
+      all = all < kFoldBytes ? all : kFoldBytes;
+      want = want > all ? want : all;
+      if (want > c->irws_bytes) {
+        void* p = want <= opt_budget(kRefineBytes) ? dalloc(c, want) : nullptr;
+        if (p) {
+          dfree(c, c->irws);
+          c->irws = p;
+          c->irws_bytes = want;
+        } else if (fold_min_bytes(c) > c->irws_bytes) {
+          c->wfold = false;
+        }
+      }
+    }
+  }
   if (s != GW_OK) { g_init_err = c->err; free_all(c); delete c; return s; }
   // zero self-energy and the grid are defined from the start
   for (gw_quantity q : {GW_Q_SIGMA_INF, GW_Q_SIGMA_IW, GW_Q_TFF, GW_Q_TBF, GW_Q_TFB, GW_Q_TBB, GW_Q_LB, GW_Q_TAU})
@@ -822,7 +1070,7 @@ extern "C" gw_status gw_set(gw_ctx* c, gw_quantity q, const void* src, size_t by
   if (!on_device) CK(cudaStreamSynchronize(c->st));
   mark(c, q);
   if (q == GW_Q_G_TAU) c->have_G = true;
-  if (q == GW_Q_P0_IW) { c->have_P0 = true; unmark(c, GW_Q_P_IW); }
+  if (q == GW_Q_P0_IW) { c->have_P0 = true; c->p0sym = false; unmark(c, GW_Q_P_IW); }
   if (q == GW_Q_P_TAU) c->have_P = true;
   if (q == GW_Q_SIGMA_INF || q == GW_Q_SIGMA_IW) c->have_sigma = true;
   return GW_OK;
@@ -1324,8 +1572,13 @@ extern "C" gw_status gw_polarization(gw_ctx* c) {
   double2* P0q = c->P0_tau + (size_t)c->q0 * ntau * na2;
   CK(polar_finish(c, c->P0_tau, red));
   // P~0(i Omega_m) = sum_j TFb[m][j] P~0(tau_j)   (Eq. P0t_to_P0w)
-  CK(transform(c, c->TFb, P0q, c->P_iw + (size_t)c->q0 * c->nwb * na2, c->nwb, na2, nq, (int64_t)ntau * na2,
-               (int64_t)c->nwb * na2));
+  c->p0sym = fold_ready(c);
+  if (c->p0sym) {
+    CK(fold_forward(c));
+  } else {
+    CK(transform(c, c->TFb, P0q, c->P_iw + (size_t)c->q0 * c->nwb * na2, c->nwb, na2, nq, (int64_t)ntau * na2,
+                 (int64_t)c->nwb * na2));
+  }
   c->have_P0 = true;
   c->have_P = false;
   mark(c, GW_Q_P0_TAU); mark(c, GW_Q_P0_IW); unmark(c, GW_Q_P_IW);
@@ -1365,7 +1618,20 @@ extern "C" gw_status gw_screened(gw_ctx* c) {
     CK(cudaMemsetAsync(c->info + 1, 0, 8, c->st));
   }
   gw_status s = GW_OK;
-  if (trs_reduce(c)) {
+  // P~0(i Omega) computed here has the symmetries of the folded block exactly; one that was
+  // handed in is looked at (not inside a capture, whose P~0 is its own), and taken as symmetric
+  // when it is to the rounding of its largest value
+  bool folded = fold_ready(c) && c->p0sym;
+  if (fold_ready(c) && !folded && !c->deferred) {
+    CK(fold_check(c->P_iw, fold_view(c), c->dscr + 16, c->st));
+    count(1);
+    CK(cudaMemcpyAsync(c->h_scr + 16, c->dscr + 16, 16, cudaMemcpyDeviceToHost, c->st));
+    CK(cudaStreamSynchronize(c->st));
+    folded = c->h_scr[16] <= kFoldTol * c->h_scr[17];
+  }
+  if (folded) {
+    CK(fold_screened(c));
+  } else if (trs_reduce(c)) {
     // time-reversal symmetry: solve the runs of irreducible q, then P~^{-q} = conj P~^q
     for (int qa = 0; qa < c->nk && s == GW_OK;) {
       if (c->kneg[(size_t)qa] < qa) { ++qa; continue; }
@@ -1599,7 +1865,16 @@ extern "C" gw_status gw_selfenergy(gw_ctx* c) {
 extern "C" gw_status gw_set_q_range(gw_ctx* c, int32_t q0, int32_t q1) {
   if (!c) return GW_ERR_ARG;
   if (q0 < 0 || q1 > c->nk || q0 >= q1) return fail(c, GW_ERR_ARG, "q range must satisfy 0 <= q0 < q1 <= nk");
-  c->q0 = q0; c->q1 = q1;
+  if (q0 != c->q0 || q1 != c->q1) {
+    c->q0 = q0; c->q1 = q1;
+    if (c->wfold) CK(fold_lists(c));
+    if (c->gexec) {   // a captured iteration is one of the previous range
+      CK(cudaStreamSynchronize(c->gst));
+      cudaGraphExecDestroy(c->gexec);
+      cudaGraphDestroy(c->graph);
+      c->gexec = nullptr; c->graph = nullptr;
+    }
+  }
   // results of another range are not those of this one
   c->have_P0 = c->have_P = false;
   for (gw_quantity q : {GW_Q_P0_TAU, GW_Q_P0_IW, GW_Q_P_IW, GW_Q_P_TAU, GW_Q_SIGMA_TAU}) unmark(c, q);

@@ -78,6 +78,28 @@ size_t screened_refine_bytes(int64_t n, int64_t chunk);
 bool screened_refine_ok(int64_t n);
 cudaError_t screened_refine(double2* X, int64_t n, int64_t count, void* work, size_t work_bytes, int nsteps,
                             int* d_info, int* d_err, cudaStream_t st, int64_t* nlaunch);
+// the same for real matrices of even order n (double)
+size_t screened_refine_real_bytes(int64_t n, int64_t chunk);
+cudaError_t screened_refine_real(double* X, int64_t n, int64_t count, void* work, size_t work_bytes, int nsteps,
+                                 int* d_info, int* d_err, cudaStream_t st, int64_t* nlaunch);
+
+// ------------------------------------------------------------------ folded bosonic block (k_fold.cu)
+struct FoldView {
+  int n, nwb, nrep, q0, q1;
+  const int *rep, *repn;   // kept frequencies and their -Omega partners (-1: none)
+  const int* neg;          // index of -q
+};
+cudaError_t fold_expand_pairs(double2* P, const FoldView& f, const int* qlist, int nz, const double2* src,
+                              cudaStream_t st);
+cudaError_t fold_expand_real(double2* P, const FoldView& f, const int* qlist, int nz, const double* src, int ne,
+                             cudaStream_t st);
+cudaError_t fold_expand_cplx(double2* P, const FoldView& f, const int* qlist, int nz, const double2* src,
+                             cudaStream_t st);
+cudaError_t fold_pack_real(const double2* P, const FoldView& f, const int* qlist, int nz, double* X, int ne,
+                           cudaStream_t st);
+cudaError_t fold_pack_cplx(const double2* P, const FoldView& f, const int* qlist, int nz, double2* X,
+                           cudaStream_t st);
+cudaError_t fold_check(const double2* P, const FoldView& f, double* out, cudaStream_t st);
 
 struct DysonArgs {
   int nao, nk, nw;
@@ -183,6 +205,8 @@ struct UmmaScale {
   int eshift;
   int64_t ea_div = 1, eb_div = 1;   // row m uses eA[z*ea_zs + m/ea_div], column n eB[z*eb_zs + (n/2)/eb_div]
   int64_t ea_mod = 0;               // > 0: row m uses eA[z*ea_zs + (m/ea_div) % ea_mod]
+  bool real_cols = false;           // column n uses eB[z*eb_zs + n/eb_div] (a real product)
+  const int* row_list = nullptr;    // outer row part o lands at row_list[o] * row_s1 (lane-per-row write-out only)
 };
 // 16-bit pieces as the output of a GEMM (C: hi, C_lo: lo, fp32-class layout in 16-bit
 // elements): D * 2^-(eO[z*eo_zs + m/eo_div] + eo_shift) in fp16 (half = 1) or bf16 (2)
@@ -214,6 +238,23 @@ size_t emul_digit_bytes(int64_t rows, int64_t K);
 cudaError_t emul_split_b(const double2* B, int64_t rows, int64_t K, int64_t ldb, void* dig, int* ex, cudaStream_t st);
 cudaError_t emul_transform(const void* Bd, const int* Be, int64_t nrow, const double2* X, int64_t K, int64_t ncol,
                            int64_t ldx, double2* Y, int64_t ldy, void* Ad, int* Ae, int* err, cudaStream_t st);
+// digits of a real matrix B [rows][K] (rows even, one exponent per row pair) as the B operand of
+// a transform whose output pairs two real rows; emul_digit_bytes(rows, (K + 1) / 2) bytes
+cudaError_t emul_split_b_real(const double* B, int64_t rows, int64_t K, void* dig, int* ex, cudaStream_t st);
+// Y[ylist ? ylist[z] : z][p][col] (double2, p < npair) = rows (2p, 2p+1) of B times the K real values
+// of column col of matrix zlist[z] of X: its K/2 complex rows (re, im), or with real_rows the real
+// parts of the K rows klist[0..K) (in place of rows 0..).  Strides zs, yzs in complex elements; the
+// rows of X and of Y are packed (ncol apart).
+cudaError_t emul_transform_multi(const void* Bd, const int* Be, int64_t npair, const double2* X, int64_t K,
+                                 bool real_rows, int64_t ncol, int64_t zs, int nz, const int* zlist,
+                                 const int* klist, double2* Y, int64_t yzs, const int* ylist, void* Ad, int* Ae,
+                                 int* err, cudaStream_t st);
+// real counterparts of the batched products (element strides in reals; K even)
+cudaError_t emul_split_cols_real(const double* B, int64_t count, int64_t K, int64_t N, int64_t ldb, int64_t sb,
+                                 void* Bd, int* Be, cudaStream_t st);
+cudaError_t emul_rgemm_batched(const void* Ad, const int* Ae, const void* Bd, const int* Be, int64_t count,
+                               int64_t M, int64_t N, int64_t K, double* C, int* err, cudaStream_t st, int nd = 8);
+int emul_launches_real(int64_t K, int nd = 8);
 // tensor-core launches of one product with complex K and nd digits (-1: K too large)
 int emul_launches(int64_t K, int nd = 8);
 cudaError_t emul_split_rows(const double2* A, int64_t count, int64_t M, int64_t K, int64_t lda, int64_t sa,
@@ -237,6 +278,9 @@ cudaError_t embed_conj_f16(const void* src, bool src_c128, int64_t rows, int64_t
                            int* ex, cudaStream_t st);
 cudaError_t embed_t_batched(const void* src, bool src_c128, int64_t count, int64_t K, int64_t N, int64_t ld,
                             int64_t zs, float* hi, float* lo, int64_t Kpad, int64_t ds, cudaStream_t st);
+// transposed real operand: row n = column n of a K x N matrix (TF32 hi / lo planes)
+cudaError_t transpose_split_batched(const void* src, bool src_f64, int64_t count, int64_t K, int64_t N, int64_t ld,
+                                    int64_t zs, float* hi, float* lo, int64_t Kpad, int64_t ds, cudaStream_t st);
 cudaError_t embed_conj_batched(const double2* src, int64_t count, int64_t ss, int64_t rows, int64_t K, float* hi,
                                float* lo, int64_t Kpad, int64_t ds, cudaStream_t st);
 cudaError_t embed_plain_batched(const double2* src, int64_t count, int64_t ss, int64_t rows, int64_t K, float* hi,

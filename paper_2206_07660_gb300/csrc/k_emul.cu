@@ -66,23 +66,35 @@ __device__ __forceinline__ int em_exponent(double m) {
 // 2k + c (re, im).  Padding columns [2K, Kp) are written as zeros.  Block: 32 rows x
 // all K; the source tile goes through shared memory so both the reads (along n)
 // and the digit writes (along k) are coalesced.
-__global__ void __launch_bounds__(256) em_split_t_kernel(const double2* __restrict__ src, int64_t K, int64_t ncol,
+// Matrix z of the batch is zlist[z] when a list is given.  RR: the K real values are the
+// real parts of K rows (klist[k], or row k), two of them taking the place of one complex
+// entry: half the digits where the source is known to be real.
+template <bool RR>
+__global__ void __launch_bounds__(256) em_split_t_kernel(const double2* __restrict__ src, int64_t Kin, int64_t ncol,
                                                          int64_t ld, int64_t zs, dig_t* __restrict__ dig,
-                                                         int* __restrict__ ex, int64_t Kp) {
+                                                         int* __restrict__ ex, int64_t Kp,
+                                                         const int* __restrict__ zlist,
+                                                         const int* __restrict__ klist) {
   __shared__ double2 tile[32][33];
   __shared__ double red[8][32];
   __shared__ int es[32];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t z = blockIdx.y;
-  const double2* X = src + z * zs;
+  const double2* X = src + (zlist ? (int64_t)zlist[z] : z) * zs;
   dig_t* D = dig + z * ncol * (int64_t)EM_S * Kp;
   int* E = ex + z * ncol;
   const int64_t n0 = (int64_t)blockIdx.x * 32;
   const int64_t n = n0 + tx;
+  const int64_t K = RR ? (Kin + 1) / 2 : Kin;
+  auto krow = [&](int64_t k) { return klist ? (int64_t)klist[k] : k; };
+  auto load = [&](int64_t j, int64_t c) {
+    if (!RR) return X[krow(j) * ld + c];
+    return make_double2(X[krow(2 * j) * ld + c].x, 2 * j + 1 < Kin ? X[krow(2 * j + 1) * ld + c].x : 0.0);
+  };
   double m = 0.0;
   if (n < ncol)
     for (int64_t j = ty; j < K; j += 8) {
-      const double2 v = X[j * ld + n];
+      const double2 v = load(j, n);
       m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
     }
   red[ty][tx] = m;
@@ -100,7 +112,7 @@ __global__ void __launch_bounds__(256) em_split_t_kernel(const double2* __restri
   for (int64_t j0 = 0; j0 < kc; j0 += 32) {
     for (int jj = ty; jj < 32; jj += 8) {
       const int64_t j = j0 + jj;
-      tile[jj][tx] = (j < K && n < ncol) ? X[j * ld + n] : make_double2(0.0, 0.0);
+      tile[jj][tx] = (j < K && n < ncol) ? load(j, n) : make_double2(0.0, 0.0);
     }
     __syncthreads();
     for (int rr = ty; rr < 32; rr += 8) {
@@ -312,7 +324,8 @@ cudaError_t emul_transform(const void* Bdv, const int* Be, int64_t nrow, const d
   const dig_t* Bd = (const dig_t*)Bdv;
   dig_t* Ad = (dig_t*)Adv;
   const int64_t Kp = emul_kpad(K);
-  em_split_t_kernel<<<dim3((unsigned)((ncol + 31) / 32), 1), 256, 0, st>>>(X, K, ncol, ldx, 0, Ad, Ae, Kp);
+  em_split_t_kernel<false><<<dim3((unsigned)((ncol + 31) / 32), 1), 256, 0, st>>>(X, K, ncol, ldx, 0, Ad, Ae, Kp,
+                                                                                   nullptr, nullptr);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int64_t ld = (int64_t)EM_S * Kp;
@@ -326,6 +339,155 @@ cudaError_t emul_transform(const void* Bdv, const int* Be, int64_t nrow, const d
     UmmaScale sc{Ae, Be, 0, 0, -EM_BETA * g};
     e = umma_gemm(oa, ob, (int)ncol, (int)(2 * nrow), (int64_t)np * Kp, 1, (void*)Y, true, 1.0, l > 0, 2, 0, 1,
                   err, st, 1, 0, 0, 2, 2 * ldy, nullptr, &sc, (int64_t)(np - 1) * Kp + 2 * K);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// Real rows of the B operand in pairs: rows 2p, 2p + 1 of a real matrix B [rows][K], digit
+// planes in reverse order, one exponent per pair, padding columns zeroed.  One block per pair.
+__global__ void __launch_bounds__(256) em_split_br_kernel(const double* __restrict__ B, int64_t K,
+                                                          dig_t* __restrict__ dig, int* __restrict__ ex, int64_t Kp) {
+  const int64_t p = blockIdx.x;
+  __shared__ double red[256];
+  double mx = 0.0;
+  for (int64_t e = threadIdx.x; e < 2 * K; e += blockDim.x) mx = fmax(mx, fabs(B[2 * p * K + e]));
+  red[threadIdx.x] = mx;
+  __syncthreads();
+  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
+    if ((int)threadIdx.x < s) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + s]);
+    __syncthreads();
+  }
+  const int e = em_exponent(red[0]);
+  if (threadIdx.x == 0) ex[p] = e;
+  const int64_t rowlen = (int64_t)EM_S * Kp;
+  for (int64_t i = threadIdx.x; i < 2 * Kp; i += blockDim.x) {
+    const int64_t r = i / Kp, k = i - r * Kp;
+    float d[EM_S];
+    em_digits(k < K ? B[(2 * p + r) * K + k] : 0.0, e, d);
+#pragma unroll
+    for (int s = 0; s < EM_S; ++s) dig[(2 * p + r) * rowlen + (int64_t)(EM_S - 1 - s) * Kp + k] = __float2half_rn(d[s]);
+  }
+}
+
+cudaError_t emul_split_b_real(const double* B, int64_t rows, int64_t K, void* dig, int* ex, cudaStream_t st) {
+  if (rows % 2) return cudaErrorInvalidValue;
+  em_split_br_kernel<<<(unsigned)(rows / 2), 256, 0, st>>>(B, K, (dig_t*)dig, ex, emul_kpad((K + 1) / 2));
+  return cudaGetLastError();
+}
+
+// One transform of several matrices at once: the (matrix, column) pairs are the rows of a
+// single GEMM, so that a small system's q-points share each of the plan's launches.
+cudaError_t emul_transform_multi(const void* Bdv, const int* Be, int64_t npair, const double2* X, int64_t K,
+                                 bool real_rows, int64_t ncol, int64_t zs, int nz, const int* zlist,
+                                 const int* klist, double2* Y, int64_t yzs, const int* ylist, void* Adv, int* Ae,
+                                 int* err, cudaStream_t st) {
+  const dig_t* Bd = (const dig_t*)Bdv;
+  dig_t* Ad = (dig_t*)Adv;
+  const int64_t Kp = emul_kpad((K + 1) / 2), rows = nz * ncol;
+  if (nz < 1 || nz > 65535 || rows > INT32_MAX || (!real_rows && K % 2)) return cudaErrorInvalidValue;
+  dim3 grid((unsigned)((ncol + 31) / 32), (unsigned)nz);
+  if (real_rows) em_split_t_kernel<true><<<grid, 256, 0, st>>>(X, K, ncol, ncol, zs, Ad, Ae, Kp, zlist, klist);
+  else em_split_t_kernel<false><<<grid, 256, 0, st>>>(X, K / 2, ncol, ncol, zs, Ad, Ae, Kp, zlist, klist);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const int64_t ld = (int64_t)EM_S * Kp;
+  EmLaunch pl[EM_MAXL];
+  const int nl = em_plan(K, pl);
+  if (nl < 0) return cudaErrorInvalidValue;
+  for (int l = 0; l < nl; ++l) {
+    const int g = pl[l].g, i0 = pl[l].i0, np = pl[l].i1 - pl[l].i0 + 1;
+    UmmaOperand oa{(const float*)(Ad + (int64_t)(i0 - 1) * Kp), nullptr, rows, 1, ld, 0, 1};
+    UmmaOperand ob{(const float*)(Bd + (int64_t)(EM_S - g + i0) * Kp), nullptr, 2 * npair, 1, ld, 0, 1};
+    UmmaScale sc{Ae, Be, 0, 0, -EM_BETA * g};
+    sc.row_list = ylist;
+    e = umma_gemm(oa, ob, (int)rows, (int)(2 * npair), (int64_t)np * Kp, 1, (void*)Y, true, 1.0, l > 0, 2, 0, 1, err,
+                  st, 1, ncol, 2 * yzs, 2, 2 * ncol, nullptr, &sc, (int64_t)(np - 1) * Kp + K);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+int emul_launches_real(int64_t K, int nd) {
+  EmLaunch pl[EM_MAXL];
+  return em_plan(K, pl, nd);
+}
+
+// Digits of the columns of real K x N matrices (one exponent per column), planes in reverse
+// order: the B operand of the real C[z] = A[z] B[z].  Layout and passes of em_split_bt_kernel.
+__global__ void __launch_bounds__(256) em_split_btr_kernel(const double* __restrict__ src, int64_t K, int64_t ncol,
+                                                           int64_t ld, int64_t zs, dig_t* __restrict__ dig,
+                                                           int* __restrict__ ex, int64_t Kp) {
+  __shared__ double tile[64][33];
+  __shared__ double red[8][32];
+  __shared__ int es[32];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int64_t z = blockIdx.y;
+  const double* X = src + z * zs;
+  const int64_t rowlen = (int64_t)EM_S * Kp;
+  dig_t* D = dig + z * ncol * rowlen;
+  int* E = ex + z * ncol;
+  const int64_t n0 = (int64_t)blockIdx.x * 32, n = n0 + tx;
+  double m = 0.0;
+  if (n < ncol)
+    for (int64_t j = ty; j < K; j += 8) m = fmax(m, fabs(X[j * ld + n]));
+  red[ty][tx] = m;
+  __syncthreads();
+  if (ty == 0) {
+    double mm = red[0][tx];
+    for (int r = 1; r < 8; ++r) mm = fmax(mm, red[r][tx]);
+    const int e = em_exponent(mm);
+    es[tx] = e;
+    if (n < ncol) E[n] = e;
+  }
+  __syncthreads();
+  for (int64_t j0 = 0; j0 < Kp; j0 += 64) {
+    for (int jj = ty; jj < 64; jj += 8) {
+      const int64_t j = j0 + jj;
+      tile[jj][tx] = (j < K && n < ncol) ? X[j * ld + n] : 0.0;
+    }
+    __syncthreads();
+    for (int rr = ty; rr < 32; rr += 8) {
+      const int64_t col = n0 + rr, j = j0 + 2 * tx;
+      if (col < ncol && j < Kp) {
+        float d0[EM_S], d1[EM_S];
+        em_digits(tile[2 * tx][rr], es[rr], d0);
+        em_digits(tile[2 * tx + 1][rr], es[rr], d1);
+        dig_t* r0 = D + col * rowlen + j;
+#pragma unroll
+        for (int i = 0; i < EM_S; ++i) *(__half2*)(r0 + (int64_t)(EM_S - 1 - i) * Kp) = __floats2half2_rn(d0[i], d1[i]);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+cudaError_t emul_split_cols_real(const double* B, int64_t count, int64_t K, int64_t N, int64_t ldb, int64_t sb,
+                                 void* Bd, int* Be, cudaStream_t st) {
+  if (count > 65535 || K % 2) return cudaErrorInvalidValue;
+  em_split_btr_kernel<<<dim3((unsigned)((N + 31) / 32), (unsigned)count), 256, 0, st>>>(B, K, N, ldb, sb, (dig_t*)Bd, Be,
+                                                                                        emul_kpad(K / 2));
+  return cudaGetLastError();
+}
+
+// C[z] (M x N real, packed) = A[z] B[z] from the digits of emul_split_rows (A's rows read as
+// K/2 complex entries) and emul_split_cols_real.
+cudaError_t emul_rgemm_batched(const void* Adv, const int* Ae, const void* Bdv, const int* Be, int64_t count,
+                               int64_t M, int64_t N, int64_t K, double* C, int* err, cudaStream_t st, int nd) {
+  const dig_t* Ad = (const dig_t*)Adv;
+  const dig_t* Bd = (const dig_t*)Bdv;
+  const int64_t Kp = emul_kpad(K / 2), ld = (int64_t)EM_S * Kp;
+  EmLaunch pl[EM_MAXL];
+  const int nl = em_plan(K, pl, nd);
+  if (nl < 0 || count > 65535) return cudaErrorInvalidValue;
+  for (int l = 0; l < nl; ++l) {
+    const int g = pl[l].g, i0 = pl[l].i0, np = pl[l].i1 - pl[l].i0 + 1;
+    UmmaOperand oa{(const float*)(Ad + (int64_t)(i0 - 1) * Kp), nullptr, M, count, ld, M * ld, 1};
+    UmmaOperand ob{(const float*)(Bd + (int64_t)(EM_S - g + i0) * Kp), nullptr, N, count, ld, N * ld, 1};
+    UmmaScale sc{Ae, Be, M, N, -EM_BETA * g};
+    sc.real_cols = true;
+    cudaError_t e = umma_gemm(oa, ob, (int)M, (int)N, (int64_t)np * Kp, (int)count, (void*)C, true, 1.0, l > 0, N,
+                              M * N, 1, err, st, 1, 0, 0, 0, 0, nullptr, &sc, (int64_t)(np - 1) * Kp + K);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -77,6 +77,7 @@ __global__ void __launch_bounds__(256) herm_fill_kernel(double2* X, int n, int n
     const bool in = nq >= q0 && nq < q1;
     const bool filled = (fold || trs) && in && (nq < q || (fold && nq == q && t >= (nt + 1) / 2));
     if (filled) continue;
+    const bool real = fold && nq == q && 2 * t == nt - 1;   // its own image: real
     double2* M = X + ((int64_t)q * nt + t) * n2;
     // mirror image (null: none)
     double2* W = nullptr;
@@ -97,7 +98,7 @@ __global__ void __launch_bounds__(256) herm_fill_kernel(double2* X, int n, int n
       int i = I * 32 + rr, j = J * 32 + tx;
       if (i < n && j < n) {
         const double2 u = a[rr][tx], v = b[tx][rr];
-        const double2 h = make_double2(0.5 * (u.x + v.x), 0.5 * (u.y - v.y));
+        const double2 h = make_double2(0.5 * (u.x + v.x), real ? 0.0 : 0.5 * (u.y - v.y));
         M[(int64_t)i * n + j] = h;
         if (W) W[(int64_t)i * n + j] = make_double2(h.x, -h.y);
       }
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(256) herm_fill_kernel(double2* X, int n, int n
         i = J * 32 + rr; j = I * 32 + tx;
         if (i < n && j < n) {
           const double2 u = b[rr][tx], v = a[tx][rr];
-          const double2 h = make_double2(0.5 * (u.x + v.x), 0.5 * (u.y - v.y));
+          const double2 h = make_double2(0.5 * (u.x + v.x), real ? 0.0 : 0.5 * (u.y - v.y));
           M[(int64_t)i * n + j] = h;
           if (W) W[(int64_t)i * n + j] = make_double2(h.x, -h.y);
         }

@@ -152,6 +152,32 @@ __global__ void embed_t_kernel(const T* __restrict__ src, int64_t K, int64_t N, 
   }
 }
 
+// Operand of C = A B^T where B[n][k] = src[z][k][n], real: rows n of Kpad floats, transposed
+// through shared memory, padding columns zeroed.  Grid: (N/32, Kpad/32, count).
+template <typename T>
+__global__ void transpose_split_kernel(const T* __restrict__ src, int64_t K, int64_t N, int64_t ld, int64_t zs,
+                                       float* hi, float* lo, int64_t Kpad, int64_t ds) {
+  __shared__ double tile[32][33];
+  const int64_t k0 = blockIdx.y * 32, nb = blockIdx.x * 32;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
+  src += (int64_t)blockIdx.z * zs;
+  hi += (int64_t)blockIdx.z * ds;
+  lo += (int64_t)blockIdx.z * ds;
+  for (int r = ty; r < 32; r += 8) {
+    const int64_t k = k0 + r, n = nb + tx;
+    tile[r][tx] = (k < K && n < N) ? (double)src[k * ld + n] : 0.0;
+  }
+  __syncthreads();
+  for (int r = ty; r < 32; r += 8) {
+    const int64_t n = nb + r, k = k0 + tx;
+    if (n >= N || k >= Kpad) continue;
+    float h, l;
+    split2(tile[tx][r], h, l);
+    hi[n * Kpad + k] = h;
+    lo[n * Kpad + k] = l;
+  }
+}
+
 static inline int nb_(int64_t n) { int64_t b = (n + 255) / 256; return (int)(b < 152 * 16 ? b : 152 * 16); }
 
 cudaError_t split_rows(const void* src, bool src_c128, int64_t rows, int64_t K, int64_t ld, bool conj, float* hi,
@@ -187,6 +213,15 @@ cudaError_t embed_plain_batched(const double2* src, int64_t count, int64_t ss, i
 cudaError_t embed_t(const void* src, bool src_c128, int64_t K, int64_t N, float* hi, float* lo, int64_t Kpad,
                     cudaStream_t st) {
   return embed_t_batched(src, src_c128, 1, K, N, N, 0, hi, lo, Kpad, 0, st);
+}
+
+cudaError_t transpose_split_batched(const void* src, bool src_f64, int64_t count, int64_t K, int64_t N, int64_t ld,
+                                    int64_t zs, float* hi, float* lo, int64_t Kpad, int64_t ds, cudaStream_t st) {
+  if (count < 1 || count > 65535) return cudaErrorInvalidValue;
+  dim3 grid((unsigned)((N + 31) / 32), (unsigned)((Kpad + 31) / 32), (unsigned)count);
+  if (src_f64) transpose_split_kernel<double><<<grid, 256, 0, st>>>((const double*)src, K, N, ld, zs, hi, lo, Kpad, ds);
+  else transpose_split_kernel<float><<<grid, 256, 0, st>>>((const float*)src, K, N, ld, zs, hi, lo, Kpad, ds);
+  return cudaGetLastError();
 }
 
 cudaError_t embed_t_batched(const void* src, bool src_c128, int64_t count, int64_t K, int64_t N, int64_t ld,

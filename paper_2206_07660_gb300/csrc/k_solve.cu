@@ -22,6 +22,9 @@ template <typename T> struct TyOf;
 template <> struct TyOf<double2> { static constexpr Ty v = Ty::C128; };
 template <> struct TyOf<float2> { static constexpr Ty v = Ty::C64; };
 
+// C(T): reals per element of T
+template <typename T> static constexpr int reals() { return gj_cplx<T>::v ? 2 : 1; }
+
 template <typename T>
 __global__ void extract_kernel(const T* __restrict__ X, int64_t n, int nb, int64_t kb, int64_t count, T* Cp, T* Rp) {
   const int64_t per = 2 * n * nb;
@@ -31,7 +34,7 @@ __global__ void extract_kernel(const T* __restrict__ X, int64_t n, int nb, int64
     if (r < n * nb) {          // column panel Cp[i][c] (rows of block b zeroed)
       int64_t i = r / nb, c = r - i * nb;
       T v = Xz[i * n + kb + c];
-      if (i >= kb && i < kb + nb) { v.x = 0; v.y = 0; }
+      if (i >= kb && i < kb + nb) v = cval<T>(0.0, 0.0);
       Cp[z * n * nb + r] = v;
     } else {                   // row panel Rp[c][j]
       r -= n * nb;
@@ -46,8 +49,7 @@ __global__ void zero_cols_kernel(T* X, int64_t n, int nb, int64_t kb, int64_t co
   const int64_t per = n * nb;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < per * count; e += (int64_t)gridDim.x * blockDim.x) {
     int64_t z = e / per, r = e - z * per, i = r / nb, c = r - i * nb;
-    T v; v.x = 0; v.y = 0;
-    X[z * n * n + i * n + kb + c] = v;
+    X[z * n * n + i * n + kb + c] = cval<T>(0.0, 0.0);
   }
 }
 
@@ -185,64 +187,82 @@ static cudaError_t gj_blocked(T* X, int64_t n, int64_t count, void* work, size_t
 static inline int64_t pad32(int64_t x) { return (x + 31) / 32 * 32; }
 
 // split planes of one block step of gj_blocked_tc, per system
+template <typename T>
 static size_t gj_tc_plane_bytes(int64_t n) {
-  const int64_t nb = n < NB ? n : NB, Kb = pad32(2 * nb);
-  return (size_t)8 * Kb * (5 * n + nb);   // hi/lo of Cp (n rows), Dinv (nb), Rp^T and Rn^T (2n each)
+  constexpr int C = reals<T>();
+  const int64_t nb = n < NB ? n : NB, Kb = pad32(C * nb);
+  return (size_t)8 * Kb * ((2 * C + 1) * n + nb);   // hi/lo of Cp (n rows), Dinv (nb), Rp^T and Rn^T (C n each)
 }
 
-// gj_blocked for complex64 storage with both products of a block step on the
-// tensor cores (split TF32, three products): Rn = Dinv Rp and X -= Cp Rn; block
-// inverses in complex64.  planes: gj_tc_plane_bytes(n) per system.
-static cudaError_t gj_blocked_tc(float2* X, int64_t n, int64_t cz, void* pan, float* planes, int* d_info, int* d_err,
+// operand planes of `rows` packed rows of nb elements / of the nb x n row panels of the batch
+// (a real row of even length is the interleaved row of nb / 2 complex entries)
+template <typename T>
+static cudaError_t rows_op(const T* x, int64_t rows, int64_t nb, float* hi, float* lo, int64_t Kp, cudaStream_t st) {
+  const int64_t k = gj_cplx<T>::v ? nb : nb / 2;
+  return split_rows(x, false, rows, k, k, false, hi, lo, Kp, st);
+}
+template <typename T>
+static cudaError_t cols_op(const T* x, int64_t cz, int64_t nb, int64_t n, float* hi, float* lo, int64_t Kp,
+                           cudaStream_t st) {
+  if (gj_cplx<T>::v) return embed_t_batched(x, false, cz, nb, n, n, n * nb, hi, lo, Kp, 2 * n * Kp, st);
+  return transpose_split_batched(x, false, cz, nb, n, n, n * nb, hi, lo, Kp, n * Kp, st);
+}
+
+// gj_blocked for FP32 storage (complex, or real with n even) with both products of a
+// block step on the tensor cores (split TF32, three products): Rn = Dinv Rp and
+// X -= Cp Rn; block inverses in T.  planes: gj_tc_plane_bytes<T>(n) per system.
+template <typename T>
+static cudaError_t gj_blocked_tc(T* X, int64_t n, int64_t cz, void* pan, float* planes, int* d_info, int* d_err,
                                  cudaStream_t st, int64_t* nlaunch) {
-  const int64_t nbmax = n < NB ? n : NB, Kb = pad32(2 * nbmax);
+  constexpr int C = reals<T>();
+  const int64_t nbmax = n < NB ? n : NB, Kb = pad32(C * nbmax);
   const int nt = 256;
-  const size_t sm = block_inv_smem<float2>(nbmax, nt);
+  const size_t sm = block_inv_smem<T>(nbmax, nt);
   cudaError_t e;
   if (sm > 48 * 1024) {
-    e = cudaFuncSetAttribute(block_inv_kernel<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    e = cudaFuncSetAttribute(block_inv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
   }
-  float2* Cp = (float2*)pan;
-  float2* Rp = Cp + cz * n * nbmax;
-  float2* Rn = Rp + cz * n * nbmax;
-  float2* Di = (float2*)((char*)pan + (((size_t)3 * cz * n * nbmax * sizeof(float2) + 255) & ~(size_t)255));
+  T* Cp = (T*)pan;
+  T* Rp = Cp + cz * n * nbmax;
+  T* Rn = Rp + cz * n * nbmax;
+  T* Di = (T*)((char*)pan + (((size_t)3 * cz * n * nbmax * sizeof(T) + 255) & ~(size_t)255));
   float* Ch = planes;
   float* Cl = Ch + cz * n * Kb;
   float* Dh = Cl + cz * n * Kb;
   float* Dl = Dh + cz * nbmax * Kb;
   float* Rh = Dl + cz * nbmax * Kb;
-  float* Rl = Rh + cz * 2 * n * Kb;
-  float* Nh = Rl + cz * 2 * n * Kb;
-  float* Nl = Nh + cz * 2 * n * Kb;
+  float* Rl = Rh + cz * C * n * Kb;
+  float* Nh = Rl + cz * C * n * Kb;
+  float* Nl = Nh + cz * C * n * Kb;
   int64_t launches = 0;
   for (int64_t kb = 0; kb < n; kb += nbmax) {
     const int nb = (int)((n - kb) < nbmax ? (n - kb) : nbmax);
-    const int64_t Kp = pad32(2 * nb);
-    extract_kernel<float2><<<grid1(2 * n * nb * cz), 256, 0, st>>>(X, n, nb, kb, cz, Cp, Rp);
-    zero_cols_kernel<float2><<<grid1(n * nb * cz), 256, 0, st>>>(X, n, nb, kb, cz);
-    block_inv_kernel<float2><<<(int)(cz < 152 * 8 ? cz : 152 * 8), nt, sm, st>>>(Rp, n, nb, kb, cz, Di, d_info);
+    const int64_t Kp = pad32(C * nb);
+    extract_kernel<T><<<grid1(2 * n * nb * cz), 256, 0, st>>>(X, n, nb, kb, cz, Cp, Rp);
+    zero_cols_kernel<T><<<grid1(n * nb * cz), 256, 0, st>>>(X, n, nb, kb, cz);
+    block_inv_kernel<T><<<(int)(cz < 152 * 8 ? cz : 152 * 8), nt, sm, st>>>(Rp, n, nb, kb, cz, Di, d_info);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // Rn[z] = Dinv[z] (nb x nb) Rp[z] (nb x n)
-    if ((e = split_rows(Di, false, cz * nb, nb, nb, false, Dh, Dl, Kp, st)) != cudaSuccess) return e;
-    if ((e = embed_t_batched(Rp, false, cz, nb, n, n, n * nb, Rh, Rl, Kp, 2 * n * Kp, st)) != cudaSuccess) return e;
+    if ((e = rows_op<T>(Di, cz * nb, nb, Dh, Dl, Kp, st)) != cudaSuccess) return e;
+    if ((e = cols_op<T>(Rp, cz, nb, n, Rh, Rl, Kp, st)) != cudaSuccess) return e;
     {
-      UmmaOperand a{Dh, Dl, nb, cz, Kp, nb * Kp}, b{Rh, Rl, 2 * n, cz, Kp, 2 * n * Kp};
-      if ((e = umma_gemm(a, b, nb, (int)(2 * n), Kp, (int)cz, Rn, false, 1.0, false, 2 * n, 2 * n * nb, 3, d_err, st,
-                         1, 0, 0, 0, 0, nullptr, nullptr, 2 * nb)) != cudaSuccess)
+      UmmaOperand a{Dh, Dl, nb, cz, Kp, nb * Kp}, b{Rh, Rl, C * n, cz, Kp, C * n * Kp};
+      if ((e = umma_gemm(a, b, nb, (int)(C * n), Kp, (int)cz, Rn, false, 1.0, false, C * n, C * n * nb, 3, d_err, st,
+                         1, 0, 0, 0, 0, nullptr, nullptr, C * nb)) != cudaSuccess)
         return e;
     }
-    put_dinv_kernel<float2><<<grid1((int64_t)nb * nb * cz), 256, 0, st>>>(Rn, Di, n, nb, kb, cz);
+    put_dinv_kernel<T><<<grid1((int64_t)nb * nb * cz), 256, 0, st>>>(Rn, Di, n, nb, kb, cz);
     // X[z] -= Cp[z] (n x nb) Rn[z] (nb x n)
-    if ((e = split_rows(Cp, false, cz * n, nb, nb, false, Ch, Cl, Kp, st)) != cudaSuccess) return e;
-    if ((e = embed_t_batched(Rn, false, cz, nb, n, n, n * nb, Nh, Nl, Kp, 2 * n * Kp, st)) != cudaSuccess) return e;
+    if ((e = rows_op<T>(Cp, cz * n, nb, Ch, Cl, Kp, st)) != cudaSuccess) return e;
+    if ((e = cols_op<T>(Rn, cz, nb, n, Nh, Nl, Kp, st)) != cudaSuccess) return e;
     {
-      UmmaOperand a{Ch, Cl, n, cz, Kp, n * Kp}, b{Nh, Nl, 2 * n, cz, Kp, 2 * n * Kp};
-      if ((e = umma_gemm(a, b, (int)n, (int)(2 * n), Kp, (int)cz, X, false, -1.0, true, 2 * n, 2 * n * n, 3, d_err,
-                         st, 1, 0, 0, 0, 0, nullptr, nullptr, 2 * nb)) != cudaSuccess)
+      UmmaOperand a{Ch, Cl, n, cz, Kp, n * Kp}, b{Nh, Nl, C * n, cz, Kp, C * n * Kp};
+      if ((e = umma_gemm(a, b, (int)n, (int)(C * n), Kp, (int)cz, X, false, -1.0, true, C * n, C * n * n, 3, d_err,
+                         st, 1, 0, 0, 0, 0, nullptr, nullptr, C * nb)) != cudaSuccess)
         return e;
     }
-    put_rows_kernel<float2><<<grid1(n * nb * cz), 256, 0, st>>>(X, Rn, n, nb, kb, cz);
+    put_rows_kernel<T><<<grid1(n * nb * cz), 256, 0, st>>>(X, Rn, n, nb, kb, cz);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     launches += 11;
   }
@@ -313,7 +333,7 @@ static size_t corr_plane_bytes(int64_t n) { return (size_t)24 * n * emul_kpad(n)
 // inversion before and those of the correction after it
 static size_t shared_plane_bytes(int64_t n) {
   size_t b = emul_digit_bytes(2 * n, n);
-  if (gj_tc_plane_bytes(n) > b) b = gj_tc_plane_bytes(n);
+  if (gj_tc_plane_bytes<float2>(n) > b) b = gj_tc_plane_bytes<float2>(n);
   if (corr_plane_bytes(n) > b) b = corr_plane_bytes(n);
   return b;
 }
@@ -394,6 +414,115 @@ cudaError_t screened_refine(double2* X, int64_t n, int64_t count, void* work, si
     if (nsteps == 0) {
       if ((e = identity_minus(Xc, n, cz, +1.0, st)) != cudaSuccess) return e;
       launches += 1;
+    }
+  }
+  if (nlaunch) *nlaunch += launches;
+  return cudaSuccess;
+}
+
+// ------------------------------------------------------------------ the same for real matrices
+// Where the folded block's matrices are real (a q that is its own negative) the inversion, the
+// residual products and the correction are real GEMMs: a quarter of the embedded complex
+// products' work and half the bytes of every pass.  Order n even, so that a row of P~0 is also
+// the interleaved row of n / 2 complex entries that the A-operand kernels read.
+
+__global__ void f_from_iminus_real_kernel(const double* __restrict__ X, float* __restrict__ F, int64_t n, int64_t tot) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = e % (n * n);
+    F[e] = (float)((r / n == r % n ? 1.0 : 0.0) - X[e]);
+  }
+}
+__global__ void x_from_f_real_kernel(const float* __restrict__ F, double* __restrict__ X, int64_t tot) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x)
+    X[e] = (double)F[e];
+}
+// T <- I - Y + T
+__global__ void resid_real_kernel(const double* __restrict__ Y, double* __restrict__ T, int64_t n, int64_t tot) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = e % (n * n);
+    T[e] = (r / n == r % n ? 1.0 : 0.0) - Y[e] + T[e];
+  }
+}
+// Y <- Y + F  (last: minus I as well)
+__global__ void y_update_real_kernel(double* __restrict__ Y, const float* __restrict__ F, int64_t n, int64_t tot,
+                                     int last) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = e % (n * n);
+    Y[e] = Y[e] + (double)F[e] - ((last && r / n == r % n) ? 1.0 : 0.0);
+  }
+}
+
+static size_t shared_plane_bytes_real(int64_t n) {
+  size_t b = emul_digit_bytes(n, n / 2);
+  if (gj_tc_plane_bytes<float>(n) > b) b = gj_tc_plane_bytes<float>(n);
+  const size_t corr = (size_t)16 * n * emul_kpad(n / 2);   // hi/lo of Y (n rows) and of E^T (n rows)
+  return corr > b ? corr : b;
+}
+
+size_t screened_refine_real_bytes(int64_t n, int64_t chunk) {
+  const int64_t n2 = n * n;
+  return al256((size_t)chunk * n2 * 4) + al256(gj_work_bytes<float>(n, chunk)) + al256((size_t)chunk * n2 * 8) +
+         al256((size_t)chunk * emul_digit_bytes(n, n / 2)) + al256((size_t)chunk * shared_plane_bytes_real(n)) +
+         2 * al256((size_t)chunk * n * sizeof(int));
+}
+
+cudaError_t screened_refine_real(double* X, int64_t n, int64_t count, void* work, size_t work_bytes, int nsteps,
+                                 int* d_info, int* d_err, cudaStream_t st, int64_t* nlaunch) {
+  if (n < 2 || n % 2 || emul_launches_real(n) < 0 || nsteps < 1) return cudaErrorInvalidValue;
+  if (count <= 0) return cudaSuccess;
+  if (screened_refine_real_bytes(n, 1) > work_bytes) return cudaErrorMemoryAllocation;
+  int64_t lo = 1, hi = count < 65535 ? count : 65535;
+  while (lo < hi) {
+    const int64_t mid = (lo + hi + 1) / 2;
+    if (screened_refine_real_bytes(n, mid) <= work_bytes) lo = mid; else hi = mid - 1;
+  }
+  const int64_t nchunks = (count + lo - 1) / lo;
+  const int64_t chunk = (count + nchunks - 1) / nchunks;
+  const int64_t n2 = n * n;
+  constexpr int kLeadDigits = 5;   // as in screened_refine
+  cudaError_t e;
+  int64_t launches = 0;
+  for (int64_t z0 = 0; z0 < count; z0 += chunk) {
+    const int64_t cz = (count - z0) < chunk ? (count - z0) : chunk;
+    const int64_t tot = cz * n2;
+    double* Xc = X + z0 * n2;
+    char* p = (char*)work;
+    float* F = (float*)p;    p += al256((size_t)chunk * n2 * 4);
+    void* pan = p;           p += al256(gj_work_bytes<float>(n, chunk));
+    double* T = (double*)p;  p += al256((size_t)chunk * n2 * 8);
+    float* Ad = (float*)p;   p += al256((size_t)chunk * emul_digit_bytes(n, n / 2));
+    float* Bd = (float*)p;   p += al256((size_t)chunk * shared_plane_bytes_real(n));
+    int* Ae = (int*)p;       p += al256((size_t)chunk * n * sizeof(int));
+    int* Be = (int*)p;
+    if ((e = emul_split_rows((const double2*)Xc, cz, n, n / 2, n / 2, n2 / 2, Ad, Ae, st)) != cudaSuccess) return e;
+    f_from_iminus_real_kernel<<<grid1(tot), 256, 0, st>>>(Xc, F, n, tot);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = gj_blocked_tc<float>(F, n, cz, pan, Bd, d_info, d_err, st, &launches)) != cudaSuccess) return e;
+    x_from_f_real_kernel<<<grid1(tot), 256, 0, st>>>(F, Xc, tot);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    launches += 3;
+    for (int s = 0; s < nsteps; ++s) {
+      if ((e = emul_split_cols_real(Xc, cz, n, n, n, n2, Bd, Be, st)) != cudaSuccess) return e;
+      const int nd = s == nsteps - 1 ? 8 : kLeadDigits;
+      if ((e = emul_rgemm_batched(Ad, Ae, Bd, Be, cz, n, n, n, T, d_err, st, nd)) != cudaSuccess) return e;
+      resid_real_kernel<<<grid1(tot), 256, 0, st>>>(Xc, T, n, tot);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      {
+        const int64_t Kp = emul_kpad(n / 2);
+        float* Yh = Bd;
+        float* Yl = Yh + cz * n * Kp;
+        float* Eh = Yl + cz * n * Kp;
+        float* El = Eh + cz * n * Kp;
+        if ((e = split_rows(Xc, true, cz * n, n / 2, n / 2, false, Yh, Yl, Kp, st)) != cudaSuccess) return e;
+        if ((e = transpose_split_batched(T, true, cz, n, n, n, n2, Eh, El, Kp, n * Kp, st)) != cudaSuccess) return e;
+        UmmaOperand a{Yh, Yl, n, cz, Kp, n * Kp}, b{Eh, El, n, cz, Kp, n * Kp};
+        if ((e = umma_gemm(a, b, (int)n, (int)n, Kp, (int)cz, F, false, 1.0, false, n, n2, 3, d_err, st, 1, 0, 0, 0, 0,
+                           nullptr, nullptr, n)) != cudaSuccess)
+          return e;
+      }
+      y_update_real_kernel<<<grid1(tot), 256, 0, st>>>(Xc, F, n, tot, s == nsteps - 1 ? 1 : 0);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      launches += 6 + emul_launches_real(n, nd);
     }
   }
   if (nlaunch) *nlaunch += launches;

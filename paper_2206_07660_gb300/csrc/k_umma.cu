@@ -76,6 +76,8 @@ struct UmmaArgs {
   const int* eB;
   int64_t ea_zs, eb_zs;
   int64_t ea_div, eb_div;
+  int eb_sh;           // column n uses exponent entry (n >> eb_sh) / eb_div: 1 complex pairs, 0 real columns
+  const int* row_list; // non-null: outer row part o lands at row_list[o] * row_s1
   int64_t ea_mod;      // > 0: row m uses eA[z*ea_zs + (m/ea_div) % ea_mod]
   int eshift;
   // o_half != 0: the fp32 output is written as 16-bit hi (C) / lo (C_lo) pieces (1 fp16, 2 bf16)
@@ -112,7 +114,7 @@ __device__ __forceinline__ int row_exp(const UmmaArgs& a, int z, int64_t m) {
   return a.eA[zlin(a, z, a.ea_zs, a.ea_zso) + i] + a.eshift;
 }
 __device__ __forceinline__ int col_exp(const UmmaArgs& a, int z, int64_t n) {
-  return a.eB ? a.eB[zlin(a, z, a.eb_zs, a.eb_zso) + exp_index(n >> 1, a.eb_div)] : 0;
+  return a.eB ? a.eB[zlin(a, z, a.eb_zs, a.eb_zso) + exp_index(n >> a.eb_sh, a.eb_div)] : 0;
 }
 __device__ __forceinline__ int out_exp(const UmmaArgs& a, int z, int64_t m) {
   return a.eO ? a.eO[zlin(a, z, a.eo_zs, a.eo_zso) + exp_index(m, a.eo_div)] + a.eo_shift : 0;
@@ -894,7 +896,8 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
         {
           const int64_t ro = a.row_inner >= ((int64_t)1 << 31) ? 0 : (int64_t)((uint32_t)row / (uint32_t)a.row_inner);
           const int64_t ri = row - ro * a.row_inner;
-          myoff = zlin(a, z, a.c_zs, a.c_zso) + ro * a.row_s1 + ri * a.c_ld;
+          const int64_t rl = a.row_list && row < a.M ? (int64_t)a.row_list[ro] : ro;
+          myoff = zlin(a, z, a.c_zs, a.c_zso) + rl * a.row_s1 + ri * a.c_ld;
         }
         const bool rok = row < a.M;
         float* C = (float*)a.C;
@@ -905,7 +908,7 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
         const int64_t ebase = a.eB ? zlin(a, z, a.eb_zs, a.eb_zso) : 0;
         const bool bconst = a.eb_div >= ((int64_t)1 << 30) || !a.eB;
         const int cconst = (a.eB && bconst) ? a.eB[ebase] : 0;
-        auto colexp = [&](int n) { return a.eB ? a.eB[ebase + exp_index(n >> 1, a.eb_div)] : 0; };
+        auto colexp = [&](int n) { return a.eB ? a.eB[ebase + exp_index(n >> a.eb_sh, a.eb_div)] : 0; };
         for (int cb = 0; cb < BW; cb += 32) {
           uint32_t v[32];
           asm volatile(
@@ -1311,6 +1314,10 @@ cudaError_t umma_gemm(const UmmaOperand& A, const UmmaOperand& B, int M, int N, 
     a.ea_div = scale->ea_div > 0 ? scale->ea_div : 1;
     a.eb_div = scale->eb_div > 0 ? scale->eb_div : 1;
     a.ea_mod = scale->ea_mod > 0 ? scale->ea_mod : 0;
+    a.eb_sh = scale->real_cols ? 0 : 1;
+    // a listed outer row is resolved by the lane-per-row write-out only
+    if (scale->row_list && !a.direct) return cudaErrorInvalidValue;
+    a.row_list = scale->row_list;
   }
   int bn = cost_model_bn(N);
   if (g_force_bn) return umma_launch(g_force_bn, A, B, Kpad, nseg, a, batch, st);

@@ -1,4 +1,4 @@
-"""P~0 folded over (q, tau) -> (-q, beta - tau): only half of the (q, tau) blocks are
+"""The bosonic block folded by its symmetries.  P~0 folded over (q, tau) -> (-q, beta - tau): only half of the (q, tau) blocks are
 contracted and the others are their conjugates.  Compared with the oracle, which
 computes every block, over meshes whose q are their own negatives or come in pairs,
 even and odd tau counts, parts of the q range, a G that is not Hermitian, and a V whose
@@ -63,3 +63,46 @@ def test_polarization_of_loosely_paired_v(precision):
     g.set("G_tau", G)
     g.polarization()
     assert rel(g.get("P0_tau"), ogw.polarization_tau(sysd["V"], G, km)) < max(TOL[precision], 1e-11)
+
+
+@pytest.mark.parametrize("kmesh,ntau,naux,qr", [((2, 2, 1), 16, 20, None), ((2, 1, 1), 15, 21, None),
+                                                ((3, 1, 1), 16, 19, None), ((3, 2, 1), 13, 33, None),
+                                                ((4, 1, 1), 14, 16, (1, 3)), ((4, 1, 1), 14, 17, (0, 4)),
+                                                ((1, 1, 1), 12, 1, None)])
+def test_screened_block(kmesh, ntau, naux, qr):
+    # P~0(i Omega), P~(i Omega) and P~(tau) from P~0(tau): frequencies +-Omega and q-points +-q folded,
+    # real matrices where q = -q (odd orders padded); FP64 accuracy of the refined solve, the last
+    # transform amplifying rounding by the condition of the grid (~1e2 here)
+    sysd = system(4, naux, kmesh, ntau, 20.0, 81)
+    km = ogw.KMesh(kmesh)
+    st = ogw.State(sysd)
+    st.G_tau = -hermitian_noise((ntau, km.nk, 4, 4), 0.05, 82) - 0.3 * np.eye(4)
+    st.sigma()
+    g = gpu(sysd)
+    if qr is not None:
+        g.set_q_range(*qr)
+    g.set("G_tau", st.G_tau)
+    g.polarization()
+    qs = list(range(km.nk) if qr is None else range(*qr))
+    assert rel(g.get("P0_iw")[qs], st.P0_iw[qs]) < 1e-11
+    g.screened()
+    assert rel(g.get("P_iw")[qs], st.P_iw[qs]) < 1e-11
+    assert rel(g.get("P_tau")[qs], st.P_tau[qs]) < 1e-10
+
+
+@pytest.mark.parametrize("defect", [0.0, 1e-3])
+def test_screened_of_a_given_p0(defect):
+    # a P~0(i Omega) that is handed in is folded only when it has the symmetries
+    kmesh, ntau, naux = (3, 2, 1), 14, 18
+    sysd = system(4, naux, kmesh, ntau, 20.0, 83)
+    km = ogw.KMesh(kmesh)
+    st = ogw.State(sysd)
+    st.G_tau = -hermitian_noise((ntau, km.nk, 4, 4), 0.05, 84) - 0.3 * np.eye(4)
+    st.sigma()
+    P0 = st.P0_iw + defect * hermitian_noise(st.P0_iw.shape, 1.0, 85)
+    g = gpu(sysd)
+    g.set("P0_iw", P0)
+    g.screened()
+    ref = ogw.screened(P0)
+    assert rel(g.get("P_iw"), ref) < 1e-11
+    assert rel(g.get("P_tau"), ogw.herm(ogw.to_matsubara(st.grid.TBb, ref, 1))) < 1e-10
