@@ -39,6 +39,8 @@ struct View {   // the context's tensors seen by the adjoint chains (same layout
   const float2* G32;
   const float2* P32;
   float2* bar32;                  // complex64 copy of the symmetrised cotangent
+  bool fold;                      // P~0^{-q}(tau_{n-1-j}) = conj P~0^q(tau_j): V is paired
+  const int* kneg;                // index of -q (host)
 };
 }  // namespace gwadj
 
@@ -49,6 +51,17 @@ static GettDesc desc(int64_t M, int64_t N, int64_t K, int64_t Z) {
   d.alpha = make_double2(1, 0); d.beta = make_double2(0, 0);
   d.ksplit = 1;
   return d;
+}
+// Split of a reduction of K terms into nao x nao outputs, Z of them: enough blocks for about four
+// rounds of the SMs (Z = ntau alone leaves most of them idle), at least 64 terms each, within the
+// workspace.
+static int split_of(const gwadj::View& v, int64_t K, int64_t Z) {
+  const int64_t per = (int64_t)v.nao * v.nao * Z * (v.c64 ? 8 : 16);
+  const int64_t tiles = (int64_t)((v.nao + 31) / 32) * ((v.nao + 31) / 32);
+  int64_t s = (4 * 152 + Z * tiles - 1) / (Z * tiles);
+  if (s > K / 64) s = K / 64;
+  if (s > (int64_t)(v.ws_bytes / per)) s = (int64_t)(v.ws_bytes / per);
+  return s < 1 ? 1 : (int)s;
 }
 // operands in the View's arithmetic type; C is an intermediate of that type, or (out)
 // one of the fp64 cotangent outputs
@@ -73,14 +86,27 @@ cudaError_t polarization_vjp(const View& v, const double2* Pbar, double2* Gbar, 
   cudaError_t e;
   double2* Pr = v.bufC;   // herm(Pbar) for one q at a time
   for (int q = 0; q < nk; ++q) {
-    if ((e = cudaMemcpyAsync(Pr, Pbar + (size_t)q * ntau * na2, (size_t)ntau * na2 * 16, cudaMemcpyDeviceToDevice,
-                             v.st)))
+    // With the fold, P~0 at (-q, beta - tau) is the conjugate of P~0 at (q, tau) for any G, so the
+    // cotangent of the first is the conjugate's contribution to that of the second and half of the
+    // (q, tau) chains are left (nao 26, naux 200, 2x1x1, ntau 92 in FP64, forward and backward:
+    // 175 -> 101 ms).
+    const int nq = v.kneg[q];
+    if (v.fold && nq < q) continue;
+    const int nt = v.fold && nq == q ? (ntau + 1) / 2 : ntau;
+    if (v.fold) {
+      if ((e = fold_cotangent(Pr, Pbar + (size_t)q * ntau * na2, Pbar + (size_t)nq * ntau * na2, na2, nt, ntau,
+                              nq == q, v.st)))
+        return e;
+      *launches += 1;
+    } else if ((e = cudaMemcpyAsync(Pr, Pbar + (size_t)q * ntau * na2, (size_t)ntau * na2 * 16,
+                                    cudaMemcpyDeviceToDevice, v.st))) {
       return e;
-    if ((e = herm_batched(Pr, naux, ntau, na2, v.st))) return e;
+    }
+    if ((e = herm_batched(Pr, naux, nt, na2, v.st))) return e;
     *launches += 1;
     const void* Pa = Pr;
     if (v.c64) {
-      if ((e = to_c64(Pr, v.bar32, (int64_t)ntau * na2, v.st))) return e;
+      if ((e = to_c64(Pr, v.bar32, (int64_t)nt * na2, v.st))) return e;
       Pa = v.bar32;
       *launches += 1;
     }
@@ -89,13 +115,13 @@ cudaError_t polarization_vjp(const View& v, const double2* Pbar, double2* Gbar, 
       const void* V1 = at(v, v.V, v.V32, ((int64_t)k * nk + kq) * slab);
       const void* V2 = at(v, v.V, v.V32, ((int64_t)kq * nk + k) * slab);
       // X[t][Q'][(d,a)] = sum_Q Pr[t][Q][Q'] conj(V1[Q][(d,a)])
-      GettDesc d1 = desc(naux, n2, naux, ntau);
+      GettDesc d1 = desc(naux, n2, naux, nt);
       d1.am = I1(1); d1.ak = I1(naux); d1.az = I1(na2);
       d1.bk = I1(n2); d1.bn = I1(1); d1.conjB = true;
       d1.cm = I1(n2); d1.cn = I1(1); d1.cz = I1(slab);
       if ((e = run(v, d1, Pa, V1, v.bufA))) return e;
       // Y[t][Q'][c][a] = sum_d conj(Gm[t][c][d]) X[t][Q'][d][a],  Gm(t) = -G^k(t_{n-1-j})
-      GettDesc d2 = desc(nao, (int64_t)naux * nao, nao, ntau);
+      GettDesc d2 = desc(nao, (int64_t)naux * nao, nao, nt);
       d2.am = I1(nao); d2.ak = I1(1); d2.az = I1(-gstep); d2.conjA = true;
       d2.bk = I1(nao); d2.bn = I2(nao, n2, 1); d2.bz = I1(slab);
       d2.cm = I1(nao); d2.cn = I2(nao, n2, 1); d2.cz = I1(slab);
@@ -103,24 +129,26 @@ cudaError_t polarization_vjp(const View& v, const double2* Pbar, double2* Gbar, 
       const void* Gm = at(v, v.G_tau, v.G32, (int64_t)(ntau - 1) * gstep + (int64_t)k * n2);
       if ((e = run(v, d2, Gm, v.bufA, v.bufB))) return e;
       // G'bar[t][a][b] += f sum_{Q',c} Y[t][Q'][c][a] conj(V2[Q'][b][c])
-      GettDesc d3 = desc(nao, nao, (int64_t)naux * nao, ntau);
+      GettDesc d3 = desc(nao, nao, (int64_t)naux * nao, nt);
       d3.am = I1(1); d3.ak = I2(nao, n2, nao); d3.az = I1(slab);
       d3.bk = I2(nao, n2, 1); d3.bn = I1(nao); d3.conjB = true;
       d3.cm = I1(nao); d3.cn = I1(1); d3.cz = I1(gstep);
       d3.alpha = make_double2(f, 0); d3.beta = make_double2(1, 0);
+      d3.ksplit = split_of(v, d3.K, nt);
       if ((e = run(v, d3, v.bufB, V2, Gbar + (size_t)kq * n2, true))) return e;
       // T[t][Q'][d][b] = sum_a X[t][Q'][d][a] conj(G'[t][a][b])
-      GettDesc d4 = desc((int64_t)naux * nao, nao, nao, ntau);
+      GettDesc d4 = desc((int64_t)naux * nao, nao, nao, nt);
       d4.am = I1(nao); d4.ak = I1(1); d4.az = I1(slab);
       d4.bk = I1(nao); d4.bn = I1(1); d4.bz = I1(gstep); d4.conjB = true;
       d4.cm = I1(nao); d4.cn = I1(1); d4.cz = I1(slab);
       if ((e = run(v, d4, v.bufA, at(v, v.G_tau, v.G32, (int64_t)kq * n2), v.bufB))) return e;
       // Gm bar[t][c][d] = f sum_{Q',b} conj(V2[Q'][b][c]) T[t][Q'][d][b];  G^k(t_{n-1-j}) gets -Gm bar(t_j)
-      GettDesc d5 = desc(nao, nao, (int64_t)naux * nao, ntau);
+      GettDesc d5 = desc(nao, nao, (int64_t)naux * nao, nt);
       d5.am = I1(1); d5.ak = I2(nao, n2, nao); d5.conjA = true;
       d5.bk = I2(nao, n2, 1); d5.bn = I1(nao); d5.bz = I1(slab);
       d5.cm = I1(nao); d5.cn = I1(1); d5.cz = I1(-gstep);
       d5.alpha = make_double2(-f, 0); d5.beta = make_double2(1, 0);
+      d5.ksplit = split_of(v, d5.K, nt);
       if ((e = run(v, d5, V2, v.bufB, Gbar + (size_t)(ntau - 1) * gstep + (size_t)k * n2, true))) return e;
       *launches += 5;
     }
@@ -169,6 +197,7 @@ cudaError_t selfenergy_vjp(const View& v, const double2* Sbar, double2* Gbar, do
       d3.bk = I2(nao, n2, 1); d3.bn = I1(nao); d3.conjB = true;
       d3.cm = I1(nao); d3.cn = I1(1); d3.cz = I1(gstep);
       d3.alpha = make_double2(f, 0); d3.beta = make_double2(1, 0);
+      d3.ksplit = split_of(v, d3.K, ntau);
       if ((e = run(v, d3, v.bufB, V2, Gbar + (size_t)kmq * n2, true))) return e;
       // H[t][Q][j][a] = sum_i Sr[t][k][i][j] conj(V1[Q][i][a])
       GettDesc d4 = desc(nao, (int64_t)naux * nao, nao, ntau);

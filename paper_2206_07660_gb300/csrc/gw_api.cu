@@ -2055,6 +2055,8 @@ struct View {
   const float2* G32;
   const float2* P32;
   float2* bar32;
+  bool fold;
+  const int* kneg;
 };
 cudaError_t polarization_vjp(const View& v, const double2* Pbar, double2* Gbar, int64_t* launches);
 cudaError_t selfenergy_vjp(const View& v, const double2* Sbar, double2* Gbar, double2* Pbar, int64_t* launches);
@@ -2103,6 +2105,7 @@ static gw_status adj_view(gw_ctx* c, gwadj::View* v) {
   v->ws = c->ws; v->ws_bytes = c->ws_bytes;
   v->bufA = c->adjA; v->bufB = c->adjB; v->bufC = c->adjC;
   v->st = c->st;
+  v->fold = c->fold; v->kneg = c->kneg.data();
   v->c64 = false; v->V32 = nullptr; v->G32 = nullptr; v->P32 = nullptr; v->bar32 = nullptr;
   return GW_OK;
 }

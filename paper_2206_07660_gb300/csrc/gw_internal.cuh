@@ -99,6 +99,10 @@ cudaError_t fold_pack_real(const double2* P, const FoldView& f, const int* qlist
                            cudaStream_t st);
 cudaError_t fold_pack_cplx(const double2* P, const FoldView& f, const int* qlist, int nz, double2* X,
                            cudaStream_t st);
+// Pr[t] = A[t] + conj B[ntau - 1 - t] for t < nt (matrices of na2 entries); with self the middle
+// of an odd ntau, its own image, is A[t] alone
+cudaError_t fold_cotangent(double2* Pr, const double2* A, const double2* B, int64_t na2, int nt, int ntau, bool self,
+                           cudaStream_t st);
 cudaError_t fold_check(const double2* P, const FoldView& f, double* out, cudaStream_t st);
 
 struct DysonArgs {

@@ -150,6 +150,26 @@ cudaError_t fold_pack_cplx(const double2* P, const FoldView& f, const int* qlist
   return cudaGetLastError();
 }
 
+__global__ void fold_cotangent_kernel(double2* __restrict__ Pr, const double2* __restrict__ A,
+                                      const double2* __restrict__ B, int64_t na2, int nt, int ntau, int self) {
+  const int64_t tot = (int64_t)nt * na2;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
+    const int t = (int)(e / na2);
+    double2 a = A[e];
+    if (!(self && 2 * t == ntau - 1)) {
+      const double2 b = B[(ntau - 1 - t) * na2 + (e - t * na2)];
+      a.x += b.x;
+      a.y -= b.y;
+    }
+    Pr[e] = a;
+  }
+}
+cudaError_t fold_cotangent(double2* Pr, const double2* A, const double2* B, int64_t na2, int nt, int ntau, bool self,
+                           cudaStream_t st) {
+  fold_cotangent_kernel<<<grid1(nt * na2), 256, 0, st>>>(Pr, A, B, na2, nt, ntau, self ? 1 : 0);
+  return cudaGetLastError();
+}
+
 __device__ __forceinline__ void amax_nonneg(double* p, double v) {
   atomicMax((unsigned long long*)p, (unsigned long long)__double_as_longlong(v));
 }

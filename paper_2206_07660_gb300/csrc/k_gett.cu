@@ -6,8 +6,8 @@
 // solve -- is a product of two tensor slices whose row, column and reduction
 // indices are each made of at most two strided parts.  One tiled kernel reads
 // all of them in place (no transposition copies).  On GB300 the fp64 pipe is
-// the bound for the fp64 instantiation, so the tile is sized for register
-// reuse (4x4 complex outputs per thread), not for bandwidth.
+// the bound for the fp64 instantiation: what a launch takes is its padded
+// multiply-adds, so the tile follows the shape.
 #include "gw_internal.cuh"
 
 namespace gwk {
@@ -29,16 +29,92 @@ __device__ __forceinline__ int64_t off2(int64_t i, const Idx2& d) {
   return o * d.s1 + (i - o * d.inner) * d.s0;
 }
 
-constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
+constexpr int BK = 16, NT = 256;
 
-template <typename TA, typename TB, typename TC, typename S>
-__global__ void __launch_bounds__(NT) gett_kernel(GettDesc d, const TA* __restrict__ A,
-                                                  const TB* __restrict__ B, TC* C,
-                                                  typename C2<S>::t* ws) {
+// One reduction step of the per-thread sums.  FP64: four multiply-adds per complex product.
+// FP32: the same four in the same order as two packed ones (fma.rn.f32x2 works on a register
+// pair at one issue slot), with A staged as (x, x, -y, y) so that only B's pair has to be
+// swapped:  (re, im) += (x, x) * (bx, by);  (re, im) += (-y, y) * (by, bx).
+template <typename S> struct Acc;
+template <> struct Acc<double> {
+  using A = double2;     // staged element of A
+  double2 v;
+  __device__ __forceinline__ static A stage(double2 a) { return a; }
+  __device__ __forceinline__ void zero() { v = make_double2(0.0, 0.0); }
+  __device__ __forceinline__ void mac(const A& a, const double2& b) {
+    v.x = fma(a.x, b.x, v.x);
+    v.x = fma(-a.y, b.y, v.x);
+    v.y = fma(a.x, b.y, v.y);
+    v.y = fma(a.y, b.x, v.y);
+  }
+  __device__ __forceinline__ double2 get() const { return v; }
+};
+template <> struct Acc<float> {
+  using A = float4;
+  unsigned long long v;
+  __device__ __forceinline__ static A stage(float2 a) { return make_float4(a.x, a.x, -a.y, a.y); }
+  __device__ __forceinline__ static unsigned long long pack(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+  }
+  __device__ __forceinline__ void zero() { v = 0ull; }
+  __device__ __forceinline__ void mac(const A& a, const float2& b) {
+    const unsigned long long ar = pack(a.x, a.y), ai = pack(a.z, a.w), bb = pack(b.x, b.y), bs = pack(b.y, b.x);
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(v) : "l"(ar), "l"(bb));
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(v) : "l"(ai), "l"(bs));
+  }
+  __device__ __forceinline__ float2 get() const {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+  }
+};
+
+// The reduction index split of an operand with a host-made reciprocal: k = o * inner + i by a
+// multiplication and a shift (exact for k < 2^31) where a 64-bit division per element took
+// longer than the FP32 products it fed.
+struct KIdx {
+  uint32_t inner, mul;   // inner 0: one stride
+  int sh;
+  int64_t s1, s0;
+};
+static KIdx kidx_of(const Idx2& d, int64_t K) {
+  KIdx r{0, 0, 0, d.s1, d.s0};
+  if (d.inner >= K) return r;
+  int s = 0;
+  while (((int64_t)1 << s) < d.inner) ++s;
+  r.inner = (uint32_t)d.inner;
+  r.sh = 31 + s;
+  r.mul = (uint32_t)((((uint64_t)1 << (31 + s)) + (uint64_t)d.inner - 1) / (uint64_t)d.inner);
+  return r;
+}
+__device__ __forceinline__ int64_t koff(uint32_t k, const KIdx& d) {
+  if (d.inner == 0) return (int64_t)k * d.s0;
+  const uint32_t o = (uint32_t)(((uint64_t)k * d.mul) >> d.sh);
+  return (int64_t)o * d.s1 + (int64_t)(k - o * d.inner) * d.s0;
+}
+
+// Output tile of (TY TM) x (TX TN), TX TY = 256 threads with TM x TN complex sums each.  The
+// shape is picked per launch (pick_tile): the orbital index of this method is 4..64, and a
+// 64-wide tile spends most of the FP64 pipe on padding there.  Whole calls before / after: an FP64
+// iteration at nao 8, naux 32, 2x2x2 63.8 -> 9.3 ms (400 launches of 146 -> 15 us), P~0 of nao 26,
+// naux 200, 3x1x1 in FP64 170 -> 110 ms (1.1 TFLOP/s in the K = nao^2 products, the pipe's rate),
+// the complex64 gradient of Sigma~ at 2x2x1 123 -> 56 ms.
+// FP32: two blocks per SM (128 registers); with one, the loads of the next K tile were not hidden
+// (36 % of the stalls) and the 128 x 64 tile that needs them was no faster than this one.
+template <typename TA, typename TC, typename S, int TX, int TY, int TM, int TN>
+__global__ void __launch_bounds__(NT, sizeof(S) == 4 ? 2 : 1) gett_kernel(const __grid_constant__ GettDesc d, const __grid_constant__ KIdx ka,
+                                                  const __grid_constant__ KIdx kb_, const TA* __restrict__ A,
+                                                  const TA* __restrict__ B, TC* C, typename C2<S>::t* ws) {
+  static_assert(TX * TY == NT, "threads");
   using CS = typename C2<S>::t;
-  __shared__ CS As[BK][BM];
-  __shared__ CS Bs[BK][BN];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  constexpr int BM = TY * TM, BN = TX * TN;
+  constexpr int LA = (BK * BM + NT - 1) / NT, LB = (BK * BN + NT - 1) / NT;   // loads per thread
+  // one column of padding: the stores of a k-contiguous operand go down the columns
+  __shared__ typename Acc<S>::A As[BK][BM + 1];
+  __shared__ CS Bs[BK][BN + 1];
+  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
   const int64_t m0 = (int64_t)blockIdx.y * BM, n0 = (int64_t)blockIdx.x * BN;
   const int ks = d.ksplit > 1 ? d.ksplit : 1;
   // loader geometry: which of (m,k) / (k,n) is the contiguous index
@@ -50,79 +126,86 @@ __global__ void __launch_bounds__(NT) gett_kernel(GettDesc d, const TA* __restri
     const int64_t z = zz / ks;
     const int split = (int)(zz - z * ks);
     const TA* Az = A + off2(z, d.az);
-    const TB* Bz = B + off2(z, d.bz);
-    int64_t kbeg = 0, kend = d.K;
+    const TA* Bz = B + off2(z, d.bz);
+    int kbeg = 0, kend = (int)d.K;
     if (ks > 1) {
-      int64_t kc = (d.K + ks - 1) / ks;
+      int kc = (kend + ks - 1) / ks;
       kc = (kc + BK - 1) / BK * BK;
-      kbeg = split * kc;
-      kend = min(d.K, kbeg + kc);
+      kbeg = min(kend, split * kc);
+      kend = min(kend, kbeg + kc);
     }
-    // per-thread load coordinates
-    int am[4], ak[4], bkk[4], bnn[4];
+    int64_t aoff[LA], boff[LB];
+    bool aok[LA], bok[LB];
+    int am[LA], ak[LA], bn[LB], bk[LB];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      if (a_kfast) { ak[r] = tid % BK; am[r] = tid / BK + 16 * r; }
-      else         { am[r] = tid % BM; ak[r] = tid / BM + 4 * r; }
-      if (b_nfast) { bnn[r] = tid % BN; bkk[r] = tid / BN + 4 * r; }
-      else         { bkk[r] = tid % BK; bnn[r] = tid / BK + 16 * r; }
+    for (int r = 0; r < LA; ++r) {
+      const int e = tid + NT * r;
+      am[r] = a_kfast ? e / BK : e % BM;
+      ak[r] = a_kfast ? e % BK : e / BM;
+      const int64_t m = m0 + am[r];
+      aok[r] = m < d.M && e < BK * BM;
+      aoff[r] = aok[r] ? off2(m, d.am) : 0;
     }
-    int64_t aoff_m[4], boff_n[4];
-    bool aok_m[4], bok_n[4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      int64_t m = m0 + am[r];
-      aok_m[r] = m < d.M;
-      aoff_m[r] = aok_m[r] ? off2(m, d.am) : 0;
-      int64_t n = n0 + bnn[r];
-      bok_n[r] = n < d.N;
-      boff_n[r] = bok_n[r] ? off2(n, d.bn) : 0;
+    for (int r = 0; r < LB; ++r) {
+      const int e = tid + NT * r;
+      bn[r] = b_nfast ? e % BN : e / BK;
+      bk[r] = b_nfast ? e / BN : e % BK;
+      const int64_t n = n0 + bn[r];
+      bok[r] = n < d.N && e < BK * BN;
+      boff[r] = bok[r] ? off2(n, d.bn) : 0;
     }
-    CS acc[4][4];
+    Acc<S> acc[TM][TN];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) { acc[i][j].x = 0; acc[i][j].y = 0; }
+      for (int j = 0; j < TN; ++j) acc[i][j].zero();
 
-    CS ra[4], rb[4];
-    auto gload = [&](int64_t kt) {
+    CS ra[LA], rb[LB];
+    auto gload = [&](int kt) {
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        int64_t k = kt + ak[r];
+      for (int r = 0; r < LA; ++r) {
+        const int k = kt + ak[r];
         CS v; v.x = 0; v.y = 0;
-        if (aok_m[r] && k < kend) { v = cvt<S>(__ldg(Az + aoff_m[r] + off2(k, d.ak))); v.y *= sa; }
+        if (aok[r] && k < kend) { v = cvt<S>(__ldg(Az + aoff[r] + koff(k, ka))); v.y *= sa; }
         ra[r] = v;
-        int64_t kb = kt + bkk[r];
+      }
+#pragma unroll
+      for (int r = 0; r < LB; ++r) {
+        const int k = kt + bk[r];
         CS w; w.x = 0; w.y = 0;
-        if (bok_n[r] && kb < kend) { w = cvt<S>(__ldg(Bz + boff_n[r] + off2(kb, d.bk))); w.y *= sb; }
+        if (bok[r] && k < kend) { w = cvt<S>(__ldg(Bz + boff[r] + koff(k, kb_))); w.y *= sb; }
         rb[r] = w;
       }
     };
+    auto step = [&](int kk) {
+      typename Acc<S>::A a[TM];
+      CS b[TN];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) a[i] = As[kk][ty + TY * i];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) b[j] = Bs[kk][tx + TX * j];
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j].mac(a[i], b[j]);
+    };
     if (kbeg < kend) gload(kbeg);
-    for (int64_t kt = kbeg; kt < kend; kt += BK) {
+    for (int kt = kbeg; kt < kend; kt += BK) {
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        As[ak[r]][am[r]] = ra[r];
-        Bs[bkk[r]][bnn[r]] = rb[r];
-      }
+      for (int r = 0; r < LA; ++r)
+        if (BK * BM % NT == 0 || tid + NT * r < BK * BM) As[ak[r]][am[r]] = Acc<S>::stage(ra[r]);
+#pragma unroll
+      for (int r = 0; r < LB; ++r)
+        if (BK * BN % NT == 0 || tid + NT * r < BK * BN) Bs[bk[r]][bn[r]] = rb[r];
       __syncthreads();
-      if (kt + BK < kend) gload(kt + BK);
-#pragma unroll
-      for (int kk = 0; kk < BK; ++kk) {
-        CS a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            acc[i][j].x = fma(a[i].x, b[j].x, acc[i][j].x);
-            acc[i][j].x = fma(-a[i].y, b[j].y, acc[i][j].x);
-            acc[i][j].y = fma(a[i].x, b[j].y, acc[i][j].y);
-            acc[i][j].y = fma(a[i].y, b[j].x, acc[i][j].y);
-          }
+      const int left = kend - kt;
+      if (left > BK) gload(kt + BK);
+      if (left >= BK) {
+#pragma unroll 4
+        for (int kk = 0; kk < BK; ++kk) step(kk);
+      } else {
+        for (int kk = 0; kk < left; ++kk) step(kk);   // a K below the tile costs what it has
       }
       __syncthreads();
     }
@@ -130,30 +213,62 @@ __global__ void __launch_bounds__(NT) gett_kernel(GettDesc d, const TA* __restri
     if (ks > 1) {
       CS* W = ws + ((int64_t)split * d.Z + z) * d.M * d.N;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        int64_t m = m0 + ty + 16 * i;
+      for (int i = 0; i < TM; ++i) {
+        const int64_t m = m0 + ty + TY * i;
         if (m >= d.M) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          int64_t n = n0 + tx + 16 * j;
-          if (n < d.N) W[m * d.N + n] = acc[i][j];
+        for (int j = 0; j < TN; ++j) {
+          const int64_t n = n0 + tx + TX * j;
+          if (n < d.N) W[m * d.N + n] = acc[i][j].get();
+        }
+      }
+    } else if (d.alpha.y == 0.0 && d.beta.y == 0.0 && (d.beta.x == 0.0 || d.beta.x == 1.0)) {
+      // real alpha, C stored or added to: what every chain asks for.  FP64 instructions (and the
+      // conversions to and from it) hold the SM's pipe 16 cycles a warp, and ten of them per output
+      // took longer than an FP32 launch's products; here two conversions and two multiply-adds
+      // are left, none for an FP32 result scaled by +-1.
+      TC* Cz = C + off2(z, d.cz);
+      const bool rd = d.beta.x != 0.0;
+      const bool unit = fabs(d.alpha.x) == 1.0;
+      const S sg = d.alpha.x < 0.0 ? (S)-1 : (S)1;
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const int64_t m = m0 + ty + TY * i;
+        if (m >= d.M) continue;
+        const int64_t cmo = off2(m, d.cm);
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+          const int64_t n = n0 + tx + TX * j;
+          if (n >= d.N) continue;
+          TC* p = Cz + cmo + off2(n, d.cn);
+          const CS av = acc[i][j].get();
+          if (sizeof(TC) == sizeof(CS) && unit && !rd) {
+            TC o;
+            o.x = (decltype(o.x))(sg * av.x);
+            o.y = (decltype(o.y))(sg * av.y);
+            *p = o;
+          } else {
+            const double cx = rd ? (double)p->x : 0.0, cy = rd ? (double)p->y : 0.0;
+            *p = cvt_out<TC, double>(fma(d.alpha.x, (double)av.x, cx), fma(d.alpha.x, (double)av.y, cy));
+          }
         }
       }
     } else {
       TC* Cz = C + off2(z, d.cz);
       const bool rd = (d.beta.x != 0.0 || d.beta.y != 0.0);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        int64_t m = m0 + ty + 16 * i;
+      for (int i = 0; i < TM; ++i) {
+        const int64_t m = m0 + ty + TY * i;
         if (m >= d.M) continue;
-        int64_t cmo = off2(m, d.cm);
+        const int64_t cmo = off2(m, d.cm);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          int64_t n = n0 + tx + 16 * j;
+        for (int j = 0; j < TN; ++j) {
+          const int64_t n = n0 + tx + TX * j;
           if (n >= d.N) continue;
           TC* p = Cz + cmo + off2(n, d.cn);
           // epilogue in double: a fp32 product slab is added to an fp64 C exactly
-          double ax = (double)acc[i][j].x, ay = (double)acc[i][j].y;
+          const CS av = acc[i][j].get();
+          double ax = (double)av.x, ay = (double)av.y;
           double re = d.alpha.x * ax - d.alpha.y * ay;
           double im = d.alpha.x * ay + d.alpha.y * ax;
           if (rd) {
@@ -200,49 +315,79 @@ size_t gett_ws_bytes(const GettDesc& d, Ty acc) {
   return (size_t)d.ksplit * d.Z * d.M * d.N * (acc == Ty::C128 ? 16 : 8);
 }
 
-template <typename TA, typename TB, typename TC, typename S>
-static cudaError_t launch(const GettDesc& d, const void* A, const void* B, void* C, void* ws,
-                          cudaStream_t st) {
-  if (d.M <= 0 || d.N <= 0 || d.Z <= 0) return cudaSuccess;
-  int ks = d.ksplit > 1 ? d.ksplit : 1;
+template <typename TA, typename TC, typename S, int TX, int TY, int TM, int TN>
+static cudaError_t launch_t(const GettDesc& d, const void* A, const void* B, void* C, void* ws, cudaStream_t st) {
+  constexpr int BM = TY * TM, BN = TX * TN;
+  const int ks = d.ksplit > 1 ? d.ksplit : 1;
   dim3 grid((unsigned)((d.N + BN - 1) / BN), (unsigned)((d.M + BM - 1) / BM),
             (unsigned)(d.Z * ks < 65535 ? d.Z * ks : 65535));
   if (grid.y > 65535) return cudaErrorInvalidConfiguration;
-  gett_kernel<TA, TB, TC, S><<<grid, NT, 0, st>>>(d, (const TA*)A, (const TB*)B, (TC*)C,
-                                                  (typename C2<S>::t*)ws);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || ks == 1) return e;
+  gett_kernel<TA, TC, S, TX, TY, TM, TN><<<grid, NT, 0, st>>>(d, kidx_of(d.ak, d.K), kidx_of(d.bk, d.K), (const TA*)A,
+                                                              (const TA*)B, (TC*)C, (typename C2<S>::t*)ws);
+  return cudaGetLastError();
+}
+
+// Tile shapes, wide ones first.  cost: time per output element of a full tile relative to the
+// widest.  In FP64 a warp's multiply-add holds the SM's pipe for 16 cycles, so the shared-memory
+// reads of small per-thread tiles hide behind it and padding decides; in FP32 the reads count.
+struct Tile { int bm, bn; float c64, c32; };
+static const Tile kTiles[] = {{64, 64, 1.00f, 1.0f}, {64, 32, 1.02f, 1.2f}, {32, 64, 1.02f, 1.2f},
+                              {32, 32, 1.04f, 1.6f}, {64, 16, 1.08f, 1.8f}, {16, 64, 1.08f, 1.8f},
+                              {16, 32, 1.12f, 2.2f}, {64, 8, 1.15f, 2.6f},  {8, 64, 1.15f, 2.6f},
+                              {16, 16, 1.25f, 3.2f}};
+static int pick_tile(const GettDesc& d, bool f64) {
+  int best = 0;
+  double bt = 1e300;
+  const int ks = d.ksplit > 1 ? d.ksplit : 1;
+  for (int i = 0; i < (int)(sizeof(kTiles) / sizeof(Tile)); ++i) {
+    const Tile& t = kTiles[i];
+    const int64_t mt = (d.M + t.bm - 1) / t.bm;
+    if (mt > 65535) continue;
+    const int64_t blocks = mt * ((d.N + t.bn - 1) / t.bn) * d.Z * ks;
+    // whole blocks per SM, or the average once there are many
+    const double per_sm = blocks < 152 * 8 ? (double)((blocks + 151) / 152) : (double)blocks / 152.0;
+    const double tt = per_sm * t.bm * t.bn * (f64 ? t.c64 : t.c32);
+    if (tt < bt * 0.999) { bt = tt; best = i; }
+  }
+  return best;
+}
+
+template <typename TA, typename TC, typename S>
+static cudaError_t launch(const GettDesc& d, const void* A, const void* B, void* C, void* ws,
+                          cudaStream_t st) {
+  if (d.M <= 0 || d.N <= 0 || d.Z <= 0) return cudaSuccess;
+  if (d.K > INT32_MAX - BK) return cudaErrorInvalidValue;
+  constexpr bool f64 = sizeof(S) == 8;
+  cudaError_t e;
+  switch (pick_tile(d, f64)) {
+    case 1: e = launch_t<TA, TC, S, 16, 16, 4, 2>(d, A, B, C, ws, st); break;
+    case 2: e = launch_t<TA, TC, S, 16, 16, 2, 4>(d, A, B, C, ws, st); break;
+    case 3: e = launch_t<TA, TC, S, 16, 16, 2, 2>(d, A, B, C, ws, st); break;
+    case 4: e = launch_t<TA, TC, S, 16, 16, 4, 1>(d, A, B, C, ws, st); break;
+    case 5: e = launch_t<TA, TC, S, 16, 16, 1, 4>(d, A, B, C, ws, st); break;
+    case 6: e = launch_t<TA, TC, S, 16, 16, 1, 2>(d, A, B, C, ws, st); break;
+    case 7: e = launch_t<TA, TC, S, 8, 32, 2, 1>(d, A, B, C, ws, st); break;
+    case 8: e = launch_t<TA, TC, S, 32, 8, 1, 2>(d, A, B, C, ws, st); break;
+    case 9: e = launch_t<TA, TC, S, 16, 16, 1, 1>(d, A, B, C, ws, st); break;
+    default: e = launch_t<TA, TC, S, 16, 16, 4, 4>(d, A, B, C, ws, st); break;
+  }
+  if (e != cudaSuccess || d.ksplit <= 1) return e;
   int64_t total = d.M * d.N * d.Z;
   int64_t nb = (total + 255) / 256; int blocks = (int)(nb < 152 * 16 ? nb : 152 * 16);
   splitk_reduce<TC, S><<<blocks, 256, 0, st>>>(d, (const typename C2<S>::t*)ws, (TC*)C);
   return cudaGetLastError();
 }
 
-template <typename TA, typename TB, typename TC>
-static cudaError_t disp_acc(const GettDesc& d, const void* A, const void* B, void* C, Ty acc, void* ws,
-                            cudaStream_t st) {
-  return acc == Ty::C128 ? launch<TA, TB, TC, double>(d, A, B, C, ws, st)
-                         : launch<TA, TB, TC, float>(d, A, B, C, ws, st);
-}
-template <typename TA, typename TB>
-static cudaError_t disp_c(const GettDesc& d, const void* A, const void* B, void* C, Ty tc, Ty acc,
-                          void* ws, cudaStream_t st) {
-  return tc == Ty::C128 ? disp_acc<TA, TB, double2>(d, A, B, C, acc, ws, st)
-                        : disp_acc<TA, TB, float2>(d, A, B, C, acc, ws, st);
-}
-template <typename TA>
-static cudaError_t disp_b(const GettDesc& d, const void* A, const void* B, Ty tb, void* C, Ty tc, Ty acc,
-                          void* ws, cudaStream_t st) {
-  return tb == Ty::C128 ? disp_c<TA, double2>(d, A, B, C, tc, acc, ws, st)
-                        : disp_c<TA, float2>(d, A, B, C, tc, acc, ws, st);
-}
-
+// the three forms in use: complex128 throughout, and complex64 operands with FP32 sums into a
+// complex64 or complex128 result
 cudaError_t gett(const GettDesc& d, const void* A, Ty ta, const void* B, Ty tb, void* C, Ty tc, Ty acc,
                  void* ws, size_t ws_bytes, cudaStream_t st) {
   if (d.ksplit > 1 && (ws == nullptr || ws_bytes < gett_ws_bytes(d, acc)))
     return cudaErrorInvalidValue;
-  return ta == Ty::C128 ? disp_b<double2>(d, A, B, tb, C, tc, acc, ws, st)
-                        : disp_b<float2>(d, A, B, tb, C, tc, acc, ws, st);
+  if (ta != tb || ta != acc) return cudaErrorInvalidValue;
+  if (ta == Ty::C128) return tc == Ty::C128 ? launch<double2, double2, double>(d, A, B, C, ws, st) : cudaErrorInvalidValue;
+  return tc == Ty::C128 ? launch<float2, double2, float>(d, A, B, C, ws, st)
+                        : launch<float2, float2, float>(d, A, B, C, ws, st);
 }
 
 }  // namespace gwk
