@@ -355,7 +355,7 @@ static cudaError_t transform(gw_ctx* c, const double2* T, const double2* X, doub
                                      Y + z * ystride, ncol, c->emA, c->emAe, c->info + 1, c->st);
       if (e != cudaSuccess) return e;
     }
-    count((int)(batch * (1 + emul_launches(K))));
+    count((int)(2 * batch));
     return cudaSuccess;
   }
   GettDesc d = base_desc(nrow, ncol, K, batch);
@@ -522,7 +522,7 @@ static cudaError_t fold_forward(gw_ctx* c) {
       if (e) return e;
       e = real ? fold_expand_pairs(c->P_iw, f, list + a, nz, Y, c->st) : fold_expand_cplx(c->P_iw, f, list + a, nz, Y, c->st);
       if (e) return e;
-      count(2 + emul_launches_real(K));
+      count(3);
     }
   }
   return cudaSuccess;
@@ -574,7 +574,7 @@ static cudaError_t fold_screened(gw_ctx* c) {
                                     (int64_t)c->nwb * na2, nz, list + a, c->d_rep, c->P_tau, (int64_t)c->ntau * na2,
                                     list + a, Ad, (int*)p, c->info + 1, c->st)))
         return e;
-      count(1 + emul_launches_real(K));
+      count(2);
     }
   }
   count(1);

@@ -209,8 +209,6 @@ struct UmmaScale {
   int eshift;
   int64_t ea_div = 1, eb_div = 1;   // row m uses eA[z*ea_zs + m/ea_div], column n eB[z*eb_zs + (n/2)/eb_div]
   int64_t ea_mod = 0;               // > 0: row m uses eA[z*ea_zs + (m/ea_div) % ea_mod]
-  bool real_cols = false;           // column n uses eB[z*eb_zs + n/eb_div] (a real product)
-  const int* row_list = nullptr;    // outer row part o lands at row_list[o] * row_s1 (lane-per-row write-out only)
 };
 // 16-bit pieces as the output of a GEMM (C: hi, C_lo: lo, fp32-class layout in 16-bit
 // elements): D * 2^-(eO[z*eo_zs + m/eo_div] + eo_shift) in fp16 (half = 1) or bf16 (2)
@@ -235,6 +233,23 @@ cudaError_t umma_gemm(const UmmaOperand& A, const UmmaOperand& B, int M, int N, 
                       int64_t col_inner = 0, int64_t col_s1 = 0, float* C_lo = nullptr,
                       const UmmaScale* scale = nullptr, int64_t kvalid = 0, const UmmaOut* out = nullptr,
                       const UmmaZ* zz = nullptr);
+// One GEMM of digit operands (k_digit.cu): C = sum over the kept digit pairs of A (M rows) and B
+// (N rows, planes in reverse order), planes of Kp reals, K of them holding data; batch entries packed.
+struct DigitGemm {
+  const void *Ad, *Bd;
+  const int *eA, *eB;            // exponents: [batch][M], [batch][N] (real_cols) or [batch][N/2]
+  int64_t batch, M, N, K, Kp;
+  int nd;                        // 8, or 5 for the leading digits
+  bool real_cols;
+  double* C;                     // [batch][M][N], or with pairs (batch 1) double2 (2p, 2p+1) of row
+  bool pairs;                    //   o * row_inner + i at row_list[o] (or o) * row_s1 + 2 i + p * col_s1
+  int64_t row_inner, row_s1, col_s1;
+  const int* row_list;
+  const double* Y;               // row-major only: C = I - Y + A B
+  int* err;
+};
+cudaError_t digit_gemm(const DigitGemm& d, cudaStream_t st);
+int64_t digit_kmax(int nd);
 // FP64 complex products on tensor cores by exact digit splitting (k_emul.cu)
 int64_t emul_kpad(int64_t K);
 size_t emul_digit_bytes(int64_t rows, int64_t K);
@@ -257,16 +272,17 @@ cudaError_t emul_transform_multi(const void* Bd, const int* Be, int64_t npair, c
 cudaError_t emul_split_cols_real(const double* B, int64_t count, int64_t K, int64_t N, int64_t ldb, int64_t sb,
                                  void* Bd, int* Be, cudaStream_t st);
 cudaError_t emul_rgemm_batched(const void* Ad, const int* Ae, const void* Bd, const int* Be, int64_t count,
-                               int64_t M, int64_t N, int64_t K, double* C, int* err, cudaStream_t st, int nd = 8);
-int emul_launches_real(int64_t K, int nd = 8);
-// tensor-core launches of one product with complex K and nd digits (-1: K too large)
-int emul_launches(int64_t K, int nd = 8);
+                               int64_t M, int64_t N, int64_t K, double* C, int* err, cudaStream_t st, int nd = 8,
+                               const double* Y = nullptr);
+// whether a product of complex K fits the digit sums
+bool emul_fits(int64_t K);
 cudaError_t emul_split_rows(const double2* A, int64_t count, int64_t M, int64_t K, int64_t lda, int64_t sa,
                             void* Ad, int* Ae, cudaStream_t st);
 cudaError_t emul_split_cols(const double2* B, int64_t count, int64_t K, int64_t N, int64_t ldb, int64_t sb,
                             void* Bd, int* Be, cudaStream_t st);
 cudaError_t emul_cgemm_batched(const void* Ad, const int* Ae, const void* Bd, const int* Be, int64_t count,
-                               int64_t M, int64_t N, int64_t K, double2* C, int* err, cudaStream_t st, int nd = 8);
+                               int64_t M, int64_t N, int64_t K, double2* C, int* err, cudaStream_t st, int nd = 8,
+                               const double2* Y = nullptr);   // Y: C = I - Y + A B
 
 // ldo: row stride of the output planes (0: Kpad)
 cudaError_t split_rows(const void* src, bool src_c128, int64_t rows, int64_t K, int64_t ld, bool conj, float* hi,

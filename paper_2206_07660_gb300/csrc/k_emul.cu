@@ -1,27 +1,21 @@
-// FP64 complex GEMMs on the TF32 tensor cores by exact digit splitting.
+// FP64 GEMMs on the tensor cores by exact digit splitting.
 //
 // Each real value x of an operand row is written x = 2^e sum_{i=1..S} d_i 2^(-7 i)
 // with one exponent e per row (max |x| <= 2^e) and integer digits d_i
 // (|d_1| <= 128, |d_i| <= 64 for i > 1, balanced rounding), i.e. 56 bits.
-// Every digit is an integer that TF32 holds exactly, every digit product has at
+// Every digit is an integer that fp16 holds exactly, every digit product has at
 // most 14 bits (|d_1 d_1| <= 2^14, |d_1 d_j| <= 2^13, |d_i d_j| <= 2^12 for i, j > 1),
-// and the pairs of one launch are chosen so that the sum over its pairs of K times
-// that bound stays <= 2^24: every partial sum is an integer below 2^24 and the
-// tensor pipe's FP32 accumulation of a launch is exact.  The product
+// and K is limited so that the sum over the pairs of one significance i + j stays
+// <= 2^24: every partial sum is an integer below 2^24 and the tensor pipe's FP32
+// accumulation is exact.  The product
 //   x_A x_B = 2^(eA + eB) sum_{i,j} d_i d_j 2^(-7 (i + j))
-// keeps the pairs with i + j <= S + 1 (36 of them); each launch covers pairs of
-// one i + j and is added into the FP64 output with the exact scale
-// 2^(eA + eB - 7 (i + j)) (the tensor-core GEMM's scaled FP64 epilogue).  The
-// dropped pairs and the truncated digits leave an error below ~2^-54 relative to
-// K max|A_row| max|B_col|, at the level of an FP64 GEMM.
+// keeps the pairs with i + j <= S + 1 (36 of them), all in one pass over the digits
+// (k_digit.cu).  The dropped pairs and the truncated digits leave an error below
+// ~2^-54 relative to K max|A_row| max|B_col|, at the level of an FP64 GEMM.
 //
 // Operand layout: digit planes of a row are stored one after another,
-// [row][S][Kp] (Kp = padded real K), so the K range of a launch is contiguous.
-// The digits are stored as fp16 (exact for |d| <= 2048) and multiplied with
-// tcgen05 kind::f16 (FP32 accumulation): half the bytes of TF32 storage and twice
-// the tensor rate, with the same exact sums.
-// B's planes are stored in reverse digit order so that the B slices that pair
-// with A slices i0..i1 of a launch are contiguous as well.
+// [row][S][Kp] (Kp = padded real K), as fp16 (tcgen05 kind::f16, FP32 accumulation);
+// B's planes in reverse digit order.
 //
 // Used for the tau <-> i nu transforms Y[z] = T X[z]: A = X[z]^T (rows = columns
 // of X, complex K = ntau), B = T (rows 2m, 2m+1 = the real 2x2 blocks of T[m][j]),
@@ -39,27 +33,51 @@ constexpr int EM_BETA = 7;
 constexpr int EM_S = 8;
 static_assert(EM_BETA == 7, "the balanced digit masks below are for 7-bit digits");
 
-// digits of x / 2^e (|x| <= 2^e): d[0..S-1].  x is rounded once to a multiple of
-// 2^(e - 7S) (an exact integer v with |v| <= 2^(7S) = 2^56), whose balanced base-128
-// digits d_S .. d_2 in [-64, 63] are peeled off with integer shifts; the rest is
-// d_1 (|d_1| <= 128).
-__device__ __forceinline__ void em_digits(double x, int e, float* d) {
-  long long v = __double2ll_rn(ldexp(x, EM_BETA * EM_S - e));
+// Digits of a pair (x, y) over 2^e (|x|, |y| <= 2^e) as half2 values d[0..S-1].  Each value is
+// rounded once to a multiple of 2^(e - 7S), an integer v with |v| <= 2^56, from the bits of the
+// double (integer shifts: the FP64 pipe and the 64-bit conversions run at 1/64 of the integer rate
+// here, and took longer than the memory traffic).  Adding 64 in every 7-bit place turns the
+// balanced digits d_S .. d_2 in [-64, 63] into plain bit fields; the rest is d_1 (|d_1| <= 128).
+// A field n becomes the fp16 value by its place in 1024 + n, whose bits are 0x6400 + n.
+__device__ __forceinline__ long long em_fixed(double x, int e) {
+  const long long b = __double_as_longlong(x);
+  const int ex = (int)(b >> 52) & 0x7ff;
+  const long long m = (b & 0xfffffffffffffll) | (ex ? 0x10000000000000ll : 0ll);
+  const int sh = (ex ? ex : 1) - 1075 + EM_BETA * EM_S - e;
+  long long v;
+  if (sh >= 0) {
+    v = m << (sh < 10 ? sh : 10);   // |x| <= 2^e: sh <= 4
+  } else if (sh >= -54) {
+    const long long half = 1ll << (-sh - 1);
+    v = (m + half - 1 + ((m >> -sh) & 1)) >> -sh;   // to nearest, ties to even
+  } else {
+    v = 0;
+  }
+  v = b < 0 ? -v : v;
+  constexpr long long kBias = 64ll * (((1ll << 49) - 1) / 127);   // 64 (1 + 128 + ... + 128^6)
+  return v + kBias;
+}
+__device__ __forceinline__ void em_digits2(double x, double y, int e, __half2* d) {
+  const long long wx = em_fixed(x, e), wy = em_fixed(y, e);
 #pragma unroll
   for (int i = EM_S - 1; i >= 1; --i) {
-    const long long di = ((v + 64) & 127) - 64;
-    d[i] = (float)di;
-    v = (v - di) >> EM_BETA;
+    const int s = EM_BETA * (EM_S - 1 - i);
+    uint32_t n = ((uint32_t)(wx >> s) & 127u) | (((uint32_t)(wy >> s) & 127u) << 16) | 0x64006400u;
+    d[i] = __hsub2(*(__half2*)&n, __floats2half2_rn(1088.f, 1088.f));
   }
-  d[0] = (float)v;
+  uint32_t n = (uint32_t)((int)(wx >> 49) + 512) | ((uint32_t)((int)(wy >> 49) + 512) << 16);
+  n += 0x64006400u;
+  d[0] = __hsub2(*(__half2*)&n, __floats2half2_rn(1536.f, 1536.f));
 }
 
-__device__ __forceinline__ int em_exponent(double m) {
-  if (!(m > 0.0)) return 0;
-  int e;
-  frexp(m, &e);   // m = f 2^e, f in [0.5, 1): m < 2^e
-  return e;
+__device__ __forceinline__ __half2 em_conj(__half2 d) {   // (re, -im)
+  uint32_t n = *(uint32_t*)&d ^ 0x80000000u;
+  return *(__half2*)&n;
 }
+
+// biased exponent of |x| (0 for zero and subnormals); the row exponent e of a largest one: m < 2^e
+__device__ __forceinline__ int em_bexp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ int em_exponent(int bexp) { return bexp ? bexp - 1022 : 0; }
 
 // A-operand digits from a transposed source: row n of the operand is column n of a
 // K x ncol complex matrix (element (n, k) at src[z*zs + k*ld + n]), real K index
@@ -76,7 +94,7 @@ __global__ void __launch_bounds__(256) em_split_t_kernel(const double2* __restri
                                                          const int* __restrict__ zlist,
                                                          const int* __restrict__ klist) {
   __shared__ double2 tile[32][33];
-  __shared__ double red[8][32];
+  __shared__ int red[8][32];
   __shared__ int es[32];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t z = blockIdx.y;
@@ -91,17 +109,17 @@ __global__ void __launch_bounds__(256) em_split_t_kernel(const double2* __restri
     if (!RR) return X[krow(j) * ld + c];
     return make_double2(X[krow(2 * j) * ld + c].x, 2 * j + 1 < Kin ? X[krow(2 * j + 1) * ld + c].x : 0.0);
   };
-  double m = 0.0;
+  int m = 0;
   if (n < ncol)
     for (int64_t j = ty; j < K; j += 8) {
       const double2 v = load(j, n);
-      m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
+      m = max(m, max(em_bexp(v.x), em_bexp(v.y)));
     }
   red[ty][tx] = m;
   __syncthreads();
   if (ty == 0) {
-    double mm = red[0][tx];
-    for (int r = 1; r < 8; ++r) mm = fmax(mm, red[r][tx]);
+    int mm = red[0][tx];
+    for (int r = 1; r < 8; ++r) mm = max(mm, red[r][tx]);
     const int e = em_exponent(mm);
     es[tx] = e;
     if (n < ncol) E[n] = e;
@@ -119,12 +137,11 @@ __global__ void __launch_bounds__(256) em_split_t_kernel(const double2* __restri
       const int64_t row = n0 + rr, j = j0 + tx;
       if (row < ncol && 2 * j < Kp) {
         const double2 v = tile[tx][rr];
-        float dr[EM_S], di[EM_S];
-        em_digits(v.x, es[rr], dr);
-        em_digits(v.y, es[rr], di);
+        __half2 d[EM_S];
+        em_digits2(v.x, v.y, es[rr], d);
         dig_t* o = D + row * rowlen + 2 * j;
 #pragma unroll
-        for (int i = 0; i < EM_S; ++i) *(__half2*)(o + (int64_t)i * Kp) = __floats2half2_rn(dr[i], di[i]);
+        for (int i = 0; i < EM_S; ++i) *(__half2*)(o + (int64_t)i * Kp) = d[i];
       }
     }
     __syncthreads();
@@ -137,16 +154,16 @@ __global__ void __launch_bounds__(256) em_split_t_kernel(const double2* __restri
 __global__ void em_split_b_kernel(const double2* __restrict__ B, int64_t rows, int64_t K, int64_t ldb,
                                   dig_t* __restrict__ dig, int* __restrict__ ex, int64_t Kp) {
   const int64_t m = blockIdx.x;
-  __shared__ double red[256];
-  double mx = 0.0;
+  __shared__ int red[256];
+  int mx = 0;
   for (int64_t j = threadIdx.x; j < K; j += blockDim.x) {
     const double2 v = B[m * ldb + j];
-    mx = fmax(mx, fmax(fabs(v.x), fabs(v.y)));
+    mx = max(mx, max(em_bexp(v.x), em_bexp(v.y)));
   }
   red[threadIdx.x] = mx;
   __syncthreads();
   for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + s]);
+    if ((int)threadIdx.x < s) red[threadIdx.x] = max(red[threadIdx.x], red[threadIdx.x + s]);
     __syncthreads();
   }
   const int e = em_exponent(red[0]);
@@ -154,16 +171,15 @@ __global__ void em_split_b_kernel(const double2* __restrict__ B, int64_t rows, i
   const int64_t rowlen = (int64_t)EM_S * Kp;
   for (int64_t j = threadIdx.x; j < K; j += blockDim.x) {
     const double2 v = B[m * ldb + j];
-    float dr[EM_S], di[EM_S];
-    em_digits(v.x, e, dr);
-    em_digits(v.y, e, di);
+    __half2 d[EM_S];
+    em_digits2(v.x, v.y, e, d);
     dig_t* r0 = dig + (2 * m) * rowlen + 2 * j;
     dig_t* r1 = dig + (2 * m + 1) * rowlen + 2 * j;
 #pragma unroll
     for (int i = 0; i < EM_S; ++i) {
       const int64_t p = (int64_t)(EM_S - 1 - i) * Kp;   // reverse digit order
-      *(__half2*)(r0 + p) = __floats2half2_rn(dr[i], -di[i]);
-      *(__half2*)(r1 + p) = __floats2half2_rn(di[i], dr[i]);
+      *(__half2*)(r0 + p) = em_conj(d[i]);
+      *(__half2*)(r1 + p) = __lowhigh2highlow(d[i]);
     }
   }
 }
@@ -179,28 +195,22 @@ __global__ void __launch_bounds__(256) em_split_r_kernel(const double2* __restri
   if (gr >= rows * count) return;
   const int64_t z = gr / rows, r = gr - z * rows;
   const double2* x = src + z * zs + r * ld;
-  double m = 0.0;
+  int m = 0;
   for (int64_t k = lane; k < K; k += 32) {
     const double2 v = x[k];
-    m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
+    m = max(m, max(em_bexp(v.x), em_bexp(v.y)));
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
   const int e = em_exponent(m);
   if (lane == 0) ex[gr] = e;
   dig_t* o = dig + gr * (int64_t)EM_S * Kp;
   for (int64_t k = lane; 2 * k < Kp; k += 32) {
-    float dr[EM_S], di[EM_S];
-    if (k < K) {
-      const double2 v = x[k];
-      em_digits(v.x, e, dr);
-      em_digits(v.y, e, di);
-    } else {
+    const double2 v = k < K ? x[k] : make_double2(0.0, 0.0);
+    __half2 d[EM_S];
+    em_digits2(v.x, v.y, e, d);
 #pragma unroll
-      for (int i = 0; i < EM_S; ++i) dr[i] = di[i] = 0.f;
-    }
-#pragma unroll
-    for (int i = 0; i < EM_S; ++i) *(__half2*)(o + (int64_t)i * Kp + 2 * k) = __floats2half2_rn(dr[i], di[i]);
+    for (int i = 0; i < EM_S; ++i) *(__half2*)(o + (int64_t)i * Kp + 2 * k) = d[i];
   }
 }
 
@@ -213,7 +223,7 @@ __global__ void __launch_bounds__(256) em_split_bt_kernel(const double2* __restr
                                                           int64_t ld, int64_t zs, dig_t* __restrict__ dig,
                                                           int* __restrict__ ex, int64_t Kp) {
   __shared__ double2 tile[32][33];
-  __shared__ double red[8][32];
+  __shared__ int red[8][32];
   __shared__ int es[32];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t z = blockIdx.y;
@@ -223,17 +233,17 @@ __global__ void __launch_bounds__(256) em_split_bt_kernel(const double2* __restr
   int* E = ex + z * ncol;
   const int64_t n0 = (int64_t)blockIdx.x * 32;
   const int64_t n = n0 + tx;
-  double m = 0.0;
+  int m = 0;
   if (n < ncol)
     for (int64_t j = ty; j < K; j += 8) {
       const double2 v = X[j * ld + n];
-      m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
+      m = max(m, max(em_bexp(v.x), em_bexp(v.y)));
     }
   red[ty][tx] = m;
   __syncthreads();
   if (ty == 0) {
-    double mm = red[0][tx];
-    for (int r = 1; r < 8; ++r) mm = fmax(mm, red[r][tx]);
+    int mm = red[0][tx];
+    for (int r = 1; r < 8; ++r) mm = max(mm, red[r][tx]);
     const int e = em_exponent(mm);
     es[tx] = e;
     if (n < ncol) E[n] = e;
@@ -250,16 +260,15 @@ __global__ void __launch_bounds__(256) em_split_bt_kernel(const double2* __restr
       const int64_t col = n0 + rr, j = j0 + tx;
       if (col < ncol && j < kc) {
         const double2 v = tile[tx][rr];
-        float dr[EM_S], di[EM_S];
-        em_digits(v.x, es[rr], dr);
-        em_digits(v.y, es[rr], di);
+        __half2 d[EM_S];
+        em_digits2(v.x, v.y, es[rr], d);
         dig_t* r0 = D + (2 * col) * rowlen + 2 * j;
         dig_t* r1 = r0 + rowlen;
 #pragma unroll
         for (int i = 0; i < EM_S; ++i) {
           const int64_t p = (int64_t)(EM_S - 1 - i) * Kp;
-          *(__half2*)(r0 + p) = __floats2half2_rn(dr[i], -di[i]);
-          *(__half2*)(r1 + p) = __floats2half2_rn(di[i], dr[i]);
+          *(__half2*)(r0 + p) = em_conj(d[i]);
+          *(__half2*)(r1 + p) = __lowhigh2highlow(d[i]);
         }
       }
     }
@@ -296,9 +305,9 @@ static int em_plan(int64_t kreal, EmLaunch* out, int nd = EM_S) {
 }
 constexpr int EM_MAXL = EM_S * EM_S;
 
-int emul_launches(int64_t K, int nd) {
+bool emul_fits(int64_t K) {
   EmLaunch pl[EM_MAXL];
-  return em_plan(2 * K, pl, nd);
+  return em_plan(2 * K, pl) > 0;
 }
 
 // real K padded to whole 128-byte k-blocks of fp16
@@ -321,27 +330,17 @@ cudaError_t emul_split_b(const double2* B, int64_t rows, int64_t K, int64_t ldb,
 cudaError_t emul_transform(const void* Bdv, const int* Be, int64_t nrow, const double2* X, int64_t K, int64_t ncol,
                            int64_t ldx, double2* Y, int64_t ldy, void* Adv, int* Ae, int* err, cudaStream_t st) {
   if (ldy != ncol) return cudaErrorInvalidValue;   // transposed lane-per-row stores assume packed rows
-  const dig_t* Bd = (const dig_t*)Bdv;
   dig_t* Ad = (dig_t*)Adv;
   const int64_t Kp = emul_kpad(K);
   em_split_t_kernel<false><<<dim3((unsigned)((ncol + 31) / 32), 1), 256, 0, st>>>(X, K, ncol, ldx, 0, Ad, Ae, Kp,
                                                                                    nullptr, nullptr);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int64_t ld = (int64_t)EM_S * Kp;
-  EmLaunch pl[EM_MAXL];
-  const int nl = em_plan(2 * K, pl);
-  if (nl < 0) return cudaErrorInvalidValue;
-  for (int l = 0; l < nl; ++l) {
-    const int g = pl[l].g, i0 = pl[l].i0, np = pl[l].i1 - pl[l].i0 + 1;
-    UmmaOperand oa{(const float*)(Ad + (int64_t)(i0 - 1) * Kp), nullptr, ncol, 1, ld, 0, 1};
-    UmmaOperand ob{(const float*)(Bd + (int64_t)(EM_S - g + i0) * Kp), nullptr, 2 * nrow, 1, ld, 0, 1};
-    UmmaScale sc{Ae, Be, 0, 0, -EM_BETA * g};
-    e = umma_gemm(oa, ob, (int)ncol, (int)(2 * nrow), (int64_t)np * Kp, 1, (void*)Y, true, 1.0, l > 0, 2, 0, 1,
-                  err, st, 1, 0, 0, 2, 2 * ldy, nullptr, &sc, (int64_t)(np - 1) * Kp + 2 * K);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  DigitGemm d{};
+  d.Ad = Ad; d.Bd = Bdv; d.eA = Ae; d.eB = Be;
+  d.batch = 1; d.M = ncol; d.N = 2 * nrow; d.K = 2 * K; d.Kp = Kp; d.nd = EM_S;
+  d.C = (double*)Y; d.pairs = true; d.col_s1 = 2 * ldy; d.err = err;
+  return digit_gemm(d, st);
 }
 
 // Real rows of the B operand in pairs: rows 2p, 2p + 1 of a real matrix B [rows][K], digit
@@ -349,13 +348,13 @@ cudaError_t emul_transform(const void* Bdv, const int* Be, int64_t nrow, const d
 __global__ void __launch_bounds__(256) em_split_br_kernel(const double* __restrict__ B, int64_t K,
                                                           dig_t* __restrict__ dig, int* __restrict__ ex, int64_t Kp) {
   const int64_t p = blockIdx.x;
-  __shared__ double red[256];
-  double mx = 0.0;
-  for (int64_t e = threadIdx.x; e < 2 * K; e += blockDim.x) mx = fmax(mx, fabs(B[2 * p * K + e]));
+  __shared__ int red[256];
+  int mx = 0;
+  for (int64_t e = threadIdx.x; e < 2 * K; e += blockDim.x) mx = max(mx, em_bexp(B[2 * p * K + e]));
   red[threadIdx.x] = mx;
   __syncthreads();
   for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + s]);
+    if ((int)threadIdx.x < s) red[threadIdx.x] = max(red[threadIdx.x], red[threadIdx.x + s]);
     __syncthreads();
   }
   const int e = em_exponent(red[0]);
@@ -363,10 +362,10 @@ __global__ void __launch_bounds__(256) em_split_br_kernel(const double* __restri
   const int64_t rowlen = (int64_t)EM_S * Kp;
   for (int64_t i = threadIdx.x; i < 2 * Kp; i += blockDim.x) {
     const int64_t r = i / Kp, k = i - r * Kp;
-    float d[EM_S];
-    em_digits(k < K ? B[(2 * p + r) * K + k] : 0.0, e, d);
+    __half2 d[EM_S];
+    em_digits2(k < K ? B[(2 * p + r) * K + k] : 0.0, 0.0, e, d);
 #pragma unroll
-    for (int s = 0; s < EM_S; ++s) dig[(2 * p + r) * rowlen + (int64_t)(EM_S - 1 - s) * Kp + k] = __float2half_rn(d[s]);
+    for (int s = 0; s < EM_S; ++s) dig[(2 * p + r) * rowlen + (int64_t)(EM_S - 1 - s) * Kp + k] = __low2half(d[s]);
   }
 }
 
@@ -382,7 +381,6 @@ cudaError_t emul_transform_multi(const void* Bdv, const int* Be, int64_t npair, 
                                  bool real_rows, int64_t ncol, int64_t zs, int nz, const int* zlist,
                                  const int* klist, double2* Y, int64_t yzs, const int* ylist, void* Adv, int* Ae,
                                  int* err, cudaStream_t st) {
-  const dig_t* Bd = (const dig_t*)Bdv;
   dig_t* Ad = (dig_t*)Adv;
   const int64_t Kp = emul_kpad((K + 1) / 2), rows = nz * ncol;
   if (nz < 1 || nz > 65535 || rows > INT32_MAX || (!real_rows && K % 2)) return cudaErrorInvalidValue;
@@ -391,26 +389,12 @@ cudaError_t emul_transform_multi(const void* Bdv, const int* Be, int64_t npair, 
   else em_split_t_kernel<false><<<grid, 256, 0, st>>>(X, K / 2, ncol, ncol, zs, Ad, Ae, Kp, zlist, klist);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int64_t ld = (int64_t)EM_S * Kp;
-  EmLaunch pl[EM_MAXL];
-  const int nl = em_plan(K, pl);
-  if (nl < 0) return cudaErrorInvalidValue;
-  for (int l = 0; l < nl; ++l) {
-    const int g = pl[l].g, i0 = pl[l].i0, np = pl[l].i1 - pl[l].i0 + 1;
-    UmmaOperand oa{(const float*)(Ad + (int64_t)(i0 - 1) * Kp), nullptr, rows, 1, ld, 0, 1};
-    UmmaOperand ob{(const float*)(Bd + (int64_t)(EM_S - g + i0) * Kp), nullptr, 2 * npair, 1, ld, 0, 1};
-    UmmaScale sc{Ae, Be, 0, 0, -EM_BETA * g};
-    sc.row_list = ylist;
-    e = umma_gemm(oa, ob, (int)rows, (int)(2 * npair), (int64_t)np * Kp, 1, (void*)Y, true, 1.0, l > 0, 2, 0, 1, err,
-                  st, 1, ncol, 2 * yzs, 2, 2 * ncol, nullptr, &sc, (int64_t)(np - 1) * Kp + K);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
-int emul_launches_real(int64_t K, int nd) {
-  EmLaunch pl[EM_MAXL];
-  return em_plan(K, pl, nd);
+  DigitGemm d{};
+  d.Ad = Ad; d.Bd = Bdv; d.eA = Ae; d.eB = Be;
+  d.batch = 1; d.M = rows; d.N = 2 * npair; d.K = K; d.Kp = Kp; d.nd = EM_S;
+  d.C = (double*)Y; d.pairs = true; d.row_inner = ncol; d.row_s1 = 2 * yzs; d.col_s1 = 2 * ncol; d.row_list = ylist;
+  d.err = err;
+  return digit_gemm(d, st);
 }
 
 // Digits of the columns of real K x N matrices (one exponent per column), planes in reverse
@@ -419,7 +403,7 @@ __global__ void __launch_bounds__(256) em_split_btr_kernel(const double* __restr
                                                            int64_t ld, int64_t zs, dig_t* __restrict__ dig,
                                                            int* __restrict__ ex, int64_t Kp) {
   __shared__ double tile[64][33];
-  __shared__ double red[8][32];
+  __shared__ int red[8][32];
   __shared__ int es[32];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t z = blockIdx.y;
@@ -428,14 +412,14 @@ __global__ void __launch_bounds__(256) em_split_btr_kernel(const double* __restr
   dig_t* D = dig + z * ncol * rowlen;
   int* E = ex + z * ncol;
   const int64_t n0 = (int64_t)blockIdx.x * 32, n = n0 + tx;
-  double m = 0.0;
+  int m = 0;
   if (n < ncol)
-    for (int64_t j = ty; j < K; j += 8) m = fmax(m, fabs(X[j * ld + n]));
+    for (int64_t j = ty; j < K; j += 8) m = max(m, em_bexp(X[j * ld + n]));
   red[ty][tx] = m;
   __syncthreads();
   if (ty == 0) {
-    double mm = red[0][tx];
-    for (int r = 1; r < 8; ++r) mm = fmax(mm, red[r][tx]);
+    int mm = red[0][tx];
+    for (int r = 1; r < 8; ++r) mm = max(mm, red[r][tx]);
     const int e = em_exponent(mm);
     es[tx] = e;
     if (n < ncol) E[n] = e;
@@ -450,12 +434,11 @@ __global__ void __launch_bounds__(256) em_split_btr_kernel(const double* __restr
     for (int rr = ty; rr < 32; rr += 8) {
       const int64_t col = n0 + rr, j = j0 + 2 * tx;
       if (col < ncol && j < Kp) {
-        float d0[EM_S], d1[EM_S];
-        em_digits(tile[2 * tx][rr], es[rr], d0);
-        em_digits(tile[2 * tx + 1][rr], es[rr], d1);
+        __half2 d[EM_S];
+        em_digits2(tile[2 * tx][rr], tile[2 * tx + 1][rr], es[rr], d);
         dig_t* r0 = D + col * rowlen + j;
 #pragma unroll
-        for (int i = 0; i < EM_S; ++i) *(__half2*)(r0 + (int64_t)(EM_S - 1 - i) * Kp) = __floats2half2_rn(d0[i], d1[i]);
+        for (int i = 0; i < EM_S; ++i) *(__half2*)(r0 + (int64_t)(EM_S - 1 - i) * Kp) = d[i];
       }
     }
     __syncthreads();
@@ -472,25 +455,15 @@ cudaError_t emul_split_cols_real(const double* B, int64_t count, int64_t K, int6
 
 // C[z] (M x N real, packed) = A[z] B[z] from the digits of emul_split_rows (A's rows read as
 // K/2 complex entries) and emul_split_cols_real.
-cudaError_t emul_rgemm_batched(const void* Adv, const int* Ae, const void* Bdv, const int* Be, int64_t count,
-                               int64_t M, int64_t N, int64_t K, double* C, int* err, cudaStream_t st, int nd) {
-  const dig_t* Ad = (const dig_t*)Adv;
-  const dig_t* Bd = (const dig_t*)Bdv;
-  const int64_t Kp = emul_kpad(K / 2), ld = (int64_t)EM_S * Kp;
-  EmLaunch pl[EM_MAXL];
-  const int nl = em_plan(K, pl, nd);
-  if (nl < 0 || count > 65535) return cudaErrorInvalidValue;
-  for (int l = 0; l < nl; ++l) {
-    const int g = pl[l].g, i0 = pl[l].i0, np = pl[l].i1 - pl[l].i0 + 1;
-    UmmaOperand oa{(const float*)(Ad + (int64_t)(i0 - 1) * Kp), nullptr, M, count, ld, M * ld, 1};
-    UmmaOperand ob{(const float*)(Bd + (int64_t)(EM_S - g + i0) * Kp), nullptr, N, count, ld, N * ld, 1};
-    UmmaScale sc{Ae, Be, M, N, -EM_BETA * g};
-    sc.real_cols = true;
-    cudaError_t e = umma_gemm(oa, ob, (int)M, (int)N, (int64_t)np * Kp, (int)count, (void*)C, true, 1.0, l > 0, N,
-                              M * N, 1, err, st, 1, 0, 0, 0, 0, nullptr, &sc, (int64_t)(np - 1) * Kp + K);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+cudaError_t emul_rgemm_batched(const void* Ad, const int* Ae, const void* Bd, const int* Be, int64_t count,
+                               int64_t M, int64_t N, int64_t K, double* C, int* err, cudaStream_t st, int nd,
+                               const double* Y) {
+  if (count > 65535 || K % 2) return cudaErrorInvalidValue;
+  DigitGemm d{};
+  d.Ad = Ad; d.Bd = Bd; d.eA = Ae; d.eB = Be;
+  d.batch = count; d.M = M; d.N = N; d.K = K; d.Kp = emul_kpad(K / 2); d.nd = nd; d.real_cols = true;
+  d.C = C; d.Y = Y; d.err = err;
+  return digit_gemm(d, st);
 }
 
 // Digits of the batched operands of C[z] = A[z] B[z] (A: count x M x K complex, row
@@ -519,25 +492,15 @@ cudaError_t emul_split_cols(const double2* B, int64_t count, int64_t K, int64_t 
 // nd = 8 digits; nd < 8 keeps the pairs with i + j <= nd + 1 of the leading nd
 // digits: each real product then errs by up to ~(nd + 1) 2^(13 - 7 (nd + 2)) of
 // max|A_row| max|B_col| (9e-11 for nd = 5).
-cudaError_t emul_cgemm_batched(const void* Adv, const int* Ae, const void* Bdv, const int* Be, int64_t count,
-                               int64_t M, int64_t N, int64_t K, double2* C, int* err, cudaStream_t st, int nd) {
-  const dig_t* Ad = (const dig_t*)Adv;
-  const dig_t* Bd = (const dig_t*)Bdv;
-  const int64_t Kp = emul_kpad(K), ld = (int64_t)EM_S * Kp;
-  EmLaunch pl[EM_MAXL];
-  const int nl = em_plan(2 * K, pl, nd);
-  if (nl < 0 || count > 65535) return cudaErrorInvalidValue;
-  for (int l = 0; l < nl; ++l) {
-    const int g = pl[l].g, i0 = pl[l].i0, np = pl[l].i1 - pl[l].i0 + 1;
-    UmmaOperand oa{(const float*)(Ad + (int64_t)(i0 - 1) * Kp), nullptr, M, count, ld, M * ld, 1};
-    UmmaOperand ob{(const float*)(Bd + (int64_t)(EM_S - g + i0) * Kp), nullptr, 2 * N, count, ld, 2 * N * ld, 1};
-    UmmaScale sc{Ae, Be, M, N, -EM_BETA * g};
-    cudaError_t e = umma_gemm(oa, ob, (int)M, (int)(2 * N), (int64_t)np * Kp, (int)count, (void*)C, true, 1.0, l > 0,
-                              2 * N, 2 * M * N, 1, err, st, 1, 0, 0, 0, 0, nullptr, &sc,
-                              (int64_t)(np - 1) * Kp + 2 * K);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+cudaError_t emul_cgemm_batched(const void* Ad, const int* Ae, const void* Bd, const int* Be, int64_t count,
+                               int64_t M, int64_t N, int64_t K, double2* C, int* err, cudaStream_t st, int nd,
+                               const double2* Y) {
+  if (count > 65535) return cudaErrorInvalidValue;
+  DigitGemm d{};
+  d.Ad = Ad; d.Bd = Bd; d.eA = Ae; d.eB = Be;
+  d.batch = count; d.M = M; d.N = 2 * N; d.K = 2 * K; d.Kp = emul_kpad(K); d.nd = nd;
+  d.C = (double*)C; d.Y = (const double*)Y; d.err = err;
+  return digit_gemm(d, st);
 }
 
 }  // namespace gwk

@@ -303,15 +303,6 @@ __global__ void x_from_f_kernel(const float2* __restrict__ F, double2* __restric
     X[e] = make_double2((double)v.x, (double)v.y);
   }
 }
-// T <- I - Y + T
-__global__ void resid_kernel(const double2* __restrict__ Y, double2* __restrict__ T, int64_t n, int64_t tot) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e % (n * n);
-    const double d = (r / n == r % n) ? 1.0 : 0.0;
-    const double2 y = Y[e], t = T[e];
-    T[e] = make_double2(d - y.x + t.x, -y.y + t.y);
-  }
-}
 // Y <- Y + F  (last: minus I as well)
 __global__ void y_update_kernel(double2* __restrict__ Y, const float2* __restrict__ F, int64_t n, int64_t tot,
                                 int last) {
@@ -348,7 +339,7 @@ size_t screened_refine_bytes(int64_t n, int64_t chunk) {
          2 * al256((size_t)chunk * n * sizeof(int));              // exponents
 }
 
-bool screened_refine_ok(int64_t n) { return n >= 1 && emul_launches(n) > 0; }
+bool screened_refine_ok(int64_t n) { return n >= 1 && emul_fits(n); }
 
 cudaError_t screened_refine(double2* X, int64_t n, int64_t count, void* work, size_t work_bytes, int nsteps,
                             int* d_info, int* d_err, cudaStream_t st, int64_t* nlaunch) {
@@ -390,9 +381,8 @@ cudaError_t screened_refine(double2* X, int64_t n, int64_t count, void* work, si
     for (int s = 0; s < nsteps; ++s) {
       if ((e = emul_split_cols(Xc, cz, n, n, n, n2, Bd, Be, st)) != cudaSuccess) return e;
       const int nd = s == nsteps - 1 ? 8 : kLeadDigits;
-      if ((e = emul_cgemm_batched(Ad, Ae, Bd, Be, cz, n, n, n, T, d_err, st, nd)) != cudaSuccess) return e;
-      resid_kernel<<<grid1(tot), 256, 0, st>>>(Xc, T, n, tot);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      // T = I - Y + P~0 Y
+      if ((e = emul_cgemm_batched(Ad, Ae, Bd, Be, cz, n, n, n, T, d_err, st, nd, Xc)) != cudaSuccess) return e;
       // F = Y E  (split TF32 on the tensor cores, FP32 output: E is small)
       {
         const int64_t Kp = emul_kpad(n);
@@ -409,7 +399,7 @@ cudaError_t screened_refine(double2* X, int64_t n, int64_t count, void* work, si
       }
       y_update_kernel<<<grid1(tot), 256, 0, st>>>(Xc, F, n, tot, s == nsteps - 1 ? 1 : 0);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      launches += 6 + emul_launches(n, nd);
+      launches += 6;
     }
     if (nsteps == 0) {
       if ((e = identity_minus(Xc, n, cz, +1.0, st)) != cudaSuccess) return e;
@@ -436,13 +426,6 @@ __global__ void x_from_f_real_kernel(const float* __restrict__ F, double* __rest
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x)
     X[e] = (double)F[e];
 }
-// T <- I - Y + T
-__global__ void resid_real_kernel(const double* __restrict__ Y, double* __restrict__ T, int64_t n, int64_t tot) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e % (n * n);
-    T[e] = (r / n == r % n ? 1.0 : 0.0) - Y[e] + T[e];
-  }
-}
 // Y <- Y + F  (last: minus I as well)
 __global__ void y_update_real_kernel(double* __restrict__ Y, const float* __restrict__ F, int64_t n, int64_t tot,
                                      int last) {
@@ -468,7 +451,7 @@ size_t screened_refine_real_bytes(int64_t n, int64_t chunk) {
 
 cudaError_t screened_refine_real(double* X, int64_t n, int64_t count, void* work, size_t work_bytes, int nsteps,
                                  int* d_info, int* d_err, cudaStream_t st, int64_t* nlaunch) {
-  if (n < 2 || n % 2 || emul_launches_real(n) < 0 || nsteps < 1) return cudaErrorInvalidValue;
+  if (n < 2 || n % 2 || !emul_fits(n / 2) || nsteps < 1) return cudaErrorInvalidValue;
   if (count <= 0) return cudaSuccess;
   if (screened_refine_real_bytes(n, 1) > work_bytes) return cudaErrorMemoryAllocation;
   int64_t lo = 1, hi = count < 65535 ? count : 65535;
@@ -504,9 +487,7 @@ cudaError_t screened_refine_real(double* X, int64_t n, int64_t count, void* work
     for (int s = 0; s < nsteps; ++s) {
       if ((e = emul_split_cols_real(Xc, cz, n, n, n, n2, Bd, Be, st)) != cudaSuccess) return e;
       const int nd = s == nsteps - 1 ? 8 : kLeadDigits;
-      if ((e = emul_rgemm_batched(Ad, Ae, Bd, Be, cz, n, n, n, T, d_err, st, nd)) != cudaSuccess) return e;
-      resid_real_kernel<<<grid1(tot), 256, 0, st>>>(Xc, T, n, tot);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      if ((e = emul_rgemm_batched(Ad, Ae, Bd, Be, cz, n, n, n, T, d_err, st, nd, Xc)) != cudaSuccess) return e;
       {
         const int64_t Kp = emul_kpad(n / 2);
         float* Yh = Bd;
@@ -522,7 +503,7 @@ cudaError_t screened_refine_real(double* X, int64_t n, int64_t count, void* work
       }
       y_update_real_kernel<<<grid1(tot), 256, 0, st>>>(Xc, F, n, tot, s == nsteps - 1 ? 1 : 0);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      launches += 6 + emul_launches_real(n, nd);
+      launches += 6;
     }
   }
   if (nlaunch) *nlaunch += launches;

@@ -30,6 +30,7 @@
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
 #include "gw_internal.cuh"
+#include "umma_ptx.cuh"
 
 #include <map>
 #include <vector>
@@ -41,7 +42,6 @@ constexpr int UM_BM = 128;
 constexpr int UM_BK = 32;          // fp32 elements per 128-byte swizzle row
 constexpr int UM_STAGES = 3;          // 3 stages x 2 resident blocks per SM
 constexpr int UM_THREADS = 192;    // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue
-constexpr uint32_t UM_SPIN_LIMIT = 1u << 26;
 constexpr int UM_FLUSH = 4;       // k-blocks per tensor-pipe accumulation chunk
 static int g_persistent = 1;      // 1: persistent tile loop (umma_pkernel); 0: one tile per block
 
@@ -76,8 +76,6 @@ struct UmmaArgs {
   const int* eB;
   int64_t ea_zs, eb_zs;
   int64_t ea_div, eb_div;
-  int eb_sh;           // column n uses exponent entry (n >> eb_sh) / eb_div: 1 complex pairs, 0 real columns
-  const int* row_list; // non-null: outer row part o lands at row_list[o] * row_s1
   int64_t ea_mod;      // > 0: row m uses eA[z*ea_zs + (m/ea_div) % ea_mod]
   int eshift;
   // o_half != 0: the fp32 output is written as 16-bit hi (C) / lo (C_lo) pieces (1 fp16, 2 bf16)
@@ -114,7 +112,7 @@ __device__ __forceinline__ int row_exp(const UmmaArgs& a, int z, int64_t m) {
   return a.eA[zlin(a, z, a.ea_zs, a.ea_zso) + i] + a.eshift;
 }
 __device__ __forceinline__ int col_exp(const UmmaArgs& a, int z, int64_t n) {
-  return a.eB ? a.eB[zlin(a, z, a.eb_zs, a.eb_zso) + exp_index(n >> a.eb_sh, a.eb_div)] : 0;
+  return a.eB ? a.eB[zlin(a, z, a.eb_zs, a.eb_zso) + exp_index(n >> 1, a.eb_div)] : 0;
 }
 __device__ __forceinline__ int out_exp(const UmmaArgs& a, int z, int64_t m) {
   return a.eO ? a.eO[zlin(a, z, a.eo_zs, a.eo_zso) + exp_index(m, a.eo_div)] + a.eo_shift : 0;
@@ -142,74 +140,6 @@ __device__ __forceinline__ void half_pieces(int fmt, float v, uint16_t& h, uint1
     h = __half_as_ushort(hh);
     l = __half_as_ushort(lh);
   }
-}
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-// bounded wait; returns false on timeout
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t limit = UM_SPIN_LIMIT) {
-  uint32_t addr = smem_u32(bar);
-  for (uint32_t i = 0; i < limit; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  }
-  return false;
-}
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1, int c2) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-      ::"r"(smem_u32(dst)), "l"((uint64_t)map), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
-      : "memory");
-}
-// L2 prefetch of one tile (no shared-memory destination, no barrier)
-__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int c0, int c1, int c2) {
-  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"((uint64_t)map), "r"(c0),
-               "r"(c1), "r"(c2)
-               : "memory");
-}
-__device__ __forceinline__ uint64_t sw128_desc(const void* p) {
-  uint64_t a = smem_u32(p);
-  return ((a & 0x3FFFFull) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
-         ((uint64_t)2 << 61);
-}
-__device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
-      : "memory");
-}
-__device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
-      : "memory");
-}
-// one K-step (32 bytes of K: 8 tf32 or 16 fp16) of the chosen kind
-__device__ __forceinline__ void umma_step(bool f16, uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t acc) {
-  if (f16) umma_f16(tmem_d, adesc, bdesc, idesc, acc);
-  else umma_tf32(tmem_d, adesc, bdesc, idesc, acc);
-}
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
 }
 
 __device__ __forceinline__ float tf32_rna_dev(float x) {
@@ -443,6 +373,7 @@ struct UpCfg {
 static int g_chunk_len = 2;
 static int g_prefetch = 0;   // L2 prefetch distance in stages (0: off)
 static uint32_t g_spin = UM_SPIN_LIMIT;   // pipeline wait limit (test hook lowers it)
+uint32_t umma_spin() { return g_spin; }
 static int g_wide = 1;       // autotuner may pick 160..256-column tiles (split 8-warp epilogue)
 static int g_force_bn = 0;   // test hook: nonzero forces this N tile (no tuning)
 // 1: the persistent kernel is launched as a programmatic dependent of the stream's previous
@@ -896,8 +827,7 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
         {
           const int64_t ro = a.row_inner >= ((int64_t)1 << 31) ? 0 : (int64_t)((uint32_t)row / (uint32_t)a.row_inner);
           const int64_t ri = row - ro * a.row_inner;
-          const int64_t rl = a.row_list && row < a.M ? (int64_t)a.row_list[ro] : ro;
-          myoff = zlin(a, z, a.c_zs, a.c_zso) + rl * a.row_s1 + ri * a.c_ld;
+          myoff = zlin(a, z, a.c_zs, a.c_zso) + ro * a.row_s1 + ri * a.c_ld;
         }
         const bool rok = row < a.M;
         float* C = (float*)a.C;
@@ -908,7 +838,7 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
         const int64_t ebase = a.eB ? zlin(a, z, a.eb_zs, a.eb_zso) : 0;
         const bool bconst = a.eb_div >= ((int64_t)1 << 30) || !a.eB;
         const int cconst = (a.eB && bconst) ? a.eB[ebase] : 0;
-        auto colexp = [&](int n) { return a.eB ? a.eB[ebase + exp_index(n >> a.eb_sh, a.eb_div)] : 0; };
+        auto colexp = [&](int n) { return a.eB ? a.eB[ebase + exp_index(n >> 1, a.eb_div)] : 0; };
         for (int cb = 0; cb < BW; cb += 32) {
           uint32_t v[32];
           asm volatile(
@@ -1080,7 +1010,7 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 
 // 3-D tensor map {kdim, rows, batch} of fp32 (or fp16) elements with row stride ld and
 // batch stride bs (elements); the box is one 128-byte row of K by box_rows rows
-static bool make_map(CUtensorMap* m, const void* base, int64_t kdim, int64_t rows, int64_t batch, int64_t ld,
+bool make_map(CUtensorMap* m, const void* base, int64_t kdim, int64_t rows, int64_t batch, int64_t ld,
                      int64_t bs, uint32_t box_rows, int f16) {
   auto fn = encode_fn();
   if (!fn) return false;
@@ -1314,10 +1244,6 @@ cudaError_t umma_gemm(const UmmaOperand& A, const UmmaOperand& B, int M, int N, 
     a.ea_div = scale->ea_div > 0 ? scale->ea_div : 1;
     a.eb_div = scale->eb_div > 0 ? scale->eb_div : 1;
     a.ea_mod = scale->ea_mod > 0 ? scale->ea_mod : 0;
-    a.eb_sh = scale->real_cols ? 0 : 1;
-    // a listed outer row is resolved by the lane-per-row write-out only
-    if (scale->row_list && !a.direct) return cudaErrorInvalidValue;
-    a.row_list = scale->row_list;
   }
   int bn = cost_model_bn(N);
   if (g_force_bn) return umma_launch(g_force_bn, A, B, Kpad, nseg, a, batch, st);
