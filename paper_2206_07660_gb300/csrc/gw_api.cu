@@ -30,7 +30,7 @@ struct gw_ctx {
   // folded bosonic block (k_fold.cu): kept frequencies and partners, q-points of the range that are
   // their own negatives (qR) and the other kept ones (qC), digits of the transforms restricted to
   // them; P_iw holds a folded P~0 / P_tau a folded P~
-  bool wfold = false, p0sym = false;
+  bool wfold = false, p0sym = false, psym = false;
   int nrep = 0, nqR = 0, nqC = 0;
   int *d_rep = nullptr, *d_repn = nullptr, *d_qR = nullptr, *d_qC = nullptr;
   void *fRd = nullptr, *fCd = nullptr, *bRd = nullptr, *bCd = nullptr;
@@ -83,7 +83,7 @@ struct gw_ctx {
   float *Y3hi = nullptr, *Y3lo = nullptr, *W3hi = nullptr, *W3lo = nullptr;   // last Sigma step
   int64_t kpadP = 0, kpadS = 0, kpad3 = 0;
   int pgroup = 1;   // k-points whose last P~0 step runs as one GEMM (K concatenated over k)
-  size_t y3bytes = 0;
+  size_t y3bytes = 0, vt_bytes = 0;
   double2 *adjA = nullptr, *adjB = nullptr, *adjC = nullptr;   // fp64 chains of the adjoints (lazy)
   float2 *adjG32 = nullptr, *adjP32 = nullptr, *adjBar32 = nullptr;   // complex64 adjoint operands (lazy)
   // captured iteration (gw_iterate_graph): status checks are deferred while capturing
@@ -99,6 +99,12 @@ struct gw_ctx {
   // k-points per launch of the 16-bit chains (their per-k operands side by side) and the
   // G blocks of k+q (or k-q) gathered in k order for such a launch
   int pbatch = 1;
+  // first Sigma~ step in 4 x 4 column blocks (nao padded to nao4), its conjugate transpose for the
+  // mirrored (k - q, -q, beta - tau), that one's row exponents, k - q per (q, k)
+  int nao4 = 0, npc = 0;   // npc: K pieces of 8 elements per row
+  float *Xb_hi = nullptr, *Xb_lo = nullptr, *Xt_hi = nullptr, *Xt_lo = nullptr;
+  size_t xb_bytes = 0;
+  int *eY3b = nullptr, *d_kminus = nullptr;
   float *Gq_hi = nullptr, *Gq_lo = nullptr;
   int* eGq = nullptr;
   int64_t kpadA = 0;
@@ -785,9 +791,15 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
     // operand buffers below hold that many blocks
     c->pbatch = chain_pbatch(nao, naux, nk, ntau);
     const size_t kb = (size_t)c->pbatch;
-    const size_t pb = (size_t)ntau * naux * c->kpadS * 2, tb = (size_t)2 * n2 * c->kpadS * 2;
+    // X in 4 x 4 column blocks where the padding to whole blocks costs less than the halved
+    // first step gains
+    const int nb4 = (nao + 3) / 4 * 4;
+    c->nao4 = 5 * nb4 * nb4 <= 8 * nao * nao ? nb4 : 0;
+    const int64_t vtrows = c->nao4 ? 2 * (int64_t)c->nao4 * c->nao4 : 2 * n2;
+    const size_t pb = (size_t)ntau * naux * c->kpadS * 2, tb = (size_t)vtrows * c->kpadS * 2;
     c->Pchi = (float*)need(A(pb)); c->Pclo = (float*)need(A(pb));
-    c->VThi = (float*)need(A(kb * tb)); c->VTlo = (float*)need(A(kb * tb));
+    c->vt_bytes = kb * tb;
+    c->VThi = (float*)need(A(c->vt_bytes)); c->VTlo = (float*)need(A(c->vt_bytes));
     const size_t vs = (size_t)naux * nao * c->kpadA * 2, ge = (size_t)nk * ntau * 2 * nao * c->kpadA * 2;
     const size_t xs = (size_t)ntau * naux * nao * c->kpadA * 2;
     c->Vs_hi = (float*)need(A(kb * vs)); c->Vs_lo = (float*)need(A(kb * vs));
@@ -799,6 +811,17 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
       c->eGq = (int*)need(A(kb * ntau * 4));
     }
     c->Xs_hi = (float*)need(A(kb * xs)); c->Xs_lo = (float*)need(A(kb * xs));
+    if (c->nao4) {
+      c->npc = 2 * ((2 * nao + 15) / 16);
+      c->xb_bytes = kb * ntau * c->npc * (size_t)naux * nao * 16 + 128 * 16;   // and one tile of rows of slack
+      c->Xb_hi = (float*)need(A(c->xb_bytes)); c->Xb_lo = (float*)need(A(c->xb_bytes));
+      c->Xt_hi = (float*)A(c->xb_bytes); c->Xt_lo = (float*)A(c->xb_bytes);
+      c->eY3b = (int*)A((size_t)ntau * 4); c->d_kminus = (int*)A((size_t)nk * nk * 4);
+      if (!c->Xt_hi || !c->Xt_lo || !c->eY3b || !c->d_kminus) {   // without room every (k, q) has its own X
+        dfree(c, c->Xt_hi); dfree(c, c->Xt_lo);
+        c->Xt_hi = c->Xt_lo = nullptr;
+      }
+    }
     c->y3bytes = (size_t)ntau * nao * c->kpad3 * 2;
     c->Y3hi = (float*)need(A(kb * c->y3bytes)); c->Y3lo = (float*)need(A(kb * c->y3bytes));
     c->W3hi = (float*)need(A(kb * 2 * nao * c->kpad3 * 2)); c->W3lo = (float*)need(A(kb * 2 * nao * c->kpad3 * 2));
@@ -929,6 +952,17 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
     const size_t xs = (size_t)c->pbatch * ntau * naux * nao * c->kpadA * 2;
     chk(cudaMemsetAsync(c->Xs_hi, 0, xs, st), "memset");
     chk(cudaMemsetAsync(c->Xs_lo, 0, xs, st), "memset");
+    if (c->nao4) {   // so do the pieces and the rows of the blocks' padding
+      chk(cudaMemsetAsync(c->Xb_hi, 0, c->xb_bytes, st), "memset");
+      chk(cudaMemsetAsync(c->Xb_lo, 0, c->xb_bytes, st), "memset");
+      chk(cudaMemsetAsync(c->VThi, 0, c->vt_bytes, st), "memset");
+      chk(cudaMemsetAsync(c->VTlo, 0, c->vt_bytes, st), "memset");
+    }
+    if (c->Xt_hi) {
+      chk(cudaMemsetAsync(c->Xt_hi, 0, c->xb_bytes, st), "memset");
+      chk(cudaMemsetAsync(c->Xt_lo, 0, c->xb_bytes, st), "memset");
+      chk(cudaMemcpyAsync(c->d_kminus, c->kminus.data(), (size_t)nk * nk * 4, cudaMemcpyHostToDevice, st), "copy");
+    }
   }
   // input checks
   chk(cudaMemsetAsync(c->dscr, 0, 64 * 8, st), "memset");
@@ -1071,7 +1105,7 @@ extern "C" gw_status gw_set(gw_ctx* c, gw_quantity q, const void* src, size_t by
   mark(c, q);
   if (q == GW_Q_G_TAU) c->have_G = true;
   if (q == GW_Q_P0_IW) { c->have_P0 = true; c->p0sym = false; unmark(c, GW_Q_P_IW); }
-  if (q == GW_Q_P_TAU) c->have_P = true;
+  if (q == GW_Q_P_TAU) { c->have_P = true; c->psym = false; }
   if (q == GW_Q_SIGMA_INF || q == GW_Q_SIGMA_IW) c->have_sigma = true;
   return GW_OK;
 }
@@ -1103,6 +1137,16 @@ extern "C" gw_status gw_reset_sigma(gw_ctx* c) {
 }
 
 // ------------------------------------------------------------------ A1: gamma, J, K
+
+// split of a long reduction into Z outputs of nao x nao: about four rounds of blocks for the SMs, at
+// least 64 terms each, at most the 64 parts the workspace holds
+static int split_blocks(int nao, int64_t Z, int64_t K) {
+  const int64_t t = (nao + 63) / 64;
+  int64_t s = (4 * 152 + Z * t * t - 1) / (Z * t * t);
+  if (s > 64) s = 64;
+  if (s > K / 64) s = K / 64;
+  return s < 1 ? 1 : (int)s;
+}
 
 static gw_status exchange(gw_ctx* c, const double2* gamma, double2* out) {
   // K^k_ij = -(1/Nk) sum_{k',Q,a,b} V^{kk'}_ia(Q) gamma^{k'}_ab V^{k'k}_bj(Q)    (Eq. HF_K)
@@ -1139,7 +1183,7 @@ static gw_status exchange(gw_ctx* c, const double2* gamma, double2* out) {
     e.bk = I1(nao); e.bn = I1(1); e.bz = I1(slab);
     e.cm = I1(nao); e.cn = I1(1); e.cz = I1(n2);
     e.alpha = make_double2(-1.0 / nk, 0); e.beta = make_double2(1, 0);
-    e.ksplit = 16;
+    e.ksplit = split_blocks(nao, nk, e.K);
     const char* Vk = (const char*)Vp + (size_t)kp * nk * slab * es;
     CK(run_gett(e, c->chA, tv, Vk, tv, out, Ty::C128, acc, c));
   }
@@ -1186,6 +1230,11 @@ static int polar_taus(const gw_ctx* c, int q) {
   return nq == q ? (c->ntau + 1) / 2 : (nq > q ? c->ntau : 0);
 }
 
+// whether this context's Sigma~ chain can take one X for both (k, q, tau) and its mirror image
+static inline bool sigma_shares(const gw_ctx* c) {
+  return c->hfmt ? c->Xt_hi != nullptr : c->cfg.contract_prec != GW_SPLIT_TF32;
+}
+
 // Symmetrises the computed part of P~0 (or its tangent) over the context's q range and fills
 // the rest from it.
 static cudaError_t polar_finish(gw_ctx* c, double2* out, bool trs) {
@@ -1201,7 +1250,8 @@ static cudaError_t polar_finish(gw_ctx* c, double2* out, bool trs) {
 // twice with the tangent in one slot.
 static gw_status polar_chain_half(gw_ctx* c, const double2* Gplus, const double2* Gminus, double2* out,
                                   bool accumulate);
-static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2* Psrc, double2* out, bool accumulate);
+static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2* Psrc, double2* out, bool accumulate,
+                                  bool psym);
 
 static gw_status polar_chain(gw_ctx* c, const double2* Gplus, const double2* Gminus, double2* out, bool accumulate) {
   if (c->hfmt) return polar_chain_half(c, Gplus, Gminus, out, accumulate);
@@ -1451,7 +1501,8 @@ static gw_status polar_chain_half(gw_ctx* c, const double2* Gplus, const double2
 // coalesced lane-per-row write-out).
 // X's rows are scaled from P~'s row sums of moduli times max |V|; Y's from max_Q' of X's
 // bounds times the row sums of G(t).
-static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2* Psrc, double2* out, bool accumulate) {
+static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2* Psrc, double2* out, bool accumulate,
+                                  bool psym) {
   const int nk = c->nk, nao = c->nao, naux = c->naux, ntau = c->ntau, fmt = c->hfmt;
   const int64_t n2 = c->n2, na2 = c->na2, slab = (int64_t)naux * n2, gstep = (int64_t)nk * n2;
   const int64_t ka = c->kpadA, per = 2 * (int64_t)nao * ka, kps = c->kpadS, kp3 = c->kpad3;
@@ -1466,19 +1517,53 @@ static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2*
     CK(half_embed_mats(Gsrc + (size_t)k * n2, ntau, gstep, nao, nao, hofs(c->Ge_hi, (int64_t)k * ntau * per),
                        hofs(c->Ge_lo, (int64_t)k * ntau * per), ka, per, fmt, false, c->eGe + (size_t)k * ntau, st));
   count(nk);
-  const double fl1 = 8.0 * ntau * naux * (double)naux * n2, fl2 = 8.0 * ntau * naux * (double)nao * n2;
-  const int64_t mt = ((int64_t)ntau * nao + 127) / 128, nt = (2 * (int64_t)nao + 159) / 160;
-  const int KB = c->pbatch;
-  const int64_t xs_blk = (int64_t)ntau * naux * nao * ka, y3_blk = (int64_t)ntau * nao * kp3;
-  const int64_t vt_blk = 2 * n2 * kps, w3_blk = 2 * (int64_t)nao * kp3;
+  // With P~^{-q}(beta - tau) = conj P~^q(tau) and the paired V, the X of (k - q, -q, beta - tau) is the
+  // conjugate of that of (k, q, tau) with i and a exchanged.  The first step, most of the chain's
+  // work, then runs over half of the (q, tau) (the kept ones of polar_taus; the middle of an odd
+  // ntau of q = -q serves both k, so it has no image) and writes X in both orders.
+  const bool share = psym && c->fold && !c->reduce && sigma_shares(c);
+  const int KB = c->pbatch, nb4 = c->nao4;
+  // X: rows (t, i, Q') of K = a, or (nao4) K pieces of those rows per t; one tau of it
+  const int npc = nb4 ? c->npc : 0;
+  const int64_t xt = nb4 ? (int64_t)naux * nao * npc * 8 : (int64_t)naux * nao * ka;
+  float *Xh = nb4 ? c->Xb_hi : c->Xs_hi, *Xl = nb4 ? c->Xb_lo : c->Xs_lo;
+  const int64_t xs_blk = ntau * xt, y3t = (int64_t)nao * kp3, y3_blk = ntau * y3t;
+  const int64_t ncol = nb4 ? 2 * (int64_t)nb4 * nb4 : 2 * n2;
+  const int64_t vt_blk = ncol * kps, w3_blk = 2 * (int64_t)nao * kp3;
+  // Sigma~ += -(1/Nk) Y V over nt tau points from t0: B = V transposed, rows j, K = (b, Q') (source
+  // rows (Q', b)); the Sigma~^k of list[z] (or of consecutive k)
+  auto last_step = [&](const int64_t* voff, int kn, int t0, int nt, const int* eY, double2* o, const int* list) -> gw_status {
+    CK(half_embed_t_multi(c->V, voff, kn, (int64_t)naux * nao, nao, c->W3hi, c->W3lo, kp3, w3_blk, fmt,
+                          c->h_Evmax - 15, st, nao, naux));
+    count(1);
+    const int64_t tiles = (((int64_t)nt * nao + 127) / 128) * ((2 * (int64_t)nao + 159) / 160) * kn;
+    int64_t ks = (304 + tiles - 1) / tiles;
+    if (ks > kp3 / 64) ks = kp3 / 64;
+    if (ks < 1) ks = 1;
+    UmmaOperand ya{hofs(c->Y3hi, t0 * y3t), hofs(c->Y3lo, t0 * y3t), (int64_t)nt * nao, kn, kp3, y3_blk, fmt};
+    UmmaOperand wb{c->W3hi, c->W3lo, 2 * (int64_t)nao, kn, kp3, w3_blk, fmt};
+    UmmaScale sc{eY + t0, c->eVall, 0, 0, 0, nao, kAll};
+    UmmaZ zz{};
+    zz.c_list = list;
+    CK(run_umma(c, 8.0 * nt * naux * (double)nao * n2 * kn, ya, wb, nt * nao, 2 * nao, kp3, kn,
+                (double*)(o + (size_t)t0 * gstep), true, -1.0 / nk, true, 2 * (int64_t)nao, 2 * n2, (int)ks, nao,
+                2 * gstep, 0, 0, nullptr, 2 * (int64_t)naux * nao, &sc, nullptr, list ? &zz : nullptr));
+    return GW_OK;
+  };
   std::vector<int> act;
   act.reserve((size_t)nk);
   for (int q = c->q0; q < c->q1; ++q) {
+    const int nq = c->kneg[(size_t)q];
+    const bool pair = share && nq >= c->q0 && nq < c->q1;
+    if (pair && nq < q) continue;
+    const int nt = pair && nq == q ? (ntau + 1) / 2 : ntau;         // tau points 0.. of X
+    const int ni = pair ? (nq == q ? ntau / 2 : ntau) : 0, t0i = ntau - ni;   // its images t0i..
+    const double fl1 = 8.0 * nt * naux * (double)naux * n2;
     // A operand of the first step: conj P~^q(t) rows (t, Q') with exact row exponents and
     // the exponents of their sums of moduli; then Y's exponent per t
-    CK(half_rows(Psrc + (size_t)q * ntau * na2, (int64_t)ntau * naux, naux, naux, true, c->Pchi, c->Pclo, kps, kps, fmt,
+    CK(half_rows(Psrc + (size_t)q * ntau * na2, (int64_t)nt * naux, naux, naux, true, c->Pchi, c->Pclo, kps, kps, fmt,
                  c->ePc, c->ePs, st));
-    CK(sigma_exps(c->ePs, shift, c->gn + ntau, ntau, naux, c->eY3, st));
+    CK(sigma_exps(c->ePs, shift, c->gn + ntau, nt, ntau, naux, c->eY3, pair ? c->eY3b : nullptr, st));
     count(2);
     act.clear();
     for (int k = 0; k < nk; ++k)
@@ -1497,17 +1582,22 @@ static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2*
         voffW[l] = ((int64_t)kmq[l] * nk + k0 + l) * slab;
       }
       // X = conj(P~) V: B = V^{k,k-q} transposed, rows (i, a), K = Q, one exponent
-      CK(half_embed_t_multi(c->V, voffX, kn, naux, n2, c->VThi, c->VTlo, kps, vt_blk, fmt, c->h_Evmax - 15, st));
+      CK(half_embed_t_multi(c->V, voffX, kn, naux, n2, c->VThi, c->VTlo, kps, vt_blk, fmt, c->h_Evmax - 15, st, 0, 0,
+                            nb4 ? nao : 0));
       count(1);
       {
-        UmmaOperand oa{c->Pchi, c->Pclo, (int64_t)ntau * naux, 1, kps, 0, fmt};
-        UmmaOperand ob{c->VThi, c->VTlo, 2 * n2, kn, kps, vt_blk, fmt};
+        UmmaOperand oa{c->Pchi, c->Pclo, (int64_t)nt * naux, 1, kps, 0, fmt};
+        UmmaOperand ob{c->VThi, c->VTlo, ncol, kn, kps, vt_blk, fmt};
         UmmaScale sc{c->ePc, c->eVall, 0, 0, 0, 1, kAll};
         UmmaOut o{fmt, c->ePs, 0, 1, shift};
+        if (nb4) {
+          o.naux = naux; o.nao = nao; o.nt = ntau; o.npc = npc;
+          if (pair) { o.C2 = c->Xt_hi; o.C2_lo = c->Xt_lo; }
+        }
         // output row (t, Q'), column (i, a re/im) -> X row (t, i, Q'), entry (a re/im); one X block per k
-        CK(run_umma(c, fl1 * kn, oa, ob, ntau * naux, (int)(2 * n2), kps, kn, c->Xs_hi, false, 1.0, false, ka,
-                    kn > 1 ? xs_blk : 0, 1, naux, (int64_t)nao * naux * ka, 2 * (int64_t)nao, (int64_t)naux * ka,
-                    c->Xs_lo, 2 * (int64_t)naux, &sc, &o));
+        CK(run_umma(c, fl1 * kn, oa, ob, nt * naux, (int)ncol, kps, kn, Xh, false, 1.0, false, ka,
+                    kn > 1 ? xs_blk : 0, 1, naux, xt, 2 * (int64_t)nao, (int64_t)naux * ka, Xl, 2 * (int64_t)naux, &sc,
+                    &o));
       }
       // Y = X G^{k-q}(t): A rows (i, Q') per (k, t) (exponent of row Q'), B = Ge[k-q][t]; row (i, Q'),
       // column (b re/im) lands at row (t, i), K entry (b, Q') of the last step's operand
@@ -1520,31 +1610,37 @@ static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2*
           count(1);
           gbh = c->Gq_hi; gbl = c->Gq_lo; gbe = c->eGq;
         }
-        UmmaOperand xa{c->Xs_hi, c->Xs_lo, (int64_t)naux * nao, (int64_t)kn * ntau, ka, (int64_t)naux * nao * ka, fmt};
+        UmmaOperand xa{Xh, Xl, (int64_t)naux * nao, (int64_t)kn * ntau, ka, xt, fmt, npc};
         UmmaOperand gb{(const float*)gbh, (const float*)gbl, 2 * (int64_t)nao, (int64_t)kn * ntau, ka, per, fmt};
         UmmaScale sc{c->ePs, gbe, naux, 1, shift, 1, kAll};
         sc.ea_mod = naux;
         UmmaOut o{fmt, c->eY3, 1, kAll, 0};
-        UmmaZ zz{ntau, ntau, 1, ntau, 1, 0, ntau, 0, y3_blk};
-        CK(run_umma(c, fl2 * kn, xa, gb, naux * nao, 2 * nao, ka, kn * ntau, c->Y3hi, false, 1.0, false, 2,
-                    (int64_t)nao * kp3, 1, naux, kp3, 2, 2 * (int64_t)naux, c->Y3lo, 2 * (int64_t)nao, &sc, &o,
+        UmmaZ zz{nt, ntau, 1, ntau, 1, 0, ntau, 0, y3_blk};
+        CK(run_umma(c, 8.0 * nt * naux * (double)nao * n2 * kn, xa, gb, naux * nao, 2 * nao, ka, kn * nt, c->Y3hi, false,
+                    1.0, false, 2, y3t, 1, naux, kp3, 2, 2 * (int64_t)naux, c->Y3lo, 2 * (int64_t)nao, &sc, &o,
                     kn > 1 ? &zz : nullptr));
       }
-      // Sigma~ += -(1/Nk) Y V^{k-q,k}: B = V^{k-q,k} transposed, rows j, K = (b, Q') (source rows (Q', b))
-      CK(half_embed_t_multi(c->V, voffW, kn, (int64_t)naux * nao, nao, c->W3hi, c->W3lo, kp3, w3_blk, fmt,
-                            c->h_Evmax - 15, st, nao, naux));
-      count(1);
+      gw_status s = last_step(voffW, kn, 0, nt, c->eY3, out + (size_t)k0 * n2, nullptr);
+      if (s != GW_OK) return s;
+      if (ni == 0) continue;
+      // the images (k - q, -q, t0i ..): Y = X^t* G^k(t'), rows (a, Q'), then Sigma~^{k-q}(t') with
+      // V^{k,k-q}; the exponents of X's rows run backwards in t'
       {
-        int64_t ks = (304 + mt * nt * kn - 1) / (mt * nt * kn);
-        if (ks > kp3 / 64) ks = kp3 / 64;
-        if (ks < 1) ks = 1;
-        UmmaOperand ya{c->Y3hi, c->Y3lo, (int64_t)ntau * nao, kn, kp3, y3_blk, fmt};
-        UmmaOperand wb{c->W3hi, c->W3lo, 2 * (int64_t)nao, kn, kp3, w3_blk, fmt};
-        UmmaScale sc{c->eY3, c->eVall, 0, 0, 0, nao, kAll};
-        CK(run_umma(c, fl2 * kn, ya, wb, ntau * nao, 2 * nao, kp3, kn, (double*)(out + (size_t)k0 * n2), true,
-                    -1.0 / nk, true, 2 * (int64_t)nao, 2 * n2, (int)ks, nao, 2 * gstep, 0, 0, nullptr,
-                    2 * (int64_t)naux * nao, &sc, nullptr));
+        UmmaOperand xa{hofs(c->Xt_hi, t0i * xt), hofs(c->Xt_lo, t0i * xt), (int64_t)naux * nao,
+                       (int64_t)(kn - 1) * ntau + ni, ka, xt, fmt, npc};
+        const int64_t g0 = (int64_t)k0 * ntau + t0i;
+        UmmaOperand gb{hofs(c->Ge_hi, g0 * per), hofs(c->Ge_lo, g0 * per), 2 * (int64_t)nao,
+                       (int64_t)(kn - 1) * ntau + ni, ka, per, fmt};
+        UmmaScale sc{c->ePs + (int64_t)(ntau - 1 - t0i) * naux, c->eGe + g0, -(int64_t)naux, 1, shift, 1, kAll};
+        sc.ea_mod = naux;
+        UmmaOut o{fmt, c->eY3b + t0i, 1, kAll, 0};
+        UmmaZ zz{ni, ntau, 1, ntau, 1, 0, ntau, 0, y3_blk};
+        CK(run_umma(c, 8.0 * ni * naux * (double)nao * n2 * kn, xa, gb, naux * nao, 2 * nao, ka, kn * ni,
+                    hofs(c->Y3hi, t0i * y3t), false, 1.0, false, 2, y3t, 1, naux, kp3, 2, 2 * (int64_t)naux,
+                    hofs(c->Y3lo, t0i * y3t), 2 * (int64_t)nao, &sc, &o, kn > 1 ? &zz : nullptr));
       }
+      s = last_step(voffX, kn, t0i, ni, c->eY3b, out, c->d_kminus + (size_t)q * nk + k0);
+      if (s != GW_OK) return s;
     }
   }
   return GW_OK;
@@ -1629,6 +1725,7 @@ extern "C" gw_status gw_screened(gw_ctx* c) {
     CK(cudaStreamSynchronize(c->st));
     folded = c->h_scr[16] <= kFoldTol * c->h_scr[17];
   }
+  c->psym = folded;
   if (folded) {
     CK(fold_screened(c));
   } else if (trs_reduce(c)) {
@@ -1669,8 +1766,9 @@ extern "C" gw_status gw_screened(gw_ctx* c) {
 // Psrc; out (ntau, nk, nao, nao) receives the unsymmetrised sum (added to its
 // contents when accumulate).  The forward map uses G_tau and P_tau; the tangent runs
 // it with the tangent in either slot.
-static gw_status sigma_chain(gw_ctx* c, const double2* Gsrc, const double2* Psrc, double2* out, bool accumulate) {
-  if (c->hfmt) return sigma_chain_half(c, Gsrc, Psrc, out, accumulate);
+static gw_status sigma_chain(gw_ctx* c, const double2* Gsrc, const double2* Psrc, double2* out, bool accumulate,
+                             bool psym) {
+  if (c->hfmt) return sigma_chain_half(c, Gsrc, Psrc, out, accumulate, psym);
   const int nk = c->nk, nao = c->nao, naux = c->naux, ntau = c->ntau;
   const int64_t n2 = c->n2, na2 = c->na2, slab = (int64_t)naux * n2, gstep = (int64_t)nk * n2;
   const bool f32 = c->cfg.contract_prec != GW_FP64;
@@ -1691,7 +1789,15 @@ static gw_status sigma_chain(gw_ctx* c, const double2* Gsrc, const double2* Psrc
     count(2);
     Gp = c->G32; Pp = c->P32;
   }
+  // one X for (k, q, tau) and (k - q, -q, beta - tau) (see sigma_chain_half); the strided kernels
+  // read its transpose in place
+  const bool share = psym && c->fold && !c->reduce && !tc;
+  if (share && !accumulate) CK(cudaMemsetAsync(out, 0, (size_t)ntau * gstep * 16, c->st));
   for (int q = c->q0; q < c->q1; ++q) {
+    const int nq = c->kneg[(size_t)q];
+    const bool pair = share && nq >= c->q0 && nq < c->q1;
+    if (pair && nq < q) continue;
+    const int nt = pair && nq == q ? (ntau + 1) / 2 : ntau, ni = pair ? (nq == q ? ntau / 2 : ntau) : 0;
     const char* Pq = (const char*)Pp + (size_t)q * ntau * na2 * es;
     if (tc) {
       // A operand of the tensor-core stage: conj P~^q(t) = P~^q(t)^T (Hermitian), split hi/lo
@@ -1723,7 +1829,7 @@ static gw_status sigma_chain(gw_ctx* c, const double2* Gsrc, const double2* Psrc
         count(1);
       } else {
       // X[t][Q'][(i,a)] = sum_Q P~^q[t][Q][Q'] V^{k,k-q}[Q][(i,a)]
-      GettDesc d1 = base_desc(naux, n2, naux, ntau);
+      GettDesc d1 = base_desc(naux, n2, naux, nt);
       d1.am = I1(1); d1.ak = I1(naux); d1.az = I1(na2);
       d1.bk = I1(n2); d1.bn = I1(1); d1.bz = I1(0);
       d1.cm = I1(n2); d1.cn = I1(1); d1.cz = I1(slab);
@@ -1741,35 +1847,26 @@ static gw_status sigma_chain(gw_ctx* c, const double2* Gsrc, const double2* Psrc
                     false, c->kpad3, (int64_t)nao * c->kpad3, 1, nao, 2 * (int64_t)nao, 0, 0, c->Y3lo,
                     2 * (int64_t)nao));
         count(1);
-      } else if (f32 && nao <= 64) {
+      } else if (tc3) {
+        // FP32 products as TF32 hi/lo rows (t, i), columns (Q', b): the A operand of the last step
+        const int64_t hk = c->kpad3 / 2;
         BsmDesc b{};
         b.M = b.N = b.K = nao; b.G = ntau; b.E = naux; b.alpha = 1.f;
         b.A = (const float2*)c->chA; b.a_gs = slab; b.a_es = n2; b.a_rs = nao; b.a_cs = 1;
         b.B = (const float2*)Gp + (size_t)kmq * n2; b.b_gs = gstep; b.b_rs = nao; b.b_cs = 1; b.b_shared = 1;
-        if (tc3) {  // TF32 hi/lo rows (t, i), columns (Q', b): the A operand of the last step
-          const int64_t hk = c->kpad3 / 2;
-          b.Chi = c->Y3hi; b.Clo = c->Y3lo; b.c_gs = nao * hk; b.c_es = nao; b.c_rs = hk;
-        } else {
-          b.C = (float2*)c->chB; b.c_gs = slab; b.c_es = nao; b.c_rs = (int64_t)naux * nao;
-        }
+        b.Chi = c->Y3hi; b.Clo = c->Y3lo; b.c_gs = nao * hk; b.c_es = nao; b.c_rs = hk;
         CK(run_bsm(c, b));
-      } else {
-      GettDesc d2 = base_desc((int64_t)naux * nao, nao, nao, ntau);
-      d2.am = I1(nao); d2.ak = I1(1); d2.az = I1(slab);
-      d2.bk = I1(nao); d2.bn = I1(1); d2.bz = I1(gstep);
-      d2.cm = I2(nao, nao, (int64_t)naux * nao); d2.cn = I1(1); d2.cz = I1(slab);
-      CK(run_gett(d2, c->chA, tv, (const char*)Gp + (size_t)kmq * n2 * es, tv, c->chB, tv, acc, c));
       }
-      // Sigma~[t][k][i][j] += -(1/Nk) sum_{(Q',b)} Y[t][i][(Q',b)] V^{k-q,k}[Q'][b][j]
       if (tc3) {
-        // one GEMM over all (t, i) rows on tensor cores, K split over blocks
+        // Sigma~[t][k][i][j] += -(1/Nk) sum_{(Q',b)} Y[t][i][(Q',b)] V^{k-q,k}[Q'][b][j]: one GEMM over
+        // all (t, i) rows on tensor cores, K split over blocks
         const int64_t kp = c->kpad3;
         CK(embed_t((const char*)c->V + ((size_t)kmq * nk + k) * slab * 16, true, (int64_t)naux * nao, nao, c->W3hi,
                    c->W3lo, kp, c->st));
         UmmaOperand oa{c->Y3hi, c->Y3lo, (int64_t)ntau * nao, 1, kp, 0};
         UmmaOperand ob{c->W3hi, c->W3lo, 2 * (int64_t)nao, 1, kp, 0};
-        const int64_t mt = ((int64_t)ntau * nao + 127) / 128, nt = (2 * (int64_t)nao + 159) / 160;
-        int64_t ks = (304 + mt * nt - 1) / (mt * nt);
+        const int64_t mt = ((int64_t)ntau * nao + 127) / 128, nt3 = (2 * (int64_t)nao + 159) / 160;
+        int64_t ks = (304 + mt * nt3 - 1) / (mt * nt3);
         if (ks > kp / 32) ks = kp / 32;
         if (ks < 1) ks = 1;
         CK(run_umma(c, 8.0 * ntau * nao * (double)nao * naux * nao, oa, ob, ntau * nao, 2 * nao, kp, 1,
@@ -1778,15 +1875,40 @@ static gw_status sigma_chain(gw_ctx* c, const double2* Gsrc, const double2* Psrc
         count(1);
         continue;
       }
-      GettDesc d3 = base_desc(nao, nao, (int64_t)naux * nao, ntau);
-      d3.am = I1((int64_t)naux * nao); d3.ak = I1(1); d3.az = I1(slab);
-      d3.bk = I1(nao); d3.bn = I1(1); d3.bz = I1(0);
-      d3.cm = I1(nao); d3.cn = I1(1); d3.cz = I1(gstep);
-      d3.alpha = make_double2(-1.0 / nk, 0);
-      d3.beta = make_double2(accumulate || q > c->q0 ? 1.0 : 0.0, 0);
-      d3.ksplit = 8;
-      const char* Vk2 = (const char*)Vp + ((size_t)kmq * nk + k) * slab * es;
-      CK(run_gett(d3, c->chB, tv, Vk2, tv, out + (size_t)k * n2, Ty::C128, acc, c));
+      for (int im = 0; im < (ni > 0 ? 2 : 1); ++im) {
+        // im = 0: Y[t][i][Q'][b] = sum_a X[t][Q'][i][a] G^{k-q}[t][a][b], then
+        //   Sigma~[t][k][i][j] += -(1/Nk) sum_{(Q',b)} Y[t][i][(Q',b)] V^{k-q,k}[Q'][b][j];
+        // im = 1, the image of t at n-1-t: Y[t][a][Q'][b] = sum_i conj X[t][Q'][i][a] G^k[n-1-t][i][b], then
+        //   Sigma~[n-1-t][k-q][a][j] += -(1/Nk) sum Y[t][a][(Q',b)] V^{k,k-q}[Q'][b][j]
+        const int zt = im ? ni : nt, kg = im ? k : kmq, ko = im ? kmq : k;
+        const int64_t t0 = im ? (int64_t)(ntau - 1) * gstep : 0, ts = im ? -gstep : gstep;
+        if (f32 && nao <= 64) {
+          BsmDesc b{};
+          b.M = b.N = b.K = nao; b.G = zt; b.E = naux; b.alpha = 1.f;
+          b.A = (const float2*)c->chA; b.a_gs = slab; b.a_es = n2;
+          b.a_rs = im ? 1 : nao; b.a_cs = im ? nao : 1; b.conjA = im;
+          b.B = (const float2*)Gp + t0 + (size_t)kg * n2; b.b_gs = ts; b.b_rs = nao; b.b_cs = 1; b.b_shared = 1;
+          b.C = (float2*)c->chB; b.c_gs = slab; b.c_es = nao; b.c_rs = (int64_t)naux * nao;
+          CK(run_bsm(c, b));
+        } else {
+          GettDesc d2 = base_desc((int64_t)naux * nao, nao, nao, zt);
+          if (im) { d2.am = I2(nao, n2, 1); d2.ak = I1(nao); d2.conjA = true; }
+          else { d2.am = I1(nao); d2.ak = I1(1); }
+          d2.az = I1(slab);
+          d2.bk = I1(nao); d2.bn = I1(1); d2.bz = I1(ts);
+          d2.cm = I2(nao, nao, (int64_t)naux * nao); d2.cn = I1(1); d2.cz = I1(slab);
+          CK(run_gett(d2, c->chA, tv, (const char*)Gp + ((size_t)t0 + (size_t)kg * n2) * es, tv, c->chB, tv, acc, c));
+        }
+        GettDesc d3 = base_desc(nao, nao, (int64_t)naux * nao, zt);
+        d3.am = I1((int64_t)naux * nao); d3.ak = I1(1); d3.az = I1(slab);
+        d3.bk = I1(nao); d3.bn = I1(1); d3.bz = I1(0);
+        d3.cm = I1(nao); d3.cn = I1(1); d3.cz = I1(ts);
+        d3.alpha = make_double2(-1.0 / nk, 0);
+        d3.beta = make_double2(accumulate || share || q > c->q0 ? 1.0 : 0.0, 0);
+        d3.ksplit = split_blocks(nao, zt, d3.K);
+        const char* Vk2 = (const char*)Vp + ((size_t)kg * nk + ko) * slab * es;
+        CK(run_gett(d3, c->chB, tv, Vk2, tv, out + t0 + (size_t)ko * n2, Ty::C128, acc, c));
+      }
     }
   }
   return GW_OK;
@@ -1799,7 +1921,15 @@ static gw_status sigma_tau_part(gw_ctx* c) {
   const bool tc = uses_tc(c);
   const bool red = trs_reduce(c);
   c->reduce = red;
-  gw_status s = sigma_chain(c, c->G_tau, c->P_tau, c->Stau, false);
+  // a P~ that was handed in is looked at for the fold (the screened solve's own has it)
+  if (c->fold && !c->psym && !red && !c->deferred && sigma_shares(c)) {
+    CK(fold_check_tau(c->P_tau, c->na2, ntau, c->q0, c->q1, c->d_kneg, c->dscr + 16, c->st));
+    count(1);
+    CK(cudaMemcpyAsync(c->h_scr + 16, c->dscr + 16, 16, cudaMemcpyDeviceToHost, c->st));
+    CK(cudaStreamSynchronize(c->st));
+    c->psym = c->h_scr[16] <= kFoldTol * c->h_scr[17];
+  }
+  gw_status s = sigma_chain(c, c->G_tau, c->P_tau, c->Stau, false, c->psym);
   c->reduce = false;
   if (s != GW_OK) return s;
   if (red) {   // Sigma~^{-k}(tau) = conj Sigma~^k(tau)
@@ -2221,8 +2351,8 @@ extern "C" gw_status gw_selfenergy_jvp(gw_ctx* c, const double* dG, const double
   if (!c->have_G) return fail(c, GW_ERR_STATE, "no Green's function yet");
   if (!c->have_P) return fail(c, GW_ERR_STATE, "no screened interaction yet");
   double2* out = (double2*)dS_tau;
-  gw_status s = sigma_chain(c, (const double2*)dG, c->P_tau, out, false);
-  if (s == GW_OK) s = sigma_chain(c, c->G_tau, (const double2*)dP_tau, out, true);
+  gw_status s = sigma_chain(c, (const double2*)dG, c->P_tau, out, false, c->psym);
+  if (s == GW_OK) s = sigma_chain(c, c->G_tau, (const double2*)dP_tau, out, true, false);
   if (s == GW_OK) s = tc_check(c);
   if (s != GW_OK) return s;
   CK(herm_batched(out, c->nao, (int64_t)c->ntau * c->nk, c->n2, c->st));
@@ -2280,8 +2410,8 @@ static gw_status sc_jvp(gw_ctx* c, const double2* dSinf, const double2* dSiw, do
   if ((s = polar_chain(c, c->G_tau, c->tGtau, c->tP, true)) != GW_OK) return s;
   CK(polar_finish(c, c->tP, false));
   if ((s = gw_screened_jvp(c, (const double*)c->tP, (double*)c->tP)) != GW_OK) return s;
-  if ((s = sigma_chain(c, c->tGtau, c->P_tau, c->tS, false)) != GW_OK) return s;
-  if ((s = sigma_chain(c, c->G_tau, c->tP, c->tS, true)) != GW_OK) return s;
+  if ((s = sigma_chain(c, c->tGtau, c->P_tau, c->tS, false, c->psym)) != GW_OK) return s;
+  if ((s = sigma_chain(c, c->G_tau, c->tP, c->tS, true, false)) != GW_OK) return s;
   if ((s = tc_check(c)) != GW_OK) return s;
   CK(herm_batched(c->tS, nao, (int64_t)c->ntau * nk, n2, c->st));
   count(1);

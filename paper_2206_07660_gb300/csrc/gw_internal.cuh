@@ -103,6 +103,10 @@ cudaError_t fold_pack_cplx(const double2* P, const FoldView& f, const int* qlist
 // of an odd ntau, its own image, is A[t] alone
 cudaError_t fold_cotangent(double2* Pr, const double2* A, const double2* B, int64_t na2, int nt, int ntau, bool self,
                            cudaStream_t st);
+// out[0] = largest deviation of P [nq][nt][n2] from P^{-q}(nt - 1 - t) = conj P^q(t) over the q in
+// [q0, q1) with a partner there (+inf: a value that is not finite), out[1] = max |P|
+cudaError_t fold_check_tau(const double2* P, int64_t n2, int nt, int q0, int q1, const int* neg, double* out,
+                           cudaStream_t st);
 cudaError_t fold_check(const double2* P, const FoldView& f, double* out, cudaStream_t st);
 
 struct DysonArgs {
@@ -183,7 +187,7 @@ cudaError_t half_embed_conj_multi(const double2* src, const int64_t* offs, int n
                                   cudaStream_t st);
 cudaError_t half_embed_t_multi(const double2* src, const int64_t* offs, int n, int64_t K, int64_t N, void* hi,
                                void* lo, int64_t Kpad, int64_t dstride, int fmt, int e, cudaStream_t st,
-                               int64_t kin = 0, int64_t kout = 0);
+                               int64_t kin = 0, int64_t kout = 0, int nao_blk = 0);   // nao_blk: rows (i, a) at block_col
 struct UmmaOperand {
   const float* hi;
   const float* lo;
@@ -191,6 +195,9 @@ struct UmmaOperand {
   int64_t ld, bs;        // row stride and batch stride in elements
   int f16 = 0;           // 1: hi/lo hold fp16 pieces, 2: bf16 pieces (cast pointers), K and strides in
                          // 16-bit elements
+  // > 0 (A, 16-bit, three products): stored as [batch][pieces][rows][8 elements], an even number of
+  // 16-byte K pieces, with 128 rows of slack behind the last one (ld and bs are not used)
+  int pieces = 0;
 };
 // ksplit > 1: the K range is split over blocks and partial results are added to
 // an fp64 C with atomics (requires accumulate).  row_inner > 0: output row m =
@@ -217,7 +224,17 @@ struct UmmaOut {
   const int* eO;
   int64_t eo_zs, eo_div;
   int eo_shift;
+  // naux > 0: columns in 4 x 4 blocks of (i, a) (block_col), rows m = (t, Q) of naux Q per t; the output
+  // goes to C / C_lo as the operand of rows (i, Q) and K = a in npc K pieces of 8 elements per t
+  // (UmmaOperand::pieces), and (C2 non-null) its conjugate to C2 / C2_lo at nt - 1 - t as that of rows
+  // (a, Q) and K = i; batch entries c_zs apart in both
+  int naux = 0, nao = 0, nt = 0, npc = 0;
+  void *C2 = nullptr, *C2_lo = nullptr;
 };
+// operand row of the matrix element (i, a) in 4 x 4 blocks, a fastest
+__host__ __device__ inline int block_col(int i, int a, int nao) {
+  return ((i >> 2) * ((nao + 3) >> 2) + (a >> 2)) * 16 + (i & 3) * 4 + (a & 3);
+}
 // Two-level batches (several k-points of a chain step in one launch): batch entry
 // z = zo * zin + zi; the TMA batch coordinate of A is zo * za_o + zi * za_i (B likewise),
 // and the exponent and output strides of the other arguments (ea_zs, eb_zs, eo_zs, c_zs)
@@ -226,6 +243,7 @@ struct UmmaZ {
   int zin;
   int za_o, za_i, zb_o, zb_i;
   int64_t ea_zso, eb_zso, eo_zso, c_zso;
+  const int* c_list = nullptr;   // the output of batch entry z goes to entry c_list[z] (zin must be 0)
 };
 cudaError_t umma_gemm(const UmmaOperand& A, const UmmaOperand& B, int M, int N, int64_t Kpad, int batch, void* C,
                       bool c_fp64, double alpha, bool accumulate, int64_t c_ld, int64_t c_zs, int nseg, int* err,
@@ -322,7 +340,8 @@ cudaError_t v_norms(const double2* V, int64_t nslab, int naux, int nao, float* v
 cudaError_t g_norms(const double2* G, int ntau, int nk, int nao, float* gmax, float* grs, cudaStream_t st);
 cudaError_t polar_exps(const float* vrs, const float* gmax_p, const float* grs_m, int ntau, int naux, int* eY, int* eZ,
                        cudaStream_t st);
-cudaError_t sigma_exps(const int* eX, int shift, const float* grs, int ntau, int naux, int* eY3, cudaStream_t st);
+cudaError_t sigma_exps(const int* eX, int shift, const float* grs, int nt, int ntau, int naux, int* eY3, int* eY3b,
+                       cudaStream_t st);
 cudaError_t max_exp(const float* v, int n, int* out, cudaStream_t st);
 cudaError_t row_exps(const float* v, int n, int* out, cudaStream_t st);
 

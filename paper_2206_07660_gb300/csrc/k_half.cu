@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(256) half_embed_conj_kernel(const double2* __r
 // e for the whole operand, transposed through shared memory.  Grid (N/32, K/32).
 __global__ void half_embed_t_kernel(const double2* __restrict__ src, int64_t K, int64_t N, uint16_t* hi, uint16_t* lo,
                                     int64_t Kpad, int fmt, int e, int64_t kin, int64_t kout, const __grid_constant__ SrcList list,
-                                    int64_t dstride) {
+                                    int64_t dstride, int nao_blk) {
   dep_wait();
   src += list.off[blockIdx.z];
   hi += blockIdx.z * dstride;
@@ -200,23 +200,25 @@ __global__ void half_embed_t_kernel(const double2* __restrict__ src, int64_t K, 
     if (n >= N || k >= K) continue;
     const double2 v = tile[tx][r];
     const int64_t kd = kin > 0 ? (k % kin) * kout + k / kin : k;   // K index in the operand
+    const int64_t nd = nao_blk > 0 ? block_col((int)n / nao_blk, (int)n % nao_blk, nao_blk) : n;   // row pair
     uint16_t a, b, c, a2, b2, c2;
     pieces(fmt, v.x, e, a, a2);
     pieces(fmt, -v.y, e, b, b2);
     pieces(fmt, v.y, e, c, c2);
-    *(uint32_t*)(hi + (2 * n) * Kpad + 2 * kd) = (uint32_t)a | ((uint32_t)b << 16);
-    *(uint32_t*)(lo + (2 * n) * Kpad + 2 * kd) = (uint32_t)a2 | ((uint32_t)b2 << 16);
-    *(uint32_t*)(hi + (2 * n + 1) * Kpad + 2 * kd) = (uint32_t)c | ((uint32_t)a << 16);
-    *(uint32_t*)(lo + (2 * n + 1) * Kpad + 2 * kd) = (uint32_t)c2 | ((uint32_t)a2 << 16);
+    *(uint32_t*)(hi + (2 * nd) * Kpad + 2 * kd) = (uint32_t)a | ((uint32_t)b << 16);
+    *(uint32_t*)(lo + (2 * nd) * Kpad + 2 * kd) = (uint32_t)a2 | ((uint32_t)b2 << 16);
+    *(uint32_t*)(hi + (2 * nd + 1) * Kpad + 2 * kd) = (uint32_t)c | ((uint32_t)a << 16);
+    *(uint32_t*)(lo + (2 * nd + 1) * Kpad + 2 * kd) = (uint32_t)c2 | ((uint32_t)a2 << 16);
   }
   // zero padding columns [2K, Kpad), by the first column of blocks
   if (blockIdx.y == 0) {
     for (int r = ty; r < 32; r += 8) {
       const int64_t n = nb + r;
       if (n >= N) continue;
+      const int64_t nd = nao_blk > 0 ? block_col((int)n / nao_blk, (int)n % nao_blk, nao_blk) : n;
       for (int64_t cc = 2 * K + tx; cc < Kpad; cc += 32) {
-        hi[(2 * n) * Kpad + cc] = 0; hi[(2 * n + 1) * Kpad + cc] = 0;
-        lo[(2 * n) * Kpad + cc] = 0; lo[(2 * n + 1) * Kpad + cc] = 0;
+        hi[(2 * nd) * Kpad + cc] = 0; hi[(2 * nd + 1) * Kpad + cc] = 0;
+        lo[(2 * nd) * Kpad + cc] = 0; lo[(2 * nd + 1) * Kpad + cc] = 0;
       }
     }
   }
@@ -351,15 +353,25 @@ __global__ void polar_exps_kernel(const float* vrs, const float* gmax_p, const f
 }
 
 // Row exponent of the Sigma~ chain's Y[t][i][(Q', b)] (uniform over Q'):
-// |Y| <= max_Q' 2^(eX[t][Q'] + 15) grs[t], with eX the exponents of X's rows.
-__global__ void sigma_exps_kernel(const int* eX, int shift, const float* grs, int ntau, int naux, int* eY3) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= ntau) return;
+// |Y| <= max_Q' 2^(eX[t][Q'] + 15) grs[t], with eX the exponents of X's rows.  eY3b (optional) gets
+// that of the conjugate X of t at the mirrored point ntau - 1 - t.  One warp per t.
+__global__ void sigma_exps_kernel(const int* eX, int shift, const float* grs, int nt, int ntau, int naux, int* eY3,
+                                  int* eY3b) {
+  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (t >= nt) return;
   int m = -100000;
-  for (int q = 0; q < naux; ++q) m = max(m, eX[(int64_t)t * naux + q]);
+  for (int q = lane; q < naux; q += 32) m = max(m, eX[(int64_t)t * naux + q]);
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane) return;
   int E = 0;
   if (grs[t] > 0.f) frexpf(grs[t], &E);
   eY3[t] = m + shift + E + 1;
+  if (eY3b) {
+    const int tm = ntau - 1 - t;
+    E = 0;
+    if (grs[tm] > 0.f) frexpf(grs[tm], &E);
+    eY3b[tm] = m + shift + E + 1;
+  }
 }
 
 __global__ void max_exp_kernel(const float* v, int n, int* out) {
@@ -444,7 +456,7 @@ cudaError_t half_embed_conj(const double2* src, int64_t rows, int64_t K, void* h
 
 cudaError_t half_embed_t_multi(const double2* src, const int64_t* offs, int n, int64_t K, int64_t N, void* hi,
                                void* lo, int64_t Kpad, int64_t dstride, int fmt, int e, cudaStream_t st, int64_t kin,
-                               int64_t kout) {
+                               int64_t kout, int nao_blk) {
   if (Kpad % 64 || K <= 0 || N <= 0 || n < 1 || n > kSrcListMax) return cudaErrorInvalidValue;
   if (kin > 0 && (K % kin || kout * kin != K)) return cudaErrorInvalidValue;   // a permutation of [0, K)
   SrcList l{};
@@ -452,7 +464,7 @@ cudaError_t half_embed_t_multi(const double2* src, const int64_t* offs, int n, i
   for (int i = 0; i < n; ++i) l.off[i] = offs ? offs[i] : 0;
   dim3 grid((unsigned)((N + 31) / 32), (unsigned)((K + 31) / 32), (unsigned)n);
   return launch_dep(half_embed_t_kernel, grid, dim3(256), st, src, K, N, (uint16_t*)hi, (uint16_t*)lo, Kpad, fmt, e,
-                    kin, kout, l, dstride);
+                    kin, kout, l, dstride, nao_blk);
 }
 
 cudaError_t half_embed_t(const double2* src, int64_t K, int64_t N, void* hi, void* lo, int64_t Kpad, int fmt, int e,
@@ -461,7 +473,7 @@ cudaError_t half_embed_t(const double2* src, int64_t K, int64_t N, void* hi, voi
   if (kin > 0 && (K % kin || kout * kin != K)) return cudaErrorInvalidValue;   // a permutation of [0, K)
   dim3 grid((unsigned)((N + 31) / 32), (unsigned)((K + 31) / 32), 1);
   return launch_dep(half_embed_t_kernel, grid, dim3(256), st, src, K, N, (uint16_t*)hi, (uint16_t*)lo, Kpad, fmt, e,
-                    kin, kout, one_src(), (int64_t)0);
+                    kin, kout, one_src(), (int64_t)0, 0);
 }
 
 cudaError_t half_embed_mats(const double2* src, int64_t count, int64_t ss, int64_t rows, int64_t K, void* hi,
@@ -495,8 +507,9 @@ cudaError_t polar_exps(const float* vrs, const float* gmax_p, const float* grs_m
   return cudaGetLastError();
 }
 
-cudaError_t sigma_exps(const int* eX, int shift, const float* grs, int ntau, int naux, int* eY3, cudaStream_t st) {
-  sigma_exps_kernel<<<nblk(ntau, 128), 128, 0, st>>>(eX, shift, grs, ntau, naux, eY3);
+cudaError_t sigma_exps(const int* eX, int shift, const float* grs, int nt, int ntau, int naux, int* eY3, int* eY3b,
+                       cudaStream_t st) {
+  sigma_exps_kernel<<<nblk(nt, 4), 128, 0, st>>>(eX, shift, grs, nt, ntau, naux, eY3, eY3b);
   return cudaGetLastError();
 }
 

@@ -32,6 +32,7 @@
 #include "gw_internal.cuh"
 #include "umma_ptx.cuh"
 
+#include <cstring>
 #include <map>
 #include <vector>
 #include <mutex>
@@ -91,6 +92,16 @@ struct UmmaArgs {
   int zin;
   int za_o, za_i, zb_o, zb_i;
   int64_t ea_zso, eb_zso, eo_zso, c_zso;
+  const int* c_list;   // non-null: the output of batch entry z goes to entry c_list[z]
+  // a_npc > 0: A is stored in K pieces of 8 elements, [batch][a_npc][a_rows][8] (UmmaOperand::pieces)
+  int a_npc;
+  int64_t a_rows;
+  const uint16_t* Ahi;
+  const uint16_t* Alo;
+  // q_naux > 0: blocked columns, the output and (C2) its conjugate transpose over (i, a) (UmmaOut)
+  int q_naux, q_nao, q_nt, q_npc;
+  void* C2;
+  void* C2_lo;
 };
 
 // index m / div of an exponent array (rows and columns fit in 32 bits; div >= 2^30
@@ -103,6 +114,10 @@ __device__ __forceinline__ int64_t zlin(const UmmaArgs& a, int z, int64_t s, int
   if (a.zin <= 0) return (int64_t)z * s;
   const int zo = (int)((uint32_t)z / (uint32_t)a.zin);
   return (int64_t)zo * so + (int64_t)(z - zo * a.zin) * s;
+}
+// output offset of batch entry z
+__device__ __forceinline__ int64_t c_zoff(const UmmaArgs& a, int z) {
+  return a.c_list ? (int64_t)a.c_list[z] * a.c_zs : zlin(a, z, a.c_zs, a.c_zso);
 }
 // exponent of the row scale of row m (output or operand side); 0 without scales
 __device__ __forceinline__ int row_exp(const UmmaArgs& a, int z, int64_t m) {
@@ -392,7 +407,7 @@ __device__ __forceinline__ void umma_write_block(const UmmaArgs& a, int z, int r
   {
     const int row = r0 + lane;
     const int64_t ro = row / a.row_inner, ri = row - ro * a.row_inner;
-    myoff = zlin(a, z, a.c_zs, a.c_zso) + ro * a.row_s1 + ri * a.c_ld;
+    myoff = c_zoff(a, z) + ro * a.row_s1 + ri * a.c_ld;
   }
   const int n = n0 + lane;
   const bool colok = lane < ncol && n < a.N;
@@ -622,7 +637,7 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
           const uint32_t ph = (g / NS) & 1u;
           if (!mbar_wait(&empty[s], ph ^ 1u, a.spin)) { atomicCAS(&s_fail, 0, 1); ok = false; break; }
           uint8_t* st = sStage + s * Cf::STAGE;
-          if (a.prefetch > 0) {   // warm L2 with the operand tiles a few stages ahead
+          if (a.prefetch > 0 && a.a_npc == 0) {   // warm L2 with the operand tiles a few stages ahead
             const int itp = it + a.prefetch;
             if (itp < nst) {
               const int kbp = three ? kb0 + itp : kb0 + 2 * itp;
@@ -637,7 +652,17 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
               }
             }
           }
-          if (three) {
+          if (a.a_npc > 0) {   // 16-bit pieces: 2 KB runs of 128 rows (three products)
+            const int kb = kb0 + it, np = min(8, a.a_npc - kb * 8);
+            mbar_expect_tx(&full[s], 2 * ((uint32_t)np * 2048u + B_BYTES));
+            const int64_t o = ((int64_t)za * a.a_npc + kb * 8) * a.a_rows + m0;
+            for (int j = 0; j < np; ++j) {
+              bulk_load(st + j * 2048, a.Ahi + (o + j * a.a_rows) * 8, 2048u, &full[s]);
+              bulk_load(st + A_BYTES + j * 2048, a.Alo + (o + j * a.a_rows) * 8, 2048u, &full[s]);
+            }
+            tma_load_3d(st + 2 * A_BYTES, &tB0, &full[s], kb * a.bke, n0, zb);
+            tma_load_3d(st + 2 * A_BYTES + B_BYTES, &tB1, &full[s], kb * a.bke, n0, zb);
+          } else if (three) {
             const int kb = kb0 + it;
             mbar_expect_tx(&full[s], 2 * (A_BYTES + B_BYTES));
             tma_load_3d(st, &tA0, &full[s], kb * a.bke, m0, za);
@@ -694,7 +719,10 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t d = tmem + (uint32_t)((grp * 2 + b) * BN);
           uint8_t* st = sStage + s * Cf::STAGE;
-          const uint64_t ah = sw128_desc(st), al = sw128_desc(st + A_BYTES);
+          const bool apc = a.a_npc > 0;
+          const uint64_t ah = apc ? piece_desc(st) : sw128_desc(st);
+          const uint64_t al = apc ? piece_desc(st + A_BYTES) : sw128_desc(st + A_BYTES);
+          const uint64_t astep = apc ? 4096 >> 4 : 2;   // 32 bytes of K: two pieces on, or along the swizzled row
           const uint64_t bh = sw128_desc(st + 2 * A_BYTES), bl = sw128_desc(st + 2 * A_BYTES + B_BYTES);
           // 32 bytes of K per MMA; the zero padding of the last k-block of the K range is skipped
           const int kb_first = three ? kb0 + it : kb0 + 2 * it;
@@ -702,11 +730,11 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
 #pragma unroll
           for (int kk = 0; kk < UM_BK / 8; ++kk) {
             if (kk < nk1) {
-              const uint64_t o = (uint64_t)(kk * 2);
-              umma_step(f16, d, ah + o, bh + o, idesc, (!chunk_first || kk > 0) ? 1u : 0u);   // hi * hi
+              const uint64_t o = (uint64_t)(kk * 2), oa = (uint64_t)kk * astep;
+              umma_step(f16, d, ah + oa, bh + o, idesc, (!chunk_first || kk > 0) ? 1u : 0u);   // hi * hi
               if (three) {
-                umma_step(f16, d, ah + o, bl + o, idesc, 1u);                                   // hi * lo
-                umma_step(f16, d, al + o, bh + o, idesc, 1u);                                   // lo * hi
+                umma_step(f16, d, ah + oa, bl + o, idesc, 1u);                                   // hi * lo
+                umma_step(f16, d, al + oa, bh + o, idesc, 1u);                                   // lo * hi
               }
             }
           }
@@ -819,7 +847,74 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
       if (!single) asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       // write-out
       const int row = m0 + quarter * 32 + lane;
-      if (a.direct && m0 + quarter * 32 < a.M) {
+      if (BW % 32 == 0 && a.q_naux > 0) {
+        // 32 columns are a 4 x 4 block of complex (i, a): each lane holds it for its row (t, Q) and
+        // stores four 16-byte pieces of rows (i, Q) and, conjugated, four of rows (a, Q) per plane;
+        // pieces of consecutive Q are contiguous, so a warp's store is 512 contiguous bytes.  With
+        // K-contiguous rows the same stores hit 32 lines each and took longer (0.26 ms per order of
+        // the 0.43 GB of a launch at nao 52, naux 400, 50 tau points) than the products (0.36 ms)
+        // leave to hide.
+        const bool rok = row < a.M;
+        const int t = row / a.q_naux, Q = row - t * a.q_naux;
+        const int64_t rows = (int64_t)a.q_naux * a.q_nao;   // rows of a K piece
+        const int64_t o1 = c_zoff(a, z) + ((int64_t)t * a.q_npc * rows + Q) * 8;
+        const int64_t o2 = c_zoff(a, z) + ((int64_t)(a.q_nt - 1 - t) * a.q_npc * rows + Q) * 8;
+        const int nb4 = (a.q_nao + 3) >> 2;
+        const float sc = rok ? (float)a.alpha * p2f(row_exp(a, z, row) - out_exp(a, z, row) + col_exp(a, z, 0)) : 0.f;
+        for (int cb = 0; cb < BW; cb += 32) {
+          const int nb = n0 + cbase + cb;
+          if (nb >= a.N) break;
+          uint32_t v[32];
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+              "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+              : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+                "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+                "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+              : "r"(tbase + (uint32_t)cb));
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          uint32_t h[16], l[16];
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const float2 x = make_float2(sc * __uint_as_float(v[2 * j]), sc * __uint_as_float(v[2 * j + 1]));
+            if (a.o_half == 2) {
+              const __nv_bfloat162 hb = __float22bfloat162_rn(x);
+              const float2 hx = __bfloat1622float2(hb);
+              const __nv_bfloat162 lb = __float22bfloat162_rn(make_float2(x.x - hx.x, x.y - hx.y));
+              h[j] = *(const uint32_t*)&hb;
+              l[j] = *(const uint32_t*)&lb;
+            } else {
+              const __half2 hb = __float22half2_rn(x);
+              const float2 hx = __half22float2(hb);
+              const __half2 lb = __float22half2_rn(make_float2(x.x - hx.x, x.y - hx.y));
+              h[j] = *(const uint32_t*)&hb;
+              l[j] = *(const uint32_t*)&lb;
+            }
+          }
+          if (!rok) continue;
+          const int blk = nb >> 5, i0 = (blk / nb4) * 4, a0 = (blk - (blk / nb4) * nb4) * 4;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            if (i0 + u < a.q_nao) {
+              const int64_t o = o1 + ((a0 >> 2) * rows + (int64_t)(i0 + u) * a.q_naux) * 8;
+              *(uint4*)((uint16_t*)a.C + o) = make_uint4(h[4 * u], h[4 * u + 1], h[4 * u + 2], h[4 * u + 3]);
+              *(uint4*)((uint16_t*)a.C_lo + o) = make_uint4(l[4 * u], l[4 * u + 1], l[4 * u + 2], l[4 * u + 3]);
+            }
+          }
+          if (a.C2) {
+            constexpr uint32_t cj = 0x80000000u;   // the sign of the imaginary piece
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              if (a0 + u < a.q_nao) {
+                const int64_t o = o2 + ((i0 >> 2) * rows + (int64_t)(a0 + u) * a.q_naux) * 8;
+                *(uint4*)((uint16_t*)a.C2 + o) = make_uint4(h[u] ^ cj, h[4 + u] ^ cj, h[8 + u] ^ cj, h[12 + u] ^ cj);
+                *(uint4*)((uint16_t*)a.C2_lo + o) = make_uint4(l[u] ^ cj, l[4 + u] ^ cj, l[8 + u] ^ cj, l[12 + u] ^ cj);
+              }
+            }
+          }
+        }
+      } else if (a.direct && m0 + quarter * 32 < a.M) {
         // complex output written transposed (real/imag column pairs land next to each
         // other, rows 2 floats apart): each lane stores its own row, so a warp's
         // float2 stores cover 256 contiguous bytes
@@ -827,7 +922,7 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
         {
           const int64_t ro = a.row_inner >= ((int64_t)1 << 31) ? 0 : (int64_t)((uint32_t)row / (uint32_t)a.row_inner);
           const int64_t ri = row - ro * a.row_inner;
-          myoff = zlin(a, z, a.c_zs, a.c_zso) + ro * a.row_s1 + ri * a.c_ld;
+          myoff = c_zoff(a, z) + ro * a.row_s1 + ri * a.c_ld;
         }
         const bool rok = row < a.M;
         float* C = (float*)a.C;
@@ -1090,9 +1185,11 @@ static cudaError_t umma_launch(int bn, const UmmaOperand& A, const UmmaOperand& 
                                const UmmaArgs& a, int batch, cudaStream_t st) {
   CUtensorMap maps[4];
   const uint32_t box = (uint32_t)bn;
+  memset(maps, 0, sizeof maps);
   const int f16 = a.f16;
-  if (!make_map(&maps[0], A.hi, Kpad, A.rows, A.batch, A.ld, A.bs, UM_BM, f16) ||
-      !make_map(&maps[1], nseg > 1 ? A.lo : A.hi, Kpad, A.rows, A.batch, A.ld, A.bs, UM_BM, f16) ||
+  const bool pcs = a.a_npc > 0;   // A is not read through a tensor map
+  if ((!pcs && !make_map(&maps[0], A.hi, Kpad, A.rows, A.batch, A.ld, A.bs, UM_BM, f16)) ||
+      (!pcs && !make_map(&maps[1], nseg > 1 ? A.lo : A.hi, Kpad, A.rows, A.batch, A.ld, A.bs, UM_BM, f16)) ||
       !make_map(&maps[2], B.hi, Kpad, B.rows, B.batch, B.ld, B.bs, box, f16) ||
       !make_map(&maps[3], nseg > 1 ? B.lo : B.hi, Kpad, B.rows, B.batch, B.ld, B.bs, box, f16))
     return cudaErrorInvalidValue;
@@ -1137,6 +1234,9 @@ static const int kBnCand[] = {128, 112, 96, 80, 64, 48, 32};
 static const int kBnWide[] = {256, 224, 192, 160};   // tried when N >= 160
 
 
+// N tiles whose halves (or whole) hold 4 x 4 blocks of complex columns
+static bool blocked_bn(int bn) { return bn % (bn > 128 ? 64 : 32) == 0; }
+
 static int cost_model_bn(int N) {
   // trade the padding of the last tile against the per-tile cost of re-reading
   // the A tile (modelled as 32 extra columns per tile)
@@ -1162,6 +1262,7 @@ static int tune_bn(const UmmaOperand& A, const UmmaOperand& B, int64_t Kpad, int
   std::vector<int> cands(kBnCand, kBnCand + sizeof(kBnCand) / sizeof(int));
   if (a.N >= 160 && g_wide) cands.insert(cands.begin(), kBnWide, kBnWide + sizeof(kBnWide) / sizeof(int));
   for (int cand : cands) {
+    if (a.q_naux > 0 && !blocked_bn(cand)) continue;
     if (umma_launch(cand, A, B, Kpad, nseg, t, batch, st) != cudaSuccess) continue;   // warm-up
     float cand_ms = 1e30f;
     for (int rep = 0; rep < 3; ++rep) {   // best of three: single timings of short launches are noisy
@@ -1188,6 +1289,8 @@ cudaError_t umma_gemm(const UmmaOperand& A, const UmmaOperand& B, int M, int N, 
   const bool f16 = A.f16 != 0;
   const int bke = f16 ? 64 : UM_BK;   // elements per 128-byte k-block
   if (B.f16 != A.f16) return cudaErrorInvalidValue;   // one MMA kind: both operands fp16 or both tf32
+  if (A.pieces > 0 && (!f16 || nseg != 3 || ksplit > 1 || A.pieces % 2 || (uintptr_t)A.hi % 16 || (uintptr_t)A.lo % 16))
+    return cudaErrorInvalidValue;
   if (f16 && (!g_persistent || !scale)) return cudaErrorInvalidValue;   // fp16 pieces carry row scales
   if (Kpad % bke) return cudaErrorInvalidValue;
   if (ksplit < 1) ksplit = 1;
@@ -1197,6 +1300,10 @@ cudaError_t umma_gemm(const UmmaOperand& A, const UmmaOperand& B, int M, int N, 
   a.M = M; a.N = N; a.kblocks = (int)(Kpad / bke); a.nseg = nseg;
   a.f16 = A.f16;
   a.bke = bke;
+  if (A.pieces > 0) {
+    a.a_npc = A.pieces; a.a_rows = A.rows;
+    a.Ahi = (const uint16_t*)A.hi; a.Alo = (const uint16_t*)A.lo;
+  }
   a.a_batched = A.batch > 1; a.b_batched = B.batch > 1;
   a.za_i = a.zb_i = 1;
   if (zz && zz->zin > 0) {
@@ -1204,6 +1311,10 @@ cudaError_t umma_gemm(const UmmaOperand& A, const UmmaOperand& B, int M, int N, 
     a.zin = zz->zin;
     a.za_o = zz->za_o; a.za_i = zz->za_i; a.zb_o = zz->zb_o; a.zb_i = zz->zb_i;
     a.ea_zso = zz->ea_zso; a.eb_zso = zz->eb_zso; a.eo_zso = zz->eo_zso; a.c_zso = zz->c_zso;
+  }
+  if (zz && zz->c_list) {
+    if (!g_persistent || zz->zin > 0) return cudaErrorInvalidValue;
+    a.c_list = zz->c_list;
   }
   a.C = C; a.c_fp64 = c_fp64; a.accumulate = accumulate; a.alpha = alpha; a.c_ld = c_ld; a.c_zs = c_zs;
   a.ksplit = ksplit;
@@ -1219,6 +1330,14 @@ cudaError_t umma_gemm(const UmmaOperand& A, const UmmaOperand& B, int M, int N, 
     if (!C_lo || !g_persistent || (out->half != 1 && out->half != 2)) return cudaErrorInvalidValue;
     a.o_half = out->half; a.eO = out->eO; a.eo_zs = out->eo_zs; a.eo_shift = out->eo_shift;
     a.eo_div = out->eo_div > 0 ? out->eo_div : 1;
+    if (out->naux > 0) {
+      // 16-byte stores of four complex pieces; B's exponent is one per batch entry
+      if (!scale || scale->eb_div < ((int64_t)1 << 30) || c_fp64 || accumulate || N % 32 || c_zs % 8 ||
+          (uintptr_t)C % 16 || (uintptr_t)C_lo % 16 || (uintptr_t)out->C2 % 16 || (uintptr_t)out->C2_lo % 16)
+        return cudaErrorInvalidValue;
+      a.q_naux = out->naux; a.q_nao = out->nao; a.q_nt = out->nt; a.q_npc = out->npc;
+      a.C2 = out->C2; a.C2_lo = out->C2_lo;
+    }
   }
   const int oes = a.o_half ? 2 : 4;   // bytes per element of an fp32-class output
   // (re, im) column pairs of a complex output that land next to each other while
@@ -1246,12 +1365,13 @@ cudaError_t umma_gemm(const UmmaOperand& A, const UmmaOperand& B, int M, int N, 
     a.ea_mod = scale->ea_mod > 0 ? scale->ea_mod : 0;
   }
   int bn = cost_model_bn(N);
-  if (g_force_bn) return umma_launch(g_force_bn, A, B, Kpad, nseg, a, batch, st);
+  if (a.q_naux > 0 && !blocked_bn(bn)) bn = bn > 96 ? 128 : bn > 64 ? 96 : bn > 32 ? 64 : 32;
+  if (g_force_bn && (a.q_naux == 0 || blocked_bn(g_force_bn))) return umma_launch(g_force_bn, A, B, Kpad, nseg, a, batch, st);
   if (g_persistent && g_autotune) {
     const TuneKey key{M, N, batch, nseg, ksplit,
                       (c_fp64 ? 1 : 0) | (accumulate ? 2 : 0) | (a.direct ? 4 : 0) | (C_lo ? 8 : 0) |
                           (a.a_batched ? 16 : 0) | (a.b_batched ? 32 : 0) | (scale ? 64 : 0) | (f16 ? 128 : 0) |
-                          (a.f16 == 2 ? 256 : 0) | (a.o_half << 9),
+                          (a.f16 == 2 ? 256 : 0) | (a.o_half << 9) | (a.q_naux > 0 ? 2048 : 0) | (a.C2 ? 4096 : 0) | (a.a_npc > 0 ? 8192 : 0),
                       Kpad};
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tuned.find(key);

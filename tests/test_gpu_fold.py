@@ -106,3 +106,51 @@ def test_screened_of_a_given_p0(defect):
     ref = ogw.screened(P0)
     assert rel(g.get("P_iw"), ref) < 1e-11
     assert rel(g.get("P_tau"), ogw.herm(ogw.to_matsubara(st.grid.TBb, ref, 1))) < 1e-10
+
+
+def _folded(P, km):
+    """P~ with the mirror symmetry P~^{-q}(beta - tau) = conj P~^q(tau), exactly."""
+    neg = [km.index(-km.vec[q]) for q in range(km.nk)]
+    return 0.5 * (P + np.conj(P[neg][:, ::-1]))
+
+
+@pytest.mark.parametrize("nao,kmesh,ntau,qr", [(4, (2, 2, 1), 6, None), (5, (2, 1, 1), 5, None), (7, (3, 1, 1), 5, None),
+                                               (13, (3, 2, 1), 4, None), (8, (4, 1, 1), 5, (1, 4)),
+                                               (3, (4, 1, 1), 4, (1, 3)), (16, (1, 1, 1), 1, None)])
+@pytest.mark.parametrize("sym", [True, False])
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "split_tf32", "split_f16", "split_bf16"])
+def test_selfenergy_blocks(nao, kmesh, ntau, qr, sym, precision):
+    # one X for (k, q, tau) and its image where P~ is symmetric, every block where it is not;
+    # nao with and without whole 4 x 4 column blocks, odd and even tau counts
+    naux = 19
+    sysd = system(nao, naux, kmesh, ntau, 20.0, 91)
+    km = ogw.KMesh(kmesh)
+    G = hermitian_noise((ntau, km.nk, nao, nao), 0.3, 92)
+    P = hermitian_noise((km.nk, ntau, naux, naux), 0.3, 93)
+    if sym:
+        P = _folded(P, km)
+    qs = list(range(km.nk) if qr is None else range(*qr))
+    ref = ogw.selfenergy_tau(sysd["V"], G, P, km, qs=qs)
+    g = gpu(sysd, precision=precision)
+    if qr is not None:
+        g.set_q_range(*qr)
+    g.set("G_tau", G)
+    g.set("P_tau", P)
+    g.selfenergy_partial()
+    assert rel(g.get("Sigma_tau"), ref) < TOL[precision]
+
+
+@pytest.mark.parametrize("kmesh,ntau", [((2, 1, 1), 5), ((3, 1, 1), 4)])
+def test_polarization_vjp_blocks(kmesh, ntau):
+    # the adjoint of the folded P~0 against the oracle's, which runs over every block
+    from oracle import adjoint as oad
+    import torch
+    sysd = system(4, 11, kmesh, ntau, 20.0, 95)
+    km = ogw.KMesh(kmesh)
+    rng = np.random.default_rng(96)
+    G = rng.standard_normal((ntau, km.nk, 4, 4)) + 1j * rng.standard_normal((ntau, km.nk, 4, 4))
+    Pbar = rng.standard_normal((km.nk, ntau, 11, 11)) + 1j * rng.standard_normal((km.nk, ntau, 11, 11))
+    g = gpu(sysd)
+    g.set("G_tau", G)
+    got = g.polarization_vjp(torch.from_numpy(Pbar).cuda()).cpu().numpy()
+    assert rel(got, oad.polarization_vjp(sysd["V"], G, km, Pbar)) < 1e-12
