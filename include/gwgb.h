@@ -264,8 +264,8 @@ gw_status gw_set_q_range(gw_ctx* ctx, int32_t q0, int32_t q1);
 
 /* Dyson equation (Eq. Dyson) with chemical-potential search: a bracketing
  * search on N(mu) = (s/Nk) sum_k tr[gamma^k S^k] (the bracket [mu_prev - 1,
- * mu_prev + 1] widened until N - n_elec changes sign, then Illinois
- * regula-falsi steps with a plain bisection every fourth step) until
+ * mu_prev + 1] widened until N - n_elec changes sign, then inverse quadratic
+ * interpolation safeguarded by bisection) until
  * |N - n_elec| <= mu_tol and the bracket is below 1e-13, then G(i w) = [(i w + mu) S - H0 - Sigma_inf -
  * Sigma~(i w)]^{-1} and G(tau) (symmetrised).  With no self-energy set this is
  * the non-interacting G0.  Synchronises.  mu_out may be NULL. */

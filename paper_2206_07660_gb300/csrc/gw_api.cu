@@ -9,6 +9,7 @@
 #include <new>
 #include <string>
 #include <vector>
+#include <algorithm>
 #include <atomic>
 #include <nvtx3/nvToolsExt.h>
 #include "gw_internal.cuh"
@@ -61,6 +62,10 @@ struct gw_ctx {
   void* irws = nullptr;
   size_t irws_bytes = 0;
   int *d_fn = nullptr, *d_bm = nullptr;
+  int* d_wpart = nullptr;   // fermionic frequency index of -w_n (-1: none), then the nwrep kept frequencies
+  int nwrep = 0;
+  bool hsherm = false;      // H0 and S are Hermitian to kAdjointTol
+  bool tfadj = false;       // TFf(-w) = conj TFf(w) to rounding
   // state
   double2 *G_tau = nullptr, *G_iw = nullptr, *G_prev = nullptr, *gamma = nullptr, *tQ = nullptr;
   double2 *Sinf = nullptr, *Sinf_new = nullptr, *Siw = nullptr, *Siw_new = nullptr, *Stau = nullptr;
@@ -702,6 +707,7 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
     }
   }
   c->r = (double2*)need(A(nwf * cb));
+  c->d_wpart = (int*)need(A((size_t)2 * nwf * 4));
   c->d_fn = (int*)need(A(nwf * 4)); c->d_bm = (int*)need(A(nwb * 4));
   const size_t gsz = (size_t)ntau * nk * n2 * cb, gszw = (size_t)nwf * nk * n2 * cb;
   c->G_tau = (double2*)need(A(gsz)); c->G_iw = (double2*)need(A(gszw)); c->G_prev = (double2*)need(A(gsz));
@@ -890,6 +896,14 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
   chk(cudaMemcpyAsync(c->H0, H0, nk * n2 * cb, kind, st), "H0 copy");
   chk(cudaMemcpyAsync(c->S, S, nk * n2 * cb, kind, st), "S copy");
   if (!(cfg->flags & GW_BORROW_V)) chk(cudaMemcpyAsync(c->V, V, vbytes, kind, st), "V copy");
+  std::vector<int> wpart((size_t)nwf, -1);   // w_n = (2n + 1) pi / beta: n and -n - 1
+  for (int i = 0; i < nwf; ++i)
+    for (int j = 0; j < nwf; ++j)
+      if (fn_h[j] == -fn_h[i] - 1) wpart[(size_t)i] = j;
+  for (int i = 0; i < nwf; ++i)
+    if (wpart[(size_t)i] < 0 || fn_h[i] >= 0) wpart.push_back(i);
+  c->nwrep = (int)wpart.size() - nwf;
+  chk(cudaMemcpyAsync(c->d_wpart, wpart.data(), wpart.size() * 4, cudaMemcpyHostToDevice, st), "index copy");
   chk(cudaMemcpyAsync(c->d_fn, fn_h, nwf * 4, cudaMemcpyHostToDevice, st), "index copy");
   chk(cudaMemcpyAsync(c->d_bm, bm_h, nwb * 4, cudaMemcpyHostToDevice, st), "index copy");
   chk(cudaMemsetAsync(c->info, 0, 64, st), "memset");
@@ -983,12 +997,12 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
       chk(check_trs(c->V, (int64_t)nk * nk, (int64_t)naux * n2, c->d_vpart, c->dscr + 14, st), "check");
       count(3);
     }
-    chk(check_herm(c->H0, nao, nk, c->dscr, st), "check");
-    chk(check_herm(c->S, nao, nk, c->dscr + 2, st), "check");
-    count(2);
   }
-  // the pairing decides whether P~0 is folded over (q, tau) -> (-q, beta - tau), so it is
-  // measured with GW_SKIP_CHECKS too (without the error)
+  // measured with GW_SKIP_CHECKS too (without the errors): the pairing decides whether P~0 is folded
+  // over (q, tau) -> (-q, beta - tau), the Hermiticity whether Dyson's negative frequencies are adjoints
+  chk(check_herm(c->H0, nao, nk, c->dscr, st), "check");
+  chk(check_herm(c->S, nao, nk, c->dscr + 2, st), "check");
+  count(2);
   chk(check_v_pairing(c->V, nk, naux, nao, c->dscr + 4, st), "check");
   count(1);
   chk(cudaMemcpyAsync(c->h_scr, c->dscr, 64 * 8, cudaMemcpyDeviceToHost, st), "copy");
@@ -1019,7 +1033,23 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
                "V^{-k,-k'} = conj V^{kk'} within 1e-10)";
     }
   }
+  c->hsherm = std::isfinite(c->h_scr[1]) && std::isfinite(c->h_scr[3]) && c->h_scr[0] <= kAdjointTol * c->h_scr[1] &&
+              c->h_scr[2] <= kAdjointTol * c->h_scr[3];
   c->fold = std::isfinite(c->h_scr[5]) && c->h_scr[4] <= kPairTol * c->h_scr[5];
+  if (s == GW_OK) {
+    std::vector<double2> F((size_t)nwf * ntau);
+    chk(cudaMemcpy(F.data(), c->TFf, F.size() * 16, cudaMemcpyDeviceToHost), "copy");
+    double dev = 0, mx = 0;
+    for (int w = 0; w < nwf; ++w)
+      for (int j = 0; j < ntau; ++j) {
+        const double2 x = F[(size_t)w * ntau + j];
+        mx = std::fmax(mx, std::fmax(std::fabs(x.x), std::fabs(x.y)));
+        if (wpart[(size_t)w] < 0) continue;
+        const double2 y = F[(size_t)wpart[(size_t)w] * ntau + j];
+        dev = std::fmax(dev, std::fmax(std::fabs(x.x - y.x), std::fabs(x.y + y.y)));
+      }
+    c->tfadj = dev <= 1e-13 * mx;
+  }
   if (s == GW_OK && c->fold && c->irws) {
     chk(fold_build(c, bm_h), "folded block");
     if (s == GW_OK && c->wfold) {
@@ -1183,7 +1213,7 @@ static gw_status exchange(gw_ctx* c, const double2* gamma, double2* out) {
     e.bk = I1(nao); e.bn = I1(1); e.bz = I1(slab);
     e.cm = I1(nao); e.cn = I1(1); e.cz = I1(n2);
     e.alpha = make_double2(-1.0 / nk, 0); e.beta = make_double2(1, 0);
-    e.ksplit = split_blocks(nao, nk, e.K);
+    e.ksplit = std::max(16, split_blocks(nao, nk, e.K));
     const char* Vk = (const char*)Vp + (size_t)kp * nk * slab * es;
     CK(run_gett(e, c->chA, tv, Vk, tv, out, Ty::C128, acc, c));
   }
@@ -1198,7 +1228,13 @@ static gw_status hf_core(gw_ctx* c, const double2* Gsrc, double2* gamma, double2
   CK(hartree_t(c->V, gamma, c->tQ, nk, naux, nao, c->st));
   CK(hartree_j(c->V, c->tQ, out, nk, naux, nao, c->spin / nk, c->st));   // Eq. HF_J
   count(3);
-  return exchange(c, gamma, out);
+  gw_status s = exchange(c, gamma, out);
+  if (s != GW_OK) return s;
+  // a Hermitian density matrix has a Hermitian Sigma_inf: the products' rounding (FP32 on the mixed
+  // paths) is averaged over (i, j) and (j, i)
+  CK(herm_like(out, gamma, nao, nk, c->dscr + 20, c->st));
+  count(2);
+  return GW_OK;
 }
 
 extern "C" gw_status gw_hf(gw_ctx* c) {
@@ -1905,7 +1941,7 @@ static gw_status sigma_chain(gw_ctx* c, const double2* Gsrc, const double2* Psrc
         d3.cm = I1(nao); d3.cn = I1(1); d3.cz = I1(ts);
         d3.alpha = make_double2(-1.0 / nk, 0);
         d3.beta = make_double2(accumulate || share || q > c->q0 ? 1.0 : 0.0, 0);
-        d3.ksplit = split_blocks(nao, zt, d3.K);
+        d3.ksplit = std::max(8, split_blocks(nao, zt, d3.K));   // (an FP32 sum is no longer than an eighth)
         const char* Vk2 = (const char*)Vp + ((size_t)kg * nk + ko) * slab * es;
         CK(run_gett(d3, c->chB, tv, Vk2, tv, out + t0 + (size_t)ko * n2, Ty::C128, acc, c));
       }
@@ -1949,9 +1985,24 @@ static gw_status sigma_tau_part(gw_ctx* c) {
   return GW_OK;
 }
 
+static DysonArgs dyson_args(gw_ctx* c) {
+  DysonArgs a{};
+  a.nao = c->nao; a.nk = c->nk; a.nw = c->nw;
+  a.H0 = c->H0; a.S = c->S; a.Sinf = c->Sinf; a.Siw = c->Siw;
+  a.wn = c->wn; a.r = c->r; a.spin = c->spin;
+  a.wpart = c->d_wpart; a.nrep = c->nwrep;
+  a.sym = c->hsherm ? c->dscr + 18 : nullptr;   // dscr[18..19], measured by dyson_begin
+  return a;
+}
+
 // Sigma~(i w_n) = sum_j TFf[n][j] Sigma~(tau_j)   (Eq. tau_to_iw) into Siw_new
 static gw_status sigma_iw_new(gw_ctx* c) {
   CK(transform(c, c->TFf, c->Stau, c->Siw_new, c->nw, (int64_t)c->nk * c->n2, 1, 0, 0));
+  if (c->tfadj) {
+    // a Hermitian Sigma~(tau) has Sigma~(-i w) = Sigma~(i w)^H: exactly so, for the Dyson solve
+    CK(siw_adjoint(dyson_args(c), c->Siw_new, c->Stau, c->ntau * c->nk, c->dscr + 20, c->st));
+    count(2);
+  }
   return GW_OK;
 }
 
@@ -2013,17 +2064,18 @@ extern "C" gw_status gw_set_q_range(gw_ctx* c, int32_t q0, int32_t q1) {
 
 // ------------------------------------------------------------------ A7: Dyson + mu
 
-static DysonArgs dyson_args(gw_ctx* c) {
-  DysonArgs a{};
-  a.nao = c->nao; a.nk = c->nk; a.nw = c->nw;
-  a.H0 = c->H0; a.S = c->S; a.Sinf = c->Sinf; a.Siw = c->Siw;
-  a.wn = c->wn; a.r = c->r; a.spin = c->spin;
-  return a;
+// measures whether the negative frequencies are the adjoints of the positive ones (on the device: the
+// inversions read it there, inside a captured iteration too)
+static cudaError_t dyson_begin(gw_ctx* c, const DysonArgs& a) {
+  if (!a.sym) return cudaSuccess;
+  count(1);
+  return dyson_sym(a, c->dscr + 18, c->st);
 }
 
 extern "C" gw_status gw_dyson(gw_ctx* c, double* mu_out) {
   if (!c) return GW_ERR_ARG;
   DysonArgs a = dyson_args(c);
+  CK(dyson_begin(c, a));
   const int64_t nsys = (int64_t)c->nw * c->nk;
   const double scale = -c->spin / c->nk;
   MuState* h = c->h_mus;
@@ -2077,6 +2129,7 @@ extern "C" gw_status gw_dyson(gw_ctx* c, double* mu_out) {
 // fixed number of (evaluate, step) pairs; converged pairs exit at once.
 static gw_status dyson_device(gw_ctx* c) {
   DysonArgs a = dyson_args(c);
+  CK(dyson_begin(c, a));
   const int64_t nsys = (int64_t)c->nw * c->nk;
   const double scale = -c->spin / c->nk;
   const int steps = c->cfg.mu_maxit < 96 ? c->cfg.mu_maxit : 96;

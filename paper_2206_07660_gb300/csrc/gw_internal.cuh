@@ -115,14 +115,31 @@ struct DysonArgs {
   const double* wn;      // fermionic frequencies [nw]
   const double2* r;      // density weights [nw] (complex)
   double spin;
+  // frequency index of -w_n (-1: none), and the deviations measured by dyson_sym: where they allow,
+  // the systems of a negative frequency are the adjoints of their positive partners
+  // nrep: frequencies to invert then, listed behind the nw entries of wpart
+  int nrep;
+  const int* wpart;
+  const double* sym;     // {deviation, largest value} (null: every system is inverted)
 };
+// sym[0] = largest deviation of Sinf [nk] from its adjoint and of Siw from Siw(-w) = Siw(w)^H,
+// sym[1] = largest magnitude of the two
+cudaError_t dyson_sym(const DysonArgs& a, double* sym, cudaStream_t st);
+constexpr double kAdjointTol = 4e-15;   // deviation, relative to the largest value, that is taken as rounding
+// Siw(w) and Siw(-w)^H <- their mean, if the `count` matrices of Stau are Hermitian to kAdjointTol
+// (a: Siw, wpart and the sizes; scr: two doubles of scratch)
+cudaError_t siw_adjoint(const DysonArgs& a, double2* Siw, const double2* Stau, int count, double* scr, cudaStream_t st);
+// X <- (X + X^H)/2 for `count` n x n matrices if the `count` matrices of g are Hermitian to kAdjointTol
+// (scr: two doubles of scratch)
+cudaError_t herm_like(double2* X, const double2* g, int n, int count, double* scr, cudaStream_t st);
 cudaError_t dyson_eval(const DysonArgs& a, const double* mu_ptr, double2* G_out, double* partial,
                        const int* done_flag, int* d_info, cudaStream_t st);
 struct MuState {
   double lo, hi, Nlo, Nhi, x, Nx, target, tol, width;
   int phase, iter, maxit, done, status;
-  double flo, fhi;   // Illinois-weighted N - target at the bracket ends
-  int side;          // which end moved last (-1 lo, +1 hi, 0 none)
+  double xa, fa, xb, fb, xc, fc;   // latest point, the bracket's other end, the point before: x and N - target
+  double w1, w2;                   // bracket widths one and two steps ago
+  int sa;                          // which end of the bracket xa is: -1 lo, +1 hi
 };
 cudaError_t mu_step(MuState* s, const double* partial, int64_t count, double scale, cudaStream_t st);
 cudaError_t dyson_tangent_rhs(const double2* dSinf, const double2* dSiw, double2* D, int64_t nk, int64_t n2,
@@ -131,7 +148,6 @@ cudaError_t dyson_tangent_finish(const double2* X, const double2* Y, const doubl
                                  int nk, int nw, double* part, double* dmu, double2* dG, cudaStream_t st);
 int rdot_blocks(int64_t n);
 cudaError_t rdot_partials(const double2* a, const double2* b, int64_t n, double* part, cudaStream_t st);
-size_t dyson_smem(int nao, int nt);
 cudaError_t mu_init_device(MuState* s, double target, double tol, double width, int maxit, cudaStream_t st);
 
 cudaError_t density_gamma(const double2* G_tau, const double* lb, double2* gamma, int ntau, int64_t nelem,

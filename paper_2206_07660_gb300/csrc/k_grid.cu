@@ -152,14 +152,12 @@ __global__ void __launch_bounds__(1024) gj_global_kernel(double2* A, int n, int*
   extern __shared__ unsigned char smem[];
   double2* f = (double2*)smem;
   int* perm = (int*)(f + n);
-  double* rv = (double*)(perm + n + (n & 1));
-  int* ri = (int*)(rv + blockDim.x);
-  int bad = gj_invert_smem(A, n, n, f, perm, rv, ri);  // A in global memory, same algorithm
+  int bad = gj_invert_smem(A, n, n, f, perm);  // A in global memory, same algorithm
   if (threadIdx.x == 0 && bad) atomicOr(info, 1);
 }
 cudaError_t invert_small_gj(double2* A, int n, int* d_info, cudaStream_t st) {
   int nt = 256;
-  size_t sm = (size_t)n * sizeof(double2) + (size_t)(n + 1) * sizeof(int) + 8 + nt * (sizeof(double) + sizeof(int));
+  size_t sm = (size_t)n * sizeof(double2) + (size_t)n * sizeof(int);
   gj_global_kernel<<<1, nt, sm, st>>>(A, n, d_info);
   return cudaGetLastError();
 }

@@ -58,20 +58,17 @@ __global__ void zero_cols_kernel(T* X, int64_t n, int nb, int64_t kb, int64_t co
 template <typename T>
 __global__ void __launch_bounds__(256) block_inv_kernel(const T* __restrict__ Rp, int64_t n, int nb, int64_t kb,
                                                         int64_t count, T* Dinv, int* info) {
-  using R = typename gj_real<T>::t;
   extern __shared__ __align__(16) unsigned char smem[];
   T* A = (T*)smem;
   T* f = A + nb * nb;
   int* perm = (int*)(f + nb);
-  R* rv = (R*)(perm + nb + (nb & 1));
-  int* ri = (int*)(rv + blockDim.x);
   for (int64_t z = blockIdx.x; z < count; z += gridDim.x) {
     for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
       int r = e / nb, c = e - r * nb;
       A[e] = Rp[z * n * nb + (int64_t)r * n + kb + c];
     }
     __syncthreads();
-    int bad = gj_invert_smem(A, nb, nb, f, perm, rv, ri);
+    int bad = gj_invert_smem(A, nb, nb, f, perm);
     if (bad && threadIdx.x == 0) atomicOr(info, 1);
     for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) Dinv[z * nb * nb + e] = A[e];
     __syncthreads();
@@ -89,10 +86,8 @@ __global__ void put_dinv_kernel(T* Rn, const T* __restrict__ Dinv, int64_t n, in
 }
 
 template <typename T>
-static size_t block_inv_smem(int64_t nb, int nt) {
-  using R = typename gj_real<T>::t;
-  return (size_t)nb * nb * sizeof(T) + (size_t)nb * sizeof(T) + (size_t)(nb + 1) * sizeof(int) + 8 +
-         (size_t)nt * (sizeof(R) + sizeof(int));
+static size_t block_inv_smem(int64_t nb) {
+  return (size_t)nb * nb * sizeof(T) + (size_t)nb * sizeof(T) + (size_t)nb * sizeof(int);
 }
 
 // X[z][kb + r][j] = Rn[z][r][j]
@@ -137,7 +132,7 @@ static cudaError_t gj_blocked(T* X, int64_t n, int64_t count, void* work, size_t
   if (chunk <= 0) return cudaErrorMemoryAllocation;
   if (chunk > 65535) chunk = 65535;
   const int nt = 256;
-  const size_t sm = block_inv_smem<T>(nbmax, nt);
+  const size_t sm = block_inv_smem<T>(nbmax);
   cudaError_t e;
   if (sm > 48 * 1024) {
     e = cudaFuncSetAttribute(block_inv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -217,7 +212,7 @@ static cudaError_t gj_blocked_tc(T* X, int64_t n, int64_t cz, void* pan, float* 
   constexpr int C = reals<T>();
   const int64_t nbmax = n < NB ? n : NB, Kb = pad32(C * nbmax);
   const int nt = 256;
-  const size_t sm = block_inv_smem<T>(nbmax, nt);
+  const size_t sm = block_inv_smem<T>(nbmax);
   cudaError_t e;
   if (sm > 48 * 1024) {
     e = cudaFuncSetAttribute(block_inv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);

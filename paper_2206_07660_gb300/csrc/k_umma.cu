@@ -545,7 +545,11 @@ __device__ __forceinline__ void umma_write_block(const UmmaArgs& a, int z, int r
   }
 }
 
-template <int BN, bool SPLIT>
+// MODE 0: the general kernel; 1: blocked columns out (UmmaOut::naux); 2: A in K pieces
+// (UmmaOperand::pieces).  Compile-time, since the other loops slow down with them (2..5 % of a
+// split-TF32 chain as run-time branches).
+enum { UM_PLAIN = 0, UM_BLOCKED = 1, UM_PIECES = 2 };
+template <int BN, bool SPLIT, int MODE>
 __global__ void __launch_bounds__(UP_THREADS, 1)
     umma_pkernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUtensorMap tA1,
                  const __grid_constant__ CUtensorMap tB0, const __grid_constant__ CUtensorMap tB1, UmmaArgs a,
@@ -637,7 +641,7 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
           const uint32_t ph = (g / NS) & 1u;
           if (!mbar_wait(&empty[s], ph ^ 1u, a.spin)) { atomicCAS(&s_fail, 0, 1); ok = false; break; }
           uint8_t* st = sStage + s * Cf::STAGE;
-          if (a.prefetch > 0 && a.a_npc == 0) {   // warm L2 with the operand tiles a few stages ahead
+          if (MODE != UM_PIECES && a.prefetch > 0) {   // warm L2 with the operand tiles a few stages ahead
             const int itp = it + a.prefetch;
             if (itp < nst) {
               const int kbp = three ? kb0 + itp : kb0 + 2 * itp;
@@ -652,7 +656,7 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
               }
             }
           }
-          if (a.a_npc > 0) {   // 16-bit pieces: 2 KB runs of 128 rows (three products)
+          if constexpr (MODE == UM_PIECES) {   // 16-bit pieces: 2 KB runs of 128 rows (three products)
             const int kb = kb0 + it, np = min(8, a.a_npc - kb * 8);
             mbar_expect_tx(&full[s], 2 * ((uint32_t)np * 2048u + B_BYTES));
             const int64_t o = ((int64_t)za * a.a_npc + kb * 8) * a.a_rows + m0;
@@ -719,10 +723,10 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t d = tmem + (uint32_t)((grp * 2 + b) * BN);
           uint8_t* st = sStage + s * Cf::STAGE;
-          const bool apc = a.a_npc > 0;
+          constexpr bool apc = MODE == UM_PIECES;
           const uint64_t ah = apc ? piece_desc(st) : sw128_desc(st);
           const uint64_t al = apc ? piece_desc(st + A_BYTES) : sw128_desc(st + A_BYTES);
-          const uint64_t astep = apc ? 4096 >> 4 : 2;   // 32 bytes of K: two pieces on, or along the swizzled row
+          constexpr uint64_t astep = apc ? 4096 >> 4 : 2;   // 32 bytes of K: two pieces on, or along the swizzled row
           const uint64_t bh = sw128_desc(st + 2 * A_BYTES), bl = sw128_desc(st + 2 * A_BYTES + B_BYTES);
           // 32 bytes of K per MMA; the zero padding of the last k-block of the K range is skipped
           const int kb_first = three ? kb0 + it : kb0 + 2 * it;
@@ -847,7 +851,8 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
       if (!single) asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       // write-out
       const int row = m0 + quarter * 32 + lane;
-      if (BW % 32 == 0 && a.q_naux > 0) {
+      if constexpr (MODE == UM_BLOCKED) {
+        static_assert(BW % 32 == 0, "whole 4 x 4 blocks of complex columns");
         // 32 columns are a 4 x 4 block of complex (i, a): each lane holds it for its row (t, Q) and
         // stores four 16-byte pieces of rows (i, Q) and, conjugated, four of rows (a, Q) per plane;
         // pieces of consecutive Q are contiguous, so a warp's store is 512 contiguous bytes.  With
@@ -1138,9 +1143,9 @@ static size_t umma_psmem() {
 
 static int g_num_sms = 0;
 
-template <int BN, bool SPLIT = (BN > 128)>
+template <int BN, int MODE = UM_PLAIN, bool SPLIT = (BN > 128)>
 static cudaError_t launch_bn(const CUtensorMap* m, const UmmaArgs& a, int batch, cudaStream_t st) {
-  if (g_persistent || BN > 128 || SPLIT) {
+  if (g_persistent || BN > 128 || SPLIT || MODE != UM_PLAIN) {
     if (!g_num_sms) {
       int dev = 0;
       cudaGetDevice(&dev);
@@ -1149,7 +1154,7 @@ static cudaError_t launch_bn(const CUtensorMap* m, const UmmaArgs& a, int batch,
     }
     size_t sm = umma_psmem<BN>();
     cudaError_t e =
-        cudaFuncSetAttribute(umma_pkernel<BN, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaFuncSetAttribute(umma_pkernel<BN, SPLIT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     const int ntn = (a.N + BN - 1) / BN, ntm = (a.M + UM_BM - 1) / UM_BM;
     const int64_t ntiles = (int64_t)ntn * ntm * batch * a.ksplit;
@@ -1165,11 +1170,11 @@ static cudaError_t launch_bn(const CUtensorMap* m, const UmmaArgs& a, int batch,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = g_pdl ? 1 : 0;
-    e = cudaLaunchKernelEx(&cfg, umma_pkernel<BN, SPLIT>, m[0], m[1], m[2], m[3], a, ntn, ntm, (int)ntiles);
+    e = cudaLaunchKernelEx(&cfg, umma_pkernel<BN, SPLIT, MODE>, m[0], m[1], m[2], m[3], a, ntn, ntm, (int)ntiles);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
   }
-  if constexpr (BN <= 128) {
+  if constexpr (BN <= 128 && MODE == UM_PLAIN) {
     size_t sm = umma_smem<BN>();
     cudaError_t e = cudaFuncSetAttribute(umma_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
@@ -1193,6 +1198,31 @@ static cudaError_t umma_launch(int bn, const UmmaOperand& A, const UmmaOperand& 
       !make_map(&maps[2], B.hi, Kpad, B.rows, B.batch, B.ld, B.bs, box, f16) ||
       !make_map(&maps[3], nseg > 1 ? B.lo : B.hi, Kpad, B.rows, B.batch, B.ld, B.bs, box, f16))
     return cudaErrorInvalidValue;
+  if (a.q_naux > 0 && pcs) return cudaErrorInvalidValue;
+  if (a.q_naux > 0) {
+    switch (bn) {
+      case 256: return launch_bn<256, UM_BLOCKED>(maps, a, batch, st);
+      case 192: return launch_bn<192, UM_BLOCKED>(maps, a, batch, st);
+      case 128: return launch_bn<128, UM_BLOCKED>(maps, a, batch, st);
+      case 96: return launch_bn<96, UM_BLOCKED>(maps, a, batch, st);
+      case 64: return launch_bn<64, UM_BLOCKED>(maps, a, batch, st);
+      case 32: return launch_bn<32, UM_BLOCKED>(maps, a, batch, st);
+      default: return cudaErrorInvalidValue;
+    }
+  }
+  if (pcs) {
+    switch (bn) {
+      case 192: return launch_bn<192, UM_PIECES>(maps, a, batch, st);
+      case 160: return launch_bn<160, UM_PIECES>(maps, a, batch, st);
+      case 128: return launch_bn<128, UM_PIECES>(maps, a, batch, st);
+      case 112: return launch_bn<112, UM_PIECES>(maps, a, batch, st);
+      case 96: return launch_bn<96, UM_PIECES>(maps, a, batch, st);
+      case 80: return launch_bn<80, UM_PIECES>(maps, a, batch, st);
+      case 64: return launch_bn<64, UM_PIECES>(maps, a, batch, st);
+      case 48: return launch_bn<48, UM_PIECES>(maps, a, batch, st);
+      default: return launch_bn<32, UM_PIECES>(maps, a, batch, st);
+    }
+  }
   switch (bn) {
     case 256: return launch_bn<256>(maps, a, batch, st);
     case 224: return launch_bn<224>(maps, a, batch, st);
@@ -1262,7 +1292,7 @@ static int tune_bn(const UmmaOperand& A, const UmmaOperand& B, int64_t Kpad, int
   std::vector<int> cands(kBnCand, kBnCand + sizeof(kBnCand) / sizeof(int));
   if (a.N >= 160 && g_wide) cands.insert(cands.begin(), kBnWide, kBnWide + sizeof(kBnWide) / sizeof(int));
   for (int cand : cands) {
-    if (a.q_naux > 0 && !blocked_bn(cand)) continue;
+    if ((a.q_naux > 0 && !blocked_bn(cand)) || (a.a_npc > 0 && cand > 192)) continue;   // N = 2 nao <= 192
     if (umma_launch(cand, A, B, Kpad, nseg, t, batch, st) != cudaSuccess) continue;   // warm-up
     float cand_ms = 1e30f;
     for (int rep = 0; rep < 3; ++rep) {   // best of three: single timings of short launches are noisy
