@@ -33,6 +33,9 @@ struct gw_ctx {
   // them; P_iw holds a folded P~0 / P_tau a folded P~
   bool wfold = false, p0sym = false, psym = false;
   int nrep = 0, nqR = 0, nqC = 0;
+  // small nao: q-points per batch of the fused P~0 chain (k_small.cu; 0: not used), k + q per (q, k)
+  int zq = 0;
+  int* d_kplus = nullptr;
   int *d_rep = nullptr, *d_repn = nullptr, *d_qR = nullptr, *d_qC = nullptr;
   void *fRd = nullptr, *fCd = nullptr, *bRd = nullptr, *bCd = nullptr;
   int *fRe = nullptr, *fCe = nullptr, *bRe = nullptr, *bCe = nullptr;
@@ -188,6 +191,8 @@ static int chain_pbatch(int nao, int naux, int nk, int ntau) {
 }
 static constexpr size_t kRefineBytes = (size_t)6 << 30;
 static constexpr size_t kFoldBytes = (size_t)1 << 30;
+// Z planes of a batch of q-points at small nao
+static constexpr size_t kSmallZBytes = (size_t)512 << 20;
 
 #define CK(x)                                                                        \
   do {                                                                               \
@@ -782,7 +787,26 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
     if (g_pgroup_cap > 0 && c->pgroup > g_pgroup_cap) c->pgroup = g_pgroup_cap;
     if (c->pgroup < 1) c->pgroup = 1;
     size_t zb = 0;
-    for (;;) {
+    if (small_z_ok(nao)) c->d_kplus = (int*)need(A((size_t)nk * nk * 4));
+    if (small_z_ok(nao) && c->pgroup == nk) {
+      // small nao: the planes of several q-points, whose chains share their launches
+      // (as many as give every SM one output tile of the last step)
+      int64_t nb = (int64_t)(opt_budget(kSmallZBytes) / (2 * zk * nk));
+      const int64_t tiles = (((int64_t)ntau * naux + 127) / 128) * ((2 * (int64_t)naux + 127) / 128);
+      if (nb > 152 / tiles) nb = 152 / tiles;
+      if (nb > nk) nb = nk;
+      if (2 * nb * nk > 65535) nb = 65535 / (2 * nk);
+      if (nb < 1) nb = 1;
+      zb = zk * nk * nb;
+      const size_t vb = vk * nk * 2 * nb;   // (twice as many q-points of half the tau points)
+      c->Zhi = (float*)A(zb); c->Zlo = (float*)A(zb); c->Vhi = (float*)A(vb); c->Vlo = (float*)A(vb);
+      if (c->Zhi && c->Zlo && c->Vhi && c->Vlo) {
+        c->zq = (int)nb;
+      } else {
+        dfree(c, c->Zhi); dfree(c, c->Zlo); dfree(c, c->Vhi); dfree(c, c->Vlo);
+      }
+    }
+    while (c->zq == 0) {
       zb = zk * c->pgroup;
       const size_t vb = vk * c->pgroup;
       c->Zhi = (float*)A(zb); c->Zlo = (float*)A(zb); c->Vhi = (float*)A(vb); c->Vlo = (float*)A(vb);
@@ -951,6 +975,8 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
   chk(fermi_freqs(nwf, cfg->beta, c->d_fn, c->wn, st), "freqs");
   count(4);
   if (lowp) { chk(to_c64(c->V, c->V32, vbytes / cb, st), "V32"); count(1); }
+  if (c->d_kplus)
+    chk(cudaMemcpyAsync(c->d_kplus, c->kplus.data(), (size_t)nk * nk * 4, cudaMemcpyHostToDevice, st), "copy");
   if (c->hfmt) {
     // V's norms per Q over every slab fix the exponents of the V operands (uniform over the
     // (k, k') pairs, so that the operands of one grouped GEMM share them)
@@ -1446,6 +1472,32 @@ static gw_status polar_chain_half(gw_ctx* c, const double2* Gplus, const double2
   }
   CK(polar_exps(c->vQrs, c->gn, grs_m, ntau, naux, c->eY, c->eZ, st));
   count(2);
+  if (c->zq > 0 && c->fold && c->wfold) {
+    // small nao: both nao-sized steps in one FP32 kernel, and the q-points of a batch in one launch of
+    // each step (the kept q of polar_taus: half of the tau points for q = -q, one q of each pair)
+    for (int pass = 0; pass < 2; ++pass) {
+      const int nq = pass ? c->nqC : c->nqR, nt = pass ? ntau : (ntau + 1) / 2;
+      const int* list = pass ? c->d_qC : c->d_qR;
+      const int nzmax = nt < ntau ? c->zq * ntau / nt : c->zq;
+      for (int a0 = 0; a0 < nq; a0 += nzmax) {
+        const int nz = nq - a0 < nzmax ? nq - a0 : nzmax;
+        const int64_t zbs = (int64_t)nt * naux * zld;
+        CK(small_z(nao, naux, nk, ntau, nt, nz, list + a0, c->d_kplus, c->V32, Gplus, Gminus, c->eZ, fmt, c->Zhi, c->Zlo,
+                   zld, kp, zbs, st));
+        CK(small_embed(nao, naux, nk, nz, list + a0, c->d_kplus, c->V, c->eVQ, fmt, c->Vhi, c->Vlo, zld, kp, st));
+        count(2);
+        UmmaOperand oa{c->Zhi, c->Zlo, (int64_t)nt * naux, nz, zld, zbs, fmt};
+        UmmaOperand ob{c->Vhi, c->Vlo, 2 * (int64_t)naux, nz, zld, 2 * naux * zld, fmt};
+        UmmaScale sc{c->eZ, c->eVQ, 0, 0, 0, 1, 1};
+        UmmaZ zz{};
+        zz.c_list = list + a0;
+        CK(run_umma(c, 8.0 * nz * nk * nt * naux * (double)naux * n2, oa, ob, nt * naux, 2 * naux, nk * kp, nz,
+                    (double*)out, true, c->spin / nk, accumulate, 2 * (int64_t)naux, 2 * ntau * c->na2, 1, 0, 0, 0, 0,
+                    nullptr, (nk - 1) * kp + 2 * n2, &sc, nullptr, &zz));
+      }
+    }
+    return GW_OK;
+  }
   // G operands per k: Ge[k][t] from G^k(t) (C = A conj(Ge)^T = A G for Hermitian G),
   // Gp[k][j] from G^k(t_{ntau-1-j}) (C = A Gp^T), one exponent per matrix
   for (int k = 0; k < nk; ++k) {

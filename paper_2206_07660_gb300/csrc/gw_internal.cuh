@@ -83,6 +83,17 @@ size_t screened_refine_real_bytes(int64_t n, int64_t chunk);
 cudaError_t screened_refine_real(double* X, int64_t n, int64_t count, void* work, size_t work_bytes, int nsteps,
                                  int* d_info, int* d_err, cudaStream_t st, int64_t* nlaunch);
 
+// ------------------------------------------------------------------ P~0 chain at small nao (k_small.cu)
+bool small_z_ok(int nao);
+// Z of every (q, k) of nz q-points as 16-bit pieces: entry zq at hi / lo + zq zbs, rows (t, Q) of stride
+// zld, columns k kp + 2 (c nao + b)
+cudaError_t small_z(int nao, int naux, int nk, int ntau, int nt, int nz, const int* qlist, const int* kplus,
+                    const float2* V, const double2* Gplus, const double2* Gminus, const int* eZ, int fmt, void* hi,
+                    void* lo, int64_t zld, int64_t kp, int64_t zbs, cudaStream_t st);
+// embedded conj V^{k,k+q}(Q') of the same pairs: entry zq at zq 2 naux zld
+cudaError_t small_embed(int nao, int naux, int nk, int nz, const int* qlist, const int* kplus, const double2* V,
+                        const int* eV, int fmt, void* hi, void* lo, int64_t zld, int64_t kp, cudaStream_t st);
+
 // ------------------------------------------------------------------ folded bosonic block (k_fold.cu)
 struct FoldView {
   int n, nwb, nrep, q0, q1;

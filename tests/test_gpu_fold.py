@@ -37,6 +37,22 @@ def test_polarization_blocks(kmesh, ntau, qr, precision):
     assert np.array_equal(got[list(qs)], np.conj(np.swapaxes(got[list(qs)], -1, -2)))
 
 
+@pytest.mark.parametrize("nao", [1, 2, 4, 7, 8, 12, 13, 16])
+@pytest.mark.parametrize("kmesh,ntau,naux", [((3, 1, 1), 5, 37), ((2, 1, 1), 4, 1), ((4, 2, 1), 3, 70)])
+@pytest.mark.parametrize("precision", ["split_f16", "split_bf16"])
+def test_polarization_of_few_orbitals(nao, kmesh, ntau, naux, precision):
+    # both nao-sized steps in one FP32 kernel and every q of a kind in one launch
+    sysd = system(nao, naux, kmesh, ntau, 20.0, 78)
+    km = ogw.KMesh(kmesh)
+    G = hermitian_noise((ntau, km.nk, nao, nao), 0.3, 79)
+    g = gpu(sysd, precision=precision)
+    g.set("G_tau", G)
+    g.polarization()
+    got, ref = g.get("P0_tau"), ogw.polarization_tau(sysd["V"], G, km)
+    for q in range(km.nk):
+        assert rel(got[q], ref[q]) < TOL[precision], q
+
+
 @pytest.mark.parametrize("kmesh,ntau", [((2, 1, 1), 7), ((3, 1, 1), 6)])
 def test_polarization_of_any_g(kmesh, ntau):
     # the fold needs no symmetry of G: a complex G without any, FP64
