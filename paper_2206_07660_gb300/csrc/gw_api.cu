@@ -36,6 +36,7 @@ struct gw_ctx {
   // small nao: q-points per batch of the fused P~0 chain (k_small.cu; 0: not used), k + q per (q, k)
   int zq = 0;
   int* d_kplus = nullptr;
+  void* Vf = nullptr;   // small nao: V of a batch of k in fragment order (the fused last steps of Sigma~)
   int *d_rep = nullptr, *d_repn = nullptr, *d_qR = nullptr, *d_qC = nullptr;
   void *fRd = nullptr, *fCd = nullptr, *bRd = nullptr, *bCd = nullptr;
   int *fRe = nullptr, *fCe = nullptr, *bRe = nullptr, *bCe = nullptr;
@@ -106,7 +107,7 @@ struct gw_ctx {
   float *Gp_hi = nullptr, *Gp_lo = nullptr;
   // k-points per launch of the 16-bit chains (their per-k operands side by side) and the
   // G blocks of k+q (or k-q) gathered in k order for such a launch
-  int pbatch = 1;
+  int pbatch = 1, sbatch = 1;   // (sbatch: of the Sigma~ chain)
   // first Sigma~ step in 4 x 4 column blocks (nao padded to nao4), its conjugate transpose for the
   // mirrored (k - q, -q, beta - tau), that one's row exponents, k - q per (q, k)
   int nao4 = 0, npc = 0;   // npc: K pieces of 8 elements per row
@@ -188,6 +189,17 @@ static int chain_pbatch(int nao, int naux, int nk, int ntau) {
   if (kb > nk) kb = nk;
   if (g_pbatch_cap > 0 && kb > g_pbatch_cap) kb = g_pbatch_cap;
   return kb < 1 ? 1 : (int)kb;
+}
+// k-points per launch of the Sigma~ chain at small nao: blocks (t, k) for four rounds of the fused
+// kernel (two per SM), as far as X and its image (xbytes per k) stay below kSmallXBytes
+static constexpr size_t kSmallXBytes = (size_t)512 << 20;
+static int chain_sbatch(int nk, int ntau, size_t xbytes, int pbatch) {
+  if (g_pbatch_cap > 0) return pbatch;
+  int64_t kb = (4 * 304 + ntau - 1) / ntau;
+  if (kb * xbytes > kSmallXBytes) kb = (int64_t)(kSmallXBytes / xbytes);
+  if (kb > kSrcListMax) kb = kSrcListMax;
+  if (kb > nk) kb = nk;
+  return kb < pbatch ? pbatch : (int)kb;
 }
 static constexpr size_t kRefineBytes = (size_t)6 << 30;
 static constexpr size_t kFoldBytes = (size_t)1 << 30;
@@ -821,14 +833,16 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
     // operand buffers below hold that many blocks
     c->pbatch = chain_pbatch(nao, naux, nk, ntau);
     const size_t kb = (size_t)c->pbatch;
-    // X in 4 x 4 column blocks where the padding to whole blocks costs less than the halved
-    // first step gains
-    const int nb4 = (nao + 3) / 4 * 4;
-    c->nao4 = 5 * nb4 * nb4 <= 8 * nao * nao ? nb4 : 0;
-    const int64_t vtrows = c->nao4 ? 2 * (int64_t)c->nao4 * c->nao4 : 2 * n2;
+    // X in 4 x 4 column blocks, padded to whole ones
+    c->nao4 = (nao + 3) / 4 * 4;
+    const int64_t vtrows = 2 * (int64_t)c->nao4 * c->nao4;
     const size_t pb = (size_t)ntau * naux * c->kpadS * 2, tb = (size_t)vtrows * c->kpadS * 2;
     c->Pchi = (float*)need(A(pb)); c->Pclo = (float*)need(A(pb));
-    c->vt_bytes = kb * tb;
+    c->npc = 2 * ((2 * nao + 15) / 16);
+    const size_t xk = (size_t)ntau * c->npc * naux * nao * 16;   // one plane of one k
+    c->sbatch = small_z_ok(nao) ? chain_sbatch(nk, ntau, 4 * xk, c->pbatch) : c->pbatch;
+    const size_t sb = (size_t)c->sbatch;
+    c->vt_bytes = sb * tb;
     c->VThi = (float*)need(A(c->vt_bytes)); c->VTlo = (float*)need(A(c->vt_bytes));
     const size_t vs = (size_t)naux * nao * c->kpadA * 2, ge = (size_t)nk * ntau * 2 * nao * c->kpadA * 2;
     const size_t xs = (size_t)ntau * naux * nao * c->kpadA * 2;
@@ -841,20 +855,21 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
       c->eGq = (int*)need(A(kb * ntau * 4));
     }
     c->Xs_hi = (float*)need(A(kb * xs)); c->Xs_lo = (float*)need(A(kb * xs));
-    if (c->nao4) {
-      c->npc = 2 * ((2 * nao + 15) / 16);
-      c->xb_bytes = kb * ntau * c->npc * (size_t)naux * nao * 16 + 128 * 16;   // and one tile of rows of slack
-      c->Xb_hi = (float*)need(A(c->xb_bytes)); c->Xb_lo = (float*)need(A(c->xb_bytes));
-      c->Xt_hi = (float*)A(c->xb_bytes); c->Xt_lo = (float*)A(c->xb_bytes);
-      c->eY3b = (int*)A((size_t)ntau * 4); c->d_kminus = (int*)A((size_t)nk * nk * 4);
-      if (!c->Xt_hi || !c->Xt_lo || !c->eY3b || !c->d_kminus) {   // without room every (k, q) has its own X
-        dfree(c, c->Xt_hi); dfree(c, c->Xt_lo);
-        c->Xt_hi = c->Xt_lo = nullptr;
-      }
+    c->xb_bytes = sb * xk + 128 * 16;   // and one tile of rows of slack
+    c->Xb_hi = (float*)need(A(c->xb_bytes)); c->Xb_lo = (float*)need(A(c->xb_bytes));
+    c->Xt_hi = (float*)A(c->xb_bytes); c->Xt_lo = (float*)A(c->xb_bytes);
+    c->eY3b = (int*)A((size_t)ntau * 4); c->d_kminus = (int*)A((size_t)nk * nk * 4);
+    if (!c->Xt_hi || !c->Xt_lo || !c->eY3b || !c->d_kminus) {   // without room every (k, q) has its own X
+      dfree(c, c->Xt_hi); dfree(c, c->Xt_lo);
+      c->Xt_hi = c->Xt_lo = nullptr;
     }
-    c->y3bytes = (size_t)ntau * nao * c->kpad3 * 2;
-    c->Y3hi = (float*)need(A(kb * c->y3bytes)); c->Y3lo = (float*)need(A(kb * c->y3bytes));
-    c->W3hi = (float*)need(A(kb * 2 * nao * c->kpad3 * 2)); c->W3lo = (float*)need(A(kb * 2 * nao * c->kpad3 * 2));
+    if (small_z_ok(nao)) {
+      c->Vf = need(A(sb * 2 * small_tail_v_bytes(nao, naux)));
+    } else {
+      c->y3bytes = (size_t)ntau * nao * c->kpad3 * 2;
+      c->Y3hi = (float*)need(A(kb * c->y3bytes)); c->Y3lo = (float*)need(A(kb * c->y3bytes));
+      c->W3hi = (float*)need(A(kb * 2 * nao * c->kpad3 * 2)); c->W3lo = (float*)need(A(kb * 2 * nao * c->kpad3 * 2));
+    }
     c->vQmax = (float*)need(A((size_t)naux * 4)); c->vQrs = (float*)need(A((size_t)naux * 4));
     c->gn = (float*)need(A((size_t)4 * ntau * 4));
     c->eVQ = (int*)need(A((size_t)naux * 4)); c->eVall = (int*)need(A(16));
@@ -987,17 +1002,18 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
     chk(cudaMemsetAsync(c->Zhi, 0, c->zbytes, st), "memset");
     chk(cudaMemsetAsync(c->Zlo, 0, c->zbytes, st), "memset");
     // the padding columns of the chain intermediates stay zero (every k block)
-    chk(cudaMemsetAsync(c->Y3hi, 0, (size_t)c->pbatch * c->y3bytes, st), "memset");
-    chk(cudaMemsetAsync(c->Y3lo, 0, (size_t)c->pbatch * c->y3bytes, st), "memset");
+    if (c->Y3hi) {
+      chk(cudaMemsetAsync(c->Y3hi, 0, (size_t)c->pbatch * c->y3bytes, st), "memset");
+      chk(cudaMemsetAsync(c->Y3lo, 0, (size_t)c->pbatch * c->y3bytes, st), "memset");
+    }
     const size_t xs = (size_t)c->pbatch * ntau * naux * nao * c->kpadA * 2;
     chk(cudaMemsetAsync(c->Xs_hi, 0, xs, st), "memset");
     chk(cudaMemsetAsync(c->Xs_lo, 0, xs, st), "memset");
-    if (c->nao4) {   // so do the pieces and the rows of the blocks' padding
-      chk(cudaMemsetAsync(c->Xb_hi, 0, c->xb_bytes, st), "memset");
-      chk(cudaMemsetAsync(c->Xb_lo, 0, c->xb_bytes, st), "memset");
-      chk(cudaMemsetAsync(c->VThi, 0, c->vt_bytes, st), "memset");
-      chk(cudaMemsetAsync(c->VTlo, 0, c->vt_bytes, st), "memset");
-    }
+    // so do the pieces and the rows of the blocks' padding
+    chk(cudaMemsetAsync(c->Xb_hi, 0, c->xb_bytes, st), "memset");
+    chk(cudaMemsetAsync(c->Xb_lo, 0, c->xb_bytes, st), "memset");
+    chk(cudaMemsetAsync(c->VThi, 0, c->vt_bytes, st), "memset");
+    chk(cudaMemsetAsync(c->VTlo, 0, c->vt_bytes, st), "memset");
     if (c->Xt_hi) {
       chk(cudaMemsetAsync(c->Xt_hi, 0, c->xb_bytes, st), "memset");
       chk(cudaMemsetAsync(c->Xt_lo, 0, c->xb_bytes, st), "memset");
@@ -1610,13 +1626,12 @@ static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2*
   // work, then runs over half of the (q, tau) (the kept ones of polar_taus; the middle of an odd
   // ntau of q = -q serves both k, so it has no image) and writes X in both orders.
   const bool share = psym && c->fold && !c->reduce && sigma_shares(c);
-  const int KB = c->pbatch, nb4 = c->nao4;
-  // X: rows (t, i, Q') of K = a, or (nao4) K pieces of those rows per t; one tau of it
-  const int npc = nb4 ? c->npc : 0;
-  const int64_t xt = nb4 ? (int64_t)naux * nao * npc * 8 : (int64_t)naux * nao * ka;
-  float *Xh = nb4 ? c->Xb_hi : c->Xs_hi, *Xl = nb4 ? c->Xb_lo : c->Xs_lo;
+  const int nb4 = c->nao4, npc = c->npc;
+  // X: K pieces (a) of rows (i, Q') per t; one tau of it
+  const int64_t xt = (int64_t)naux * nao * npc * 8;
+  float *Xh = c->Xb_hi, *Xl = c->Xb_lo;
   const int64_t xs_blk = ntau * xt, y3t = (int64_t)nao * kp3, y3_blk = ntau * y3t;
-  const int64_t ncol = nb4 ? 2 * (int64_t)nb4 * nb4 : 2 * n2;
+  const int64_t ncol = 2 * (int64_t)nb4 * nb4;
   const int64_t vt_blk = ncol * kps, w3_blk = 2 * (int64_t)nao * kp3;
   // Sigma~ += -(1/Nk) Y V over nt tau points from t0: B = V transposed, rows j, K = (b, Q') (source
   // rows (Q', b)); the Sigma~^k of list[z] (or of consecutive k)
@@ -1656,6 +1671,8 @@ static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2*
     act.clear();
     for (int k = 0; k < nk; ++k)
       if (!(c->reduce && c->kneg[(size_t)k] < k)) act.push_back(k);   // else the conjugate of Sigma~^{-k}
+    // launches of equally many k
+    const int nb = ((int)act.size() + c->sbatch - 1) / c->sbatch, KB = nb > 0 ? ((int)act.size() + nb - 1) / nb : 1;
     for (size_t b0 = 0; b0 < act.size();) {
       // a run of consecutive k (their Sigma~^k blocks are equally spaced), KB at most
       int kn = 1;
@@ -1671,21 +1688,35 @@ static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2*
       }
       // X = conj(P~) V: B = V^{k,k-q} transposed, rows (i, a), K = Q, one exponent
       CK(half_embed_t_multi(c->V, voffX, kn, naux, n2, c->VThi, c->VTlo, kps, vt_blk, fmt, c->h_Evmax - 15, st, 0, 0,
-                            nb4 ? nao : 0));
+                            nao));
       count(1);
       {
         UmmaOperand oa{c->Pchi, c->Pclo, (int64_t)nt * naux, 1, kps, 0, fmt};
         UmmaOperand ob{c->VThi, c->VTlo, ncol, kn, kps, vt_blk, fmt};
         UmmaScale sc{c->ePc, c->eVall, 0, 0, 0, 1, kAll};
         UmmaOut o{fmt, c->ePs, 0, 1, shift};
-        if (nb4) {
-          o.naux = naux; o.nao = nao; o.nt = ntau; o.npc = npc;
-          if (pair) { o.C2 = c->Xt_hi; o.C2_lo = c->Xt_lo; }
-        }
+        o.naux = naux; o.nao = nao; o.nt = ntau; o.npc = npc;
+        if (pair) { o.C2 = c->Xt_hi; o.C2_lo = c->Xt_lo; }
         // output row (t, Q'), column (i, a re/im) -> X row (t, i, Q'), entry (a re/im); one X block per k
         CK(run_umma(c, fl1 * kn, oa, ob, nt * naux, (int)ncol, kps, kn, Xh, false, 1.0, false, ka,
                     kn > 1 ? xs_blk : 0, 1, naux, xt, 2 * (int64_t)nao, (int64_t)naux * ka, Xl, 2 * (int64_t)naux, &sc,
                     &o));
+      }
+      if (c->Vf) {   // small nao: the other two steps in one kernel
+        const int* kmq_d = c->d_kplus + (size_t)nq * nk;   // k - q = k + (-q)
+        const int ev = c->h_Evmax - 15;
+        CK(small_tail_v(c->V, kmq_d, nao, naux, nk, k0, kn, fmt, ev, c->Vf, st));
+        SmallTail d{nao, naux, nk, ntau, nt, 0, k0, kn, npc, fmt, false, Xh, Xl, c->Vf, kmq_d, c->Ge_hi, c->Ge_lo, per, ka,
+                    c->eGe, c->ePs, c->eY3, shift, ev, -1.0 / nk, out};
+        CK(small_tail(d, st));
+        count(2);
+        if (ni > 0) {
+          d.nt = ni; d.t0 = t0i; d.image = true; d.xhi = c->Xt_hi; d.xlo = c->Xt_lo; d.eY = c->eY3b;
+          d.vf = (const char*)c->Vf + kn * small_tail_v_bytes(nao, naux);
+          CK(small_tail(d, st));
+          count(1);
+        }
+        continue;
       }
       // Y = X G^{k-q}(t): A rows (i, Q') per (k, t) (exponent of row Q'), B = Ge[k-q][t]; row (i, Q'),
       // column (b re/im) lands at row (t, i), K entry (b, Q') of the last step's operand

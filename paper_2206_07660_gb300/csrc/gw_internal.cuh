@@ -93,6 +93,26 @@ cudaError_t small_z(int nao, int naux, int nk, int ntau, int nt, int nz, const i
 // embedded conj V^{k,k+q}(Q') of the same pairs: entry zq at zq 2 naux zld
 cudaError_t small_embed(int nao, int naux, int nk, int nz, const int* qlist, const int* kplus, const double2* V,
                         const int* eV, int fmt, void* hi, void* lo, int64_t zld, int64_t kp, cudaStream_t st);
+// The last two Sigma~ steps of nl k-points from k0 and one q at the tau points t0 .. t0 + nt - 1
+// (image: of (k - q, -q) from the transposed conjugate X)
+struct SmallTail {
+  int nao, naux, nk, ntau, nt, t0, k0, nl, npc, fmt;
+  bool image;
+  const void *xhi, *xlo;       // X in K pieces, [nl][ntau][npc][nao naux rows]
+  const void* vf;              // small_tail_v's entries of this direction
+  const int* kmq;              // device: k - q of every k
+  const void *ghi, *glo;       // Ge [nk][ntau] of gper elements, rows of ka
+  int64_t gper, ka;
+  const int *eG, *eX, *eY;     // exponents: [nk][ntau], [ntau][naux] (of X's own tau), [ntau]
+  int shift, ev;               // X's rows carry eX + shift, vf carries ev
+  double alpha;
+  double2* out;                // (ntau, nk, nao, nao)
+};
+cudaError_t small_tail(const SmallTail& d, cudaStream_t st);
+int64_t small_tail_v_bytes(int nao, int naux);   // per k and direction
+// V^{k-q,k} of nl k-points from k0, then V^{k,k-q} of the same
+cudaError_t small_tail_v(const double2* V, const int* kmq, int nao, int naux, int nk, int k0, int nl, int fmt, int e,
+                         void* out, cudaStream_t st);
 
 // ------------------------------------------------------------------ folded bosonic block (k_fold.cu)
 struct FoldView {

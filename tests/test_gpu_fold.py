@@ -156,6 +156,26 @@ def test_selfenergy_blocks(nao, kmesh, ntau, qr, sym, precision):
     assert rel(g.get("Sigma_tau"), ref) < TOL[precision]
 
 
+@pytest.mark.parametrize("nao", [1, 2, 4, 7, 8, 9, 12, 15, 16, 17, 20])
+@pytest.mark.parametrize("kmesh,ntau,naux", [((3, 1, 1), 5, 37), ((2, 1, 1), 3, 1), ((3, 2, 1), 2, 16)])
+@pytest.mark.parametrize("sym", [True, False])
+@pytest.mark.parametrize("precision", ["split_f16", "split_bf16"])
+def test_selfenergy_of_few_orbitals(nao, kmesh, ntau, naux, sym, precision):
+    # the last two steps in one kernel up to nao 16 (one or two auxiliary functions per warp), GEMMs above
+    sysd = system(nao, naux, kmesh, ntau, 20.0, 97)
+    km = ogw.KMesh(kmesh)
+    G = hermitian_noise((ntau, km.nk, nao, nao), 0.3, 98)
+    P = hermitian_noise((km.nk, ntau, naux, naux), 0.3, 99)
+    if sym:
+        P = _folded(P, km)
+    ref = ogw.selfenergy_tau(sysd["V"], G, P, km, qs=list(range(km.nk)))
+    g = gpu(sysd, precision=precision)
+    g.set("G_tau", G)
+    g.set("P_tau", P)
+    g.selfenergy_partial()
+    assert rel(g.get("Sigma_tau"), ref) < TOL[precision]
+
+
 @pytest.mark.parametrize("kmesh,ntau", [((2, 1, 1), 5), ((3, 1, 1), 4)])
 def test_polarization_vjp_blocks(kmesh, ntau):
     # the adjoint of the folded P~0 against the oracle's, which runs over every block
