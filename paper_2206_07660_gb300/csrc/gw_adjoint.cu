@@ -41,6 +41,7 @@ struct View {   // the context's tensors seen by the adjoint chains (same layout
   float2* bar32;                  // complex64 copy of the symmetrised cotangent
   bool fold;                      // P~0^{-q}(tau_{n-1-j}) = conj P~0^q(tau_j): V is paired
   const int* kneg;                // index of -q (host)
+  DigitWs dg;                     // digits of the FP64 products (no A: not used)
 };
 }  // namespace gwadj
 
@@ -110,16 +111,23 @@ cudaError_t polarization_vjp(const View& v, const double2* Pbar, double2* Gbar, 
       Pa = v.bar32;
       *launches += 1;
     }
+    bool P_ready = false;   // the digits of Pr are in place
     for (int k = 0; k < nk; ++k) {
       const int kq = v.kplus[(size_t)q * nk + k];
       const void* V1 = at(v, v.V, v.V32, ((int64_t)k * nk + kq) * slab);
       const void* V2 = at(v, v.V, v.V32, ((int64_t)kq * nk + k) * slab);
       // X[t][Q'][(d,a)] = sum_Q Pr[t][Q][Q'] conj(V1[Q][(d,a)])
+      if (!v.c64 && emul_pays(v.dg, (int64_t)nt * naux, n2, naux, naux)) {
+        if ((e = emul_zgemm_cols(v.dg, Pr, nt, naux, (const double2*)V1, n2, 1, v.bufA, P_ready, v.st, launches))) return e;
+        P_ready = true;
+      } else {
       GettDesc d1 = desc(naux, n2, naux, nt);
       d1.am = I1(1); d1.ak = I1(naux); d1.az = I1(na2);
       d1.bk = I1(n2); d1.bn = I1(1); d1.conjB = true;
       d1.cm = I1(n2); d1.cn = I1(1); d1.cz = I1(slab);
       if ((e = run(v, d1, Pa, V1, v.bufA))) return e;
+      *launches += 1;
+      }
       // Y[t][Q'][c][a] = sum_d conj(Gm[t][c][d]) X[t][Q'][d][a],  Gm(t) = -G^k(t_{n-1-j})
       GettDesc d2 = desc(nao, (int64_t)naux * nao, nao, nt);
       d2.am = I1(nao); d2.ak = I1(1); d2.az = I1(-gstep); d2.conjA = true;
@@ -150,7 +158,7 @@ cudaError_t polarization_vjp(const View& v, const double2* Pbar, double2* Gbar, 
       d5.alpha = make_double2(-f, 0); d5.beta = make_double2(1, 0);
       d5.ksplit = split_of(v, d5.K, nt);
       if ((e = run(v, d5, V2, v.bufB, Gbar + (size_t)(ntau - 1) * gstep + (size_t)k * n2, true))) return e;
-      *launches += 5;
+      *launches += 4;
     }
   }
   return cudaSuccess;
@@ -174,17 +182,28 @@ cudaError_t selfenergy_vjp(const View& v, const double2* Sbar, double2* Gbar, do
   }
   for (int q = 0; q < nk; ++q) {
     const void* Pq = at(v, v.P_tau, v.P32, (int64_t)q * ntau * na2);
+    bool P_ready = false;
     for (int k = 0; k < nk; ++k) {
       const int kmq = v.kminus[(size_t)q * nk + k];
       const void* V1 = at(v, v.V, v.V32, ((int64_t)k * nk + kmq) * slab);
       const void* V2 = at(v, v.V, v.V32, ((int64_t)kmq * nk + k) * slab);
       const void* Sk = at(v, Sr, v.bar32, (int64_t)k * n2);
       // E[t][Q'][(i,a)] = sum_Q conj(P[t][Q][Q']) conj(V1[Q][(i,a)])
+      // (the last product's rows share the workspace: one that takes the digits too leaves P's to redo)
+      const bool dig6 = !v.c64 && v.fold && emul_pays(v.dg, (int64_t)ntau * naux, naux, n2, 1);
+      if (!v.c64 && emul_pays(v.dg, (int64_t)ntau * naux, n2, naux, naux)) {
+        if ((e = emul_zgemm_cols(v.dg, (const double2*)Pq, ntau, naux, (const double2*)V1, n2, 2, v.bufA, P_ready, v.st,
+                                 launches)))
+          return e;
+        P_ready = !dig6;
+      } else {
       GettDesc d1 = desc(naux, n2, naux, ntau);
       d1.am = I1(1); d1.ak = I1(naux); d1.az = I1(na2); d1.conjA = true;
       d1.bk = I1(n2); d1.bn = I1(1); d1.conjB = true;
       d1.cm = I1(n2); d1.cn = I1(1); d1.cz = I1(slab);
       if ((e = run(v, d1, Pq, V1, v.bufA))) return e;
+      *launches += 1;
+      }
       // F[t][Q'][a][j] = sum_i E[t][Q'][i][a] Sr[t][k][i][j]
       GettDesc d2 = desc((int64_t)naux * nao, nao, nao, ntau);
       d2.am = I2(nao, n2, 1); d2.ak = I1(nao); d2.az = I1(slab);
@@ -212,13 +231,20 @@ cudaError_t selfenergy_vjp(const View& v, const double2* Sbar, double2* Gbar, do
       d5.cm = I1(nao); d5.cn = I1(1); d5.cz = I1(slab);
       if ((e = run(v, d5, v.bufA, at(v, v.G_tau, v.G32, (int64_t)kmq * n2), v.bufB))) return e;
       // Pbar^q[t][Q][Q'] += f sum_{(j,b)} W[t][Q][(j,b)] conj(V2[Q'][b][j])
+      if (dig6) {   // with the paired V, conj(V2[Q'][b][j]) = V1[Q'][j][b]: packed rows
+        if ((e = emul_zgemm_rows(v.dg, v.bufB, (int64_t)ntau * naux, n2, (const double2*)V1, naux, false,
+                                 Pbar + (size_t)q * ntau * na2, f, true, v.st, launches)))
+          return e;
+        *launches += 4;
+        continue;
+      }
       GettDesc d6 = desc((int64_t)ntau * naux, naux, n2, 1);
       d6.am = I1(n2); d6.ak = I1(1);
       d6.bk = I2(nao, 1, nao); d6.bn = I1(n2); d6.conjB = true;
       d6.cm = I1(naux); d6.cn = I1(1);
       d6.alpha = make_double2(f, 0); d6.beta = make_double2(1, 0);
       if ((e = run(v, d6, v.bufB, V2, Pbar + (size_t)q * ntau * na2, true))) return e;
-      *launches += 6;
+      *launches += 5;
     }
   }
   return cudaSuccess;

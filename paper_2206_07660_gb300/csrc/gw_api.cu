@@ -36,6 +36,7 @@ struct gw_ctx {
   // small nao: q-points per batch of the fused P~0 chain (k_small.cu; 0: not used), k + q per (q, k)
   int zq = 0;
   int* d_kplus = nullptr;
+  DigitWs dg;           // digits of the FP64 chains' products (no A: not used)
   void* Vf = nullptr;   // small nao: V of a batch of k in fragment order (the fused last steps of Sigma~)
   int *d_rep = nullptr, *d_repn = nullptr, *d_qR = nullptr, *d_qC = nullptr;
   void *fRd = nullptr, *fCd = nullptr, *bRd = nullptr, *bCd = nullptr;
@@ -242,6 +243,30 @@ static size_t opt_budget(size_t cap) {
   return fr / 32 < cap ? fr / 32 : cap;
 }
 
+// Digit workspaces of the FP64 chains' large products: at context creation for GW_FP64 contractions
+// (so that nothing is allocated inside a capture), with the first FP64 adjoint otherwise.  Without
+// room, or where no product is large enough, the native kernels stay.
+static void digit_ws(gw_ctx* c) {
+  if (c->dg.A || !c->emul) return;
+  const int64_t naux = c->naux, n2 = c->n2, rows = c->ntau * naux;
+  const size_t ra = emul_digit_bytes(1, n2), rb = emul_digit_bytes(1, naux);   // bytes of a row
+  DigitWs w;
+  w.A_bytes = (size_t)rows * (ra > rb ? ra : rb);
+  const size_t cap = opt_budget(kFoldBytes);
+  if (w.A_bytes > cap) w.A_bytes = cap;
+  w.B_bytes = 2 * (naux * ra > n2 * rb ? naux * ra : n2 * rb);
+  w.A = &w;   // (for the rule alone)
+  if (!emul_pays(w, rows, naux, n2, 1) && !emul_pays(w, rows, n2, naux, naux)) return;
+  w.A = dalloc(c, w.A_bytes); w.B = dalloc(c, w.B_bytes);
+  w.Ae = (int*)dalloc(c, (size_t)rows * 4); w.Be = (int*)dalloc(c, (size_t)(naux > n2 ? naux : n2) * 4);
+  w.err = c->info + 1;
+  if (!w.A || !w.B || !w.Ae || !w.Be) {
+    dfree(c, w.A); dfree(c, w.B); dfree(c, w.Ae); dfree(c, w.Be);
+    return;
+  }
+  c->dg = w;
+}
+
 static void free_all(gw_ctx* c) {
   if (c->st) cudaStreamSynchronize(c->st); else cudaDeviceSynchronize();
   for (void* p : c->owned) {
@@ -267,7 +292,7 @@ static inline void count(int n) { g_launches += n; }
 
 // contractions on the tensor cores (the wait-timeout flag is then meaningful)
 static inline bool uses_tc(const gw_ctx* c) {
-  return c->cfg.contract_prec == GW_SPLIT_TF32 || c->hfmt != 0;
+  return c->cfg.contract_prec == GW_SPLIT_TF32 || c->hfmt != 0 || c->dg.A != nullptr;
 }
 // the time-reversal reduction applies to forward stages over the full q range
 static inline bool trs_reduce(const gw_ctx* c) { return c->trs && c->q0 == 0 && c->q1 == c->nk; }
@@ -905,6 +930,7 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
   c->mus = (MuState*)need(A(sizeof(MuState)));
   c->info = (int*)need(A(64));
   c->dscr = (double*)need(A(64 * 8));
+  if (ok && cfg->contract_prec == GW_FP64) digit_ws(c);
   if (ok && c->emul && screened_refine_ok(naux)) {
     // refined screened solve: as many (q, Omega) systems per batch as the budget
     // allows; without room for one system the FP64 Gauss-Jordan solve is used
@@ -1447,6 +1473,13 @@ static gw_status polar_chain(gw_ctx* c, const double2* Gplus, const double2* Gmi
         }
         continue;
       }
+      if (!f32 && emul_pays(c->dg, (int64_t)nt * naux, naux, n2, 1)) {
+        int64_t nl = 0;
+        CK(emul_zgemm_rows(c->dg, (const double2*)c->chB, (int64_t)nt * naux, n2, (const double2*)Vkq, naux, true, Pq,
+                           c->spin / nk, accumulate || k > 0, c->st, &nl));
+        count((int)nl);
+        continue;
+      }
       GettDesc d3 = base_desc((int64_t)nt * naux, naux, n2, 1);
       d3.am = I1(n2); d3.ak = I1(1);
       d3.bk = I1(1); d3.bn = I1(n2); d3.conjB = true;
@@ -1918,6 +1951,7 @@ static gw_status sigma_chain(gw_ctx* c, const double2* Gsrc, const double2* Psrc
     if (pair && nq < q) continue;
     const int nt = pair && nq == q ? (ntau + 1) / 2 : ntau, ni = pair ? (nq == q ? ntau / 2 : ntau) : 0;
     const char* Pq = (const char*)Pp + (size_t)q * ntau * na2 * es;
+    bool P_ready = false;   // the digits of P~^q are in place
     if (tc) {
       // A operand of the tensor-core stage: conj P~^q(t) = P~^q(t)^T (Hermitian), split hi/lo
       CK(split_rows(Psrc + (size_t)q * ntau * na2, true, (int64_t)ntau * naux, naux, naux, true, c->Pchi,
@@ -1948,12 +1982,20 @@ static gw_status sigma_chain(gw_ctx* c, const double2* Gsrc, const double2* Psrc
         count(1);
       } else {
       // X[t][Q'][(i,a)] = sum_Q P~^q[t][Q][Q'] V^{k,k-q}[Q][(i,a)]
+      const char* Vkk = (const char*)Vp + ((size_t)k * nk + kmq) * slab * es;
+      if (!f32 && emul_pays(c->dg, (int64_t)nt * naux, n2, naux, naux)) {
+        int64_t nl = 0;
+        CK(emul_zgemm_cols(c->dg, (const double2*)Pq, nt, naux, (const double2*)Vkk, n2, 0, (double2*)c->chA, P_ready,
+                           c->st, &nl));
+        count((int)nl);
+        P_ready = true;
+      } else {
       GettDesc d1 = base_desc(naux, n2, naux, nt);
       d1.am = I1(1); d1.ak = I1(naux); d1.az = I1(na2);
       d1.bk = I1(n2); d1.bn = I1(1); d1.bz = I1(0);
       d1.cm = I1(n2); d1.cn = I1(1); d1.cz = I1(slab);
-      const char* Vkk = (const char*)Vp + ((size_t)k * nk + kmq) * slab * es;
       CK(run_gett(d1, Pq, tv, Vkk, tv, c->chA, tv, acc, c));
+      }
       }
       // Y[t][i][Q'][b] = sum_a X[t][Q'][i][a] G^{k-q}[t][a][b]
       if (tc2) {
@@ -2323,6 +2365,7 @@ struct View {
   float2* bar32;
   bool fold;
   const int* kneg;
+  DigitWs dg;
 };
 cudaError_t polarization_vjp(const View& v, const double2* Pbar, double2* Gbar, int64_t* launches);
 cudaError_t selfenergy_vjp(const View& v, const double2* Sbar, double2* Gbar, double2* Pbar, int64_t* launches);
@@ -2372,7 +2415,20 @@ static gw_status adj_view(gw_ctx* c, gwadj::View* v) {
   v->bufA = c->adjA; v->bufB = c->adjB; v->bufC = c->adjC;
   v->st = c->st;
   v->fold = c->fold; v->kneg = c->kneg.data();
+  digit_ws(c);
+  v->dg = c->dg;
   v->c64 = false; v->V32 = nullptr; v->G32 = nullptr; v->P32 = nullptr; v->bar32 = nullptr;
+  return GW_OK;
+}
+
+// whether a product of the tensor cores gave up waiting
+static gw_status tc_check(gw_ctx* c) {
+  if (!uses_tc(c) || c->deferred) return GW_OK;
+  int h = 0;
+  CK(cudaMemcpyAsync(c->h_scr, c->info + 1, 4, cudaMemcpyDeviceToHost, c->st));
+  CK(cudaStreamSynchronize(c->st));
+  memcpy(&h, c->h_scr, 4);
+  if (h) return fail(c, GW_ERR_TIMEOUT, "tensor-core contraction gave up waiting (code " + std::to_string(h) + ")");
   return GW_OK;
 }
 
@@ -2385,9 +2441,10 @@ static gw_status polarization_vjp_impl(gw_ctx* c, const double* Pbar, double* Gb
   if (s != GW_OK) return s;
   CK(cudaMemsetAsync(Gbar, 0, (size_t)c->ntau * c->nk * c->n2 * 16, c->st));
   int64_t l = 0;
+  if (c->dg.A && !c->deferred) CK(cudaMemsetAsync(c->info + 1, 0, 4, c->st));
   CK(gwadj::polarization_vjp(v, (const double2*)Pbar, (double2*)Gbar, &l));
   count((int)l);
-  return GW_OK;
+  return c64 || !c->dg.A ? GW_OK : tc_check(c);
 }
 
 extern "C" gw_status gw_polarization_vjp(gw_ctx* c, const double* Pbar, double* Gbar) {
@@ -2408,9 +2465,10 @@ static gw_status selfenergy_vjp_impl(gw_ctx* c, const double* Sbar, double* Gbar
   CK(cudaMemsetAsync(Gbar, 0, (size_t)c->ntau * c->nk * c->n2 * 16, c->st));
   CK(cudaMemsetAsync(Pbar, 0, (size_t)c->nk * c->ntau * c->na2 * 16, c->st));
   int64_t l = 0;
+  if (c->dg.A && !c->deferred) CK(cudaMemsetAsync(c->info + 1, 0, 4, c->st));
   CK(gwadj::selfenergy_vjp(v, (const double2*)Sbar, (double2*)Gbar, (double2*)Pbar, &l));
   count((int)l);
-  return GW_OK;
+  return c64 || !c->dg.A ? GW_OK : tc_check(c);
 }
 
 extern "C" gw_status gw_selfenergy_vjp(gw_ctx* c, const double* Sbar, double* Gbar, double* Pbar) {
@@ -2425,16 +2483,6 @@ extern "C" gw_status gw_selfenergy_vjp_c64(gw_ctx* c, const double* Sbar, double
 // Tangents of the contraction chains at the context's precision: the forward chains
 // with the tangent in one G (or P~) slot at a time (P~0 is quadratic in G, Sigma~
 // bilinear in (G, P~)), then the symmetrisation.
-static gw_status tc_check(gw_ctx* c) {
-  if (!uses_tc(c) || c->deferred) return GW_OK;
-  int h = 0;
-  CK(cudaMemcpyAsync(c->h_scr, c->info + 1, 4, cudaMemcpyDeviceToHost, c->st));
-  CK(cudaStreamSynchronize(c->st));
-  memcpy(&h, c->h_scr, 4);
-  if (h) return fail(c, GW_ERR_TIMEOUT, "tensor-core contraction gave up waiting (code " + std::to_string(h) + ")");
-  return GW_OK;
-}
-
 extern "C" gw_status gw_polarization_jvp(gw_ctx* c, const double* dG, double* dP0) {
   if (!c || !dG || !dP0) return fail(c, GW_ERR_ARG, "null argument");
   if (!c->have_G) return fail(c, GW_ERR_STATE, "no Green's function yet");

@@ -312,6 +312,8 @@ struct DigitGemm {
   const int* row_list;
   const double* Y;               // row-major only: C = I - Y + A B
   int* err;
+  double alpha = 1.0;            // C = alpha A B
+  bool acc = false;              // added to C
 };
 cudaError_t digit_gemm(const DigitGemm& d, cudaStream_t st);
 int64_t digit_kmax(int nd);
@@ -339,6 +341,26 @@ cudaError_t emul_split_cols_real(const double* B, int64_t count, int64_t K, int6
 cudaError_t emul_rgemm_batched(const void* Ad, const int* Ae, const void* Bd, const int* Be, int64_t count,
                                int64_t M, int64_t N, int64_t K, double* C, int* err, cudaStream_t st, int nd = 8,
                                const double* Y = nullptr);
+// FP64-accurate complex products in digits for the contraction chains: workspaces of both operands
+struct DigitWs {
+  void* A = nullptr;
+  size_t A_bytes = 0;
+  int* Ae = nullptr;
+  void* B = nullptr;
+  size_t B_bytes = 0;
+  int* Be = nullptr;
+  int* err = nullptr;
+};
+// whether a product of M x N complex outputs over K terms takes the digits (its operands fit, and
+// it is large enough)
+bool emul_pays(const DigitWs& w, int64_t M, int64_t N, int64_t K, int64_t rows);
+// C (M x N, packed) = or (acc) += alpha A op(B)^T, A: M x K and B: N x K packed rows, op = conj or none
+cudaError_t emul_zgemm_rows(const DigitWs& w, const double2* A, int64_t M, int64_t K, const double2* B, int64_t N,
+                            bool conjB, double2* C, double alpha, bool acc, cudaStream_t st, int64_t* nlaunch);
+// C[t] (K x N, packed) = P[t]^T op(V), t < nt, P[t]: K x K and V: K x N packed; mode 0: op none, 1: conj V,
+// 2: conj of the whole product.  P_ready: the digits of P are those of the call before.
+cudaError_t emul_zgemm_cols(const DigitWs& w, const double2* P, int64_t nt, int64_t K, const double2* V, int64_t N,
+                            int mode, double2* C, bool P_ready, cudaStream_t st, int64_t* nlaunch);
 // whether a product of complex K fits the digit sums
 bool emul_fits(int64_t K);
 cudaError_t emul_split_rows(const double2* A, int64_t count, int64_t M, int64_t K, int64_t lda, int64_t sa,

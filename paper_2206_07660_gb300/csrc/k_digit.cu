@@ -44,6 +44,8 @@ struct DigitArgs {
   int pairs;            // 1: columns (2p, 2p + 1) of row r form the double2 at p * col_s1 + r's offset
   int64_t row_inner, row_s1, col_s1;
   const int* row_list;
+  double alpha;
+  int scaled, acc;      // alpha differs from 1; the output is added to
   const double* Y;      // row-major: the output is I - Y + A B (identity of complex matrices with eb_sh = 1)
   int* err;
   uint32_t spin;
@@ -60,8 +62,10 @@ __device__ __forceinline__ void tmem_ld8(uint32_t addr, uint32_t* r) {
 // exact double of an integer |v| < 2^51, less the bias 1.5 2^52 (one FP64 subtraction instead of
 // a conversion)
 __device__ __forceinline__ double biased(long long v) { return __longlong_as_double(v + 0x4338000000000000ll); }
-// 2^e as a double (exponents stay far inside the range; clamped)
+// 2^e as a double (exponents stay far inside the range; clamped); NaN with the exponent of a row that
+// is not finite (k_emul.cu: em_exponent)
 __device__ __forceinline__ double pow2d(int e) {
+  if (e > 8192) return __longlong_as_double(0x7ff8000000000000ll);
   e = e < -1022 ? -1022 : (e > 1023 ? 1023 : e);
   return __longlong_as_double((long long)(e + 1023) << 52);
 }
@@ -229,7 +233,11 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
               v[u] = fma(h, 268435456.0, l) * pow2d(rexp + ce);
             }
             double2* p = a.pairs ? (double2*)(a.C + off + (int64_t)(n >> 1) * a.col_s1) : (double2*)(a.C + off + n);
-            if (rg > 0) {
+            if (a.scaled) {
+              v[0] *= a.alpha;
+              v[1] *= a.alpha;
+            }
+            if (rg > 0 || a.acc) {
               const double2 o = *p;
               v[0] += o.x;
               v[1] += o.y;
@@ -321,6 +329,7 @@ cudaError_t digit_gemm(const DigitGemm& d, cudaStream_t st) {
   a.pairs = d.pairs ? 1 : 0;
   a.row_inner = d.row_inner > 0 ? d.row_inner : d.M; a.row_s1 = d.row_s1; a.col_s1 = d.col_s1; a.row_list = d.row_list;
   a.Y = d.Y;
+  a.alpha = d.alpha; a.scaled = d.alpha != 1.0; a.acc = d.acc ? 1 : 0;
   a.err = d.err;
   a.spin = umma_spin();
   CUtensorMap tA, tB;

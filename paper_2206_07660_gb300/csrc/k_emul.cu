@@ -75,9 +75,18 @@ __device__ __forceinline__ __half2 em_conj(__half2 d) {   // (re, -im)
   return *(__half2*)&n;
 }
 
-// biased exponent of |x| (0 for zero and subnormals); the row exponent e of a largest one: m < 2^e
+// biased exponent of |x| (0 for zero and subnormals); the row exponent e of a largest one: m < 2^e, or
+// 2^14 for a row that is not finite (its digits are zeros, its products NaN)
 __device__ __forceinline__ int em_bexp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-__device__ __forceinline__ int em_exponent(int bexp) { return bexp ? bexp - 1022 : 0; }
+__device__ __forceinline__ int em_exponent(int bexp) { return bexp == 0x7ff ? 1 << 14 : bexp ? bexp - 1022 : 0; }
+// doubled rows (2j, 2j + 1) of a B entry d = (Br, Bi): mode 0: B, 1: conj B, 2: the conjugate of the product
+__device__ __forceinline__ void em_double(__half2 d, int mode, __half2& r0, __half2& r1) {
+  const __half2 w = __lowhigh2highlow(d);
+  const uint32_t x0 = *(const uint32_t*)&d ^ (mode == 1 ? 0u : 0x80000000u);
+  const uint32_t x1 = *(const uint32_t*)&w ^ (mode == 0 ? 0u : mode == 1 ? 0x00008000u : 0x80008000u);
+  r0 = *(const __half2*)&x0;
+  r1 = *(const __half2*)&x1;
+}
 
 // A-operand digits from a transposed source: row n of the operand is column n of a
 // K x ncol complex matrix (element (n, k) at src[z*zs + k*ld + n]), real K index
@@ -152,7 +161,7 @@ __global__ void __launch_bounds__(256) em_split_t_kernel(const double2* __restri
 // ldb): rows 2m = (Br, -Bi), 2m+1 = (Bi, Br) along the real K index 2j + c;
 // digit planes in reverse order; one exponent per complex row m.
 __global__ void em_split_b_kernel(const double2* __restrict__ B, int64_t rows, int64_t K, int64_t ldb,
-                                  dig_t* __restrict__ dig, int* __restrict__ ex, int64_t Kp) {
+                                  dig_t* __restrict__ dig, int* __restrict__ ex, int64_t Kp, int mode) {
   const int64_t m = blockIdx.x;
   __shared__ int red[256];
   int mx = 0;
@@ -178,8 +187,7 @@ __global__ void em_split_b_kernel(const double2* __restrict__ B, int64_t rows, i
 #pragma unroll
     for (int i = 0; i < EM_S; ++i) {
       const int64_t p = (int64_t)(EM_S - 1 - i) * Kp;   // reverse digit order
-      *(__half2*)(r0 + p) = em_conj(d[i]);
-      *(__half2*)(r1 + p) = __lowhigh2highlow(d[i]);
+      em_double(d[i], mode, *(__half2*)(r0 + p), *(__half2*)(r1 + p));
     }
   }
 }
@@ -221,7 +229,7 @@ __global__ void __launch_bounds__(256) em_split_r_kernel(const double2* __restri
 // digit writes along k); padding columns [2K, Kp) are written as zeros.
 __global__ void __launch_bounds__(256) em_split_bt_kernel(const double2* __restrict__ src, int64_t K, int64_t ncol,
                                                           int64_t ld, int64_t zs, dig_t* __restrict__ dig,
-                                                          int* __restrict__ ex, int64_t Kp) {
+                                                          int* __restrict__ ex, int64_t Kp, int mode) {
   __shared__ double2 tile[32][33];
   __shared__ int red[8][32];
   __shared__ int es[32];
@@ -267,8 +275,7 @@ __global__ void __launch_bounds__(256) em_split_bt_kernel(const double2* __restr
 #pragma unroll
         for (int i = 0; i < EM_S; ++i) {
           const int64_t p = (int64_t)(EM_S - 1 - i) * Kp;
-          *(__half2*)(r0 + p) = em_conj(d[i]);
-          *(__half2*)(r1 + p) = __lowhigh2highlow(d[i]);
+          em_double(d[i], mode, *(__half2*)(r0 + p), *(__half2*)(r1 + p));
         }
       }
     }
@@ -319,7 +326,7 @@ cudaError_t emul_split_b(const double2* B, int64_t rows, int64_t K, int64_t ldb,
   const int64_t Kp = emul_kpad(K);
   cudaError_t e = cudaMemsetAsync(dig, 0, emul_digit_bytes(2 * rows, K), st);
   if (e != cudaSuccess) return e;
-  em_split_b_kernel<<<(unsigned)rows, 256, 0, st>>>(B, rows, K, ldb, (dig_t*)dig, ex, Kp);
+  em_split_b_kernel<<<(unsigned)rows, 256, 0, st>>>(B, rows, K, ldb, (dig_t*)dig, ex, Kp, 0);
   return cudaGetLastError();
 }
 
@@ -483,8 +490,65 @@ cudaError_t emul_split_cols(const double2* B, int64_t count, int64_t K, int64_t 
   const int64_t Kp = emul_kpad(K);
   if (count > 65535) return cudaErrorInvalidValue;
   em_split_bt_kernel<<<dim3((unsigned)((N + 31) / 32), (unsigned)count), 256, 0, st>>>(B, K, N, ldb, sb, (dig_t*)Bd,
-                                                                                        Be, Kp);
+                                                                                        Be, Kp, 0);
   return cudaGetLastError();
+}
+
+// Products of the FP64 contraction chains.  Native FP64 runs at 1.1 TFLOP/s here; 36 digit products
+// of 16-bit operands at a thousand times that are ten times as fast, the digits included, and as
+// accurate (a row's 56 bits against the rounding of a sum; ranges longer than digit_kmax are added in
+// FP64).  Below ~2e8 flops the three launches cost more than they save.
+bool emul_pays(const DigitWs& w, int64_t M, int64_t N, int64_t K, int64_t rows) {
+  return w.A && 8.0 * M * N * K >= 2e8 && (size_t)rows * EM_S * emul_kpad(K) * sizeof(dig_t) <= w.A_bytes &&
+         emul_digit_bytes(2 * N, K) <= w.B_bytes;
+}
+cudaError_t emul_zgemm_rows(const DigitWs& w, const double2* A, int64_t M, int64_t K, const double2* B, int64_t N,
+                            bool conjB, double2* C, double alpha, bool acc, cudaStream_t st, int64_t* nlaunch) {
+  const int64_t Kp = emul_kpad(K), rowb = EM_S * Kp * (int64_t)sizeof(dig_t);
+  cudaError_t e = cudaMemsetAsync(w.B, 0, emul_digit_bytes(2 * N, K), st);
+  if (e != cudaSuccess) return e;
+  em_split_b_kernel<<<(unsigned)N, 256, 0, st>>>(B, N, K, K, (dig_t*)w.B, w.Be, Kp, conjB ? 1 : 0);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  *nlaunch += 1;
+  const int64_t mc = (int64_t)(w.A_bytes / rowb);   // rows at a time
+  for (int64_t m0 = 0; m0 < M; m0 += mc) {
+    const int64_t m = M - m0 < mc ? M - m0 : mc;
+    if ((e = emul_split_rows(A + m0 * K, 1, m, K, K, 0, w.A, w.Ae, st)) != cudaSuccess) return e;
+    DigitGemm d{};
+    d.Ad = w.A; d.Bd = w.B; d.eA = w.Ae; d.eB = w.Be;
+    d.batch = 1; d.M = m; d.N = 2 * N; d.K = 2 * K; d.Kp = Kp; d.nd = EM_S;
+    d.C = (double*)(C + m0 * N); d.err = w.err; d.alpha = alpha; d.acc = acc;
+    if ((e = digit_gemm(d, st)) != cudaSuccess) return e;
+    *nlaunch += 2;
+  }
+  return cudaSuccess;
+}
+cudaError_t emul_zgemm_cols(const DigitWs& w, const double2* P, int64_t nt, int64_t K, const double2* V, int64_t N,
+                            int mode, double2* C, bool P_ready, cudaStream_t st, int64_t* nlaunch) {
+  const int64_t Kp = emul_kpad(K), rowb = EM_S * Kp * (int64_t)sizeof(dig_t);
+  em_split_bt_kernel<<<dim3((unsigned)((N + 31) / 32), 1), 256, 0, st>>>(V, K, N, N, 0, (dig_t*)w.B, w.Be, Kp, mode);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  *nlaunch += 1;
+  int64_t tc = (int64_t)(w.A_bytes / (K * rowb));   // matrices at a time
+  if (tc > nt) tc = nt;
+  if (tc < 1) return cudaErrorInvalidValue;
+  for (int64_t t0 = 0; t0 < nt; t0 += tc) {
+    const int64_t n = nt - t0 < tc ? nt - t0 : tc;
+    if (!P_ready || tc < nt) {
+      em_split_t_kernel<false><<<dim3((unsigned)((K + 31) / 32), (unsigned)n), 256, 0, st>>>(
+          P + t0 * K * K, K, K, K, K * K, (dig_t*)w.A, w.Ae, Kp, nullptr, nullptr);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      *nlaunch += 1;
+    }
+    DigitGemm d{};
+    d.Ad = w.A; d.Bd = w.B; d.eA = w.Ae; d.eB = w.Be;
+    d.batch = 1; d.M = n * K; d.N = 2 * N; d.K = 2 * K; d.Kp = Kp; d.nd = EM_S;
+    d.C = (double*)(C + t0 * K * N); d.err = w.err;
+    if ((e = digit_gemm(d, st)) != cudaSuccess) return e;
+    *nlaunch += 1;
+  }
+  return cudaSuccess;
 }
 
 // C[z] (M x N complex, row-major, row stride N, batch stride M N) = A[z] B[z] from the

@@ -1,0 +1,67 @@
+"""The large products of the FP64 contraction chains in digits on the tensor cores (the default of
+FP64-accurate arithmetic) against the oracle: the last P~0 step, the first Sigma~ step, and those of
+the two adjoints.  Sizes above the rule's 2e8 flops with odd orders, K longer and shorter than one
+exact range, native FP64 arithmetic as the other side, and values that are not finite."""
+import numpy as np
+import pytest
+
+from gpu_helpers import gpu, hermitian_noise, rel, system
+from oracle import adjoint as oad
+from oracle import gw as ogw
+
+pytestmark = pytest.mark.gpu
+
+# sums of ~1e3 products of order one: 2^-53 sqrt(1e3) per term of the largest sum, with margin
+TOL = 1e-12
+SIZES = [(13, 97, (2, 1, 1), 41), (17, 75, (3, 1, 1), 40), (5, 200, (1, 1, 1), 50)]
+
+
+@pytest.mark.parametrize("nao,naux,kmesh,ntau", SIZES)
+@pytest.mark.parametrize("arith", ["tensor", "native"])
+def test_contractions(nao, naux, kmesh, ntau, arith):
+    sysd = system(nao, naux, kmesh, ntau, 20.0, 101)
+    km = ogw.KMesh(kmesh)
+    G = hermitian_noise((ntau, km.nk, nao, nao), 0.3, 102)
+    P = hermitian_noise((km.nk, ntau, naux, naux), 0.3, 103)
+    g = gpu(sysd, fp64_gemm=arith)
+    g.set("G_tau", G)
+    g.polarization()
+    assert rel(g.get("P0_tau"), ogw.polarization_tau(sysd["V"], G, km)) < TOL
+    g.set("P_tau", P)
+    g.selfenergy_partial()
+    assert rel(g.get("Sigma_tau"), ogw.selfenergy_tau(sysd["V"], G, P, km, qs=list(range(km.nk)))) < TOL
+
+
+@pytest.mark.parametrize("nao,naux,kmesh,ntau", SIZES[:2])
+@pytest.mark.parametrize("precision", ["fp64", "split_f16"])
+def test_adjoints(nao, naux, kmesh, ntau, precision):
+    import torch
+    sysd = system(nao, naux, kmesh, ntau, 20.0, 104)
+    km = ogw.KMesh(kmesh)
+    rng = np.random.default_rng(105)
+    noise = lambda *s: rng.standard_normal(s) + 1j * rng.standard_normal(s)
+    G, P = hermitian_noise((ntau, km.nk, nao, nao), 0.3, 106), hermitian_noise((km.nk, ntau, naux, naux), 0.3, 107)
+    g = gpu(sysd, precision=precision)
+    g.set("G_tau", G)
+    g.set("P_tau", P)
+    Pbar, Sbar = noise(km.nk, ntau, naux, naux), noise(ntau, km.nk, nao, nao)
+    got = g.polarization_vjp(torch.from_numpy(Pbar).cuda()).cpu().numpy()
+    assert rel(got, oad.polarization_vjp(sysd["V"], G, km, Pbar)) < TOL
+    gb, pb = g.selfenergy_vjp(torch.from_numpy(Sbar).cuda())
+    rg, rp = oad.selfenergy_vjp(sysd["V"], G, P, km, Sbar)
+    assert rel(gb.cpu().numpy(), rg) < TOL and rel(pb.cpu().numpy(), rp) < TOL
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+def test_values_that_are_not_finite_stay_so(value):
+    nao, naux, kmesh, ntau = SIZES[2]
+    sysd = system(nao, naux, kmesh, ntau, 20.0, 108)
+    G = hermitian_noise((ntau, 1, nao, nao), 0.3, 109)
+    G[3, 0, 2, 2] = value
+    g = gpu(sysd)
+    g.set("G_tau", G)
+    g.polarization()
+    P0 = g.get("P0_tau")[0]
+    bad = [3, ntau - 1 - 3]
+    assert not np.isfinite(P0[bad]).any()
+    assert np.isfinite(np.delete(P0, bad, axis=0)).all()
