@@ -89,7 +89,8 @@ enum {
   GW_SMALL_SIMT   = 1u << 4, /* GW_SPLIT_TF32, nao <= 64: those steps on the FP32
                                 SIMT small-product kernel.  Neither flag: library default */
   GW_FP64_NATIVE  = 1u << 5, /* FP64 SIMT arithmetic for the tau <-> i nu transforms
-                                and the screened solve, instead of the defaults:
+                                and the screened solve, the GW_FP64 contractions and
+                                the fp64 adjoints, instead of the defaults:
                                 FP64-accurate digit-split products on the tensor cores
                                 and a complex64 inversion refined to FP64 accuracy    */
   GW_TRS          = 1u << 6  /* the system is time-reversal symmetric: H0(-k) =
@@ -330,8 +331,10 @@ gw_status gw_profile_read(gw_ctx* ctx, double* out6);
  * respect to G(tau), at the context's current G: Gbar = sum conj(dP~0/dG) Pbar
  * for a real loss (PyTorch's conjugate-Wirtinger convention).  Pbar
  * [nq][ntau][naux][naux] and Gbar [ntau][nk][nao][nao] are device pointers;
- * Gbar is overwritten.  Runs in fp64 whatever contract_prec is; allocates
- * three chain buffers of ntau*naux*nao^2 complex on first use. */
+ * Gbar is overwritten.  Runs in fp64 whatever contract_prec is (large products
+ * as exact digits on the tensor cores, without GW_FP64_NATIVE; the call then
+ * synchronises, except inside a stream capture); allocates three chain buffers of
+ * ntau*naux*nao^2 complex, and up to 1 GB for the digits, on first use. */
 gw_status gw_polarization_vjp(gw_ctx* ctx, const double* Pbar, double* Gbar);
 
 /* Adjoint of gw_selfenergy's Sigma~(tau) (Eq. tilde_sigma2, symmetrised) with

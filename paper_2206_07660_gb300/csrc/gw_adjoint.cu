@@ -129,16 +129,26 @@ cudaError_t polarization_vjp(const View& v, const double2* Pbar, double2* Gbar, 
       *launches += 1;
       }
       // Y[t][Q'][c][a] = sum_d conj(Gm[t][c][d]) X[t][Q'][d][a],  Gm(t) = -G^k(t_{n-1-j})
+      // (in digits as Y[t][Q'][a][c], rows the columns of X)
+      const bool dig = !v.c64 && emul_pays_batch(v.dg, nt, (int64_t)naux * nao, nao, nao);
       GettDesc d2 = desc(nao, (int64_t)naux * nao, nao, nt);
       d2.am = I1(nao); d2.ak = I1(1); d2.az = I1(-gstep); d2.conjA = true;
       d2.bk = I1(nao); d2.bn = I2(nao, n2, 1); d2.bz = I1(slab);
       d2.cm = I1(nao); d2.cn = I2(nao, n2, 1); d2.cz = I1(slab);
       d2.alpha = make_double2(-1, 0);
       const void* Gm = at(v, v.G_tau, v.G32, (int64_t)(ntau - 1) * gstep + (int64_t)k * n2);
-      if ((e = run(v, d2, Gm, v.bufA, v.bufB))) return e;
+      if (dig) {
+        if ((e = emul_zgemm_batch(v.dg, EmulA::cols, v.bufA, nao, false, (const double2*)Gm, -gstep, 1, nt,
+                                  (int64_t)naux * nao, nao, nao, v.bufB, -1.0, v.st, launches)))
+          return e;
+        P_ready = false;
+      } else if ((e = run(v, d2, Gm, v.bufA, v.bufB))) {
+        return e;
+      }
       // G'bar[t][a][b] += f sum_{Q',c} Y[t][Q'][c][a] conj(V2[Q'][b][c])
       GettDesc d3 = desc(nao, nao, (int64_t)naux * nao, nt);
       d3.am = I1(1); d3.ak = I2(nao, n2, nao); d3.az = I1(slab);
+      if (dig) { d3.am = I1(nao); d3.ak = I2(nao, n2, 1); }
       d3.bk = I2(nao, n2, 1); d3.bn = I1(nao); d3.conjB = true;
       d3.cm = I1(nao); d3.cn = I1(1); d3.cz = I1(gstep);
       d3.alpha = make_double2(f, 0); d3.beta = make_double2(1, 0);
@@ -149,7 +159,14 @@ cudaError_t polarization_vjp(const View& v, const double2* Pbar, double2* Gbar, 
       d4.am = I1(nao); d4.ak = I1(1); d4.az = I1(slab);
       d4.bk = I1(nao); d4.bn = I1(1); d4.bz = I1(gstep); d4.conjB = true;
       d4.cm = I1(nao); d4.cn = I1(1); d4.cz = I1(slab);
-      if ((e = run(v, d4, v.bufA, at(v, v.G_tau, v.G32, (int64_t)kq * n2), v.bufB))) return e;
+      const void* Gq = at(v, v.G_tau, v.G32, (int64_t)kq * n2);
+      if (dig) {
+        if ((e = emul_zgemm_batch(v.dg, EmulA::rows, v.bufA, 0, true, (const double2*)Gq, gstep, 1, nt,
+                                  (int64_t)naux * nao, nao, nao, v.bufB, 1.0, v.st, launches)))
+          return e;
+      } else if ((e = run(v, d4, v.bufA, Gq, v.bufB))) {
+        return e;
+      }
       // Gm bar[t][c][d] = f sum_{Q',b} conj(V2[Q'][b][c]) T[t][Q'][d][b];  G^k(t_{n-1-j}) gets -Gm bar(t_j)
       GettDesc d5 = desc(nao, nao, (int64_t)naux * nao, nt);
       d5.am = I1(1); d5.ak = I2(nao, n2, nao); d5.conjA = true;
@@ -158,7 +175,7 @@ cudaError_t polarization_vjp(const View& v, const double2* Pbar, double2* Gbar, 
       d5.alpha = make_double2(-f, 0); d5.beta = make_double2(1, 0);
       d5.ksplit = split_of(v, d5.K, nt);
       if ((e = run(v, d5, V2, v.bufB, Gbar + (size_t)(ntau - 1) * gstep + (size_t)k * n2, true))) return e;
-      *launches += 4;
+      *launches += dig ? 2 : 4;
     }
   }
   return cudaSuccess;

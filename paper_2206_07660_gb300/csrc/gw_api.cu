@@ -255,10 +255,12 @@ static void digit_ws(gw_ctx* c) {
   const size_t cap = opt_budget(kFoldBytes);
   if (w.A_bytes > cap) w.A_bytes = cap;
   w.B_bytes = 2 * (naux * ra > n2 * rb ? naux * ra : n2 * rb);
+  w.A_rows = rows * c->nao;
+  w.B_rows = std::max(std::max(naux, n2), (int64_t)c->ntau * c->nao);
   w.A = &w;   // (for the rule alone)
   if (!emul_pays(w, rows, naux, n2, 1) && !emul_pays(w, rows, n2, naux, naux)) return;
   w.A = dalloc(c, w.A_bytes); w.B = dalloc(c, w.B_bytes);
-  w.Ae = (int*)dalloc(c, (size_t)rows * 4); w.Be = (int*)dalloc(c, (size_t)(naux > n2 ? naux : n2) * 4);
+  w.Ae = (int*)dalloc(c, (size_t)w.A_rows * 4); w.Be = (int*)dalloc(c, (size_t)w.B_rows * 4);
   w.err = c->info + 1;
   if (!w.A || !w.B || !w.Ae || !w.Be) {
     dfree(c, w.A); dfree(c, w.B); dfree(c, w.Ae); dfree(c, w.Be);
@@ -290,9 +292,14 @@ static void free_all(gw_ctx* c) {
 
 static inline void count(int n) { g_launches += n; }
 
-// contractions on the tensor cores (the wait-timeout flag is then meaningful)
+// whether the caller captures the context's stream (its FP64 stages without a host read can be)
+static bool capturing(const gw_ctx* c) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(c->st, &s) == cudaSuccess && s != cudaStreamCaptureStatusNone;
+}
+// contractions on the tensor cores (the wait-timeout flag is then meaningful, and read)
 static inline bool uses_tc(const gw_ctx* c) {
-  return c->cfg.contract_prec == GW_SPLIT_TF32 || c->hfmt != 0 || c->dg.A != nullptr;
+  return c->cfg.contract_prec == GW_SPLIT_TF32 || c->hfmt != 0 || (c->dg.A != nullptr && !capturing(c));
 }
 // the time-reversal reduction applies to forward stages over the full q range
 static inline bool trs_reduce(const gw_ctx* c) { return c->trs && c->q0 == 0 && c->q1 == c->nk; }
@@ -1389,6 +1396,8 @@ static gw_status polar_chain(gw_ctx* c, const double2* Gplus, const double2* Gmi
     const int nt = polar_taus(c, q);   // tau points computed; the others are conjugates
     if (nt == 0) continue;
     double2* Pq = out + (size_t)q * ntau * na2;
+    const bool zdig = !f32 && emul_pays(c->dg, (int64_t)nt * naux, naux, n2, 1) &&
+                      emul_pays_batch(c->dg, nt, (int64_t)naux * nao, nao, nao);
     for (int k = 0; k < nk; ++k) {
       const int kq = c->kplus[(size_t)q * nk + k];
       const int j = k % G;                      // column block of this k in its group
@@ -1415,6 +1424,16 @@ static gw_status polar_chain(gw_ctx* c, const double2* Gplus, const double2* Gmi
                        per};
         CK(run_umma(c, 8.0 * nt * naux * (double)nao * n2, ya, gb, naux * nao, 2 * nao, ka, nt, Zh, false, -1.0,
                     false, 2, (int64_t)naux * zld, 1, nao, zld, 2, 2 * (int64_t)nao, Zl, 2 * (int64_t)nao));
+      } else if (zdig) {
+        // FP64: both steps in digits (nao 26, naux 200, 3x1x1, ntau 92: 1.0 ms a (q, k) pair on average, native 4.5), the second
+        // with the rows (Q, b) of Y's columns, Z[t][Q][b][c] = sum_d Y_db (-G^k_cd(t_{ntau-1-j})): the last
+        // step then takes the rows V^{k+q,k}_bc
+        int64_t nl = 0;
+        CK(emul_zgemm_batch(c->dg, EmulA::shared, (const double2*)Vkq, 0, true, (const double2*)Gp + (size_t)kq * n2, gstep,
+                            0, nt, (int64_t)naux * nao, nao, nao, (double2*)c->chA, 1.0, c->st, &nl));
+        CK(emul_zgemm_batch(c->dg, EmulA::cols, (const double2*)c->chA, nao, false, (const double2*)Gm, -gstep, 0, nt,
+                            (int64_t)naux * nao, nao, nao, (double2*)c->chB, -1.0, c->st, &nl));
+        count((int)nl);
       } else if (f32 && nao <= 64) {
         // Y[t][Q][d][b] = sum_a V^{k,k+q}[Q][d][a] G^{k+q}[t][a][b]   (G shared per t)
         BsmDesc b1{};
@@ -1475,7 +1494,8 @@ static gw_status polar_chain(gw_ctx* c, const double2* Gplus, const double2* Gmi
       }
       if (!f32 && emul_pays(c->dg, (int64_t)nt * naux, naux, n2, 1)) {
         int64_t nl = 0;
-        CK(emul_zgemm_rows(c->dg, (const double2*)c->chB, (int64_t)nt * naux, n2, (const double2*)Vkq, naux, true, Pq,
+        CK(emul_zgemm_rows(c->dg, (const double2*)c->chB, (int64_t)nt * naux, n2,
+                           zdig ? c->V + ((size_t)kq * nk + k) * slab : (const double2*)Vkq, naux, !zdig, Pq,
                            c->spin / nk, accumulate || k > 0, c->st, &nl));
         count((int)nl);
         continue;
@@ -2043,6 +2063,7 @@ static gw_status sigma_chain(gw_ctx* c, const double2* Gsrc, const double2* Psrc
         //   Sigma~[n-1-t][k-q][a][j] += -(1/Nk) sum Y[t][a][(Q',b)] V^{k,k-q}[Q'][b][j]
         const int zt = im ? ni : nt, kg = im ? k : kmq, ko = im ? kmq : k;
         const int64_t t0 = im ? (int64_t)(ntau - 1) * gstep : 0, ts = im ? -gstep : gstep;
+        const bool ydig = !f32 && emul_pays_batch(c->dg, zt, (int64_t)naux * nao, nao, nao);
         if (f32 && nao <= 64) {
           BsmDesc b{};
           b.M = b.N = b.K = nao; b.G = zt; b.E = naux; b.alpha = 1.f;
@@ -2051,6 +2072,13 @@ static gw_status sigma_chain(gw_ctx* c, const double2* Gsrc, const double2* Psrc
           b.B = (const float2*)Gp + t0 + (size_t)kg * n2; b.b_gs = ts; b.b_rs = nao; b.b_cs = 1; b.b_shared = 1;
           b.C = (float2*)c->chB; b.c_gs = slab; b.c_es = nao; b.c_rs = (int64_t)naux * nao;
           CK(run_bsm(c, b));
+        } else if (ydig) {   // as Y[t][Q'][i or a][b]
+          int64_t nl = 0;
+          CK(emul_zgemm_batch(c->dg, im ? EmulA::cols : EmulA::rows, (const double2*)c->chA, nao, true,
+                              (const double2*)Gp + t0 + (size_t)kg * n2, ts, im ? 3 : 0, zt, (int64_t)naux * nao, nao, nao,
+                              (double2*)c->chB, 1.0, c->st, &nl));
+          count((int)nl);
+          P_ready = false;
         } else {
           GettDesc d2 = base_desc((int64_t)naux * nao, nao, nao, zt);
           if (im) { d2.am = I2(nao, n2, 1); d2.ak = I1(nao); d2.conjA = true; }
@@ -2062,6 +2090,7 @@ static gw_status sigma_chain(gw_ctx* c, const double2* Gsrc, const double2* Psrc
         }
         GettDesc d3 = base_desc(nao, nao, (int64_t)naux * nao, zt);
         d3.am = I1((int64_t)naux * nao); d3.ak = I1(1); d3.az = I1(slab);
+        if (ydig) { d3.am = I1(nao); d3.ak = I2(nao, n2, 1); }
         d3.bk = I1(nao); d3.bn = I1(1); d3.bz = I1(0);
         d3.cm = I1(nao); d3.cn = I1(1); d3.cz = I1(ts);
         d3.alpha = make_double2(-1.0 / nk, 0);
@@ -2083,7 +2112,7 @@ static gw_status sigma_tau_part(gw_ctx* c) {
   const bool red = trs_reduce(c);
   c->reduce = red;
   // a P~ that was handed in is looked at for the fold (the screened solve's own has it)
-  if (c->fold && !c->psym && !red && !c->deferred && sigma_shares(c)) {
+  if (c->fold && !c->psym && !red && !c->deferred && !capturing(c) && sigma_shares(c)) {
     CK(fold_check_tau(c->P_tau, c->na2, ntau, c->q0, c->q1, c->d_kneg, c->dscr + 16, c->st));
     count(1);
     CK(cudaMemcpyAsync(c->h_scr + 16, c->dscr + 16, 16, cudaMemcpyDeviceToHost, c->st));
@@ -2444,7 +2473,7 @@ static gw_status polarization_vjp_impl(gw_ctx* c, const double* Pbar, double* Gb
   if (c->dg.A && !c->deferred) CK(cudaMemsetAsync(c->info + 1, 0, 4, c->st));
   CK(gwadj::polarization_vjp(v, (const double2*)Pbar, (double2*)Gbar, &l));
   count((int)l);
-  return c64 || !c->dg.A ? GW_OK : tc_check(c);
+  return c64 || !c->dg.A || capturing(c) ? GW_OK : tc_check(c);
 }
 
 extern "C" gw_status gw_polarization_vjp(gw_ctx* c, const double* Pbar, double* Gbar) {
@@ -2468,7 +2497,7 @@ static gw_status selfenergy_vjp_impl(gw_ctx* c, const double* Sbar, double* Gbar
   if (c->dg.A && !c->deferred) CK(cudaMemsetAsync(c->info + 1, 0, 4, c->st));
   CK(gwadj::selfenergy_vjp(v, (const double2*)Sbar, (double2*)Gbar, (double2*)Pbar, &l));
   count((int)l);
-  return c64 || !c->dg.A ? GW_OK : tc_check(c);
+  return c64 || !c->dg.A || capturing(c) ? GW_OK : tc_check(c);
 }
 
 extern "C" gw_status gw_selfenergy_vjp(gw_ctx* c, const double* Sbar, double* Gbar, double* Pbar) {

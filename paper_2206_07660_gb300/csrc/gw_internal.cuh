@@ -314,6 +314,7 @@ struct DigitGemm {
   int* err;
   double alpha = 1.0;            // C = alpha A B
   bool acc = false;              // added to C
+  bool a_shared = false;         // one A for the whole batch
 };
 cudaError_t digit_gemm(const DigitGemm& d, cudaStream_t st);
 int64_t digit_kmax(int nd);
@@ -346,19 +347,29 @@ struct DigitWs {
   void* A = nullptr;
   size_t A_bytes = 0;
   int* Ae = nullptr;
+  int64_t A_rows = 0;   // exponents of A
   void* B = nullptr;
   size_t B_bytes = 0;
+  int64_t B_rows = 0;   // exponents of B (complex rows)
   int* Be = nullptr;
   int* err = nullptr;
 };
 // whether a product of M x N complex outputs over K terms takes the digits (its operands fit, and
-// it is large enough)
+// it is large enough), `rows` rows of A at least at a time
 bool emul_pays(const DigitWs& w, int64_t M, int64_t N, int64_t K, int64_t rows);
 // C (M x N, packed) = or (acc) += alpha A op(B)^T, A: M x K and B: N x K packed rows, op = conj or none
 cudaError_t emul_zgemm_rows(const DigitWs& w, const double2* A, int64_t M, int64_t K, const double2* B, int64_t N,
                             bool conjB, double2* C, double alpha, bool acc, cudaStream_t st, int64_t* nlaunch);
+// C_z (M x N, packed) = alpha A_z op(B_z), z < nz.  A: one M x K matrix for all z, packed M x K matrices,
+// or per z M / inner packed K x inner matrices whose columns are the rows.  B_z (at B + z b_zs): K x N packed
+// (bcols), or its transpose; mode as emul_zgemm_cols.
+enum class EmulA { shared, rows, cols };
+bool emul_pays_batch(const DigitWs& w, int64_t nz, int64_t M, int64_t N, int64_t K);
+cudaError_t emul_zgemm_batch(const DigitWs& w, EmulA akind, const double2* A, int64_t inner, bool bcols, const double2* B,
+                             int64_t b_zs, int mode, int64_t nz, int64_t M, int64_t N, int64_t K, double2* C, double alpha,
+                             cudaStream_t st, int64_t* nlaunch);
 // C[t] (K x N, packed) = P[t]^T op(V), t < nt, P[t]: K x K and V: K x N packed; mode 0: op none, 1: conj V,
-// 2: conj of the whole product.  P_ready: the digits of P are those of the call before.
+// 2: conj of the whole product, 3: conj P.  P_ready: the digits of P are those of the call before.
 cudaError_t emul_zgemm_cols(const DigitWs& w, const double2* P, int64_t nt, int64_t K, const double2* V, int64_t N,
                             int mode, double2* C, bool P_ready, cudaStream_t st, int64_t* nlaunch);
 // whether a product of complex K fits the digit sums

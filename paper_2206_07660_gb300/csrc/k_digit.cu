@@ -319,12 +319,12 @@ cudaError_t digit_gemm(const DigitGemm& d, cudaStream_t st) {
   a.kbr = d.K <= km ? a.nkb : (int)(km / DG_BK);
   a.nranges = (a.nkb + a.kbr - 1) / a.kbr;
   a.kbr = (a.nkb + a.nranges - 1) / a.nranges;
-  a.a_batched = d.batch > 1; a.b_batched = d.batch > 1;
+  a.a_batched = d.batch > 1 && !d.a_shared; a.b_batched = d.batch > 1;
   a.ntm = (a.M + DG_BM - 1) / DG_BM; a.ntn = (a.N + DG_BN - 1) / DG_BN;
   const int64_t nt = (int64_t)a.ntm * a.ntn * d.batch;
   if (nt > INT32_MAX || (d.pairs && d.batch != 1)) return cudaErrorInvalidValue;
   a.ntiles = (int)nt;
-  a.eA = d.eA; a.eB = d.eB; a.ea_zs = d.M; a.eb_sh = d.real_cols ? 0 : 1; a.eb_zs = d.real_cols ? d.N : d.N / 2;
+  a.eA = d.eA; a.eB = d.eB; a.ea_zs = d.a_shared ? 0 : d.M; a.eb_sh = d.real_cols ? 0 : 1; a.eb_zs = d.real_cols ? d.N : d.N / 2;
   a.C = d.C; a.c_ld = d.N; a.c_zs = d.M * d.N;
   a.pairs = d.pairs ? 1 : 0;
   a.row_inner = d.row_inner > 0 ? d.row_inner : d.M; a.row_s1 = d.row_s1; a.col_s1 = d.col_s1; a.row_list = d.row_list;
@@ -334,7 +334,7 @@ cudaError_t digit_gemm(const DigitGemm& d, cudaStream_t st) {
   a.spin = umma_spin();
   CUtensorMap tA, tB;
   const int64_t ld = (int64_t)DG_S * d.Kp;
-  if (!make_map(&tA, d.Ad, ld, d.M, d.batch, ld, d.M * ld, DG_BM, 1) ||
+  if (!make_map(&tA, d.Ad, ld, d.M, d.a_shared ? 1 : d.batch, ld, d.M * ld, DG_BM, 1) ||
       !make_map(&tB, d.Bd, ld, d.N, d.batch, ld, d.N * ld, DG_BN, 1))
     return cudaErrorInvalidValue;
   return d.nd == 8 ? launch<8>(tA, tB, a, st) : launch<5>(tA, tB, a, st);

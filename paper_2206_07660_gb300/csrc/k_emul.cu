@@ -21,8 +21,10 @@
 // of X, complex K = ntau), B = T (rows 2m, 2m+1 = the real 2x2 blocks of T[m][j]),
 // output written transposed into Y (lane-per-row FP64 stores); and for the batched
 // square products C[z] = A[z] B[z] of the screened solve's refinement (A split from
-// its rows, B from its columns, output row-major).
+// its rows, B from its columns, output row-major); and for the large products of the FP64
+// contraction chains and adjoints (the emul_zgemm functions).
 #include <cuda_fp16.h>
+#include <algorithm>
 #include "gw_internal.cuh"
 
 namespace gwk {
@@ -79,11 +81,11 @@ __device__ __forceinline__ __half2 em_conj(__half2 d) {   // (re, -im)
 // 2^14 for a row that is not finite (its digits are zeros, its products NaN)
 __device__ __forceinline__ int em_bexp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 __device__ __forceinline__ int em_exponent(int bexp) { return bexp == 0x7ff ? 1 << 14 : bexp ? bexp - 1022 : 0; }
-// doubled rows (2j, 2j + 1) of a B entry d = (Br, Bi): mode 0: B, 1: conj B, 2: the conjugate of the product
+// doubled rows (2j, 2j + 1) of a B entry d = (Br, Bi): mode 0: A B, 1: A conj B, 2: conj (A B), 3: conj A  B
 __device__ __forceinline__ void em_double(__half2 d, int mode, __half2& r0, __half2& r1) {
   const __half2 w = __lowhigh2highlow(d);
-  const uint32_t x0 = *(const uint32_t*)&d ^ (mode == 1 ? 0u : 0x80000000u);
-  const uint32_t x1 = *(const uint32_t*)&w ^ (mode == 0 ? 0u : mode == 1 ? 0x00008000u : 0x80008000u);
+  const uint32_t x0 = *(const uint32_t*)&d ^ (mode & 1 ? 0u : 0x80000000u);
+  const uint32_t x1 = *(const uint32_t*)&w ^ (mode == 0 ? 0u : mode == 1 ? 0x00008000u : mode == 2 ? 0x80008000u : 0x80000000u);
   r0 = *(const __half2*)&x0;
   r1 = *(const __half2*)&x1;
 }
@@ -157,16 +159,17 @@ __global__ void __launch_bounds__(256) em_split_t_kernel(const double2* __restri
   }
 }
 
-// B operand of C = A B^T from a small complex matrix B[m][j] (rows x K, row stride
-// ldb): rows 2m = (Br, -Bi), 2m+1 = (Bi, Br) along the real K index 2j + c;
+// B operand of C = A B^T from small complex matrices B[m][j] (per x K, row stride ldb; rows from
+// m = per on in the next one, zs away): rows 2m = (Br, -Bi), 2m+1 = (Bi, Br) along the real K index 2j + c;
 // digit planes in reverse order; one exponent per complex row m.
-__global__ void em_split_b_kernel(const double2* __restrict__ B, int64_t rows, int64_t K, int64_t ldb,
+__global__ void em_split_b_kernel(const double2* __restrict__ B0, int64_t per, int64_t zs, int64_t K, int64_t ldb,
                                   dig_t* __restrict__ dig, int* __restrict__ ex, int64_t Kp, int mode) {
   const int64_t m = blockIdx.x;
+  const double2* B = B0 + (m / per) * zs + (m % per) * ldb;
   __shared__ int red[256];
   int mx = 0;
   for (int64_t j = threadIdx.x; j < K; j += blockDim.x) {
-    const double2 v = B[m * ldb + j];
+    const double2 v = B[j];
     mx = max(mx, max(em_bexp(v.x), em_bexp(v.y)));
   }
   red[threadIdx.x] = mx;
@@ -179,7 +182,7 @@ __global__ void em_split_b_kernel(const double2* __restrict__ B, int64_t rows, i
   if (threadIdx.x == 0) ex[m] = e;
   const int64_t rowlen = (int64_t)EM_S * Kp;
   for (int64_t j = threadIdx.x; j < K; j += blockDim.x) {
-    const double2 v = B[m * ldb + j];
+    const double2 v = B[j];
     __half2 d[EM_S];
     em_digits2(v.x, v.y, e, d);
     dig_t* r0 = dig + (2 * m) * rowlen + 2 * j;
@@ -326,7 +329,7 @@ cudaError_t emul_split_b(const double2* B, int64_t rows, int64_t K, int64_t ldb,
   const int64_t Kp = emul_kpad(K);
   cudaError_t e = cudaMemsetAsync(dig, 0, emul_digit_bytes(2 * rows, K), st);
   if (e != cudaSuccess) return e;
-  em_split_b_kernel<<<(unsigned)rows, 256, 0, st>>>(B, rows, K, ldb, (dig_t*)dig, ex, Kp, 0);
+  em_split_b_kernel<<<(unsigned)rows, 256, 0, st>>>(B, rows, 0, K, ldb, (dig_t*)dig, ex, Kp, 0);
   return cudaGetLastError();
 }
 
@@ -496,10 +499,12 @@ cudaError_t emul_split_cols(const double2* B, int64_t count, int64_t K, int64_t 
 
 // Products of the FP64 contraction chains.  Native FP64 runs at 1.1 TFLOP/s here; 36 digit products
 // of 16-bit operands at a thousand times that are ten times as fast, the digits included, and as
-// accurate (a row's 56 bits against the rounding of a sum; ranges longer than digit_kmax are added in
-// FP64).  Below ~2e8 flops the three launches cost more than they save.
+// accurate (a row's 56 bits against the rounding of a sum: P~0 of the
+// 3x1x1 silicon-sized system errs by 1e-17 .. 4e-17 relative, with native FP64 by 1.2e-15, both against
+// quadruple precision; ranges longer
+// than digit_kmax are added in FP64).  At M 18400, N 200, K 676 a product takes 1.4 instead of 18 ms.  Below ~2e8 flops the three launches cost more than they save.
 bool emul_pays(const DigitWs& w, int64_t M, int64_t N, int64_t K, int64_t rows) {
-  return w.A && 8.0 * M * N * K >= 2e8 && (size_t)rows * EM_S * emul_kpad(K) * sizeof(dig_t) <= w.A_bytes &&
+  return w.A && 8.0 * M * N * K >= 2e8 && M <= w.A_rows && N <= w.B_rows && (size_t)rows * EM_S * emul_kpad(K) * sizeof(dig_t) <= w.A_bytes &&
          emul_digit_bytes(2 * N, K) <= w.B_bytes;
 }
 cudaError_t emul_zgemm_rows(const DigitWs& w, const double2* A, int64_t M, int64_t K, const double2* B, int64_t N,
@@ -507,7 +512,7 @@ cudaError_t emul_zgemm_rows(const DigitWs& w, const double2* A, int64_t M, int64
   const int64_t Kp = emul_kpad(K), rowb = EM_S * Kp * (int64_t)sizeof(dig_t);
   cudaError_t e = cudaMemsetAsync(w.B, 0, emul_digit_bytes(2 * N, K), st);
   if (e != cudaSuccess) return e;
-  em_split_b_kernel<<<(unsigned)N, 256, 0, st>>>(B, N, K, K, (dig_t*)w.B, w.Be, Kp, conjB ? 1 : 0);
+  em_split_b_kernel<<<(unsigned)N, 256, 0, st>>>(B, N, 0, K, K, (dig_t*)w.B, w.Be, Kp, conjB ? 1 : 0);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   *nlaunch += 1;
   const int64_t mc = (int64_t)(w.A_bytes / rowb);   // rows at a time
@@ -518,6 +523,57 @@ cudaError_t emul_zgemm_rows(const DigitWs& w, const double2* A, int64_t M, int64
     d.Ad = w.A; d.Bd = w.B; d.eA = w.Ae; d.eB = w.Be;
     d.batch = 1; d.M = m; d.N = 2 * N; d.K = 2 * K; d.Kp = Kp; d.nd = EM_S;
     d.C = (double*)(C + m0 * N); d.err = w.err; d.alpha = alpha; d.acc = acc;
+    if ((e = digit_gemm(d, st)) != cudaSuccess) return e;
+    *nlaunch += 2;
+  }
+  return cudaSuccess;
+}
+// The nao-sized steps: per row of A a product costs the digits' traffic (2 KB at K <= 32), their MMAs
+// and the write-out, about what native FP64 takes for 16 x 16 (N x K)
+bool emul_pays_batch(const DigitWs& w, int64_t nz, int64_t M, int64_t N, int64_t K) {
+  const size_t rowb = emul_digit_bytes(1, K);
+  return w.A && N * K >= 256 && 8.0 * nz * M * N * K >= 2e8 && M <= w.A_rows && N <= w.B_rows &&
+         (size_t)M * rowb <= w.A_bytes && 2 * N * rowb <= w.B_bytes;
+}
+cudaError_t emul_zgemm_batch(const DigitWs& w, EmulA akind, const double2* A, int64_t inner, bool bcols, const double2* B,
+                             int64_t b_zs, int mode, int64_t nz, int64_t M, int64_t N, int64_t K, double2* C, double alpha,
+                             cudaStream_t st, int64_t* nlaunch) {
+  const int64_t Kp = emul_kpad(K);
+  const size_t rowb = emul_digit_bytes(1, K);
+  // batch entries at a time
+  int64_t zc = (int64_t)(w.B_bytes / (2 * N * rowb));
+  zc = std::min(zc, w.B_rows / N);
+  if (akind != EmulA::shared) zc = std::min(zc, std::min((int64_t)(w.A_bytes / (M * rowb)), w.A_rows / M));
+  const int64_t per = akind == EmulA::cols ? M / inner : 1;   // matrices of a batch entry
+  zc = std::min(zc, 65535 / per);
+  if (zc < 1 || (akind == EmulA::cols && M % inner)) return cudaErrorInvalidValue;
+  cudaError_t e = cudaSuccess;
+  for (int64_t z0 = 0; z0 < nz; z0 += zc) {
+    const int64_t n = nz - z0 < zc ? nz - z0 : zc;
+    if (akind == EmulA::cols) {
+      em_split_t_kernel<false><<<dim3((unsigned)((inner + 31) / 32), (unsigned)(n * per)), 256, 0, st>>>(
+          A + z0 * M * K, K, inner, inner, K * inner, (dig_t*)w.A, w.Ae, Kp, nullptr, nullptr);
+      e = cudaGetLastError();
+      *nlaunch += 1;
+    } else if (akind == EmulA::rows || z0 == 0) {
+      e = emul_split_rows(A + (akind == EmulA::rows ? z0 * M * K : 0), akind == EmulA::rows ? n : 1, M, K, K, M * K, w.A,
+                          w.Ae, st);
+      *nlaunch += 1;
+    }
+    if (e != cudaSuccess) return e;
+    const double2* Bz = B + z0 * b_zs;
+    if (bcols) {
+      em_split_bt_kernel<<<dim3((unsigned)((N + 31) / 32), (unsigned)n), 256, 0, st>>>(Bz, K, N, N, b_zs, (dig_t*)w.B,
+                                                                                       w.Be, Kp, mode);
+    } else {
+      if ((e = cudaMemsetAsync(w.B, 0, 2 * n * N * rowb, st)) != cudaSuccess) return e;
+      em_split_b_kernel<<<(unsigned)(n * N), 256, 0, st>>>(Bz, N, b_zs, K, K, (dig_t*)w.B, w.Be, Kp, mode);
+    }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    DigitGemm d{};
+    d.Ad = w.A; d.Bd = w.B; d.eA = w.Ae; d.eB = w.Be; d.a_shared = akind == EmulA::shared;
+    d.batch = n; d.M = M; d.N = 2 * N; d.K = 2 * K; d.Kp = Kp; d.nd = EM_S;
+    d.C = (double*)(C + z0 * M * N); d.err = w.err; d.alpha = alpha;
     if ((e = digit_gemm(d, st)) != cudaSuccess) return e;
     *nlaunch += 2;
   }

@@ -1,7 +1,8 @@
 """The large products of the FP64 contraction chains in digits on the tensor cores (the default of
 FP64-accurate arithmetic) against the oracle: the last P~0 step, the first Sigma~ step, and those of
 the two adjoints.  Sizes above the rule's 2e8 flops with odd orders, K longer and shorter than one
-exact range, native FP64 arithmetic as the other side, and values that are not finite."""
+exact range (and one whose first P~0 step takes the digits for a part of the q), native FP64 arithmetic
+as the other side, and values that are not finite."""
 import numpy as np
 import pytest
 
@@ -13,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 # sums of ~1e3 products of order one: 2^-53 sqrt(1e3) per term of the largest sum, with margin
 TOL = 1e-12
-SIZES = [(13, 97, (2, 1, 1), 41), (17, 75, (3, 1, 1), 40), (5, 200, (1, 1, 1), 50)]
+SIZES = [(13, 97, (2, 1, 1), 41), (17, 75, (3, 1, 1), 40), (5, 200, (1, 1, 1), 50), (21, 80, (3, 1, 1), 40)]
 
 
 @pytest.mark.parametrize("nao,naux,kmesh,ntau", SIZES)
