@@ -498,13 +498,13 @@ cudaError_t emul_split_cols(const double2* B, int64_t count, int64_t K, int64_t 
 }
 
 // Products of the FP64 contraction chains.  Native FP64 runs at 1.1 TFLOP/s here; 36 digit products
-// of 16-bit operands at a thousand times that are ten times as fast, the digits included, and as
-// accurate (a row's 56 bits against the rounding of a sum: P~0 of the
-// 3x1x1 silicon-sized system errs by 1e-17 .. 4e-17 relative, with native FP64 by 1.2e-15, both against
-// quadruple precision; ranges longer
-// than digit_kmax are added in FP64).  At M 18400, N 200, K 676 a product takes 1.4 instead of 18 ms.  Below ~2e8 flops the three launches cost more than they save.
+// of 16-bit operands at a thousand times that are ten times as fast, the digits included: at M 18400,
+// N 200, K 676 1.4 instead of 18 ms.  And more accurate, a row's 56 bits against the rounding of a sum:
+// P~0 of the 3x1x1 silicon-sized system errs by 1e-17 .. 4e-17 relative, with native FP64 by 1.2e-15,
+// both against quadruple precision (ranges longer than digit_kmax are added in FP64).  Below ~2e8 flops
+// the three launches cost more than they save.
 bool emul_pays(const DigitWs& w, int64_t M, int64_t N, int64_t K, int64_t rows) {
-  return w.A && 8.0 * M * N * K >= 2e8 && M <= w.A_rows && N <= w.B_rows && (size_t)rows * EM_S * emul_kpad(K) * sizeof(dig_t) <= w.A_bytes &&
+  return w.A && 8.0 * M * N * K >= 2e8 && M <= w.A_rows && N <= w.B_rows && emul_digit_bytes(rows, K) <= w.A_bytes &&
          emul_digit_bytes(2 * N, K) <= w.B_bytes;
 }
 cudaError_t emul_zgemm_rows(const DigitWs& w, const double2* A, int64_t M, int64_t K, const double2* B, int64_t N,
