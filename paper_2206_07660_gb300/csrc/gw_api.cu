@@ -1653,9 +1653,9 @@ static gw_status polar_chain_half(gw_ctx* c, const double2* Gplus, const double2
 //   X[t][Q'][(i,a)] = sum_Q conj P~^q_Q'Q(t) V^{k,k-q}_ia(Q)         (rows (t, Q'))
 //   Y[t][i][(b,Q')] = sum_a X[t][Q'][i][a] G^{k-q}_ab(t)             (rows (i, Q'), batch t)
 //   Sigma~[t][k][i][j] += -(1/Nk) sum_(b,Q') Y[t][i][(b,Q')] V^{k-q,k}_bj(Q')
-// X is written as rows (t, i, Q') and the last step's K runs over (b, Q'), so that the
-// middle step's consecutive rows Q' are adjacent complex entries of its output (the
-// coalesced lane-per-row write-out).
+// X is written as rows (i, Q') per t in K pieces (UmmaOut) and the last step's K runs over
+// (b, Q'), so that the middle step's consecutive rows Q' are adjacent complex entries of its
+// output (the coalesced lane-per-row write-out).  Up to nao 16 small_tail takes the last two steps.
 // X's rows are scaled from P~'s row sums of moduli times max |V|; Y's from max_Q' of X's
 // bounds times the row sums of G(t).
 static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2* Psrc, double2* out, bool accumulate,
@@ -1750,7 +1750,7 @@ static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2*
         UmmaOut o{fmt, c->ePs, 0, 1, shift};
         o.naux = naux; o.nao = nao; o.nt = ntau; o.npc = npc;
         if (pair) { o.C2 = c->Xt_hi; o.C2_lo = c->Xt_lo; }
-        // output row (t, Q'), column (i, a re/im) -> X row (t, i, Q'), entry (a re/im); one X block per k
+        // output row (t, Q'), column block (i, a re/im) -> X row (i, Q') of t, piece of a; one X block per k
         CK(run_umma(c, fl1 * kn, oa, ob, nt * naux, (int)ncol, kps, kn, Xh, false, 1.0, false, ka,
                     kn > 1 ? xs_blk : 0, 1, naux, xt, 2 * (int64_t)nao, (int64_t)naux * ka, Xl, 2 * (int64_t)naux, &sc,
                     &o));
@@ -1955,10 +1955,9 @@ static gw_status sigma_chain(gw_ctx* c, const double2* Gsrc, const double2* Psrc
   const bool tc2 = tc3 && c->Xs_hi != nullptr;   // middle step on tensor cores too
   if (tc2) CK(build_gemb(c, Gsrc, nullptr));
   const size_t es = f32 ? 8 : 16;
-  if (f32) {
-    CK(to_c64(Gsrc, c->G32, (int64_t)ntau * gstep, c->st));
-    CK(to_c64(Psrc, c->P32, (int64_t)nk * ntau * na2, c->st));
-    count(2);
+  if (f32) {   // complex64 copies for the steps in FP32 (the tensor cores' operands are cut from the FP64 arrays)
+    if (!tc2) { CK(to_c64(Gsrc, c->G32, (int64_t)ntau * gstep, c->st)); count(1); }
+    if (!tc) { CK(to_c64(Psrc, c->P32, (int64_t)nk * ntau * na2, c->st)); count(1); }
     Gp = c->G32; Pp = c->P32;
   }
   // one X for (k, q, tau) and (k - q, -q, beta - tau) (see sigma_chain_half); the strided kernels
