@@ -1895,7 +1895,7 @@ extern "C" gw_status gw_screened(gw_ctx* c) {
     count(1);
     CK(cudaMemcpyAsync(c->h_scr + 16, c->dscr + 16, 16, cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
-    folded = c->h_scr[16] <= kFoldTol * c->h_scr[17];
+    folded = sym_holds(c->h_scr + 16, kFoldTol);
   }
   c->psym = folded;
   if (folded) {
@@ -2116,7 +2116,7 @@ static gw_status sigma_tau_part(gw_ctx* c) {
     count(1);
     CK(cudaMemcpyAsync(c->h_scr + 16, c->dscr + 16, 16, cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
-    c->psym = c->h_scr[16] <= kFoldTol * c->h_scr[17];
+    c->psym = sym_holds(c->h_scr + 16, kFoldTol);
   }
   gw_status s = sigma_chain(c, c->G_tau, c->P_tau, c->Stau, false, c->psym);
   c->reduce = false;

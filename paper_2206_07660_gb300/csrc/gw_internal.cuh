@@ -140,6 +140,12 @@ cudaError_t fold_check_tau(const double2* P, int64_t n2, int nt, int q0, int q1,
                            cudaStream_t st);
 cudaError_t fold_check(const double2* P, const FoldView& f, double* out, cudaStream_t st);
 
+// s = {deviation, largest value} of a symmetry check: whether the data have it to `tol`.  Data with a value
+// that is not finite (an infinite largest value would pass any deviation) do not.
+__host__ __device__ inline bool sym_holds(const double* s, double tol) {
+  return s[1] <= 1.7976931348623157e308 && s[0] <= tol * s[1];
+}
+
 struct DysonArgs {
   int nao, nk, nw;
   const double2* H0; const double2* S; const double2* Sinf; const double2* Siw; // Siw [nw][nk][nao2]

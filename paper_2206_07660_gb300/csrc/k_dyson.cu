@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(256) dyson_kernel(DysonArgs a, const double* m
   // A(-i w) = A(i w)^H with Hermitian H0, S, Sigma_inf and Sigma~(-i w) = Sigma~(i w)^H: the block
   // of a positive frequency writes both.  The first blocks take the kept frequencies (blocks that
   // return at once in front of them left the others on half of the SMs)
-  const bool sym = a.sym && a.sym[0] <= kAdjointTol * a.sym[1];
+  const bool sym = a.sym && sym_holds(a.sym, kAdjointTol);
   const int64_t nwork = sym ? (int64_t)a.nrep * a.nk : nsys;
   for (int64_t it = blockIdx.x; it < nwork; it += gridDim.x) {
     const int wi = (int)(it / a.nk), k = (int)(it - (int64_t)wi * a.nk);
@@ -146,7 +146,7 @@ __global__ void herm_dev_kernel(const double2* __restrict__ g, int n, double* ou
   put_dev(dev, mx, out);
 }
 __global__ void herm_like_kernel(double2* X, int n, const double* s) {
-  if (!(s[0] <= kAdjointTol * s[1])) return;
+  if (!sym_holds(s, kAdjointTol)) return;
   double2* x = X + (int64_t)blockIdx.x * n * n;
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
     const int i = e / n, j = e - i * n;
@@ -166,7 +166,7 @@ cudaError_t herm_like(double2* X, const double2* g, int n, int count, double* sc
 }
 
 __global__ void siw_adjoint_kernel(DysonArgs a, double2* S, const double* s) {
-  if (!(s[0] <= kAdjointTol * s[1])) return;
+  if (!sym_holds(s, kAdjointTol)) return;
   const int n = a.nao;
   const int64_t n2 = (int64_t)n * n, per = (int64_t)a.nk * n2, tot = (int64_t)a.nw * per;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {

@@ -1,0 +1,65 @@
+"""The symmetries that the folded routes rest on are looked at before they are used: data without them,
+or with a value that is not finite, take the route over every block."""
+import numpy as np
+import pytest
+
+from gpu_helpers import gpu, hermitian_noise, system
+from oracle import gw as ogw
+
+pytestmark = pytest.mark.gpu
+
+NAO, NAUX, KMESH, NTAU = 4, 18, (3, 1, 1), 14
+
+
+def _context(**kw):
+    return gpu(system(NAO, NAUX, KMESH, NTAU, 20.0, 121), **kw)
+
+
+def _fails_or_not_finite(call, result):
+    """An error of the library, or a result that shows the value."""
+    from paper_2206_07660_gb300.gw import GWError
+    try:
+        call()
+    except GWError:
+        return True
+    return not np.isfinite(result()).all()
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("q,m", [(0, 0), (1, 0), (2, NTAU - 1), (0, NTAU - 1)])
+def test_p0_iw_that_is_not_finite(value, q, m):
+    # frequencies and q-points that the fold keeps, and ones that it takes from their partners
+    sysd = system(NAO, NAUX, KMESH, NTAU, 20.0, 121)
+    st = ogw.State(sysd)
+    st.G_tau = -hermitian_noise((NTAU, 3, NAO, NAO), 0.05, 122) - 0.3 * np.eye(NAO)
+    st.sigma()
+    P0 = st.P0_iw.copy()
+    P0[q, m, 2, 3] = value
+    g = gpu(sysd)
+    g.set("P0_iw", P0)
+    assert _fails_or_not_finite(g.screened, lambda: g.get("P_iw")[q, m])
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("q,t", [(0, 0), (0, NTAU - 1), (2, 3)])
+@pytest.mark.parametrize("precision", ["fp64", "split_f16"])
+def test_p_tau_that_is_not_finite(value, q, t, precision):
+    km = ogw.KMesh(KMESH)
+    P = hermitian_noise((km.nk, NTAU, NAUX, NAUX), 0.3, 123)
+    neg = [km.index(-km.vec[i]) for i in range(km.nk)]
+    P = 0.5 * (P + np.conj(P[neg][:, ::-1]))
+    P[q, t, 1, 1] = value
+    g = _context(precision=precision)
+    g.set("G_tau", hermitian_noise((NTAU, km.nk, NAO, NAO), 0.3, 124))
+    g.set("P_tau", P)
+    assert _fails_or_not_finite(g.selfenergy_partial, lambda: g.get("Sigma_tau")[t])
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("w", [0, NTAU - 1])
+def test_sigma_iw_that_is_not_finite(value, w):
+    g = _context()
+    S = np.zeros(g.shape_of("Sigma_iw"), dtype=np.complex128)
+    S[w, 1, 2, 2] = value
+    g.set("Sigma_iw", S)
+    assert _fails_or_not_finite(g.dyson, lambda: g.get("G_iw")[w])
