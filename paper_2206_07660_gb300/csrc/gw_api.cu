@@ -297,6 +297,9 @@ static bool capturing(const gw_ctx* c) {
   cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
   return cudaStreamIsCapturing(c->st, &s) == cudaSuccess && s != cudaStreamCaptureStatusNone;
 }
+// whether the Sigma~ chain may rest on P_tau's mirror symmetry.  A caller's captured stage is replayed on a
+// P~ that is handed in later and that nothing looks at: it runs over every block.
+static inline bool psym_now(const gw_ctx* c) { return c->psym && (c->deferred || !capturing(c)); }
 // contractions on the tensor cores (the wait-timeout flag is then meaningful, and read)
 static inline bool uses_tc(const gw_ctx* c) {
   return c->cfg.contract_prec == GW_SPLIT_TF32 || c->hfmt != 0 || (c->dg.A != nullptr && !capturing(c));
@@ -1840,8 +1843,9 @@ extern "C" gw_status gw_polarization(gw_ctx* c) {
   double2* P0q = c->P0_tau + (size_t)c->q0 * ntau * na2;
   CK(polar_finish(c, c->P0_tau, red));
   // P~0(i Omega_m) = sum_j TFb[m][j] P~0(tau_j)   (Eq. P0t_to_P0w)
-  c->p0sym = fold_ready(c);
-  if (c->p0sym) {
+  const bool folded = fold_ready(c);
+  c->p0sym = folded && (c->deferred || !capturing(c));   // (a caller's capture computes nothing yet)
+  if (folded) {
     CK(fold_forward(c));
   } else {
     CK(transform(c, c->TFb, P0q, c->P_iw + (size_t)c->q0 * c->nwb * na2, c->nwb, na2, nq, (int64_t)ntau * na2,
@@ -2118,7 +2122,7 @@ static gw_status sigma_tau_part(gw_ctx* c) {
     CK(cudaStreamSynchronize(c->st));
     c->psym = sym_holds(c->h_scr + 16, kFoldTol);
   }
-  gw_status s = sigma_chain(c, c->G_tau, c->P_tau, c->Stau, false, c->psym);
+  gw_status s = sigma_chain(c, c->G_tau, c->P_tau, c->Stau, false, psym_now(c));
   c->reduce = false;
   if (s != GW_OK) return s;
   if (red) {   // Sigma~^{-k}(tau) = conj Sigma~^k(tau)
@@ -2563,7 +2567,7 @@ extern "C" gw_status gw_selfenergy_jvp(gw_ctx* c, const double* dG, const double
   if (!c->have_G) return fail(c, GW_ERR_STATE, "no Green's function yet");
   if (!c->have_P) return fail(c, GW_ERR_STATE, "no screened interaction yet");
   double2* out = (double2*)dS_tau;
-  gw_status s = sigma_chain(c, (const double2*)dG, c->P_tau, out, false, c->psym);
+  gw_status s = sigma_chain(c, (const double2*)dG, c->P_tau, out, false, psym_now(c));
   if (s == GW_OK) s = sigma_chain(c, c->G_tau, (const double2*)dP_tau, out, true, false);
   if (s == GW_OK) s = tc_check(c);
   if (s != GW_OK) return s;
@@ -2622,7 +2626,7 @@ static gw_status sc_jvp(gw_ctx* c, const double2* dSinf, const double2* dSiw, do
   if ((s = polar_chain(c, c->G_tau, c->tGtau, c->tP, true)) != GW_OK) return s;
   CK(polar_finish(c, c->tP, false));
   if ((s = gw_screened_jvp(c, (const double*)c->tP, (double*)c->tP)) != GW_OK) return s;
-  if ((s = sigma_chain(c, c->tGtau, c->P_tau, c->tS, false, c->psym)) != GW_OK) return s;
+  if ((s = sigma_chain(c, c->tGtau, c->P_tau, c->tS, false, psym_now(c))) != GW_OK) return s;
   if ((s = sigma_chain(c, c->G_tau, c->tP, c->tS, true, false)) != GW_OK) return s;
   if ((s = tc_check(c)) != GW_OK) return s;
   CK(herm_batched(c->tS, nao, (int64_t)c->ntau * nk, n2, c->st));

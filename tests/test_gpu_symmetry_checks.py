@@ -63,3 +63,46 @@ def test_sigma_iw_that_is_not_finite(value, w):
     S[w, 1, 2, 2] = value
     g.set("Sigma_iw", S)
     assert _fails_or_not_finite(g.dyson, lambda: g.get("G_iw")[w])
+
+
+@pytest.mark.parametrize("stage", ["forward", "tangent"])
+def test_captured_selfenergy_is_replayed_on_other_p_tau(stage):
+    # a stage captured after a symmetric P~ serves a P~ without the symmetry that is handed in later
+    import torch
+    km = ogw.KMesh(KMESH)
+    sysd = system(NAO, NAUX, KMESH, NTAU, 20.0, 121)
+    neg = [km.index(-km.vec[i]) for i in range(km.nk)]
+    G = hermitian_noise((NTAU, km.nk, NAO, NAO), 0.3, 125)
+    P = hermitian_noise((km.nk, NTAU, NAUX, NAUX), 0.3, 126)
+    sym = 0.5 * (P + np.conj(P[neg][:, ::-1]))
+    dG, dP = hermitian_noise(G.shape, 0.3, 127), hermitian_noise(P.shape, 0.3, 128)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        g = gpu(sysd)
+        dGd, dPd = torch.from_numpy(dG).cuda(), torch.from_numpy(dP).cuda()
+        out = {}
+
+        def run():
+            if stage == "forward":
+                g.selfenergy_partial()
+            else:
+                out["S"] = g.selfenergy_jvp(dGd, dPd)
+
+        g.set("G_tau", G)
+        g.set("P_tau", sym)
+        g.selfenergy_partial()
+        run()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            run()
+        g.set("P_tau", P)
+        graph.replay()
+        torch.cuda.synchronize()
+        got = g.get("Sigma_tau") if stage == "forward" else out["S"].cpu().numpy()
+    qs = list(range(km.nk))
+    if stage == "forward":
+        ref = ogw.selfenergy_tau(sysd["V"], G, P, km, qs=qs)
+    else:
+        ref = ogw.selfenergy_tau(sysd["V"], dG, P, km, qs=qs) + ogw.selfenergy_tau(sysd["V"], G, dP, km, qs=qs)
+    assert np.abs(got - ref).max() < 1e-12 * np.abs(ref).max()
