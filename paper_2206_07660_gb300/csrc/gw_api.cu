@@ -32,6 +32,7 @@ struct gw_ctx {
   // their own negatives (qR) and the other kept ones (qC), digits of the transforms restricted to
   // them; P_iw holds a folded P~0 / P_tau a folded P~
   bool wfold = false, p0sym = false, psym = false;
+  bool gpsym = false;   // psym after a replay of the captured iteration
   int nrep = 0, nqR = 0, nqC = 0;
   // small nao: q-points per batch of the fused P~0 chain (k_small.cu; 0: not used), k + q per (q, k)
   int zq = 0;
@@ -2892,6 +2893,8 @@ static gw_status capture_iteration(gw_ctx* c) {
   }
   const int64_t gsz = (int64_t)c->ntau * c->nk * c->n2;
   cudaStream_t keep = c->st;
+  // the symmetries of the arrays are those of before until the graph has run
+  const bool p0sym = c->p0sym, psym = c->psym;
   c->st = c->gst;
   c->deferred = true;
   gw_status s = GW_OK;
@@ -2929,6 +2932,9 @@ static gw_status capture_iteration(gw_ctx* c) {
   }
   c->deferred = false;
   c->st = keep;
+  c->gpsym = c->psym;
+  c->p0sym = p0sym;
+  c->psym = psym;
   return s;
 }
 
@@ -2936,6 +2942,7 @@ static gw_status launch_graph(gw_ctx* c) {
   CK(cudaEventRecord(c->gev[0], c->st));
   CK(cudaStreamWaitEvent(c->gst, c->gev[0], 0));
   CK(cudaGraphLaunch(c->gexec, c->gst));
+  c->psym = c->gpsym;
   g_launches += c->graph_kernels;
   CK(cudaEventRecord(c->gev[1], c->gst));
   CK(cudaStreamWaitEvent(c->st, c->gev[1], 0));

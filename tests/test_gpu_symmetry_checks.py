@@ -106,3 +106,18 @@ def test_captured_selfenergy_is_replayed_on_other_p_tau(stage):
     else:
         ref = ogw.selfenergy_tau(sysd["V"], dG, P, km, qs=qs) + ogw.selfenergy_tau(sysd["V"], G, dP, km, qs=qs)
     assert np.abs(got - ref).max() < 1e-12 * np.abs(ref).max()
+
+
+def test_capture_of_the_iteration_leaves_a_given_p_tau_unfolded():
+    # the graph is captured without being run: the P~ that is in place is still the caller's
+    km = ogw.KMesh(KMESH)
+    sysd = system(NAO, NAUX, KMESH, 24, 20.0, 129)
+    g = gpu(sysd)
+    g.iterate(1)
+    G = g.get("G_tau")
+    P = hermitian_noise((km.nk, 24, NAUX, NAUX), 0.3, 130)
+    g.set("P_tau", P)
+    g.iterate_graph(0)
+    g.selfenergy_partial()
+    ref = ogw.selfenergy_tau(sysd["V"], G, P, km, qs=list(range(km.nk)))
+    assert np.abs(g.get("Sigma_tau") - ref).max() < 1e-12 * np.abs(ref).max()
