@@ -62,12 +62,15 @@ __device__ __forceinline__ void tmem_ld8(uint32_t addr, uint32_t* r) {
 // exact double of an integer |v| < 2^51, less the bias 1.5 2^52 (one FP64 subtraction instead of
 // a conversion)
 __device__ __forceinline__ double biased(long long v) { return __longlong_as_double(v + 0x4338000000000000ll); }
-// 2^e as a double (exponents stay far inside the range; clamped); NaN with the exponent of a row that
-// is not finite (k_emul.cu: em_exponent)
-__device__ __forceinline__ double pow2d(int e) {
+// v 2^e for |v| < 2^72; NaN with the exponent of a row that is not finite (k_emul.cu: em_exponent).  An e
+// outside the normal range (rows that are tiny together) is applied in two steps, the first of them
+// exact, so that the result is the rounded product, subnormal or zero.
+__device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+__device__ __forceinline__ double scaled(double v, int e) {
+  if ((unsigned)(e + 1022) <= 2045u) return v * pow2d(e);
   if (e > 8192) return __longlong_as_double(0x7ff8000000000000ll);
-  e = e < -1022 ? -1022 : (e > 1023 ? 1023 : e);
-  return __longlong_as_double((long long)(e + 1023) << 52);
+  const int h = e < 0 ? -500 : 500;
+  return v * pow2d(h) * pow2d(max(-1022, min(1023, e - h)));
 }
 
 // ND: digits kept.  The loops over significances are compile-time so that the accumulators of
@@ -230,7 +233,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
               const double bias = 6755399441055744.0;   // 1.5 2^52
               const double h = biased(H) - bias, l = biased(L) - bias;
               const int ce = a.eB[z * a.eb_zs + ((n + u) >> a.eb_sh)];
-              v[u] = fma(h, 268435456.0, l) * pow2d(rexp + ce);
+              v[u] = scaled(fma(h, 268435456.0, l), rexp + ce);
             }
             double2* p = a.pairs ? (double2*)(a.C + off + (int64_t)(n >> 1) * a.col_s1) : (double2*)(a.C + off + n);
             if (a.scaled) {

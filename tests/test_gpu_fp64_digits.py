@@ -66,3 +66,20 @@ def test_values_that_are_not_finite_stay_so(value):
     bad = [3, ntau - 1 - 3]
     assert not np.isfinite(P0[bad]).any()
     assert np.isfinite(np.delete(P0, bad, axis=0)).all()
+
+
+@pytest.mark.parametrize("scale", [1e-146, 1e-200])
+def test_products_near_the_smallest_number(scale):
+    # rows whose product is 1e-292, or underflows: the number itself (the last bits of sums of 1e3 terms of
+    # which those below 1e-308 are lost, 1e-16 of the largest), not one of the smallest scale
+    nao, naux, kmesh, ntau = SIZES[0]
+    sysd = system(nao, naux, kmesh, ntau, 20.0, 110)
+    km = ogw.KMesh(kmesh)
+    G = hermitian_noise((ntau, km.nk, nao, nao), 0.3, 111) * scale
+    g = gpu(sysd)
+    g.set("G_tau", G)
+    g.polarization()
+    ref = ogw.polarization_tau(sysd["V"], G, km)
+    T = ogw.State(sysd).grid.TFb
+    for name, x in (("P0_tau", ref), ("P0_iw", ogw.to_matsubara(T, ref, 1))):
+        assert np.abs(g.get(name) - x).max() <= 1e-12 * np.abs(x).max(), name
