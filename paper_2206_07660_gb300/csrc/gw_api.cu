@@ -258,13 +258,18 @@ static void digit_ws(gw_ctx* c) {
   w.B_bytes = 2 * (naux * ra > n2 * rb ? naux * ra : n2 * rb);
   w.A_rows = rows * c->nao;
   w.B_rows = std::max(std::max(naux, n2), (int64_t)c->ntau * c->nao);
+  w.tiles = std::max(std::max(digit_tiles(rows, naux, 1), digit_tiles(rows, n2, 1)),
+                     digit_tiles(naux * c->nao, c->nao, c->ntau));
   w.A = &w;   // (for the rule alone)
   if (!emul_pays(w, rows, naux, n2, 1) && !emul_pays(w, rows, n2, naux, naux)) return;
   w.A = dalloc(c, w.A_bytes); w.B = dalloc(c, w.B_bytes);
   w.Ae = (int*)dalloc(c, (size_t)w.A_rows * 4); w.Be = (int*)dalloc(c, (size_t)w.B_rows * 4);
+  w.Aq = dalloc(c, w.A_bytes / 16); w.Bq = dalloc(c, w.B_bytes / 32);
+  w.tile = (int*)dalloc(c, (size_t)w.tiles * 4);
   w.err = c->info + 1;
-  if (!w.A || !w.B || !w.Ae || !w.Be) {
+  if (!w.A || !w.B || !w.Ae || !w.Be || !w.Aq || !w.Bq || !w.tile) {
     dfree(c, w.A); dfree(c, w.B); dfree(c, w.Ae); dfree(c, w.Be);
+    dfree(c, w.Aq); dfree(c, w.Bq); dfree(c, w.tile);
     return;
   }
   c->dg = w;

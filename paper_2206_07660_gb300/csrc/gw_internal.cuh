@@ -36,7 +36,10 @@ struct GettDesc {
   bool conjA, conjB;
   double2 alpha, beta;      // beta == 0 -> C is not read
   int ksplit;               // > 1: deterministic split-K through a workspace
+  // non-null (ksplit 1): only the flagged output tiles of kTileM x kTileN, [z][m tile][n tile]
+  const int* tiles;
 };
+constexpr int kTileM = 128, kTileN = 32;   // a tile of the digit products (k_digit.cu), in complex outputs
 
 // element type tags for the contraction kernels
 enum class Ty : int { C64 = 0, C128 = 1 };
@@ -321,6 +324,7 @@ struct DigitGemm {
   double alpha = 1.0;            // C = alpha A B
   bool acc = false;              // added to C
   bool a_shared = false;         // one A for the whole batch
+  const int* skip = nullptr;     // non-null: tiles [z][kTileM rows][2 kTileN columns] left alone where not 0
 };
 cudaError_t digit_gemm(const DigitGemm& d, cudaStream_t st);
 int64_t digit_kmax(int nd);
@@ -358,8 +362,17 @@ struct DigitWs {
   size_t B_bytes = 0;
   int64_t B_rows = 0;   // exponents of B (complex rows)
   int* Be = nullptr;
+  // squared moduli of both operands (2 bytes per complex entry, A_bytes / 16 and B_bytes / 32) and the
+  // tiles left to FP64 arithmetic
+  void *Aq = nullptr, *Bq = nullptr;
+  int* tile = nullptr;
+  int64_t tiles = 0;
   int* err = nullptr;
 };
+// tiles of nz products of M x N complex outputs
+inline int64_t digit_tiles(int64_t M, int64_t N, int64_t nz) {
+  return nz * ((M + kTileM - 1) / kTileM) * ((N + kTileN - 1) / kTileN);
+}
 // whether a product of M x N complex outputs over K terms takes the digits (its operands fit, and
 // it is large enough), `rows` rows of A at least at a time
 bool emul_pays(const DigitWs& w, int64_t M, int64_t N, int64_t K, int64_t rows);
@@ -381,7 +394,7 @@ cudaError_t emul_zgemm_cols(const DigitWs& w, const double2* P, int64_t nt, int6
 // whether a product of complex K fits the digit sums
 bool emul_fits(int64_t K);
 cudaError_t emul_split_rows(const double2* A, int64_t count, int64_t M, int64_t K, int64_t lda, int64_t sa,
-                            void* Ad, int* Ae, cudaStream_t st);
+                            void* Ad, int* Ae, cudaStream_t st, void* sq = nullptr);   // sq: squares (DigitWs)
 cudaError_t emul_split_cols(const double2* B, int64_t count, int64_t K, int64_t N, int64_t ldb, int64_t sb,
                             void* Bd, int* Be, cudaStream_t st);
 cudaError_t emul_cgemm_batched(const void* Ad, const int* Ae, const void* Bd, const int* Be, int64_t count,

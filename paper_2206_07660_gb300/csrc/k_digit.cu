@@ -25,7 +25,7 @@ namespace gwk {
 namespace {
 
 constexpr int DG_S = 8, DG_BETA = 7;
-constexpr int DG_BM = 128, DG_BN = 64, DG_BK = 64;
+constexpr int DG_BM = kTileM, DG_BN = 2 * kTileN, DG_BK = 64;
 constexpr uint32_t DG_A = DG_BM * DG_BK * 2, DG_B = DG_BN * DG_BK * 2;   // bytes of one plane tile
 constexpr int DG_RA = 4;                                                  // A ring
 constexpr int DG_THREADS = 192;   // warp 0 TMA, warp 1 MMA, warps 2..5 write-out
@@ -46,6 +46,7 @@ struct DigitArgs {
   const int* row_list;
   double alpha;
   int scaled, acc;      // alpha differs from 1; the output is added to
+  const int* skip;      // tiles left alone (by the order of `decode`)
   const double* Y;      // row-major: the output is I - Y + A B (identity of complex matrices with eb_sh = 1)
   int* err;
   uint32_t spin;
@@ -119,11 +120,18 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
     z = r / a.ntm;
   };
 
+  // each role walks the same tiles; the flag of the next one is read a tile ahead
+  auto flag = [&](int t) { return a.skip && t < a.ntiles ? a.skip[t] : 0; };
+
   if (warp == 0) {
     if (lane == 0) {
       uint32_t ga = 0, gb = 0;
       bool ok = true;
+      int fl = flag(blockIdx.x);
       for (int t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x) {
+        const int left = fl;
+        fl = flag(t + gridDim.x);
+        if (left) continue;
         int m0, n0, z;
         decode(t, m0, n0, z);
         const int za = a.a_batched ? z : 0, zb = a.b_batched ? z : 0;
@@ -153,7 +161,11 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
       const uint32_t idesc = (1u << 4) | ((uint32_t)(DG_BN >> 3) << 17) | ((uint32_t)(DG_BM >> 4) << 24);
       uint32_t ga = 0, gb = 0, ni = 0;
       bool ok = true;
+      int fl = flag(blockIdx.x);
       for (int t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x) {
+        const int left = fl;
+        fl = flag(t + gridDim.x);
+        if (left) continue;
         for (int rg = 0; rg < a.nranges && ok; ++rg, ++ni) {
           const int kb0 = rg * a.kbr, kb1 = min(a.nkb, kb0 + a.kbr);
           if (ni > 0 && !mbar_wait(acce, (ni - 1) & 1u, a.spin)) { atomicCAS(&s_fail, 0, 4); ok = false; break; }
@@ -190,7 +202,11 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
     const int quarter = warp & 3;
     uint32_t ni = 0;
     bool ok = true;
+    int fl = flag(blockIdx.x);
     for (int t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x) {
+      const int left = fl;
+      fl = flag(t + gridDim.x);
+      if (left) continue;
       int m0, n0, z;
       decode(t, m0, n0, z);
       const int row = m0 + quarter * 32 + lane;
@@ -331,7 +347,7 @@ cudaError_t digit_gemm(const DigitGemm& d, cudaStream_t st) {
   a.C = d.C; a.c_ld = d.N; a.c_zs = d.M * d.N;
   a.pairs = d.pairs ? 1 : 0;
   a.row_inner = d.row_inner > 0 ? d.row_inner : d.M; a.row_s1 = d.row_s1; a.col_s1 = d.col_s1; a.row_list = d.row_list;
-  a.Y = d.Y;
+  a.Y = d.Y; a.skip = d.skip;
   a.alpha = d.alpha; a.scaled = d.alpha != 1.0; a.acc = d.acc ? 1 : 0;
   a.err = d.err;
   a.spin = umma_spin();

@@ -72,15 +72,22 @@ __device__ __forceinline__ void em_digits2(double x, double y, int e, __half2* d
   d[0] = __hsub2(*(__half2*)&n, __floats2half2_rn(1536.f, 1536.f));
 }
 
-__device__ __forceinline__ __half2 em_conj(__half2 d) {   // (re, -im)
-  uint32_t n = *(uint32_t*)&d ^ 0x80000000u;
-  return *(__half2*)&n;
-}
-
 // biased exponent of |x| (0 for zero and subnormals); the row exponent e of a largest one: m < 2^e, or
 // 2^14 for a row that is not finite (its digits are zeros, its products NaN)
 __device__ __forceinline__ int em_bexp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 __device__ __forceinline__ int em_exponent(int bexp) { return bexp == 0x7ff ? 1 << 14 : bexp ? bexp - 1022 : 0; }
+// |x + iy|^2 4^(7 - e) as fp16 (row exponent e: below 2^15), at least the smallest one, 2^-38 of the largest, for
+// a value that is not zero
+__device__ __forceinline__ float em_frac(double x, int e) {
+  const int h = __double2hiint(x) & 0x7fffffff, d = (h >> 20) - 1023 + 7 - e;
+  const float f = __int_as_float(((max(d, -60) + 127) << 23) | ((h & 0xfffff) << 3));
+  return h >= (1 << 20) ? f : (__double_as_longlong(x) << 1) ? 1e-18f : 0.f;
+}
+__device__ __forceinline__ uint16_t em_square(double2 v, int e) {
+  const float x = em_frac(v.x, e), y = em_frac(v.y, e), s = x * x + y * y;
+  const uint16_t h = __half_as_ushort(__float2half_rn(s));
+  return h == 0 && s > 0.f ? 1 : h;
+}
 // doubled rows (2j, 2j + 1) of a B entry d = (Br, Bi): mode 0: A B, 1: A conj B, 2: conj (A B), 3: conj A  B
 __device__ __forceinline__ void em_double(__half2 d, int mode, __half2& r0, __half2& r1) {
   const __half2 w = __lowhigh2highlow(d);
@@ -103,7 +110,8 @@ __global__ void __launch_bounds__(256) em_split_t_kernel(const double2* __restri
                                                          int64_t ld, int64_t zs, dig_t* __restrict__ dig,
                                                          int* __restrict__ ex, int64_t Kp,
                                                          const int* __restrict__ zlist,
-                                                         const int* __restrict__ klist) {
+                                                         const int* __restrict__ klist,
+                                                         uint16_t* __restrict__ sq) {
   __shared__ double2 tile[32][33];
   __shared__ int red[8][32];
   __shared__ int es[32];
@@ -153,6 +161,7 @@ __global__ void __launch_bounds__(256) em_split_t_kernel(const double2* __restri
         dig_t* o = D + row * rowlen + 2 * j;
 #pragma unroll
         for (int i = 0; i < EM_S; ++i) *(__half2*)(o + (int64_t)i * Kp) = d[i];
+        if (sq) sq[(z * ncol + row) * (Kp / 2) + j] = em_square(v, es[rr]);
       }
     }
     __syncthreads();
@@ -163,7 +172,8 @@ __global__ void __launch_bounds__(256) em_split_t_kernel(const double2* __restri
 // m = per on in the next one, zs away): rows 2m = (Br, -Bi), 2m+1 = (Bi, Br) along the real K index 2j + c;
 // digit planes in reverse order; one exponent per complex row m.
 __global__ void em_split_b_kernel(const double2* __restrict__ B0, int64_t per, int64_t zs, int64_t K, int64_t ldb,
-                                  dig_t* __restrict__ dig, int* __restrict__ ex, int64_t Kp, int mode) {
+                                  dig_t* __restrict__ dig, int* __restrict__ ex, int64_t Kp, int mode,
+                                  uint16_t* __restrict__ sq) {
   const int64_t m = blockIdx.x;
   const double2* B = B0 + (m / per) * zs + (m % per) * ldb;
   __shared__ int red[256];
@@ -193,6 +203,8 @@ __global__ void em_split_b_kernel(const double2* __restrict__ B0, int64_t per, i
       em_double(d[i], mode, *(__half2*)(r0 + p), *(__half2*)(r1 + p));
     }
   }
+  if (sq)
+    for (int64_t j = threadIdx.x; j < Kp / 2; j += blockDim.x) sq[m * (Kp / 2) + j] = j < K ? em_square(B[j], e) : 0;
 }
 
 // A-operand digits from complex rows: row r of batch z is src[z*zs + r*ld + k],
@@ -200,7 +212,8 @@ __global__ void em_split_b_kernel(const double2* __restrict__ B0, int64_t per, i
 // written as zeros.
 __global__ void __launch_bounds__(256) em_split_r_kernel(const double2* __restrict__ src, int64_t rows, int64_t K,
                                                          int64_t ld, int64_t zs, int64_t count,
-                                                         dig_t* __restrict__ dig, int* __restrict__ ex, int64_t Kp) {
+                                                         dig_t* __restrict__ dig, int* __restrict__ ex, int64_t Kp,
+                                                         uint16_t* __restrict__ sq) {
   const int lane = threadIdx.x & 31;
   const int64_t gr = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (gr >= rows * count) return;
@@ -222,6 +235,7 @@ __global__ void __launch_bounds__(256) em_split_r_kernel(const double2* __restri
     em_digits2(v.x, v.y, e, d);
 #pragma unroll
     for (int i = 0; i < EM_S; ++i) *(__half2*)(o + (int64_t)i * Kp + 2 * k) = d[i];
+    if (sq) sq[gr * (Kp / 2) + k] = em_square(v, e);
   }
 }
 
@@ -232,7 +246,8 @@ __global__ void __launch_bounds__(256) em_split_r_kernel(const double2* __restri
 // digit writes along k); padding columns [2K, Kp) are written as zeros.
 __global__ void __launch_bounds__(256) em_split_bt_kernel(const double2* __restrict__ src, int64_t K, int64_t ncol,
                                                           int64_t ld, int64_t zs, dig_t* __restrict__ dig,
-                                                          int* __restrict__ ex, int64_t Kp, int mode) {
+                                                          int* __restrict__ ex, int64_t Kp, int mode,
+                                                          uint16_t* __restrict__ sq) {
   __shared__ double2 tile[32][33];
   __shared__ int red[8][32];
   __shared__ int es[32];
@@ -280,6 +295,7 @@ __global__ void __launch_bounds__(256) em_split_bt_kernel(const double2* __restr
           const int64_t p = (int64_t)(EM_S - 1 - i) * Kp;
           em_double(d[i], mode, *(__half2*)(r0 + p), *(__half2*)(r1 + p));
         }
+        if (sq) sq[(z * ncol + col) * (Kp / 2) + j] = em_square(v, es[rr]);
       }
     }
     __syncthreads();
@@ -329,7 +345,7 @@ cudaError_t emul_split_b(const double2* B, int64_t rows, int64_t K, int64_t ldb,
   const int64_t Kp = emul_kpad(K);
   cudaError_t e = cudaMemsetAsync(dig, 0, emul_digit_bytes(2 * rows, K), st);
   if (e != cudaSuccess) return e;
-  em_split_b_kernel<<<(unsigned)rows, 256, 0, st>>>(B, rows, 0, K, ldb, (dig_t*)dig, ex, Kp, 0);
+  em_split_b_kernel<<<(unsigned)rows, 256, 0, st>>>(B, rows, 0, K, ldb, (dig_t*)dig, ex, Kp, 0, nullptr);
   return cudaGetLastError();
 }
 
@@ -343,7 +359,7 @@ cudaError_t emul_transform(const void* Bdv, const int* Be, int64_t nrow, const d
   dig_t* Ad = (dig_t*)Adv;
   const int64_t Kp = emul_kpad(K);
   em_split_t_kernel<false><<<dim3((unsigned)((ncol + 31) / 32), 1), 256, 0, st>>>(X, K, ncol, ldx, 0, Ad, Ae, Kp,
-                                                                                   nullptr, nullptr);
+                                                                                   nullptr, nullptr, nullptr);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   DigitGemm d{};
@@ -395,8 +411,8 @@ cudaError_t emul_transform_multi(const void* Bdv, const int* Be, int64_t npair, 
   const int64_t Kp = emul_kpad((K + 1) / 2), rows = nz * ncol;
   if (nz < 1 || nz > 65535 || rows > INT32_MAX || (!real_rows && K % 2)) return cudaErrorInvalidValue;
   dim3 grid((unsigned)((ncol + 31) / 32), (unsigned)nz);
-  if (real_rows) em_split_t_kernel<true><<<grid, 256, 0, st>>>(X, K, ncol, ncol, zs, Ad, Ae, Kp, zlist, klist);
-  else em_split_t_kernel<false><<<grid, 256, 0, st>>>(X, K / 2, ncol, ncol, zs, Ad, Ae, Kp, zlist, klist);
+  if (real_rows) em_split_t_kernel<true><<<grid, 256, 0, st>>>(X, K, ncol, ncol, zs, Ad, Ae, Kp, zlist, klist, nullptr);
+  else em_split_t_kernel<false><<<grid, 256, 0, st>>>(X, K / 2, ncol, ncol, zs, Ad, Ae, Kp, zlist, klist, nullptr);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   DigitGemm d{};
@@ -481,11 +497,11 @@ cudaError_t emul_rgemm_batched(const void* Ad, const int* Ae, const void* Bd, co
 // Ad/Ae: emul_digit_bytes(M, K) and M ints per batch; Bd/Be: emul_digit_bytes(2N, K)
 // and N ints per batch.
 cudaError_t emul_split_rows(const double2* A, int64_t count, int64_t M, int64_t K, int64_t lda, int64_t sa,
-                            void* Ad, int* Ae, cudaStream_t st) {
+                            void* Ad, int* Ae, cudaStream_t st, void* sq) {
   const int64_t Kp = emul_kpad(K);
   const int64_t nb = (M * count + 7) / 8;
   if (nb > INT32_MAX) return cudaErrorInvalidValue;
-  em_split_r_kernel<<<(unsigned)nb, 256, 0, st>>>(A, M, K, lda, sa, count, (dig_t*)Ad, Ae, Kp);
+  em_split_r_kernel<<<(unsigned)nb, 256, 0, st>>>(A, M, K, lda, sa, count, (dig_t*)Ad, Ae, Kp, (uint16_t*)sq);
   return cudaGetLastError();
 }
 cudaError_t emul_split_cols(const double2* B, int64_t count, int64_t K, int64_t N, int64_t ldb, int64_t sb,
@@ -493,38 +509,156 @@ cudaError_t emul_split_cols(const double2* B, int64_t count, int64_t K, int64_t 
   const int64_t Kp = emul_kpad(K);
   if (count > 65535) return cudaErrorInvalidValue;
   em_split_bt_kernel<<<dim3((unsigned)((N + 31) / 32), (unsigned)count), 256, 0, st>>>(B, K, N, ldb, sb, (dig_t*)Bd,
-                                                                                        Be, Kp, 0);
+                                                                                        Be, Kp, 0, nullptr);
   return cudaGetLastError();
 }
 
 // Products of the FP64 contraction chains.  Native FP64 runs at 1.1 TFLOP/s here; 36 digit products
 // of 16-bit operands at a thousand times that are ten times as fast, the digits included: at M 18400,
-// N 200, K 676 1.4 instead of 18 ms.  And more accurate, a row's 56 bits against the rounding of a sum:
-// P~0 of the 3x1x1 silicon-sized system errs by 1e-17 .. 4e-17 relative, with native FP64 by 1.2e-15,
-// both against quadruple precision (ranges longer than digit_kmax are added in FP64).  Below ~2e8 flops
-// the three launches cost more than they save.
+// N 200, K 676 1.4 instead of 18 ms.  Below ~2e8 flops the launches cost more than they save.
+//
+// A row is cut to 56 bits below its largest entry, so a digit product errs by about
+// 0.46 2^-57 sqrt(2 K) of 2^(eA + eB), whatever the sum comes to, where FP64 arithmetic rounds each
+// partial sum.  With large entries meeting large ones the digits are 2 to 30 times more accurate; where
+// the two rows are graded over K in opposite directions they lose what the grading takes.  The break-even
+// lies at sums of 0.13 2^(eA + eB) (ungraded rows of 10 to 400 terms, exponential grading of one row, of
+// both, and in opposite directions by 10 to 1e4, against extended precision: with the sum's size taken
+// from S = sum_k |a_k|^2 |b_k|^2 4^-(eA + eB), random phases, the ratio of the two errors is 0.3 to 1.1 at
+// S = 1/64 and 8 at 1e-4).  range_kernel forms S of every output from 16-bit squares, at 1/144 of the digits' MMAs,
+// and leaves a tile to FP64 arithmetic where a row or a column of it has a mean S below 1/64, or an output one
+// below 2^-14: every row and every column of a product is as accurate as in FP64, and a single small output
+// keeps a relative error of 1e-14.  So are tiles with a row that is not finite.
+// (Orbitals of one scale, G of random levels, V decaying over the auxiliary index: 0 to 2 % of the tiles.)
 bool emul_pays(const DigitWs& w, int64_t M, int64_t N, int64_t K, int64_t rows) {
   return w.A && 8.0 * M * N * K >= 2e8 && M <= w.A_rows && N <= w.B_rows && emul_digit_bytes(rows, K) <= w.A_bytes &&
-         emul_digit_bytes(2 * N, K) <= w.B_bytes;
+         emul_digit_bytes(2 * N, K) <= w.B_bytes && digit_tiles(M, N, 1) <= w.tiles;
 }
+
+constexpr int kNotFinite = 1 << 14;   // em_exponent of a row that is not finite
+
+// One block per tile, eight warps of 16 rows each; S by mma.m16n8k16, K in chunks of 32 whose order within
+// a lane's 16 bytes is the same for both operands.  Q: squares, rows of Kq entries.
+__global__ void __launch_bounds__(256) range_kernel(const uint16_t* __restrict__ Aq, const uint16_t* __restrict__ Bq,
+                                                    const int* __restrict__ eA, const int* __restrict__ eB, int64_t M,
+                                                    int64_t N, int Kq, int64_t a_zs, int ntm, int ntn,
+                                                    int* __restrict__ tile) {
+  __shared__ float cs[8][kTileN];
+  __shared__ int cn[8][kTileN];
+  const int tn = blockIdx.x % ntn, r0 = blockIdx.x / ntn, z = r0 / ntm;
+  const int64_t m0 = (int64_t)(r0 % ntm) * kTileM, n0 = (int64_t)tn * kTileN;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, tg = lane & 3;
+  Aq += z * a_zs * Kq; eA += z * a_zs;
+  Bq += z * N * Kq; eB += z * N;
+  const int64_t ra = m0 + w * 16 + g, rb = ra + 8;
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  float s[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) s[i][c] = 0.f;
+  for (int k = tg * 8; k < Kq; k += 32) {
+    const uint4 x = ra < M ? *(const uint4*)(Aq + ra * Kq + k) : zero, y = rb < M ? *(const uint4*)(Aq + rb * Kq + k) : zero;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int64_t n = n0 + 8 * i + g;
+      const uint4 b = n < N ? *(const uint4*)(Bq + n * Kq + k) : zero;
+      asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+          : "+f"(s[i][0]), "+f"(s[i][1]), "+f"(s[i][2]), "+f"(s[i][3]) : "r"(x.x), "r"(y.x), "r"(x.y), "r"(y.y), "r"(b.x), "r"(b.y));
+      asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+          : "+f"(s[i][0]), "+f"(s[i][1]), "+f"(s[i][2]), "+f"(s[i][3]) : "r"(x.z), "r"(y.z), "r"(x.w), "r"(y.w), "r"(b.z), "r"(b.w));
+    }
+  }
+  // over the outputs that are not exactly zero (those are exact in digits too); the squares carry 2^28
+  constexpr float kMean = 4194304.f, kLeast = 16384.f;
+  int bad = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) bad |= s[i][c] > 0.f && s[i][c] < kLeast;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float sum = 0.f;
+    int cnt = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) { sum += s[i][2 * h + c]; cnt += s[i][2 * h + c] > 0.f; }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+      sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    }
+    if (sum < kMean * cnt) bad = 1;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      float sum = s[i][c] + s[i][2 + c];
+      int cnt = (s[i][c] > 0.f) + (s[i][2 + c] > 0.f);
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+      }
+      if (g == 0) { cs[w][8 * i + 2 * tg + c] = sum; cn[w][8 * i + 2 * tg + c] = cnt; }
+    }
+  if (threadIdx.x < kTileM && m0 + threadIdx.x < M && eA[m0 + threadIdx.x] == kNotFinite) bad = 1;
+  __syncthreads();
+  if (threadIdx.x < kTileN) {
+    float sum = 0.f;
+    int cnt = 0;
+    for (int i = 0; i < 8; ++i) { sum += cs[i][threadIdx.x]; cnt += cn[i][threadIdx.x]; }
+    if (sum < kMean * cnt || (n0 + threadIdx.x < N && eB[n0 + threadIdx.x] == kNotFinite)) bad = 1;
+  }
+  bad = __syncthreads_or(bad);
+  if (threadIdx.x == 0) tile[blockIdx.x] = bad;
+}
+
+// One launch of digit products (d: Ad .. Kp, C, alpha, acc, batch, a_shared) with the tiles that range_kernel
+// names in FP64 arithmetic (n: the same product's strides, on A and B)
+static cudaError_t ranged_gemm(const DigitWs& w, DigitGemm d, GettDesc n, const double2* A, const double2* B,
+                               cudaStream_t st, int64_t* nlaunch) {
+  const int64_t N = d.N / 2;
+  const int ntm = (int)((d.M + kTileM - 1) / kTileM), ntn = (int)((N + kTileN - 1) / kTileN);
+  const int64_t nt = digit_tiles(d.M, N, d.batch);
+  if (nt > w.tiles || nt > INT32_MAX) return cudaErrorInvalidValue;
+  range_kernel<<<(unsigned)nt, 256, 0, st>>>((const uint16_t*)w.Aq, (const uint16_t*)w.Bq, d.eA, d.eB, d.M, N,
+                                             (int)(d.Kp / 2), d.a_shared ? 0 : d.M, ntm, ntn, w.tile);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  d.skip = w.tile;
+  if ((e = digit_gemm(d, st)) != cudaSuccess) return e;
+  n.M = d.M; n.N = N; n.K = d.K / 2; n.Z = d.batch;
+  n.cm = I1(N); n.cn = I1(1); n.cz = I1(d.M * N);
+  n.alpha = make_double2(d.alpha, 0); n.beta = make_double2(d.acc ? 1 : 0, 0);
+  n.ksplit = 1;
+  n.tiles = w.tile;
+  *nlaunch += 3;
+  return gett(n, A, Ty::C128, B, Ty::C128, d.C, Ty::C128, Ty::C128, nullptr, 0, st);
+}
+
 cudaError_t emul_zgemm_rows(const DigitWs& w, const double2* A, int64_t M, int64_t K, const double2* B, int64_t N,
                             bool conjB, double2* C, double alpha, bool acc, cudaStream_t st, int64_t* nlaunch) {
   const int64_t Kp = emul_kpad(K), rowb = EM_S * Kp * (int64_t)sizeof(dig_t);
   cudaError_t e = cudaMemsetAsync(w.B, 0, emul_digit_bytes(2 * N, K), st);
   if (e != cudaSuccess) return e;
-  em_split_b_kernel<<<(unsigned)N, 256, 0, st>>>(B, N, 0, K, K, (dig_t*)w.B, w.Be, Kp, conjB ? 1 : 0);
+  em_split_b_kernel<<<(unsigned)N, 256, 0, st>>>(B, N, 0, K, K, (dig_t*)w.B, w.Be, Kp, conjB ? 1 : 0, (uint16_t*)w.Bq);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   *nlaunch += 1;
+  GettDesc n{};
+  n.am = I1(K); n.ak = I1(1); n.az = I1(0);
+  n.bn = I1(K); n.bk = I1(1); n.bz = I1(0); n.conjB = conjB;
   const int64_t mc = (int64_t)(w.A_bytes / rowb);   // rows at a time
   for (int64_t m0 = 0; m0 < M; m0 += mc) {
     const int64_t m = M - m0 < mc ? M - m0 : mc;
-    if ((e = emul_split_rows(A + m0 * K, 1, m, K, K, 0, w.A, w.Ae, st)) != cudaSuccess) return e;
+    if ((e = emul_split_rows(A + m0 * K, 1, m, K, K, 0, w.A, w.Ae, st, w.Aq)) != cudaSuccess) return e;
     DigitGemm d{};
     d.Ad = w.A; d.Bd = w.B; d.eA = w.Ae; d.eB = w.Be;
     d.batch = 1; d.M = m; d.N = 2 * N; d.K = 2 * K; d.Kp = Kp; d.nd = EM_S;
     d.C = (double*)(C + m0 * N); d.err = w.err; d.alpha = alpha; d.acc = acc;
-    if ((e = digit_gemm(d, st)) != cudaSuccess) return e;
-    *nlaunch += 2;
+    *nlaunch += 1;
+    if ((e = ranged_gemm(w, d, n, A + m0 * K, B, st, nlaunch)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
@@ -533,7 +667,7 @@ cudaError_t emul_zgemm_rows(const DigitWs& w, const double2* A, int64_t M, int64
 bool emul_pays_batch(const DigitWs& w, int64_t nz, int64_t M, int64_t N, int64_t K) {
   const size_t rowb = emul_digit_bytes(1, K);
   return w.A && N * K >= 256 && 8.0 * nz * M * N * K >= 2e8 && M <= w.A_rows && N <= w.B_rows &&
-         (size_t)M * rowb <= w.A_bytes && 2 * N * rowb <= w.B_bytes;
+         (size_t)M * rowb <= w.A_bytes && 2 * N * rowb <= w.B_bytes && digit_tiles(M, N, nz) <= w.tiles;
 }
 cudaError_t emul_zgemm_batch(const DigitWs& w, EmulA akind, const double2* A, int64_t inner, bool bcols, const double2* B,
                              int64_t b_zs, int mode, int64_t nz, int64_t M, int64_t N, int64_t K, double2* C, double alpha,
@@ -547,53 +681,68 @@ cudaError_t emul_zgemm_batch(const DigitWs& w, EmulA akind, const double2* A, in
   const int64_t per = akind == EmulA::cols ? M / inner : 1;   // matrices of a batch entry
   zc = std::min(zc, 65535 / per);
   if (zc < 1 || (akind == EmulA::cols && M % inner)) return cudaErrorInvalidValue;
+  GettDesc g{};
+  if (akind == EmulA::cols) { g.am = I2(inner, K * inner, 1); g.ak = I1(inner); }
+  else { g.am = I1(K); g.ak = I1(1); }
+  g.az = I1(akind == EmulA::shared ? 0 : M * K);
+  if (bcols) { g.bk = I1(N); g.bn = I1(1); }
+  else { g.bk = I1(1); g.bn = I1(K); }
+  g.bz = I1(b_zs);
+  g.conjA = mode >= 2; g.conjB = mode == 1 || mode == 2;
   cudaError_t e = cudaSuccess;
   for (int64_t z0 = 0; z0 < nz; z0 += zc) {
     const int64_t n = nz - z0 < zc ? nz - z0 : zc;
+    const double2* Az = akind == EmulA::shared ? A : A + z0 * M * K;
     if (akind == EmulA::cols) {
       em_split_t_kernel<false><<<dim3((unsigned)((inner + 31) / 32), (unsigned)(n * per)), 256, 0, st>>>(
-          A + z0 * M * K, K, inner, inner, K * inner, (dig_t*)w.A, w.Ae, Kp, nullptr, nullptr);
+          Az, K, inner, inner, K * inner, (dig_t*)w.A, w.Ae, Kp, nullptr, nullptr, (uint16_t*)w.Aq);
       e = cudaGetLastError();
       *nlaunch += 1;
     } else if (akind == EmulA::rows || z0 == 0) {
-      e = emul_split_rows(A + (akind == EmulA::rows ? z0 * M * K : 0), akind == EmulA::rows ? n : 1, M, K, K, M * K, w.A,
-                          w.Ae, st);
+      e = emul_split_rows(Az, akind == EmulA::rows ? n : 1, M, K, K, M * K, w.A, w.Ae, st, w.Aq);
       *nlaunch += 1;
     }
     if (e != cudaSuccess) return e;
     const double2* Bz = B + z0 * b_zs;
     if (bcols) {
       em_split_bt_kernel<<<dim3((unsigned)((N + 31) / 32), (unsigned)n), 256, 0, st>>>(Bz, K, N, N, b_zs, (dig_t*)w.B,
-                                                                                       w.Be, Kp, mode);
+                                                                                       w.Be, Kp, mode, (uint16_t*)w.Bq);
     } else {
       if ((e = cudaMemsetAsync(w.B, 0, 2 * n * N * rowb, st)) != cudaSuccess) return e;
-      em_split_b_kernel<<<(unsigned)(n * N), 256, 0, st>>>(Bz, N, b_zs, K, K, (dig_t*)w.B, w.Be, Kp, mode);
+      em_split_b_kernel<<<(unsigned)(n * N), 256, 0, st>>>(Bz, N, b_zs, K, K, (dig_t*)w.B, w.Be, Kp, mode,
+                                                           (uint16_t*)w.Bq);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     DigitGemm d{};
     d.Ad = w.A; d.Bd = w.B; d.eA = w.Ae; d.eB = w.Be; d.a_shared = akind == EmulA::shared;
     d.batch = n; d.M = M; d.N = 2 * N; d.K = 2 * K; d.Kp = Kp; d.nd = EM_S;
     d.C = (double*)(C + z0 * M * N); d.err = w.err; d.alpha = alpha;
-    if ((e = digit_gemm(d, st)) != cudaSuccess) return e;
-    *nlaunch += 2;
+    *nlaunch += 1;
+    if ((e = ranged_gemm(w, d, g, Az, Bz, st, nlaunch)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 cudaError_t emul_zgemm_cols(const DigitWs& w, const double2* P, int64_t nt, int64_t K, const double2* V, int64_t N,
                             int mode, double2* C, bool P_ready, cudaStream_t st, int64_t* nlaunch) {
   const int64_t Kp = emul_kpad(K), rowb = EM_S * Kp * (int64_t)sizeof(dig_t);
-  em_split_bt_kernel<<<dim3((unsigned)((N + 31) / 32), 1), 256, 0, st>>>(V, K, N, N, 0, (dig_t*)w.B, w.Be, Kp, mode);
+  em_split_bt_kernel<<<dim3((unsigned)((N + 31) / 32), 1), 256, 0, st>>>(V, K, N, N, 0, (dig_t*)w.B, w.Be, Kp, mode,
+                                                                         (uint16_t*)w.Bq);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   *nlaunch += 1;
   int64_t tc = (int64_t)(w.A_bytes / (K * rowb));   // matrices at a time
   if (tc > nt) tc = nt;
   if (tc < 1) return cudaErrorInvalidValue;
+  GettDesc g{};
+  g.am = I2(K, K * K, 1); g.ak = I1(K); g.az = I1(0);
+  g.bk = I1(N); g.bn = I1(1); g.bz = I1(0);
+  g.conjA = mode >= 2; g.conjB = mode == 1 || mode == 2;
   for (int64_t t0 = 0; t0 < nt; t0 += tc) {
     const int64_t n = nt - t0 < tc ? nt - t0 : tc;
+    const double2* Pt = P + t0 * K * K;
     if (!P_ready || tc < nt) {
       em_split_t_kernel<false><<<dim3((unsigned)((K + 31) / 32), (unsigned)n), 256, 0, st>>>(
-          P + t0 * K * K, K, K, K, K * K, (dig_t*)w.A, w.Ae, Kp, nullptr, nullptr);
+          Pt, K, K, K, K * K, (dig_t*)w.A, w.Ae, Kp, nullptr, nullptr, (uint16_t*)w.Aq);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       *nlaunch += 1;
     }
@@ -601,8 +750,7 @@ cudaError_t emul_zgemm_cols(const DigitWs& w, const double2* P, int64_t nt, int6
     d.Ad = w.A; d.Bd = w.B; d.eA = w.Ae; d.eB = w.Be;
     d.batch = 1; d.M = n * K; d.N = 2 * N; d.K = 2 * K; d.Kp = Kp; d.nd = EM_S;
     d.C = (double*)(C + t0 * K * N); d.err = w.err;
-    if ((e = digit_gemm(d, st)) != cudaSuccess) return e;
-    *nlaunch += 1;
+    if ((e = ranged_gemm(w, d, g, Pt, V, st, nlaunch)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }

@@ -103,7 +103,10 @@ __device__ __forceinline__ int64_t koff(uint32_t k, const KIdx& d) {
 // the complex64 gradient of Sigma~ at 2x2x1 123 -> 56 ms.
 // FP32: two blocks per SM (128 registers); with one, the loads of the next K tile were not hidden
 // (36 % of the stalls) and the 128 x 64 tile that needs them was no faster than this one.
-template <typename TA, typename TC, typename S, int TX, int TY, int TM, int TN>
+// LIST: the flagged tiles of d.tiles only.  A block looks at the flags of every gridDim.x-th tile, 256 at a
+// time: as a launch of a block per tile the 7544 empty ones of Y at nao 26, naux 200, 92 tau points took
+// longer (one block of these registers per SM) than the check of the ranges.
+template <typename TA, typename TC, typename S, int TX, int TY, int TM, int TN, bool LIST>
 __global__ void __launch_bounds__(NT, sizeof(S) == 4 ? 2 : 1) gett_kernel(const __grid_constant__ GettDesc d, const __grid_constant__ KIdx ka,
                                                   const __grid_constant__ KIdx kb_, const TA* __restrict__ A,
                                                   const TA* __restrict__ B, TC* C, typename C2<S>::t* ws) {
@@ -115,16 +118,40 @@ __global__ void __launch_bounds__(NT, sizeof(S) == 4 ? 2 : 1) gett_kernel(const 
   __shared__ typename Acc<S>::A As[BK][BM + 1];
   __shared__ CS Bs[BK][BN + 1];
   const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
-  const int64_t m0 = (int64_t)blockIdx.y * BM, n0 = (int64_t)blockIdx.x * BN;
-  const int ks = d.ksplit > 1 ? d.ksplit : 1;
+  int64_t m0 = (int64_t)blockIdx.y * BM, n0 = (int64_t)blockIdx.x * BN;
+  const int ks = LIST ? 1 : d.ksplit > 1 ? d.ksplit : 1;
   // loader geometry: which of (m,k) / (k,n) is the contiguous index
   const bool a_kfast = (d.ak.s0 == 1);
   const bool b_nfast = (d.bn.s0 == 1);
   const S sa = d.conjA ? (S)-1 : (S)1, sb = d.conjB ? (S)-1 : (S)1;
 
-  for (int64_t zz = blockIdx.z; zz < d.Z * ks; zz += gridDim.z) {
-    const int64_t z = zz / ks;
-    const int split = (int)(zz - z * ks);
+  static_assert(!LIST || (kTileM % BM == 0 && kTileN == BN), "whole tiles");
+  constexpr int SUB = LIST ? kTileM / BM : 1;
+  __shared__ int flags[LIST ? NT : 1];
+  const int64_t lmt = (d.M + kTileM - 1) / kTileM, lnt = (d.N + kTileN - 1) / kTileN, ltiles = d.Z * lmt * lnt;
+  // LIST: pass zz looks at part zz % SUB of tile (zz / SUB) gridDim.x + blockIdx.x
+  const int64_t zend = LIST ? (ltiles + gridDim.x - 1) / gridDim.x * SUB : d.Z * ks;
+  for (int64_t zz = LIST ? 0 : blockIdx.z; zz < zend; zz += LIST ? 1 : gridDim.z) {
+    if constexpr (LIST) {
+      const int at = (int)(zz % (NT * SUB));
+      if (at == 0) {
+        const int64_t t = (zz / SUB + tid) * gridDim.x + blockIdx.x;
+        const int f = t < ltiles ? d.tiles[t] : 0;
+        __syncthreads();   // the flags of before are read
+        flags[tid] = f;
+        if (!__syncthreads_or(f)) { zz += NT * SUB - 1; continue; }
+      }
+      if (!flags[at / SUB]) { zz += SUB - 1; continue; }
+    }
+    const int64_t lt = LIST ? (zz / SUB) * gridDim.x + blockIdx.x : 0;
+    const int64_t z = LIST ? lt / (lmt * lnt) : zz / ks;
+    const int split = (int)(LIST ? 0 : zz - z * ks);
+    if constexpr (LIST) {
+      const int64_t r = lt - z * (lmt * lnt);
+      m0 = r / lnt * kTileM + zz % SUB * BM;
+      n0 = r % lnt * kTileN;
+      if (m0 >= d.M) continue;
+    }
     const TA* Az = A + off2(z, d.az);
     const TA* Bz = B + off2(z, d.bz);
     int kbeg = 0, kend = (int)d.K;
@@ -315,14 +342,18 @@ size_t gett_ws_bytes(const GettDesc& d, Ty acc) {
   return (size_t)d.ksplit * d.Z * d.M * d.N * (acc == Ty::C128 ? 16 : 8);
 }
 
-template <typename TA, typename TC, typename S, int TX, int TY, int TM, int TN>
+template <typename TA, typename TC, typename S, int TX, int TY, int TM, int TN, bool LIST = false>
 static cudaError_t launch_t(const GettDesc& d, const void* A, const void* B, void* C, void* ws, cudaStream_t st) {
   constexpr int BM = TY * TM, BN = TX * TN;
   const int ks = d.ksplit > 1 ? d.ksplit : 1;
   dim3 grid((unsigned)((d.N + BN - 1) / BN), (unsigned)((d.M + BM - 1) / BM),
             (unsigned)(d.Z * ks < 65535 ? d.Z * ks : 65535));
+  if (LIST) {
+    const int64_t t = digit_tiles(d.M, d.N, d.Z);
+    grid = dim3((unsigned)(t < 304 ? t : 304));
+  }
   if (grid.y > 65535) return cudaErrorInvalidConfiguration;
-  gett_kernel<TA, TC, S, TX, TY, TM, TN><<<grid, NT, 0, st>>>(d, kidx_of(d.ak, d.K), kidx_of(d.bk, d.K), (const TA*)A,
+  gett_kernel<TA, TC, S, TX, TY, TM, TN, LIST><<<grid, NT, 0, st>>>(d, kidx_of(d.ak, d.K), kidx_of(d.bk, d.K), (const TA*)A,
                                                               (const TA*)B, (TC*)C, (typename C2<S>::t*)ws);
   return cudaGetLastError();
 }
@@ -359,6 +390,10 @@ static cudaError_t launch(const GettDesc& d, const void* A, const void* B, void*
   if (d.K > INT32_MAX - BK) return cudaErrorInvalidValue;
   constexpr bool f64 = sizeof(S) == 8;
   cudaError_t e;
+  if (d.tiles) {
+    if (!f64 || d.ksplit > 1) return cudaErrorInvalidValue;
+    return launch_t<double2, double2, double, 16, 16, 4, 2, true>(d, A, B, C, ws, st);
+  }
   switch (pick_tile(d, f64)) {
     case 1: e = launch_t<TA, TC, S, 16, 16, 4, 2>(d, A, B, C, ws, st); break;
     case 2: e = launch_t<TA, TC, S, 16, 16, 2, 4>(d, A, B, C, ws, st); break;

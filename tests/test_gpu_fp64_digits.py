@@ -83,3 +83,61 @@ def test_products_near_the_smallest_number(scale):
     T = ogw.State(sysd).grid.TFb
     for name, x in (("P0_tau", ref), ("P0_iw", ogw.to_matsubara(T, ref, 1))):
         assert np.abs(g.get(name) - x).max() <= 1e-12 * np.abs(x).max(), name
+
+
+def _scales(n, seed):
+    """Powers of two from 2^-13 to 2^13 in random order (exact, and 1e8 between the ends)."""
+    return 2.0 ** np.random.default_rng(seed).permutation(np.round(np.linspace(-13, 13, n)))
+
+
+@pytest.mark.parametrize("nao,naux,kmesh,ntau", [SIZES[0], SIZES[3]])
+def test_orbitals_and_auxiliaries_of_different_scale(nao, naux, kmesh, ntau):
+    # V carries the scales of both indices, G and P~ their inverses: FP64 arithmetic does not see them
+    # (scaling by powers of two), and the results are the unscaled ones'
+    import torch
+    sysd = system(nao, naux, kmesh, ntau, 20.0, 112)
+    km = ogw.KMesh(kmesh)
+    G, P = hermitian_noise((ntau, km.nk, nao, nao), 0.3, 113), hermitian_noise((km.nk, ntau, naux, naux), 0.3, 114)
+    V = sysd["V"]
+    rng = np.random.default_rng(115)
+    noise = lambda *s: rng.standard_normal(s) + 1j * rng.standard_normal(s)
+    Pbar, Sbar = noise(km.nk, ntau, naux, naux), noise(ntau, km.nk, nao, nao)
+    s, u = np.outer(*[_scales(nao, 116)] * 2), np.outer(*[_scales(naux, 117)] * 2)
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    ref_p0 = ogw.polarization_tau(V, G, km)
+    ref_pg = oad.polarization_vjp(V, G, km, Pbar)
+    ref_s = ogw.selfenergy_tau(V, G, P, km, qs=list(range(km.nk)))
+    ref_sg, ref_sp = oad.selfenergy_vjp(V, G, P, km, Sbar)
+    g = gpu(dict(sysd, V=V * s))
+    g.set("G_tau", G / s)
+    g.polarization()
+    assert rel(g.get("P0_tau"), ref_p0) < TOL
+    assert rel(g.polarization_vjp(dev(Pbar)).cpu().numpy() / s, ref_pg) < TOL
+    g = gpu(dict(sysd, V=V * s * np.sqrt(np.diag(u))[:, None, None]))
+    g.set("G_tau", G / s)
+    g.set("P_tau", P / u)
+    g.selfenergy_partial()
+    assert rel(g.get("Sigma_tau") / s, ref_s) < TOL
+    gb, pb = g.selfenergy_vjp(dev(Sbar / s))
+    assert rel(gb.cpu().numpy() / s, ref_sg) < TOL and rel(pb.cpu().numpy() / u, ref_sp) < TOL
+
+
+def test_one_tau_point_of_another_scale():
+    # one tau point and one auxiliary function graded: tiles in digits and in FP64 in one product
+    nao, naux, kmesh, ntau = SIZES[3]
+    sysd = system(nao, naux, kmesh, ntau, 20.0, 118)
+    km = ogw.KMesh(kmesh)
+    G = hermitian_noise((ntau, km.nk, nao, nao), 0.3, 119)
+    s = _scales(nao, 120)
+    G[7] /= np.outer(s, s)
+    G[ntau - 1 - 7] *= np.outer(s, s)
+    V = sysd["V"].copy()
+    V[:, :, 5] *= np.outer(s, s)
+    g = gpu(dict(sysd, V=V))
+    g.set("G_tau", G)
+    g.polarization()
+    got, ref = g.get("P0_tau"), ogw.polarization_tau(V, G, km)
+    for t in (0, 7, 20, ntau - 1 - 7):
+        for Q in (slice(0, 5), slice(5, 6), slice(6, None)):
+            for R in (slice(0, 5), slice(5, 6), slice(6, None)):
+                assert rel(got[:, t, Q, R], ref[:, t, Q, R]) < TOL, (t, Q, R)
