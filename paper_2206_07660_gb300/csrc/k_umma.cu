@@ -897,27 +897,29 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
               l[j] = *(const uint32_t*)&lb;
             }
           }
-          if (!rok) continue;
-          const int blk = nb >> 5, i0 = (blk / nb4) * 4, a0 = (blk - (blk / nb4) * nb4) * 4;
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            if (i0 + u < a.q_nao) {
-              const int64_t o = o1 + ((a0 >> 2) * rows + (int64_t)(i0 + u) * a.q_naux) * 8;
-              *(uint4*)((uint16_t*)a.C + o) = make_uint4(h[4 * u], h[4 * u + 1], h[4 * u + 2], h[4 * u + 3]);
-              *(uint4*)((uint16_t*)a.C_lo + o) = make_uint4(l[4 * u], l[4 * u + 1], l[4 * u + 2], l[4 * u + 3]);
-            }
-          }
-          if (a.C2) {
-            constexpr uint32_t cj = 0x80000000u;   // the sign of the imaginary piece
+          if (rok) {
+            const int blk = nb >> 5, i0 = (blk / nb4) * 4, a0 = (blk - (blk / nb4) * nb4) * 4;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-              if (a0 + u < a.q_nao) {
-                const int64_t o = o2 + ((i0 >> 2) * rows + (int64_t)(a0 + u) * a.q_naux) * 8;
-                *(uint4*)((uint16_t*)a.C2 + o) = make_uint4(h[u] ^ cj, h[4 + u] ^ cj, h[8 + u] ^ cj, h[12 + u] ^ cj);
-                *(uint4*)((uint16_t*)a.C2_lo + o) = make_uint4(l[u] ^ cj, l[4 + u] ^ cj, l[8 + u] ^ cj, l[12 + u] ^ cj);
+              if (i0 + u < a.q_nao) {
+                const int64_t o = o1 + ((a0 >> 2) * rows + (int64_t)(i0 + u) * a.q_naux) * 8;
+                *(uint4*)((uint16_t*)a.C + o) = make_uint4(h[4 * u], h[4 * u + 1], h[4 * u + 2], h[4 * u + 3]);
+                *(uint4*)((uint16_t*)a.C_lo + o) = make_uint4(l[4 * u], l[4 * u + 1], l[4 * u + 2], l[4 * u + 3]);
+              }
+            }
+            if (a.C2) {
+              constexpr uint32_t cj = 0x80000000u;   // the sign of the imaginary piece
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                if (a0 + u < a.q_nao) {
+                  const int64_t o = o2 + ((i0 >> 2) * rows + (int64_t)(a0 + u) * a.q_naux) * 8;
+                  *(uint4*)((uint16_t*)a.C2 + o) = make_uint4(h[u] ^ cj, h[4 + u] ^ cj, h[8 + u] ^ cj, h[12 + u] ^ cj);
+                  *(uint4*)((uint16_t*)a.C2_lo + o) = make_uint4(l[u] ^ cj, l[4 + u] ^ cj, l[8 + u] ^ cj, l[12 + u] ^ cj);
+                }
               }
             }
           }
+          __syncwarp();   // tcgen05.ld wants the whole warp, with the rows beyond M
         }
       } else if (a.direct && m0 + quarter * 32 < a.M) {
         // complex output written transposed (real/imag column pairs land next to each
@@ -1048,6 +1050,7 @@ __global__ void __launch_bounds__(UP_THREADS, 1)
               }
             }
           }
+          __syncwarp();   // as above
         }
       } else if (m0 + quarter * 32 < a.M) {
         for (int cb = 0; cb < BW; cb += 32) {
