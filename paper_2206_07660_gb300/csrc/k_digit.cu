@@ -68,7 +68,7 @@ __device__ __forceinline__ double biased(long long v) { return __longlong_as_dou
 // exact, so that the result is the rounded product, subnormal or zero.
 __device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 __device__ __forceinline__ double scaled(double v, int e) {
-  if ((unsigned)(e + 1022) <= 2045u) return v * pow2d(e);
+  if (abs(e) <= 1000) return v * pow2d(e);
   if (e > 8192) return __longlong_as_double(0x7ff8000000000000ll);
   const int h = e < 0 ? -500 : 500;
   return v * pow2d(h) * pow2d(max(-1022, min(1023, e - h)));
@@ -220,62 +220,71 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
       } else {
         off = z * a.c_zs + (int64_t)row * a.c_ld;
       }
+      // A tile whose scales may leave the normal range has a loop of its own.  (The clamp that was here, and more
+      // so a branch at each output, cost the write-out instructions, which it is bound by.)
+      int far = abs(rexp);
+      for (int n = n0 + lane; n < n0 + DG_BN && n < a.N; n += 32) far = max(far, abs(a.eB[z * a.eb_zs + (n >> a.eb_sh)]));
+      const bool odd = __any_sync(0xffffffffu, far > 500);
       for (int rg = 0; rg < a.nranges && ok; ++rg, ++ni) {
         if (!__all_sync(0xffffffffu, mbar_wait(accf, ni & 1u, a.spin))) { atomicCAS(&s_fail, 0, 3); ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        auto columns = [&](auto wide) {
 #pragma unroll 1
-        for (int c0 = 0; c0 < DG_BN; c0 += 8) {
-          if (n0 + c0 >= a.N) break;
-          uint32_t r[ND][8];
+          for (int c0 = 0; c0 < DG_BN; c0 += 8) {
+            if (n0 + c0 >= a.N) break;
+            uint32_t r[ND][8];
 #pragma unroll
-          for (int g = 0; g < ND; ++g)
-            tmem_ld8(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(g * DG_BN + c0), r[g]);
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          if (rok) {
+            for (int g = 0; g < ND; ++g)
+              tmem_ld8(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(g * DG_BN + c0), r[g]);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            if (rok) {
 #pragma unroll
-            for (int q = 0; q < 8; q += 2) {
-              const int n = n0 + c0 + q;
-              if (n >= a.N) break;
-              double v[2];
+              for (int q = 0; q < 8; q += 2) {
+                const int n = n0 + c0 + q;
+                if (n >= a.N) break;
+                double v[2];
 #pragma unroll
-              for (int u = 0; u < 2; ++u) {
-                long long H = 0, L = 0;
+                for (int u = 0; u < 2; ++u) {
+                  long long H = 0, L = 0;
 #pragma unroll
-                for (int g = 0; g < ND; ++g) {
-                  const long long s = (long long)__float2int_rn(__uint_as_float(r[g][q + u]));
-                  if (g < ND - 4) H += s << (DG_BETA * (ND - 5 - g));
-                  else L += s << (DG_BETA * (ND - 1 - g));
+                  for (int g = 0; g < ND; ++g) {
+                    const long long s = (long long)__float2int_rn(__uint_as_float(r[g][q + u]));
+                    if (g < ND - 4) H += s << (DG_BETA * (ND - 5 - g));
+                    else L += s << (DG_BETA * (ND - 1 - g));
+                  }
+                  const double bias = 6755399441055744.0;   // 1.5 2^52
+                  const double h = biased(H) - bias, l = biased(L) - bias;
+                  const int ce = a.eB[z * a.eb_zs + ((n + u) >> a.eb_sh)];
+                  const double x = fma(h, 268435456.0, l);
+                  v[u] = wide() ? scaled(x, rexp + ce) : x * pow2d(rexp + ce);
                 }
-                const double bias = 6755399441055744.0;   // 1.5 2^52
-                const double h = biased(H) - bias, l = biased(L) - bias;
-                const int ce = a.eB[z * a.eb_zs + ((n + u) >> a.eb_sh)];
-                v[u] = scaled(fma(h, 268435456.0, l), rexp + ce);
-              }
-              double2* p = a.pairs ? (double2*)(a.C + off + (int64_t)(n >> 1) * a.col_s1) : (double2*)(a.C + off + n);
-              if (a.scaled) {
-                v[0] *= a.alpha;
-                v[1] *= a.alpha;
-              }
-              if (rg > 0 || a.acc) {
-                const double2 o = *p;
-                v[0] += o.x;
-                v[1] += o.y;
-              } else if (a.Y) {
-                const double2 y = *(const double2*)(a.Y + off + n);
-                v[0] -= y.x;
-                v[1] -= y.y;
-                if (a.eb_sh) {
-                  if (n == 2 * row) v[0] += 1.0;
-                } else {
-                  if (n == row) v[0] += 1.0;
-                  if (n + 1 == row) v[1] += 1.0;
+                double2* p = a.pairs ? (double2*)(a.C + off + (int64_t)(n >> 1) * a.col_s1) : (double2*)(a.C + off + n);
+                if (a.scaled) {
+                  v[0] *= a.alpha;
+                  v[1] *= a.alpha;
                 }
+                if (rg > 0 || a.acc) {
+                  const double2 o = *p;
+                  v[0] += o.x;
+                  v[1] += o.y;
+                } else if (a.Y) {
+                  const double2 y = *(const double2*)(a.Y + off + n);
+                  v[0] -= y.x;
+                  v[1] -= y.y;
+                  if (a.eb_sh) {
+                    if (n == 2 * row) v[0] += 1.0;
+                  } else {
+                    if (n == row) v[0] += 1.0;
+                    if (n + 1 == row) v[1] += 1.0;
+                  }
+                }
+                *p = make_double2(v[0], v[1]);
               }
-              *p = make_double2(v[0], v[1]);
             }
+            __syncwarp();   // tcgen05.ld wants the whole warp, with the rows beyond M
           }
-          __syncwarp();   // tcgen05.ld wants the whole warp, with the rows beyond M
-        }
+        };
+        if (odd) columns([] { return true; }); else columns([] { return false; });
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
         if (lane == 0) arrive(acce);
