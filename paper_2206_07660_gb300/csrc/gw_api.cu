@@ -308,7 +308,8 @@ static bool capturing(const gw_ctx* c) {
 static inline bool psym_now(const gw_ctx* c) { return c->psym && (c->deferred || !capturing(c)); }
 // contractions on the tensor cores (the wait-timeout flag is then meaningful, and read)
 static inline bool uses_tc(const gw_ctx* c) {
-  return c->cfg.contract_prec == GW_SPLIT_TF32 || c->hfmt != 0 || (c->dg.A != nullptr && !capturing(c));
+  return c->cfg.contract_prec == GW_SPLIT_TF32 || c->hfmt != 0 ||
+         (c->cfg.contract_prec == GW_FP64 && c->dg.A != nullptr && !capturing(c));
 }
 // the time-reversal reduction applies to forward stages over the full q range
 static inline bool trs_reduce(const gw_ctx* c) { return c->trs && c->q0 == 0 && c->q1 == c->nk; }
@@ -2434,7 +2435,8 @@ static gw_status adj_c64(gw_ctx* c, gwadj::View* v) {
   return GW_OK;
 }
 
-static gw_status adj_view(gw_ctx* c, gwadj::View* v) {
+// digits: for the chains whose FP64 products take them (the FP64 adjoints)
+static gw_status adj_view(gw_ctx* c, gwadj::View* v, bool digits = false) {
   const int64_t n2 = c->n2;
   const size_t tw = (size_t)(c->ntau > c->nwf ? (c->ntau > c->nwb ? c->ntau : c->nwb) : (c->nwf > c->nwb ? c->nwf : c->nwb));
   size_t need = (size_t)c->ntau * c->naux * n2;
@@ -2453,15 +2455,17 @@ static gw_status adj_view(gw_ctx* c, gwadj::View* v) {
   v->bufA = c->adjA; v->bufB = c->adjB; v->bufC = c->adjC;
   v->st = c->st;
   v->fold = c->fold; v->kneg = c->kneg.data();
-  digit_ws(c);
-  v->dg = c->dg;
+  if (digits) {
+    digit_ws(c);
+    v->dg = c->dg;
+  }
   v->c64 = false; v->V32 = nullptr; v->G32 = nullptr; v->P32 = nullptr; v->bar32 = nullptr;
   return GW_OK;
 }
 
 // whether a product of the tensor cores gave up waiting
-static gw_status tc_check(gw_ctx* c) {
-  if (!uses_tc(c) || c->deferred) return GW_OK;
+static gw_status tc_check(gw_ctx* c, bool used) {
+  if (!used || c->deferred) return GW_OK;
   int h = 0;
   CK(cudaMemcpyAsync(c->h_scr, c->info + 1, 4, cudaMemcpyDeviceToHost, c->st));
   CK(cudaStreamSynchronize(c->st));
@@ -2474,15 +2478,15 @@ static gw_status polarization_vjp_impl(gw_ctx* c, const double* Pbar, double* Gb
   if (!c || !Pbar || !Gbar) return fail(c, GW_ERR_ARG, "null argument");
   if (!c->have_G) return fail(c, GW_ERR_STATE, "no Green's function yet");
   gwadj::View v;
-  gw_status s = adj_view(c, &v);
+  gw_status s = adj_view(c, &v, !c64);
   if (s == GW_OK && c64) s = adj_c64(c, &v);
   if (s != GW_OK) return s;
   CK(cudaMemsetAsync(Gbar, 0, (size_t)c->ntau * c->nk * c->n2 * 16, c->st));
   int64_t l = 0;
-  if (c->dg.A && !c->deferred) CK(cudaMemsetAsync(c->info + 1, 0, 4, c->st));
+  if (v.dg.A && !c->deferred) CK(cudaMemsetAsync(c->info + 1, 0, 4, c->st));
   CK(gwadj::polarization_vjp(v, (const double2*)Pbar, (double2*)Gbar, &l));
   count((int)l);
-  return c64 || !c->dg.A || capturing(c) ? GW_OK : tc_check(c);
+  return tc_check(c, v.dg.A && !capturing(c));
 }
 
 extern "C" gw_status gw_polarization_vjp(gw_ctx* c, const double* Pbar, double* Gbar) {
@@ -2497,16 +2501,16 @@ static gw_status selfenergy_vjp_impl(gw_ctx* c, const double* Sbar, double* Gbar
   if (!c->have_G) return fail(c, GW_ERR_STATE, "no Green's function yet");
   if (!c->have_P) return fail(c, GW_ERR_STATE, "no screened interaction yet");
   gwadj::View v;
-  gw_status s = adj_view(c, &v);
+  gw_status s = adj_view(c, &v, !c64);
   if (s == GW_OK && c64) s = adj_c64(c, &v);
   if (s != GW_OK) return s;
   CK(cudaMemsetAsync(Gbar, 0, (size_t)c->ntau * c->nk * c->n2 * 16, c->st));
   CK(cudaMemsetAsync(Pbar, 0, (size_t)c->nk * c->ntau * c->na2 * 16, c->st));
   int64_t l = 0;
-  if (c->dg.A && !c->deferred) CK(cudaMemsetAsync(c->info + 1, 0, 4, c->st));
+  if (v.dg.A && !c->deferred) CK(cudaMemsetAsync(c->info + 1, 0, 4, c->st));
   CK(gwadj::selfenergy_vjp(v, (const double2*)Sbar, (double2*)Gbar, (double2*)Pbar, &l));
   count((int)l);
-  return c64 || !c->dg.A || capturing(c) ? GW_OK : tc_check(c);
+  return tc_check(c, v.dg.A && !capturing(c));
 }
 
 extern "C" gw_status gw_selfenergy_vjp(gw_ctx* c, const double* Sbar, double* Gbar, double* Pbar) {
@@ -2528,7 +2532,7 @@ extern "C" gw_status gw_polarization_jvp(gw_ctx* c, const double* dG, double* dP
   double2* out = (double2*)dP0;
   gw_status s = polar_chain(c, g, c->G_tau, out, false);
   if (s == GW_OK) s = polar_chain(c, c->G_tau, g, out, true);
-  if (s == GW_OK) s = tc_check(c);
+  if (s == GW_OK) s = tc_check(c, uses_tc(c));
   if (s != GW_OK) return s;
   CK(polar_finish(c, out, false));
   return GW_OK;
@@ -2575,7 +2579,7 @@ extern "C" gw_status gw_selfenergy_jvp(gw_ctx* c, const double* dG, const double
   double2* out = (double2*)dS_tau;
   gw_status s = sigma_chain(c, (const double2*)dG, c->P_tau, out, false, psym_now(c));
   if (s == GW_OK) s = sigma_chain(c, c->G_tau, (const double2*)dP_tau, out, true, false);
-  if (s == GW_OK) s = tc_check(c);
+  if (s == GW_OK) s = tc_check(c, uses_tc(c));
   if (s != GW_OK) return s;
   CK(herm_batched(out, c->nao, (int64_t)c->ntau * c->nk, c->n2, c->st));
   count(1);
@@ -2634,7 +2638,7 @@ static gw_status sc_jvp(gw_ctx* c, const double2* dSinf, const double2* dSiw, do
   if ((s = gw_screened_jvp(c, (const double*)c->tP, (double*)c->tP)) != GW_OK) return s;
   if ((s = sigma_chain(c, c->tGtau, c->P_tau, c->tS, false, psym_now(c))) != GW_OK) return s;
   if ((s = sigma_chain(c, c->G_tau, c->tP, c->tS, true, false)) != GW_OK) return s;
-  if ((s = tc_check(c)) != GW_OK) return s;
+  if ((s = tc_check(c, uses_tc(c))) != GW_OK) return s;
   CK(herm_batched(c->tS, nao, (int64_t)c->ntau * nk, n2, c->st));
   count(1);
   // dSigma'(i w) = TFf dSigma~(tau)
