@@ -121,3 +121,22 @@ def test_capture_of_the_iteration_leaves_a_given_p_tau_unfolded():
     g.selfenergy_partial()
     ref = ogw.selfenergy_tau(sysd["V"], G, P, km, qs=list(range(km.nk)))
     assert np.abs(g.get("Sigma_tau") - ref).max() < 1e-12 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("defect", [0.0, 5e-12])
+def test_sigma_inf_of_loosely_paired_v(defect):
+    # Sigma_inf is made Hermitian where V is paired; a pairing defect that the checks accept stays in it
+    sysd = system(NAO, NAUX, KMESH, 24, 20.0, 136)
+    rng = np.random.default_rng(137)
+    V = sysd["V"] * (1.0 + defect * rng.standard_normal(sysd["V"].shape))
+    st = ogw.State(sysd)
+    G = -hermitian_noise((24, 3, NAO, NAO), 0.05, 138) - 0.3 * np.eye(NAO)
+    gamma = ogw.density_matrix(st.grid, G)
+    ref = ogw.hartree(V, gamma) + ogw.exchange(V, gamma)
+    g = gpu(dict(sysd, V=V))
+    g.set("G_tau", G)
+    g.hf()
+    got = g.get("Sigma_inf_new")
+    assert np.abs(got - ref).max() < 2e-14 * np.abs(ref).max()
+    if defect == 0.0:
+        assert np.array_equal(got, np.conj(np.swapaxes(got, -1, -2)))
