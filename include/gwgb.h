@@ -174,7 +174,10 @@ typedef struct {
  * is given by its values at the ntau points; X(i w_n) = sum_j TFf[n][j] X(tau_j)
  * at the nwf fermionic points, X(tau_j) = sum_n TBf[j][n] X(i w_n) back (and TFb,
  * TBb at the nwb bosonic points); X(beta^-) = sum_j lb[j] X(tau_j) gives the
- * density matrix.  Complex matrices are interleaved (re, im) doubles, row-major. */
+ * density matrix.  Complex matrices are interleaved (re, im) doubles, row-major.
+ * They are applied as given: the library uses their symmetries (tau -> beta - tau,
+ * i w -> -i w as complex conjugation) only where they hold to 4e-15 of the largest
+ * entry. */
 typedef struct {
   int32_t ntau;            /* tau points (must equal the config's ntau)            */
   int32_t nwf, nwb;        /* fermionic / bosonic Matsubara points                  */

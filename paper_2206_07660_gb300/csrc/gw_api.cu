@@ -488,8 +488,10 @@ static cudaError_t fold_lists(gw_ctx* c) {
 //   (w = 2; 1 for a tau point that is its own image), of the others rows T_mj;
 //   P(tau_j) = herm(sum_m c_jm P(i Omega_m)) over the kept m, c_jm = T'_jm + conj T'_j,-m (T'_jm
 //   alone for a frequency without a partner or Omega = 0).
-// wfold stays false when a matrix misses the symmetries T_m,n-1-j = conj T_mj, T_-m,j = conj T_mj.
-static cudaError_t fold_build(gw_ctx* c, const int32_t* bm) {
+// wfold stays false when a matrix misses the symmetries T_m,n-1-j = conj T_mj, T_-m,j = conj T_mj: the
+// library's own grid has them to the rounding of its inverse, amplified by its condition (2e-14 at 32 points);
+// a caller's matrices are applied as they are unless they have them to kFoldTol.
+static cudaError_t fold_build(gw_ctx* c, const int32_t* bm, bool own) {
   const int nt = c->ntau, nw = c->nwb, h = (nt + 1) / 2;
   std::vector<double2> F((size_t)nw * nt), B((size_t)nt * nw);
   cudaError_t e = cudaMemcpyAsync(F.data(), c->TFb, F.size() * 16, cudaMemcpyDeviceToHost, c->st);
@@ -509,10 +511,11 @@ static cudaError_t fold_build(gw_ctx* c, const int32_t* bm) {
       dF = std::fmax(dF, dev(f, F[(size_t)m * nt + nt - 1 - j]));
       if (part[(size_t)m] >= 0) dF = std::fmax(dF, dev(f, F[(size_t)part[(size_t)m] * nt + j]));
       dB = std::fmax(dB, dev(b, B[(size_t)(nt - 1 - j) * nw + m]));
-      mF = std::fmax(mF, mag(f));
-      mB = std::fmax(mB, mag(b));
+      mF = std::fmax(mF, std::isnan(f.x + f.y) ? INFINITY : mag(f));
+      mB = std::fmax(mB, std::isnan(b.x + b.y) ? INFINITY : mag(b));
     }
-  if (!(dF <= 1e-13 * mF && dB <= 1e-11 * mB)) return cudaSuccess;
+  const double tF = own ? 1e-13 : kFoldTol, tB = own ? 1e-11 : kFoldTol;
+  if (!std::isfinite(mF) || !std::isfinite(mB) || !(dF <= tF * mF && dB <= tB * mB)) return cudaSuccess;
   for (int m = 0; m < nw; ++m)
     if (part[(size_t)m] < 0 || bm[m] > 0) { rep.push_back(m); repn.push_back(part[(size_t)m]); }
   const int nr = c->nrep = (int)rep.size(), nr2 = (nr + 1) / 2 * 2;
@@ -1133,10 +1136,10 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
         const double2 y = F[(size_t)wpart[(size_t)w] * ntau + j];
         dev = std::fmax(dev, std::fmax(std::fabs(x.x - y.x), std::fabs(x.y + y.y)));
       }
-    c->tfadj = dev <= 1e-13 * mx;
+    c->tfadj = std::isfinite(mx) && dev <= (grid ? kFoldTol : 1e-13) * mx;
   }
   if (s == GW_OK && c->fold && c->irws) {
-    chk(fold_build(c, bm_h), "folded block");
+    chk(fold_build(c, bm_h, !grid), "folded block");
     if (s == GW_OK && c->wfold) {
       // a small system's refinement workspace may be too small for a transform's digits: all
       // kept q of it share a launch where kFoldBytes hold them

@@ -140,3 +140,32 @@ def test_sigma_inf_of_loosely_paired_v(defect):
     assert np.abs(got - ref).max() < 2e-14 * np.abs(ref).max()
     if defect == 0.0:
         assert np.array_equal(got, np.conj(np.swapaxes(got, -1, -2)))
+
+
+@pytest.mark.parametrize("matrix", ["TBb", "TFb", "TFf"])
+def test_callers_grid_is_applied_as_given(matrix):
+    # transforms that miss their mirror symmetry by more than rounding are not replaced by their symmetric part
+    sysd = system(NAO, NAUX, KMESH, NTAU, 20.0, 139)
+    st = ogw.State(sysd)
+    grid = {k: np.array(getattr(st.grid, k)) for k in ("tau", "TFf", "TBf", "TFb", "TBb", "lb")}
+    grid["fermi_n"], grid["bose_m"] = sysd["fermi_n"], sysd["bose_m"]
+    rng = np.random.default_rng(140)
+    defect = {"TBb": 4e-12, "TFb": 3e-14, "TFf": 3e-14}[matrix]
+    grid[matrix] = grid[matrix] + defect * np.abs(grid[matrix]).max() * rng.uniform(-1, 1, grid[matrix].shape)
+    import torch
+    from paper_2206_07660_gb300 import GW
+    torch.cuda.set_device(0)
+    g = GW(sysd["H0"], sysd["S"], sysd["V"], KMESH, NTAU, 20.0, n_elec=sysd["n_elec"], grid=grid, damping=1.0)
+    g.set("G_tau", -hermitian_noise((NTAU, 3, NAO, NAO), 0.05, 141) - 0.3 * np.eye(NAO))
+    g.polarization()
+    p0_tau, p0_iw = g.get("P0_tau"), g.get("P0_iw")
+    g.screened()
+    p_iw, p_tau = g.get("P_iw"), g.get("P_tau")
+    g.selfenergy()
+    for T, x, y, axis in ((grid["TFb"], p0_tau, p0_iw, 1), (grid["TBb"], p_iw, p_tau, 1),
+                          (grid["TFf"], g.get("Sigma_tau"), g.get("Sigma_iw"), 0)):
+        ref = ogw.to_matsubara(T, x, axis)
+        if axis == 1 and T is grid["TBb"]:
+            ref = ogw.herm(ref)
+        # sums of 14 terms: a few units in the last place of the largest possible one
+        assert np.abs(y - ref).max() < 1e-15 * np.abs(T).sum(1).max() * np.abs(x).max()
