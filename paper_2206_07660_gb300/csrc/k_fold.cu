@@ -229,14 +229,14 @@ __global__ void fold_check_kernel(const double2* __restrict__ P, int n, int nwb,
 __global__ void fold_check_tau_kernel(const double2* __restrict__ P, int64_t n2, int nt, int q0, int q1,
                                       const int* __restrict__ neg, double* out) {
   FoldDev f;
-  // matrices (q, t) by blocks, each pair of images once
+  // matrices (q, t) by blockIdx.x, parts of each by blockIdx.y, each pair of images once
   for (int m = blockIdx.x; m < (q1 - q0) * nt; m += gridDim.x) {
     const int q = q0 + m / nt, t = m % nt, nq = neg[q];
     const bool pair = nq >= q0 && nq < q1;
     if (pair && (nq < q || (nq == q && 2 * t > nt - 1))) continue;
     const double2* x = P + ((int64_t)q * nt + t) * n2;
     const double2* y = pair ? P + ((int64_t)nq * nt + nt - 1 - t) * n2 : nullptr;
-    for (int64_t i = threadIdx.x; i < n2; i += blockDim.x) {
+    for (int64_t i = blockIdx.y * (int64_t)blockDim.x + threadIdx.x; i < n2; i += (int64_t)gridDim.y * blockDim.x) {
       const double2 a = x[i];
       f.seen(a);
       if (y) f.pair(a, y[i], true);
@@ -248,8 +248,13 @@ cudaError_t fold_check_tau(const double2* P, int64_t n2, int nt, int q0, int q1,
                            cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(out, 0, 16, st);
   if (e != cudaSuccess) return e;
+  // Few q leave a block per matrix too few blocks (half of them images: 32 at one q and 64 tau points, 0.66 ms for
+  // 0.16 GB): parts of at least 1024 entries, for about sixteen blocks per SM.
   const int cnt = (q1 - q0) * nt;
-  fold_check_tau_kernel<<<cnt < 152 * 8 ? cnt : 152 * 8, 256, 0, st>>>(P, n2, nt, q0, q1, neg, out);
+  int64_t parts = (152 * 16 + cnt - 1) / cnt;
+  if (parts > (n2 + 1023) / 1024) parts = (n2 + 1023) / 1024;
+  const dim3 grid((unsigned)(cnt < 152 * 8 ? cnt : 152 * 8), (unsigned)(parts < 1 ? 1 : parts));
+  fold_check_tau_kernel<<<grid, 256, 0, st>>>(P, n2, nt, q0, q1, neg, out);
   return cudaGetLastError();
 }
 
