@@ -114,7 +114,8 @@ struct gw_ctx {
   // mirrored (k - q, -q, beta - tau), that one's row exponents, k - q per (q, k)
   int nao4 = 0, npc = 0;   // npc: K pieces of 8 elements per row
   float *Xb_hi = nullptr, *Xb_lo = nullptr, *Xt_hi = nullptr, *Xt_lo = nullptr;
-  size_t xb_bytes = 0;
+  size_t xb_bytes = 0, xs_bytes = 0;
+  bool xalias = false;   // Xb lies in Xs (no room for both): zeroed by each chain that takes it
   int *eY3b = nullptr, *d_kminus = nullptr;
   float *Gq_hi = nullptr, *Gq_lo = nullptr;
   int* eGq = nullptr;
@@ -223,7 +224,10 @@ static void* dalloc(gw_ctx* c, size_t bytes) {
   if (bytes == 0) bytes = 16;
   void* p = nullptr;
   if (c->cfg.dev_alloc) p = c->cfg.dev_alloc(c->cfg.alloc_user, bytes);
-  else if (cudaMalloc(&p, bytes) != cudaSuccess) p = nullptr;
+  else if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    p = nullptr;
+    cudaGetLastError();   // (an optional workspace that does not fit is not the next launch's error)
+  }
   if (p) c->owned.push_back(p);
   return p;
 }
@@ -675,8 +679,18 @@ extern "C" gw_status gw_init_grid(const gw_config* cfg, const gw_grid* grid, con
   return init_impl(cfg, grid, H0, S, V, out);
 }
 
+static gw_status init_once(const gw_config* cfg, const gw_grid* grid, const double* H0, const double* S,
+                           const double* V, gw_ctx** out, bool lean);
 static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const double* H0, const double* S,
                            const double* V, gw_ctx** out) {
+  gw_status s = init_once(cfg, grid, H0, S, V, out, false);
+  const bool half = s == GW_ERR_OOM && (cfg->contract_prec == GW_SPLIT_F16 || cfg->contract_prec == GW_SPLIT_BF16);
+  return half ? init_once(cfg, grid, H0, S, V, out, true) : s;
+}
+
+// lean: the 16-bit chains without the workspaces that only save launches and traffic
+static gw_status init_once(const gw_config* cfg, const gw_grid* grid, const double* H0, const double* S,
+                           const double* V, gw_ctx** out, bool lean) {
   if (!out) return fail(nullptr, GW_ERR_ARG, "out is NULL");
   *out = nullptr;
   if (!cfg || !H0 || !S || !V) return fail(nullptr, GW_ERR_ARG, "null config or input pointer");
@@ -845,7 +859,7 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
     if (c->pgroup < 1) c->pgroup = 1;
     size_t zb = 0;
     if (small_z_ok(nao)) c->d_kplus = (int*)need(A((size_t)nk * nk * 4));
-    if (small_z_ok(nao) && c->pgroup == nk) {
+    if (small_z_ok(nao) && c->pgroup == nk && !lean) {
       // small nao: the planes of several q-points, whose chains share their launches
       // (as many as give every SM one output tile of the last step)
       int64_t nb = (int64_t)(opt_budget(kSmallZBytes) / (2 * zk * nk));
@@ -885,7 +899,7 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
     c->Pchi = (float*)need(A(pb)); c->Pclo = (float*)need(A(pb));
     c->npc = 2 * ((2 * nao + 15) / 16);
     const size_t xk = (size_t)ntau * c->npc * naux * nao * 16;   // one plane of one k
-    c->sbatch = small_z_ok(nao) ? chain_sbatch(nk, ntau, 4 * xk, c->pbatch) : c->pbatch;
+    c->sbatch = small_z_ok(nao) && !lean ? chain_sbatch(nk, ntau, 4 * xk, c->pbatch) : c->pbatch;
     const size_t sb = (size_t)c->sbatch;
     c->vt_bytes = sb * tb;
     c->VThi = (float*)need(A(c->vt_bytes)); c->VTlo = (float*)need(A(c->vt_bytes));
@@ -899,10 +913,19 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
       c->Gq_hi = (float*)need(A(gq)); c->Gq_lo = (float*)need(A(gq));
       c->eGq = (int*)need(A(kb * ntau * 4));
     }
-    c->Xs_hi = (float*)need(A(kb * xs)); c->Xs_lo = (float*)need(A(kb * xs));
     c->xb_bytes = sb * xk + 128 * 16;   // and one tile of rows of slack
-    c->Xb_hi = (float*)need(A(c->xb_bytes)); c->Xb_lo = (float*)need(A(c->xb_bytes));
-    c->Xt_hi = (float*)A(c->xb_bytes); c->Xt_lo = (float*)A(c->xb_bytes);
+    c->xs_bytes = kb * xs;
+    if (lean) {   // X's pieces (of one chain) in the rows of the other, never longer: 32 ceil(nao / 8) bytes, 128 ceil(nao / 32)
+      c->xalias = true;
+      if (c->xs_bytes < c->xb_bytes) c->xs_bytes = c->xb_bytes;
+    }
+    c->Xs_hi = (float*)need(A(c->xs_bytes)); c->Xs_lo = (float*)need(A(c->xs_bytes));
+    if (lean) {
+      c->Xb_hi = c->Xs_hi; c->Xb_lo = c->Xs_lo;
+    } else {
+      c->Xb_hi = (float*)need(A(c->xb_bytes)); c->Xb_lo = (float*)need(A(c->xb_bytes));
+      c->Xt_hi = (float*)A(c->xb_bytes); c->Xt_lo = (float*)A(c->xb_bytes);
+    }
     c->eY3b = (int*)A((size_t)ntau * 4); c->d_kminus = (int*)A((size_t)nk * nk * 4);
     if (!c->Xt_hi || !c->Xt_lo || !c->eY3b || !c->d_kminus) {   // without room every (k, q) has its own X
       dfree(c, c->Xt_hi); dfree(c, c->Xt_lo);
@@ -1052,12 +1075,13 @@ static gw_status init_impl(const gw_config* cfg, const gw_grid* grid, const doub
       chk(cudaMemsetAsync(c->Y3hi, 0, (size_t)c->pbatch * c->y3bytes, st), "memset");
       chk(cudaMemsetAsync(c->Y3lo, 0, (size_t)c->pbatch * c->y3bytes, st), "memset");
     }
-    const size_t xs = (size_t)c->pbatch * ntau * naux * nao * c->kpadA * 2;
-    chk(cudaMemsetAsync(c->Xs_hi, 0, xs, st), "memset");
-    chk(cudaMemsetAsync(c->Xs_lo, 0, xs, st), "memset");
+    chk(cudaMemsetAsync(c->Xs_hi, 0, c->xs_bytes, st), "memset");
+    chk(cudaMemsetAsync(c->Xs_lo, 0, c->xs_bytes, st), "memset");
     // so do the pieces and the rows of the blocks' padding
-    chk(cudaMemsetAsync(c->Xb_hi, 0, c->xb_bytes, st), "memset");
-    chk(cudaMemsetAsync(c->Xb_lo, 0, c->xb_bytes, st), "memset");
+    if (!c->xalias) {
+      chk(cudaMemsetAsync(c->Xb_hi, 0, c->xb_bytes, st), "memset");
+      chk(cudaMemsetAsync(c->Xb_lo, 0, c->xb_bytes, st), "memset");
+    }
     chk(cudaMemsetAsync(c->VThi, 0, c->vt_bytes, st), "memset");
     chk(cudaMemsetAsync(c->VTlo, 0, c->vt_bytes, st), "memset");
     if (c->Xt_hi) {
@@ -1536,6 +1560,12 @@ static gw_status polar_chain(gw_ctx* c, const double2* Gplus, const double2* Gmi
 //   P[t][Q][Q'] += (s/Nk) sum_(c,b) Z[t][Q][(c,b)] conj V^{k,k+q}_cb(Q')   (group of k-points)
 // Y and Z are written by the GEMM epilogues directly as the next GEMM's 16-bit operand,
 // scaled by 2^-e with e from the bounds |Y| <= vrs(Q) max|G(t)| and |Z| <= rowsum|G(-t)| |Y|.
+// the padding columns of the chains' intermediates are zeros: again so where two chains share the memory
+static cudaError_t x_zero(gw_ctx* c) {
+  if (!c->xalias) return cudaSuccess;
+  cudaError_t e = cudaMemsetAsync(c->Xs_hi, 0, c->xs_bytes, c->st);
+  return e ? e : cudaMemsetAsync(c->Xs_lo, 0, c->xs_bytes, c->st);
+}
 static gw_status polar_chain_half(gw_ctx* c, const double2* Gplus, const double2* Gminus, double2* out,
                                   bool accumulate) {
   const int nk = c->nk, nao = c->nao, naux = c->naux, ntau = c->ntau, fmt = c->hfmt;
@@ -1556,6 +1586,7 @@ static gw_status polar_chain_half(gw_ctx* c, const double2* Gplus, const double2
   }
   CK(polar_exps(c->vQrs, c->gn, grs_m, ntau, naux, c->eY, c->eZ, st));
   count(2);
+  CK(x_zero(c));
   if (c->zq > 0 && c->fold && c->wfold) {
     // small nao: both nao-sized steps in one FP32 kernel, and the q-points of a batch in one launch of
     // each step (the kept q of polar_taus: half of the tau points for q = -q, one q of each pair)
@@ -1683,6 +1714,7 @@ static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2*
   cudaStream_t st = c->st;
   if (!c->deferred) CK(cudaMemsetAsync(c->info + 1, 0, 4, st));
   if (!accumulate) CK(cudaMemsetAsync(out, 0, (size_t)ntau * gstep * 16, st));
+  CK(x_zero(c));
   CK(g_norms(Gsrc, ntau, nk, nao, c->gn, c->gn + ntau, st));
   count(1);
   for (int k = 0; k < nk; ++k)
