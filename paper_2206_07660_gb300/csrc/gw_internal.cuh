@@ -391,7 +391,7 @@ cudaError_t emul_zgemm_batch(const DigitWs& w, EmulA akind, const double2* A, in
 // 2: conj of the whole product, 3: conj P.  P_ready: the digits of P are those of the call before.
 cudaError_t emul_zgemm_cols(const DigitWs& w, const double2* P, int64_t nt, int64_t K, const double2* V, int64_t N,
                             int mode, double2* C, bool P_ready, cudaStream_t st, int64_t* nlaunch);
-// whether a product of complex K fits the digit sums
+// whether every digit pair of a product of complex K sums exactly over all of K (the refined solve's limit)
 bool emul_fits(int64_t K);
 cudaError_t emul_split_rows(const double2* A, int64_t count, int64_t M, int64_t K, int64_t lda, int64_t sa,
                             void* Ad, int* Ae, cudaStream_t st, void* sq = nullptr);   // sq: squares (DigitWs)

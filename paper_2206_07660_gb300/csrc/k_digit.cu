@@ -337,18 +337,23 @@ int64_t digit_kmax(int nd) {
   return ((int64_t)1 << 24) / (2 * (1 << 13) + (int64_t)(nd - 2) * (1 << 12));
 }
 
+// k-blocks of a real K, those of a range, and the ranges, equally long and within digit_kmax
+static void digit_ranges(int64_t K, int nd, int* nkb, int* kbr, int* nranges) {
+  *nkb = (int)((K + DG_BK - 1) / DG_BK);
+  const int64_t km = digit_kmax(nd);
+  *kbr = K <= km ? *nkb : (int)(km / DG_BK);
+  *nranges = (*nkb + *kbr - 1) / *kbr;
+  *kbr = (*nkb + *nranges - 1) / *nranges;
+}
+
 cudaError_t digit_gemm(const DigitGemm& d, cudaStream_t st) {
   if ((d.nd != 8 && d.nd != 5) || d.K < 1 || d.M < 1 || d.N < 1 || d.N % 2 || d.Kp % DG_BK || d.K > d.Kp)
     return cudaErrorInvalidValue;
   if (d.M > INT32_MAX - DG_BM || d.N > INT32_MAX - DG_BN || d.Kp * DG_S > INT32_MAX) return cudaErrorInvalidValue;
   DigitArgs a{};
   a.M = (int)d.M; a.N = (int)d.N; a.nd = d.nd; a.Kp = d.Kp;
-  a.nkb = (int)((d.K + DG_BK - 1) / DG_BK);
+  digit_ranges(d.K, d.nd, &a.nkb, &a.kbr, &a.nranges);
   a.klast = (int)((d.K - (int64_t)(a.nkb - 1) * DG_BK + 15) / 16);
-  const int64_t km = digit_kmax(d.nd);
-  a.kbr = d.K <= km ? a.nkb : (int)(km / DG_BK);
-  a.nranges = (a.nkb + a.kbr - 1) / a.kbr;
-  a.kbr = (a.nkb + a.nranges - 1) / a.nranges;
   a.a_batched = d.batch > 1 && !d.a_shared; a.b_batched = d.batch > 1;
   a.ntm = (a.M + DG_BM - 1) / DG_BM; a.ntn = (a.N + DG_BN - 1) / DG_BN;
   const int64_t nt = (int64_t)a.ntm * a.ntn * d.batch;
@@ -371,3 +376,10 @@ cudaError_t digit_gemm(const DigitGemm& d, cudaStream_t st) {
 }
 
 }  // namespace gwk
+
+// Host-only view of the ranges of a digit product (no GPU needed): reals per k-block, k-blocks, k-blocks of a
+// range, ranges.
+extern "C" void gwdbg_digit_ranges(int64_t kreal, int nd, int* out) {
+  out[0] = gwk::DG_BK;
+  gwk::digit_ranges(kreal, nd, &out[1], &out[2], &out[3]);
+}

@@ -5,13 +5,15 @@
 // (|d_1| <= 128, |d_i| <= 64 for i > 1, balanced rounding), i.e. 56 bits.
 // Every digit is an integer that fp16 holds exactly, every digit product has at
 // most 14 bits (|d_1 d_1| <= 2^14, |d_1 d_j| <= 2^13, |d_i d_j| <= 2^12 for i, j > 1),
-// and K is limited so that the sum over the pairs of one significance i + j stays
-// <= 2^24: every partial sum is an integer below 2^24 and the tensor pipe's FP32
+// and K is taken in ranges in which the sum over the pairs of one significance i + j stays
+// <= 2^24 (k_digit.cu): every partial sum is an integer below 2^24 and the tensor pipe's FP32
 // accumulation is exact.  The product
 //   x_A x_B = 2^(eA + eB) sum_{i,j} d_i d_j 2^(-7 (i + j))
 // keeps the pairs with i + j <= S + 1 (36 of them), all in one pass over the digits
 // (k_digit.cu).  The dropped pairs and the truncated digits leave an error below
-// ~2^-54 relative to K max|A_row| max|B_col|, at the level of an FP64 GEMM.
+// ~2^-54 relative to K max|A_row| max|B_col|: the level of an FP64 GEMM where large entries meet
+// large ones, not where the rows are graded in opposite directions (the products of the contraction chains
+// look at that: range_kernel).
 //
 // Operand layout: digit planes of a row are stored one after another,
 // [row][S][Kp] (Kp = padded real K), as fp16 (tcgen05 kind::f16, FP32 accumulation);
@@ -302,11 +304,11 @@ __global__ void __launch_bounds__(256) em_split_bt_kernel(const double2* __restr
   }
 }
 
-// Launch plan of the digit-pair products for a real K extent kreal, keeping the
-// pairs with i + j <= nd + 1 of the first nd digits: launches of pairs (i, g - i),
-// i = i0..i1 (1-based digits), one significance g each, smallest contributions
-// first, each summing at most 2^24 in magnitude (exact in FP32).  Returns the number
-// of launches, or -1 when one pair alone could round (kreal > 1024).
+// Partition of the digit pairs with i + j <= nd + 1 of the first nd digits into FP32 sums over the whole of a
+// real K extent kreal that are exact: pairs (i, g - i), i = i0..i1 (1-based digits), one significance g each,
+// smallest contributions first, at most 2^24 in magnitude.  Returns their number, or -1 when one pair alone
+// could round (kreal > 1024).  digit_gemm takes K in ranges instead; what is left of this is the limit up to
+// which the screened solve is the refined one (emul_fits: naux 512).
 struct EmLaunch { int g, i0, i1; };
 static int em_plan(int64_t kreal, EmLaunch* out, int nd = EM_S) {
   if (kreal * (int64_t)(1 << 14) > ((int64_t)1 << 24) || nd < 1 || nd > EM_S) return -1;
@@ -828,9 +830,8 @@ extern "C" int gwdbg_emul_cgemm(const double2* A, const double2* B, double2* C, 
   return e ? (int)e : herr;
 }
 
-// Host-only view of the launch plan of a digit-split product (no GPU needed): writes
-// up to cap launches as (g, i0, i1) triples into out and returns their number (-1
-// when kreal is too large for exact sums).
+// Host-only view of that partition (no GPU needed): writes up to cap sums as (g, i0, i1)
+// triples into out and returns their number (-1 when kreal is too large for exact ones).
 extern "C" int gwdbg_emul_plan(int64_t kreal, int nd, int* out, int cap) {
   using namespace gwk;
   EmLaunch pl[EM_MAXL];
