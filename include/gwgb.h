@@ -92,7 +92,10 @@ enum {
                                 and the screened solve, the GW_FP64 contractions and
                                 the fp64 adjoints, instead of the defaults:
                                 FP64-accurate digit-split products on the tensor cores
-                                and a complex64 inversion refined to FP64 accuracy    */
+                                (in the contractions and adjoints only where the
+                                operands' ranges allow FP64 accuracy, looked at on the
+                                device) and a complex64 inversion refined to FP64
+                                accuracy                                              */
   GW_TRS          = 1u << 6  /* the system is time-reversal symmetric: H0(-k) =
                                 conj H0(k), S(-k) = conj S(k), V^{-k,-k'}(Q) =
                                 conj V^{kk'}(Q) (checked by gw_init unless
@@ -215,7 +218,11 @@ gw_status gw_destroy(gw_ctx* ctx);
  * GW_ERR_STATE for a quantity that neither gw_set nor the call computing it
  * has written yet (Sigma_inf, Sigma(i w), the grid and the transforms are
  * defined from gw_init on; P~0(i Omega) stops being readable once gw_screened
- * has replaced it by P~(i Omega)). */
+ * has replaced it by P~(i Omega)).
+ * A P~0(i Omega), P~(tau), Sigma_inf or Sigma~(i w) that is handed in is looked at
+ * (with H0, S and V of gw_init): one that has its mirror symmetries (Hermitian, q -> -q,
+ * beta - tau, -i w) to 4e-15 of its largest value, and no value that is not
+ * finite, is taken as having them exactly; every other one goes through as it is. */
 gw_status gw_set(gw_ctx* ctx, gw_quantity which, const void* src, size_t bytes, int on_device);
 gw_status gw_get(gw_ctx* ctx, gw_quantity which, void* dst, size_t bytes, int on_device);
 
@@ -337,7 +344,7 @@ gw_status gw_profile_read(gw_ctx* ctx, double* out6);
  * Gbar is overwritten.  Runs in fp64 whatever contract_prec is (large products
  * as exact digits on the tensor cores, without GW_FP64_NATIVE; the call then
  * synchronises, except inside a stream capture); allocates three chain buffers of
- * ntau*naux*nao^2 complex, and up to 1 GB for the digits, on first use. */
+ * ntau*naux*nao^2 complex, and up to 1.2 GB for the digits, on first use. */
 gw_status gw_polarization_vjp(gw_ctx* ctx, const double* Pbar, double* Gbar);
 
 /* Adjoint of gw_selfenergy's Sigma~(tau) (Eq. tilde_sigma2, symmetrised) with
