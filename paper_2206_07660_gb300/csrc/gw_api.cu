@@ -1731,6 +1731,10 @@ static gw_status sigma_chain_half(gw_ctx* c, const double2* Gsrc, const double2*
   const int64_t xt = (int64_t)naux * nao * npc * 8;
   float *Xh = c->Xb_hi, *Xl = c->Xb_lo;
   const int64_t xs_blk = ntau * xt, y3t = (int64_t)nao * kp3, y3_blk = ntau * y3t;
+  // (Whole blocks at every nao: where nothing is shared, GW_TRS or a P~ without the symmetry, the padded columns
+  // of this step, 2.56 times its products at nao 5, cost less than the pieces save behind it.  Sigma~ at ntau 64, split
+  // fp16, nothing shared, rows / blocks: nao 5, naux 40, 2x2x2 0.60 / 0.43 ms, nao 17, naux 136, 3x2x1 2.85 / 2.56,
+  // nao 26, naux 200, 2x2x1 3.35 / 2.95, nao 33, naux 264, 2x1x1 1.65 / 1.54.)
   const int64_t ncol = 2 * (int64_t)nb4 * nb4;
   const int64_t vt_blk = ncol * kps, w3_blk = 2 * (int64_t)nao * kp3;
   // Sigma~ += -(1/Nk) Y V over nt tau points from t0: B = V transposed, rows j, K = (b, Q') (source

@@ -92,3 +92,35 @@ def test_trs_at_any_orbital_count(nao, kmesh, precision, tol):
     g.set("P_tau", P)
     g.selfenergy_partial()
     assert rel(g.get("Sigma_tau"), ogw.selfenergy_tau(sysd["V"], G, P, km, qs=list(range(km.nk)))) < tol
+
+
+def test_fp64_stages_in_a_callers_capture():
+    # digit products, their range check and the tiles left to FP64 arithmetic, replayed on level and graded G
+    import torch
+    nao, naux, kmesh, ntau = 17, 75, (3, 1, 1), 40
+    sysd = system(nao, naux, kmesh, ntau, 20.0, 191)
+    km = ogw.KMesh(kmesh)
+    G, P = hermitian_noise((ntau, km.nk, nao, nao), 0.3, 192), hermitian_noise((km.nk, ntau, naux, naux), 0.3, 193)
+    s = 2.0 ** np.random.default_rng(194).permutation(np.round(np.linspace(-10, 10, nao)))
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        g = gpu(sysd)
+        g.set("G_tau", hermitian_noise(G.shape, 0.3, 195))
+        graphs = []
+        for stage in (g.polarization, g.selfenergy_partial):
+            g.set("P_tau", P)
+            stage()
+            torch.cuda.synchronize()
+            graphs.append(torch.cuda.CUDAGraph())
+            with torch.cuda.graph(graphs[-1], stream=stream):
+                stage()
+            g.set("P_tau", P)
+        for X in (G, G / np.outer(s, s)):
+            g.set("G_tau", X)
+            graphs[0].replay()
+            torch.cuda.synchronize()
+            assert rel(g.get("P0_tau"), ogw.polarization_tau(sysd["V"], X, km)) < TOL
+            g.set("P_tau", P)
+            graphs[1].replay()
+            torch.cuda.synchronize()
+            assert rel(g.get("Sigma_tau"), ogw.selfenergy_tau(sysd["V"], X, P, km, qs=list(range(km.nk)))) < TOL
