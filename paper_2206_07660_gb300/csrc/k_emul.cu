@@ -539,8 +539,10 @@ bool emul_pays(const DigitWs& w, int64_t M, int64_t N, int64_t K, int64_t rows) 
 constexpr int kNotFinite = 1 << 14;   // em_exponent of a row that is not finite
 
 // One block per tile, eight warps of 16 rows each; S by mma.m16n8k16, K in chunks of 32 whose order within
-// a lane's 16 bytes is the same for both operands.  Q: squares, rows of Kq entries.
-__global__ void __launch_bounds__(256) range_kernel(const uint16_t* __restrict__ Aq, const uint16_t* __restrict__ Bq,
+// a lane's 16 bytes is the same for both operands.  Bound by latency: loads, the sums of rows and columns, the barrier.
+// 64 registers (108 left two blocks per SM).  At M 18400, N 200, K 676 14 us, 71 over all of K; at M 5200, N 26,
+// K 26 and 92 tau points 25; the products themselves 1690 and 540 us.
+__global__ void __launch_bounds__(256, 4) range_kernel(const uint16_t* __restrict__ Aq, const uint16_t* __restrict__ Bq,
                                                     const int* __restrict__ eA, const int* __restrict__ eB, int64_t M,
                                                     int64_t N, int Kq, int64_t a_zs, int ntm, int ntn,
                                                     int* __restrict__ tile) {
@@ -558,7 +560,59 @@ __global__ void __launch_bounds__(256) range_kernel(const uint16_t* __restrict__
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int c = 0; c < 4; ++c) s[i][c] = 0.f;
-  for (int k = tg * 8; k < Kq; k += 32) {
+  // over the outputs that are not exactly zero (those are exact in digits too); the squares carry 2^28.
+  // whole: a zero of an output that exists counts as too small
+  constexpr float kMean = 4194304.f, kLeast = 16384.f;
+  auto judge = [&](bool whole) {
+    int bad = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const bool out = whole && (c < 2 ? ra : rb) < M && n0 + 8 * i + 2 * tg + (c & 1) < N;
+        bad |= (out || s[i][c] > 0.f) && s[i][c] < kLeast;
+      }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float sum = 0.f;
+      int cnt = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) { sum += s[i][2 * h + c]; cnt += s[i][2 * h + c] > 0.f; }
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+      }
+      if (sum < kMean * cnt) bad = 1;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        float sum = s[i][c] + s[i][2 + c];
+        int cnt = (s[i][c] > 0.f) + (s[i][2 + c] > 0.f);
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+          sum += __shfl_xor_sync(0xffffffffu, sum, o);
+          cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+        }
+        if (g == 0) { cs[w][8 * i + 2 * tg + c] = sum; cn[w][8 * i + 2 * tg + c] = cnt; }
+      }
+    if (threadIdx.x < kTileM && m0 + threadIdx.x < M && eA[m0 + threadIdx.x] == kNotFinite) bad = 1;
+    __syncthreads();
+    if (threadIdx.x < kTileN) {
+      float sum = 0.f;
+      int cnt = 0;
+      for (int i = 0; i < 8; ++i) { sum += cs[i][threadIdx.x]; cnt += cn[i][threadIdx.x]; }
+      if (sum < kMean * cnt || (n0 + threadIdx.x < N && eB[n0 + threadIdx.x] == kNotFinite)) bad = 1;
+    }
+    return __syncthreads_or(bad);
+  };
+  int bad = 1;
+  for (int k0 = 0; k0 < Kq && bad; k0 += 32) {
+    const int k = k0 + tg * 8;
     const uint4 x = ra < M ? *(const uint4*)(Aq + ra * Kq + k) : zero, y = rb < M ? *(const uint4*)(Aq + rb * Kq + k) : zero;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -569,51 +623,10 @@ __global__ void __launch_bounds__(256) range_kernel(const uint16_t* __restrict__
       asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
           : "+f"(s[i][0]), "+f"(s[i][1]), "+f"(s[i][2]), "+f"(s[i][3]) : "r"(x.z), "r"(y.z), "r"(x.w), "r"(y.w), "r"(b.z), "r"(b.w));
     }
+    // the terms are not negative: a tile whose first 32 or 128 already suffice at every output needs no others
+    const bool last = k0 + 32 >= Kq;
+    if (k0 == 0 || k0 == 96 || last) bad = judge(!last);
   }
-  // over the outputs that are not exactly zero (those are exact in digits too); the squares carry 2^28
-  constexpr float kMean = 4194304.f, kLeast = 16384.f;
-  int bad = 0;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) bad |= s[i][c] > 0.f && s[i][c] < kLeast;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    float sum = 0.f;
-    int cnt = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int c = 0; c < 2; ++c) { sum += s[i][2 * h + c]; cnt += s[i][2 * h + c] > 0.f; }
-#pragma unroll
-    for (int o = 1; o < 4; o <<= 1) {
-      sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    }
-    if (sum < kMean * cnt) bad = 1;
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      float sum = s[i][c] + s[i][2 + c];
-      int cnt = (s[i][c] > 0.f) + (s[i][2 + c] > 0.f);
-#pragma unroll
-      for (int o = 4; o < 32; o <<= 1) {
-        sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-      }
-      if (g == 0) { cs[w][8 * i + 2 * tg + c] = sum; cn[w][8 * i + 2 * tg + c] = cnt; }
-    }
-  if (threadIdx.x < kTileM && m0 + threadIdx.x < M && eA[m0 + threadIdx.x] == kNotFinite) bad = 1;
-  __syncthreads();
-  if (threadIdx.x < kTileN) {
-    float sum = 0.f;
-    int cnt = 0;
-    for (int i = 0; i < 8; ++i) { sum += cs[i][threadIdx.x]; cnt += cn[i][threadIdx.x]; }
-    if (sum < kMean * cnt || (n0 + threadIdx.x < N && eB[n0 + threadIdx.x] == kNotFinite)) bad = 1;
-  }
-  bad = __syncthreads_or(bad);
   if (threadIdx.x == 0) tile[blockIdx.x] = bad;
 }
 
